@@ -3,12 +3,14 @@
 Argument marshalling only: every function takes torch CUDA tensors (device
 memory and streams are PyTorch's job), checks dtypes, passes raw pointers to the
 entry point of the same name and raises :class:`SpqtError` on a non-zero status.
-No arithmetic of the method happens in Python and there is no CPU fallback: if
+The per-token calls and the conversions do this in a native module
+(``csrc/spqt_python.cpp``), the rest through ctypes.  No arithmetic of the method happens in Python and there is no CPU fallback: if
 ``libspqt.so`` has not been built, the first call raises.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from dataclasses import dataclass
 
@@ -16,6 +18,7 @@ import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libspqt.so")
+NATIVE_PATH = os.path.join(_HERE, "_native.so")
 
 EXPORTS = (
     "spqt_status_string", "spqt_version", "spqt_packed_sizes", "spqt_pack", "spqt_unpack",
@@ -24,6 +27,7 @@ EXPORTS = (
 )
 
 _lib = None
+_native = None
 
 
 class SpqtError(RuntimeError):
@@ -103,6 +107,21 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+def native():
+    """The native marshalling of the per-token calls (``csrc/spqt_python.cpp``), loaded once."""
+    global _native
+    if _native is None:
+        lib()
+        spec = importlib.util.spec_from_file_location(__package__ + "._native", NATIVE_PATH) if os.path.exists(NATIVE_PATH) else None
+        if spec is None:
+            raise RuntimeError("_native.so is missing: build it with `python -m paper_2511_04477_b200.build`")
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        module.set_error(SpqtError)
+        _native = module
+    return _native
+
+
 def status_string(status: int) -> str:
     return lib().spqt_status_string(int(status)).decode()
 
@@ -172,17 +191,8 @@ def new_workspace(m: int, n: int, bits: int = 4, group: int = 128, device=None) 
 
 
 def spqt_pack(W: torch.Tensor, bits: int = 4, group: int = 128, stream=None) -> Packed:
-    if W.dim() != 2 or W.stride(1) != 1:
-        raise ValueError("W must be 2-D with unit column stride")
-    if not W.is_cuda or W.dtype != torch.float16:
-        raise TypeError("W must be a CUDA float16 tensor")
-    m, n = W.shape
-    sz = spqt_packed_sizes(m, n, bits, group)
-    codes = torch.empty(sz.codes_bytes, dtype=torch.uint8, device=W.device)
-    scale_zero = torch.empty(sz.scale_zero_bytes // 2, dtype=torch.float16, device=W.device)
-    _ok(lib().spqt_pack(W.data_ptr(), m, n, W.stride(0), bits, group, codes.data_ptr(),
-                        scale_zero.data_ptr(), _stream(stream)), "spqt_pack")
-    return Packed(codes, scale_zero, m, n, bits, group)
+    codes, scale_zero = native().pack(W, bits, group, stream)
+    return Packed(codes, scale_zero, W.shape[0], W.shape[1], bits, group)
 
 
 def spqt_unpack(p: Packed, stream=None) -> torch.Tensor:
@@ -195,31 +205,12 @@ def spqt_unpack(p: Packed, stream=None) -> torch.Tensor:
 def spqt_sparsify(x: torch.Tensor, t: float, idx: torch.Tensor = None, count: torch.Tensor = None,
                   stream=None):
     """-> (idx int32[n] of which the first count[0] entries are valid, count int32[1]), both on the device."""
-    n = x.numel()
-    if idx is None:
-        idx = torch.empty(max(n, 1), dtype=torch.int32, device=x.device)
-    if count is None:
-        count = torch.empty(1, dtype=torch.int32, device=x.device)
-    if idx.numel() < n:
-        raise ValueError("idx must hold n entries")
-    _ok(lib().spqt_sparsify(_dev(x, torch.float16, "x"), n, float(t), _dev(idx, torch.int32, "idx"),
-                            _dev(count, torch.int32, "count"), _stream(stream)), "spqt_sparsify")
-    return idx, count
+    return native().sparsify(x, t, idx, count, stream)
 
 
 def spqt_sparse_gemv(p: Packed, x: torch.Tensor, idx: torch.Tensor, count: torch.Tensor,
                      workspace: torch.Tensor, y: torch.Tensor = None, stream=None) -> torch.Tensor:
-    if y is None:
-        y = torch.empty(p.m, dtype=torch.float16, device=x.device)
-    if x.numel() != p.n or y.numel() != p.m:
-        raise ValueError("x must have n entries and y m entries")
-    _ok(lib().spqt_sparse_gemv(
-        _dev(p.codes, torch.uint8, "codes"), _dev(p.scale_zero, torch.float16, "scale_zero"),
-        p.m, p.n, p.bits, p.group,
-        _dev(x, torch.float16, "x"), _dev(idx, torch.int32, "idx"), _dev(count, torch.int32, "count"),
-        _dev(y, torch.float16, "y"), _dev(workspace, torch.uint8, "workspace"), workspace.numel(),
-        _stream(stream)), "spqt_sparse_gemv")
-    return y
+    return native().sparse_gemv(p, x, idx, count, workspace, y, stream)
 
 
 def spqt_sparse_gemv_static(p: Packed, x: torch.Tensor, idx: torch.Tensor, count: torch.Tensor,
@@ -240,35 +231,12 @@ def spqt_sparse_gemv_static(p: Packed, x: torch.Tensor, idx: torch.Tensor, count
 def spqt_sparsify_gemv(p: Packed, x: torch.Tensor, t: float, workspace: torch.Tensor,
                        idx: torch.Tensor = None, count: torch.Tensor = None, y: torch.Tensor = None, stream=None):
     """Index collection and sparse GEMV in one launch -> (y, idx, count)."""
-    if idx is None:
-        idx = torch.empty(p.n, dtype=torch.int32, device=x.device)
-    if count is None:
-        count = torch.empty(1, dtype=torch.int32, device=x.device)
-    if y is None:
-        y = torch.empty(p.m, dtype=torch.float16, device=x.device)
-    if x.numel() != p.n or y.numel() != p.m or idx.numel() < p.n:
-        raise ValueError("x and idx must have n entries and y m entries")
-    _ok(lib().spqt_sparsify_gemv(
-        _dev(p.codes, torch.uint8, "codes"), _dev(p.scale_zero, torch.float16, "scale_zero"),
-        p.m, p.n, p.bits, p.group,
-        _dev(x, torch.float16, "x"), float(t), _dev(idx, torch.int32, "idx"), _dev(count, torch.int32, "count"),
-        _dev(y, torch.float16, "y"), _dev(workspace, torch.uint8, "workspace"), workspace.numel(),
-        _stream(stream)), "spqt_sparsify_gemv")
-    return y, idx, count
+    return native().sparsify_gemv(p, x, t, workspace, idx, count, y, stream)
 
 
 def spqt_dense_gemv(p: Packed, x: torch.Tensor, workspace: torch.Tensor, y: torch.Tensor = None,
                     stream=None) -> torch.Tensor:
-    if y is None:
-        y = torch.empty(p.m, dtype=torch.float16, device=x.device)
-    if x.numel() != p.n or y.numel() != p.m:
-        raise ValueError("x must have n entries and y m entries")
-    _ok(lib().spqt_dense_gemv(
-        _dev(p.codes, torch.uint8, "codes"), _dev(p.scale_zero, torch.float16, "scale_zero"),
-        p.m, p.n, p.bits, p.group,
-        _dev(x, torch.float16, "x"), _dev(y, torch.float16, "y"),
-        _dev(workspace, torch.uint8, "workspace"), workspace.numel(), _stream(stream)), "spqt_dense_gemv")
-    return y
+    return native().dense_gemv(p, x, workspace, y, stream)
 
 
 class HostLinear:
@@ -326,7 +294,7 @@ class HostStep:
         _ok(lib().spqt_host_step_create(ctypes.cast(arr, ctypes.c_void_p), len(self.hs), ctypes.byref(self.handle)), "spqt_host_step_create")
 
     def launch(self, stream=None) -> None:
-        _ok(lib().spqt_host_step_launch(self.handle, _stream(stream)), "spqt_host_step_launch")
+        native().host_step_launch(self.handle.value, stream)
 
     def close(self) -> None:
         if self.handle:
@@ -368,41 +336,14 @@ def new_gemm_small_workspace(p: Packed) -> torch.Tensor:
     return torch.zeros(int(out.value), dtype=torch.uint8, device=p.codes.device)
 
 
-def _batch(p: Packed, X: torch.Tensor, Y: torch.Tensor):
-    if X.dim() != 2 or X.stride(1) != 1 or X.shape[1] != p.n or not (1 <= X.shape[0] <= 8):
-        raise ValueError("X must be [batch <= 8][n] with unit column stride")
-    if Y is None:
-        Y = torch.empty((X.shape[0], p.m), dtype=torch.float16, device=X.device)
-    if Y.dtype != torch.float16 or X.dtype != torch.float16 or not X.is_cuda or not Y.is_cuda:
-        raise TypeError("X and Y must be CUDA float16 tensors")
-    if Y.shape != (X.shape[0], p.m) or Y.stride(1) != 1:
-        raise ValueError("Y must be [batch][m] with unit column stride")
-    return Y
-
-
 def spqt_sparse_gemm_small(p: Packed, X: torch.Tensor, t: float, workspace: torch.Tensor, idx: torch.Tensor = None,
                            count: torch.Tensor = None, Y: torch.Tensor = None, stream=None):
     """2..8 decode rows over the union of their active sets -> (Y [batch][m], idx, count)."""
-    Y = _batch(p, X, Y)
-    if idx is None:
-        idx = torch.empty(p.n, dtype=torch.int32, device=X.device)
-    if count is None:
-        count = torch.empty(1, dtype=torch.int32, device=X.device)
-    _ok(lib().spqt_sparse_gemm_small(
-        _dev(p.codes, torch.uint8, "codes"), _dev(p.scale_zero, torch.float16, "scale_zero"), p.m, p.n, p.bits, p.group,
-        X.data_ptr(), X.stride(0), X.shape[0], float(t), _dev(idx, torch.int32, "idx"), _dev(count, torch.int32, "count"),
-        Y.data_ptr(), Y.stride(0), _dev(workspace, torch.uint8, "workspace"), workspace.numel(), _stream(stream)),
-        "spqt_sparse_gemm_small")
-    return Y, idx, count
+    return native().sparse_gemm_small(p, X, t, workspace, idx, count, Y, stream)
 
 
 def spqt_dense_gemm_small(p: Packed, X: torch.Tensor, workspace: torch.Tensor, Y: torch.Tensor = None, stream=None):
-    Y = _batch(p, X, Y)
-    _ok(lib().spqt_dense_gemm_small(
-        _dev(p.codes, torch.uint8, "codes"), _dev(p.scale_zero, torch.float16, "scale_zero"), p.m, p.n, p.bits, p.group,
-        X.data_ptr(), X.stride(0), X.shape[0], Y.data_ptr(), Y.stride(0),
-        _dev(workspace, torch.uint8, "workspace"), workspace.numel(), _stream(stream)), "spqt_dense_gemm_small")
-    return Y
+    return native().dense_gemm_small(p, X, workspace, Y, stream)
 
 
 @dataclass
@@ -469,15 +410,7 @@ def spqt_kq_packed_sizes(m: int, n: int):
 
 
 def spqt_kq_pack(W: torch.Tensor, stream=None) -> KqPacked:
-    if W.dim() != 2 or W.stride(1) != 1:
-        raise ValueError("W must be 2-D with unit column stride")
-    if not W.is_cuda or W.dtype != torch.float16:
-        raise TypeError("W must be a CUDA float16 tensor")
-    m, n = W.shape
-    rb, _ = spqt_kq_packed_sizes(m, n)
-    records = torch.empty(rb, dtype=torch.uint8, device=W.device)
-    _ok(lib().spqt_kq_pack(W.data_ptr(), m, n, W.stride(0), records.data_ptr(), _stream(stream)), "spqt_kq_pack")
-    return KqPacked(records, m, n)
+    return KqPacked(native().kqw_pack(W, 4, stream, "spqt_kq_pack"), W.shape[0], W.shape[1])
 
 
 def spqt_kqw_packed_sizes(m: int, n: int, bits: int):
@@ -488,35 +421,16 @@ def spqt_kqw_packed_sizes(m: int, n: int, bits: int):
 
 def spqt_kqw_pack(W: torch.Tensor, bits: int, stream=None) -> KqPacked:
     """The two-level format with 2-, 4-, 5-, 6- or 8-bit codes."""
-    if W.dim() != 2 or W.stride(1) != 1:
-        raise ValueError("W must be 2-D with unit column stride")
-    if not W.is_cuda or W.dtype != torch.float16:
-        raise TypeError("W must be a CUDA float16 tensor")
-    m, n = W.shape
-    rb, _ = spqt_kqw_packed_sizes(m, n, bits)
-    records = torch.empty(rb, dtype=torch.uint8, device=W.device)
-    _ok(lib().spqt_kqw_pack(W.data_ptr(), m, n, W.stride(0), bits, records.data_ptr(), _stream(stream)), "spqt_kqw_pack")
-    return KqPacked(records, m, n, bits)
+    return KqPacked(native().kqw_pack(W, bits, stream, "spqt_kqw_pack"), W.shape[0], W.shape[1], bits)
 
 
 def spqt_kqw_sparse_gemv(p: KqPacked, x: torch.Tensor, idx: torch.Tensor, count: torch.Tensor, workspace: torch.Tensor,
                          y: torch.Tensor = None, stream=None) -> torch.Tensor:
-    if y is None:
-        y = torch.empty(p.m, dtype=torch.float16, device=x.device)
-    _ok(lib().spqt_kqw_sparse_gemv(
-        _dev(p.records, torch.uint8, "records"), p.m, p.n, p.bits, _dev(x, torch.float16, "x"),
-        _dev(idx, torch.int32, "idx"), _dev(count, torch.int32, "count"), _dev(y, torch.float16, "y"),
-        _dev(workspace, torch.uint8, "workspace"), workspace.numel(), _stream(stream)), "spqt_kqw_sparse_gemv")
-    return y
+    return native().kqw_gemv(p, x, idx, count, workspace, y, stream, "spqt_kqw_sparse_gemv")
 
 
 def spqt_kqw_dense_gemv(p: KqPacked, x: torch.Tensor, workspace: torch.Tensor, y: torch.Tensor = None, stream=None) -> torch.Tensor:
-    if y is None:
-        y = torch.empty(p.m, dtype=torch.float16, device=x.device)
-    _ok(lib().spqt_kqw_dense_gemv(
-        _dev(p.records, torch.uint8, "records"), p.m, p.n, p.bits, _dev(x, torch.float16, "x"), _dev(y, torch.float16, "y"),
-        _dev(workspace, torch.uint8, "workspace"), workspace.numel(), _stream(stream)), "spqt_kqw_dense_gemv")
-    return y
+    return native().kqw_gemv(p, x, None, None, workspace, y, stream, "spqt_kqw_dense_gemv")
 
 
 def new_kq_workspace(p: KqPacked) -> torch.Tensor:
@@ -527,22 +441,11 @@ def new_kq_workspace(p: KqPacked) -> torch.Tensor:
 
 def spqt_kq_sparse_gemv(p: KqPacked, x: torch.Tensor, idx: torch.Tensor, count: torch.Tensor, workspace: torch.Tensor,
                         y: torch.Tensor = None, stream=None) -> torch.Tensor:
-    if y is None:
-        y = torch.empty(p.m, dtype=torch.float16, device=x.device)
-    _ok(lib().spqt_kq_sparse_gemv(
-        _dev(p.records, torch.uint8, "records"), p.m, p.n, _dev(x, torch.float16, "x"), _dev(idx, torch.int32, "idx"),
-        _dev(count, torch.int32, "count"), _dev(y, torch.float16, "y"), _dev(workspace, torch.uint8, "workspace"),
-        workspace.numel(), _stream(stream)), "spqt_kq_sparse_gemv")
-    return y
+    return native().kqw_gemv(p, x, idx, count, workspace, y, stream, "spqt_kq_sparse_gemv")
 
 
 def spqt_kq_dense_gemv(p: KqPacked, x: torch.Tensor, workspace: torch.Tensor, y: torch.Tensor = None, stream=None) -> torch.Tensor:
-    if y is None:
-        y = torch.empty(p.m, dtype=torch.float16, device=x.device)
-    _ok(lib().spqt_kq_dense_gemv(
-        _dev(p.records, torch.uint8, "records"), p.m, p.n, _dev(x, torch.float16, "x"), _dev(y, torch.float16, "y"),
-        _dev(workspace, torch.uint8, "workspace"), workspace.numel(), _stream(stream)), "spqt_kq_dense_gemv")
-    return y
+    return native().kqw_gemv(p, x, None, None, workspace, y, stream, "spqt_kq_dense_gemv")
 
 
 def spqt_rowwise_thresholded_gemv(p: RowwisePacked, x: torch.Tensor, t: float, y: torch.Tensor = None, stream=None) -> torch.Tensor:
