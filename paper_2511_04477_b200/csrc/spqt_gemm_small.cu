@@ -1,19 +1,18 @@
 // Small batch (2..8 decode rows at once: beams, speculative tokens): the sparse product over the UNION
-// of the rows' active sets, and its dense twin.  Every active block is fetched once for the whole
-// batch and its codes are extracted once; only the FMAs are repeated per row, so the byte and the
-// integer-instruction cost per row falls with the batch size.
+// of the rows' active sets, and its dense twin.  Every active block is fetched once for the whole batch.
 //
-//   sparsify_rows_kernel    (spqt_sparsify.cu) one CTA; "active" = |X[b][k]| > t in at least one row b.
-//   gemm_small_kernel       grid (S, R): CTA (s, r) takes the s-th of S equal slices of the union list
-//                           for block-row r; its 8 warps take the slice's chunks of 32 entries in turn,
-//                           each with three chunk buffers (the next chunks' copies fly during the
-//                           arithmetic).  Lane e of a chunk holds entry e: it loads the entry's column,
-//                           its (scale, zero) pair and the batch's x values and writes the packed
-//                           multiplier pairs of every row; then the warp does the dequantize-FMA work,
-//                           four rows per pass.  Partial sums go warp -> CTA (shared memory) -> block-row
-//                           (fp32 partials in the workspace, arrive-only counter, the last CTA adds them
-//                           in slice order: bit-reproducible).
-// Batches of 5..8 rows run as two passes of up to four rows over the same union list.
+//   sparsify_rows_kernel    (spqt_sparsify.cu) "active" = |X[b][k]| > t in at least one row b; leaves the list and,
+//                           list entry after list entry, the rows' x values (gathered once, not once per block-row).
+//   gemm_small_kernel       a thread-block cluster of S CTAs of 8 warps per block-row; CTA s takes the s-th of S equal
+//                           slices of the list, every warp a contiguous part of it, streamed through its own ring of
+//                           chunks of 32 entries (cp.async).  Lane e of a chunk holds entry e: it multiplies the
+//                           batch's x values by the entry's scale and leaves them as fp16 pairs for the tensor cores
+//                           (spqt_mma.cuh), which take the codes as they are.  At the end the warps' sums meet in
+//                           shared memory and the CTAs' sums in one another's, added in a fixed order.
+//
+// What bounds it: instruction issue around the code stream (270 warp instructions per chunk), then the fixed cost of a
+// launch.  The batch is the N = 8 side of the matrix instructions, so the instruction count hardly grows with the
+// rows (the packed-FMA form before it paid 64 FMAs per chunk and row and two passes from five rows up).
 #include <cstddef>
 
 #include "spqt_common.cuh"
@@ -22,322 +21,422 @@ namespace spqt {
 constexpr unsigned long long kWaitNs = 1000000000ull;
 }
 #include "spqt_gemv_device.cuh"
+#include "spqt_mma.cuh"
 
 namespace spqt {
 
-constexpr int kSmallWarps = 8;
+constexpr int kSmallWarps = 8;      // warps of a CTA
 constexpr int kSmallThreads = kSmallWarps * 32;
-constexpr int kSmallRows = 4;      // batch rows per pass at most (a pass of one or two rows keeps two sets of sums)
-constexpr int kSmallMaxSplit = 8;  // slices per block-row at most
-constexpr int kSmallChunk = 32;    // list entries per chunk
-#ifndef SPQT_SMALL_DEPTH
-#define SPQT_SMALL_DEPTH 3
-#endif
-constexpr int kSmallDepth = SPQT_SMALL_DEPTH;     // chunk buffers per warp
+constexpr int kSmallCtasPerSm = 2;
+constexpr int kSmallMaxSplit = 8;   // CTAs of a block-row: the largest portable cluster
+constexpr int kSmallChunk = 32;     // list entries per chunk
 
 template <int G, int BITS, int ROWS>
 struct SmallSmem {
-    static constexpr int B = G * BITS / 8;
-    alignas(16) unsigned char codes[kSmallWarps][kSmallDepth][kSmallChunk * B];
-    alignas(16) float mult[kSmallWarps][kSmallChunk][ROWS][2];   // (a, a) * 2^93 per entry and batch row
-    alignas(16) unsigned ent[kSmallWarps][kSmallDepth][kSmallChunk][ROWS + 1];  // per entry: its (scale, zero) pair and the words holding the rows' x values
-    alignas(16) float red[kSmallWarps][ROWS][G];
-    float red_z[kSmallWarps][ROWS];
-    int last;
+    static constexpr int kRow = MmaStage<G, BITS>::kRow;
+    static constexpr int kDepth = G == 64 ? 5 : (ROWS == 8 ? 3 : 4);   // chunks per warp: 2.2 to 2.7 KB each (G = 64: half that)
+    static constexpr int kPad = G + 4;
+    struct Stage {
+        alignas(16) unsigned char codes[kSmallChunk * kRow];
+        alignas(16) unsigned meta[kSmallChunk];                 // (scale, zero) pair of entry e
+        alignas(16) unsigned short x[kSmallChunk * ROWS];       // given list: entry after entry; dense: row after row
+    };
+    Stage stage[kSmallWarps][kDepth];
+    alignas(16) unsigned short b[kSmallWarps][ROWS == 8 ? 2 : 1][kSmallChunk][8];   // B of the chunk in work, entry after entry
+    alignas(16) float red[kSmallWarps][ROWS][kPad];
+    float red_z[kSmallWarps][8];
+    float sum_z[8];
 };
 
-// idx == nullptr: the dense product (the list is 0, 1, .., n-1 and count is n).
-// CTAs resident per SM: the sums of four rows take 64 registers of a thread, which leaves room for two CTAs.
-constexpr int small_ctas_per_sm(int rows) { return rows <= 2 ? 3 : 2; }
+struct SmallArgs {
+    const uint8_t* codes;
+    const unsigned* meta;
+    int n;
+    const uint8_t* x;            // gathered x (ROWS values per list entry), or X itself (DIRECT)
+    int ldx, batch;
+    const int32_t* idx;          // nullptr: the list is 0, 1, .., n-1
+    const int32_t* count;
+    __half* Y;
+    int ldy;
+};
 
-template <int G, int BITS, int ROWS>
-__global__ void __launch_bounds__(kSmallThreads, small_ctas_per_sm(ROWS))
-gemm_small_kernel(const uint8_t* __restrict__ codes, const unsigned* __restrict__ meta, int n,
-                  const __half* __restrict__ X, int ldx, int batch,
-                  const int32_t* __restrict__ idx, const int32_t* __restrict__ count_ptr,
-                  __half* __restrict__ Y, int ldy, float* __restrict__ partials, int* __restrict__ counters)
+// DIRECT: the dense product with x read from X itself, 8 columns of a row per 16-byte copy (n and ldx multiples of 8,
+// X 16-byte aligned); otherwise x comes gathered.
+template <int G, int BITS, int ROWS, bool DIRECT>
+__global__ void __launch_bounds__(kSmallThreads, kSmallCtasPerSm)
+gemm_small_kernel(const SmallArgs a)
 {
-    constexpr int B = G * BITS / 8;
-    constexpr int CH = kSmallChunk;
-    constexpr int CB = (B % 16 == 0) ? 16 : 8;        // bytes per copy
-    constexpr int NC = CH * B / CB / 32;              // copies per lane and chunk
-    constexpr int LM = G / 16;                        // arithmetic: lanes per block, 16 codes each
-    constexpr int SLM = 32 / LM;                      // blocks per step
-    constexpr int MSUBS = CH / SLM;                   // steps per chunk
-    constexpr int KEEP = 16 / SLM;
+    using Smem = SmallSmem<G, BITS, ROWS>;
+    using Layout = MmaStage<G, BITS>;
+    constexpr int B = G * BITS / 8, CH = kSmallChunk, D = Smem::kDepth, SP = Layout::kSp;
+    constexpr bool TWO = ROWS == 8;
+    constexpr int CB = (B % 16 == 0) ? 16 : 8;          // bytes per copy
+    constexpr int NC = CH * B / CB / 32;                // copies per lane and chunk
+    constexpr bool kTwice = BITS == 3 && G == 64;       // the 1-bit plane is copied twice
     extern __shared__ __align__(16) unsigned char small_raw[];
-    SmallSmem<G, BITS, ROWS>& sm = *reinterpret_cast<SmallSmem<G, BITS, ROWS>*>(small_raw);
+    Smem& sm = *reinterpret_cast<Smem*>(small_raw);
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
-    const int s = blockIdx.x, S = gridDim.x, r = blockIdx.y;
-    const int mslot = lane / LM, mh = lane % LM;
+    const int g = lane >> 2, t4 = lane & 3;
+    const int n = a.n;
+
+    const int split = blockIdx.x, S = gridDim.x, r = blockIdx.y;
+    const typename Layout::Lane ll(lane);
+    const unsigned stage0 = smem_u32(&sm.stage[warp][0]);
+    constexpr unsigned kStageBytes = (unsigned)sizeof(typename Smem::Stage);
+    constexpr unsigned kMetaOff = (unsigned)offsetof(typename Smem::Stage, meta);
+    constexpr unsigned kXOff = (unsigned)offsetof(typename Smem::Stage, x);
+    const unsigned bbuf = smem_u32(&sm.b[warp][0][0][0]);
+    // where this lane's copies of a chunk come from and go to
+    int copy_e[NC], copy_part[NC];
+    unsigned copy_dst[NC];
+#pragma unroll
+    for (int q = 0; q < NC; ++q) {
+        const int p = q * 32 + lane;
+        const int e = p / (B / CB), part = p % (B / CB);
+        copy_e[q] = e;
+        copy_part[q] = part * CB;
+        if (BITS == 4 && G == 128) copy_dst[q] = e * 64 + ((part ^ ((e >> 1) & 3)) << 4);
+        else if (BITS == 4) copy_dst[q] = e * 32 + ((part ^ ((e >> 2) & 1)) << 4);
+        else copy_dst[q] = e * Layout::kRow + part * CB;
+    }
+    // x: this lane's share of a chunk (DIRECT: 16 bytes of one row; a row past the batch repeats the last one)
+    const uint8_t* const xsrc = DIRECT ? a.x + 2 * ((size_t)min(lane >> 2, a.batch - 1) * a.ldx + 8 * (lane & 3)) : a.x + 2 * ROWS * lane;
+    const unsigned xdst = kXOff + (DIRECT ? 16u : 2u * ROWS) * lane;
 
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-    const int count = idx ? __ldg(count_ptr) : n;
-    const int lo = (int)(((long long)s * count) / S), hi = (int)(((long long)(s + 1) * count) / S);
-    const size_t row_base = (size_t)r * (size_t)n;
-    const uint8_t* row_codes = codes + row_base * B;
-    const unsigned* row_meta = meta + row_base;
-    const unsigned cbuf = smem_u32(&sm.codes[warp][0][0]);
-    const unsigned mbuf = smem_u32(&sm.mult[warp][0][0][0]);
-    constexpr unsigned kBufBytes = CH * B;
+    // this warp's part [pos, end) of the CTA's slice; in units of 8 entries (DIRECT: 16-byte pieces of x)
+    int pos, end;
+    {
+        const int count = (!DIRECT && a.idx) ? __ldg(a.count) : n;
+        const int units = (count + 7) >> 3;
+        const int lo = (int)(((long long)split * units) / S), hi = (int)(((long long)(split + 1) * units) / S);
+        pos = 8 * (lo + ((hi - lo) * warp) / kSmallWarps);
+        end = min(8 * (lo + ((hi - lo) * (warp + 1)) / kSmallWarps), count);
+    }
+    const uint8_t* const row_codes = a.codes + (size_t)r * (size_t)n * B;
+    const unsigned* const row_meta = a.meta + (size_t)r * (size_t)n;
 
-    unsigned long long acc[ROWS][8];
-    float zl[ROWS];
+    float acc[SP][4][4];
+    unsigned long long zl[ROWS / 2], scale[ROWS / 2];   // pairs of rows
 #pragma unroll
-    for (int b = 0; b < ROWS; ++b) {
-        zl[b] = 0.0f;
+    for (int s = 0; s < SP; ++s)
 #pragma unroll
-        for (int i = 0; i < 8; ++i) acc[b][i] = 0ull;
+        for (int i = 0; i < 16; ++i) acc[s][i >> 2][i & 3] = 0.0f;
+#pragma unroll
+    for (int b = 0; b < ROWS / 2; ++b) {
+        zl[b] = 0ull;
+        scale[b] = pack2(kMmaNoScale, kMmaNoScale);
     }
 
-    // column of the entry this lane holds in the chunk at list position pos (past the end: the last entry again)
-    auto column_at = [&](int pos) -> int {
-        const int e = min(pos + lane, hi - 1);
-        return idx ? __ldg(idx + e) : e;
+    // The columns of the lane's entries in the chunks that the copies come to next (past the end of the part: its last
+    // entry again), fetched kAhead chunks early.
+    constexpr int kAhead = 4;
+    int coming[kAhead];
+    int ipos = pos;               // where the copies stand; the arithmetic is D - 1 chunks behind
+    auto column_at = [&](int p) -> int {
+        const int e = min(p + lane, end - 1);
+        return (!DIRECT && a.idx) ? __ldg(a.idx + e) : e;
     };
-    // the chunk's code blocks into one of the warp's buffers, lane after lane
-    auto copy_codes = [&](int col, unsigned dst) {
 #pragma unroll
-        for (int q = 0; q < NC; ++q) {
-            const int off = (q * 32 + lane) * CB;
-            const int e = off / B, part = off % B;
-            const int cu = __shfl_sync(0xffffffffu, col, e);
-            const uint8_t* src = row_codes + (size_t)cu * B + part;
-            if (CB == 16) cp_async_16_l2_64(dst + off, src);
-            else cp_async_8(dst + off, src);
+    for (int d = 0; d < kAhead; ++d) coming[d] = pos < end ? column_at(pos + d * CH) : 0;
+    unsigned rc = 0, ri = 0;      // byte offsets of the arithmetic's and the copies' stage
+    auto issue = [&]() {          // the copies of the next chunk, if there is one
+        if (ipos < end) {
+            const int col = coming[0];
+            const unsigned st = stage0 + ri;
+            cp_async_4(st + kMetaOff + 4u * lane, row_meta + col);
+            if (DIRECT) {
+                if (ROWS == 8 || lane < 16) cp_async_16_left(st + xdst, xsrc + 2 * (size_t)(unsigned)ipos, n - ipos - 8 * (lane & 3));
+            } else if (ROWS == 8) {
+                cp_async_16(st + xdst, xsrc + (size_t)(unsigned)ipos * 16);
+            } else {
+                cp_async_8(st + xdst, xsrc + (size_t)(unsigned)ipos * 8);
+            }
+#pragma unroll
+            for (int q = 0; q < NC; ++q) {
+                const unsigned cu = (unsigned)__shfl_sync(0xffffffffu, col, copy_e[q]);
+                const uint8_t* s = row_codes + ((size_t)cu * B + copy_part[q]);
+                if (CB == 16) cp_async_16_l2_64(st + copy_dst[q], s);
+                else cp_async_8(st + copy_dst[q], s);
+            }
+            if (kTwice) cp_async_8(st + lane * Layout::kRow + 24, row_codes + ((size_t)(unsigned)col * B + 16));
+            ri = ri + kStageBytes == D * kStageBytes ? 0u : ri + kStageBytes;
+            ipos += CH;
+#pragma unroll
+            for (int d = 0; d + 1 < kAhead; ++d) coming[d] = coming[d + 1];
+            coming[kAhead - 1] = column_at(ipos + (kAhead - 1) * CH);
         }
         cp_async_commit();
     };
+#pragma unroll 1
+    for (int d = 0; d < D - 1; ++d) issue();
 
-    // One step: the lane's 16 codes become eight packed operand pairs ONCE (masks and shifts), then every
-    // row of the batch multiplies them with its own multiplier pair.
-    auto step = [&](unsigned cb, int u) {
-        const unsigned ent = (unsigned)(u * SLM + mslot);
-        uint2 wv;
-        if (BITS == 4) {
-            wv = lds_v2(cb + lane * 8 + u * 256);
-        } else {
-            const unsigned blk = cb + ent * B;
-            const unsigned w2 = lds_u32(blk + 4u * mh);
-            const unsigned w1 = lds_u32(blk + (G / 4) + 4u * (mh % (LM / 2))) >> (mh / (LM / 2));
-            wv.x = (w2 & 0x33333333u) | ((w1 << 2) & 0x44444444u);     // the two planes widened to nibble codes
-            wv.y = ((w2 >> 2) & 0x33333333u) | (w1 & 0x44444444u);
-        }
-        unsigned long long op[8];
+#pragma unroll 1
+    for (; pos < end; pos += CH) {
+        issue();
+        // ---- B of the chunk that is due: lane e's entry, every row of the batch
+        const unsigned st = stage0 + rc;
+        cp_async_wait<D - 1>();
+        __syncwarp();
         {
-            const unsigned w = wv.x, v = wv.x >> 16, w2b = wv.y, v2 = wv.y >> 16;
-            // the cumulative values of every half-word (its low 4, 8, 12 and 16 bits), as in the batch-1 kernel
-            op[0] = pack2(__uint_as_float(w & 0x0000000fu), __uint_as_float(w & 0x000000ffu));
-            op[1] = pack2(__uint_as_float(w & 0x00000fffu), __uint_as_float(w & 0x0000ffffu));
-            op[2] = pack2(__uint_as_float(v & 0x0000000fu), __uint_as_float(v & 0x000000ffu));
-            op[3] = pack2(__uint_as_float(v & 0x00000fffu), __uint_as_float(v));
-            op[4] = pack2(__uint_as_float(w2b & 0x0000000fu), __uint_as_float(w2b & 0x000000ffu));
-            op[5] = pack2(__uint_as_float(w2b & 0x00000fffu), __uint_as_float(w2b & 0x0000ffffu));
-            op[6] = pack2(__uint_as_float(v2 & 0x0000000fu), __uint_as_float(v2 & 0x000000ffu));
-            op[7] = pack2(__uint_as_float(v2 & 0x00000fffu), __uint_as_float(v2));
-        }
+            const bool on = pos + lane < end;
+            const unsigned mz = lds_u32(st + kMetaOff + 4u * lane);
+            const float sf = __half2float(__ushort_as_half((unsigned short)(mz & 0xffffu)));
+            const float zf = __half2float(__ushort_as_half((unsigned short)(mz >> 16)));
+            unsigned xw[ROWS / 2];   // the entry's x values, two rows a word
+            if (DIRECT) {
 #pragma unroll
-        for (int b = 0; b < ROWS; ++b) {
-            const unsigned long long mm = lds_u64(mbuf + 8u * (ent * ROWS + b));
+                for (int b = 0; b < ROWS / 2; ++b)
+                    xw[b] = lds_u16(st + kXOff + 128u * b + 2u * lane) | (lds_u16(st + kXOff + 128u * b + 64u + 2u * lane) << 16);
+            } else if (ROWS == 8) {
+                const uint4 v = lds_v4(st + xdst);
+                xw[0] = v.x;
+                xw[1] = v.y;
+                xw[ROWS / 2 - 2] = v.z;
+                xw[ROWS / 2 - 1] = v.w;
+            } else {
+                const uint2 v = lds_v2(st + xdst);
+                xw[0] = v.x;
+                xw[1] = v.y;
+            }
+            unsigned long long am[ROWS / 2], p[ROWS / 2];
+            float top = 0.0f;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) ffma2(acc[b][i], op[i], mm);
-        }
-    };
-
-    // The (scale, zero) pair and the x values of an entry travel like its codes: asynchronous copies into
-    // shared memory, one chunk ahead (held in registers across a chunk's arithmetic they made the compiler
-    // move the loads next to their use, and every chunk then waited for a round of gathers).  x is fetched as
-    // the aligned 4-byte word that holds the value; without that alignment the values are loaded directly.
-    const bool xw_ok = (reinterpret_cast<uintptr_t>(X) & 3) == 0 && (ldx & 1) == 0;
-    const unsigned ebuf = smem_u32(&sm.ent[warp][0][0][0]);
-    constexpr unsigned kEntBytes = CH * (ROWS + 1) * 4;
-    auto issue_chunk = [&](int col, unsigned which) {
-        const unsigned ed = ebuf + which * kEntBytes + (unsigned)lane * (ROWS + 1) * 4u;
-        cp_async_4(ed, row_meta + col);
-        if (xw_ok) {
+            for (int b = 0; b < ROWS / 2; ++b) {
+                const unsigned w = on ? xw[b] : 0u;
+                const float2 xf = __half22float2(*reinterpret_cast<const __half2*>(&w));
+                const unsigned long long x2 = pack2(xf.x, xf.y);
+                ffma2(zl[b], x2, pack2(zf, zf));
+                am[b] = fmul2(x2, pack2(sf, sf));     // exact
+                p[b] = fmul2(am[b], scale[b]);        // powers of two
+                float p0, p1;
+                unpack2(p[b], p0, p1);
+                top = fmaxf(top, fmaxf(fabsf(p0), fabsf(p1)));
+            }
+            if (__any_sync(0xffffffffu, top > kMmaLimit)) {
+                // a larger entry than the range holds: new scales for the rows concerned
 #pragma unroll
-            for (int b = 0; b < ROWS; ++b)
-                if (b < batch) cp_async_4(ed + 4u * (1 + b), reinterpret_cast<const unsigned*>(X + (size_t)b * ldx + (col & ~1)));
-        }
-        copy_codes(col, cbuf + which * kBufBytes);   // (commits the group)
-    };
-
-    // kSmallDepth buffers per warp: the copies of the next kSmallDepth - 1 chunks fly during a chunk's arithmetic
-    const int first = lo + warp * CH, stride = kSmallWarps * CH;
-    if (first < hi) {
-        constexpr int D = kSmallDepth;
-        int cols[D];   // columns of this lane's entry in the chunks at pos, pos + stride, ..
+                for (int b = 0; b < ROWS / 2; ++b) {
+                    float av[2], sv[2], fv[2] = {1.0f, 1.0f};
+                    unpack2(am[b], av[0], av[1]);
+                    unpack2(scale[b], sv[0], sv[1]);
 #pragma unroll
-        for (int d = 0; d < D; ++d) cols[d] = first + d * stride < hi ? column_at(first + d * stride) : 0;
-#pragma unroll
-        for (int d = 0; d < D - 1; ++d) {
-            if (first + d * stride < hi) issue_chunk(cols[d], (unsigned)d);
-            else cp_async_commit();
-        }
-        unsigned cur = 0;
-        for (int pos = first; pos < hi; pos += stride) {
-            const unsigned nxt = cur + (D - 1) >= (unsigned)D ? cur + (D - 1) - D : cur + (D - 1);
-            if (pos + (D - 1) * stride < hi) issue_chunk(cols[D - 1], nxt);
-            else cp_async_commit();
-            const int col_after = pos + D * stride < hi ? column_at(pos + D * stride) : 0;
-            const int col = cols[0];
-            cp_async_wait<D - 1>();   // this chunk's copies have landed (the later chunks' may still fly)
-            __syncwarp();
-            // lane e: the multiplier pair of every row for its entry
-            {
-                const bool on = pos + lane < hi;
-                const unsigned ea = ebuf + cur * kEntBytes + (unsigned)lane * (ROWS + 1) * 4u;
-                const unsigned mz = lds_u32(ea);
-                const float sf = __half2float(__ushort_as_half((unsigned short)(mz & 0xffffu)));
-                const float zf = __half2float(__ushort_as_half((unsigned short)(mz >> 16)));
-#pragma unroll
-                for (int b = 0; b < ROWS; ++b) {
-                    unsigned short xb = 0;
-                    if (on && b < batch) {
-                        if (xw_ok) {
-                            const unsigned w = lds_u32(ea + 4u * (1 + b));
-                            xb = (unsigned short)((col & 1) ? (w >> 16) : (w & 0xffffu));
-                        } else {
-                            xb = __ldg(reinterpret_cast<const unsigned short*>(X) + (size_t)b * ldx + col);
+                    for (int j = 0; j < 2; ++j) {
+                        const unsigned bits = __float_as_uint(av[j]) & 0x7fffffffu;
+                        const unsigned m = __reduce_max_sync(0xffffffffu, bits < 0x7f800000u ? bits : 0u);   // finite ones
+                        if (__uint_as_float(m) * sv[j] > kMmaLimit) {
+                            const float next = __uint_as_float((264u - (m >> 23)) << 23);   // m goes to 2^10 .. 2^11
+                            fv[j] = next * power_of_two_inverse(sv[j]);
+                            sv[j] = next;
                         }
                     }
-                    const float xf = __half2float(__ushort_as_half(xb));
-                    const float am = xf * sf;       // exact
-                    zl[b] += xf * zf;               // exact product
-                    const unsigned long long aa = pack2(am, am);
-                    sts_u64(mbuf + 8u * (lane * ROWS + b), fmul2(aa, pack2(0x1p93f, 0x1p93f)));
+                    scale[b] = pack2(sv[0], sv[1]);
+                    p[b] = fmul2(am[b], scale[b]);
+                    if ((t4 & (ROWS / 2 - 1)) == b) {   // the lane's columns are rows 2b and 2b + 1
+#pragma unroll
+                        for (int s = 0; s < SP; ++s)
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) acc[s][i >> 2][i & 3] *= fv[i & 1];
+                    }
                 }
             }
-            __syncwarp();
-            const unsigned cb = cbuf + cur * kBufBytes;
-            const int valid = min(CH, hi - pos);
-            if (valid == CH) {
+            unsigned hi[ROWS / 2], lo[ROWS / 2];
 #pragma unroll
-                for (int u = 0; u < MSUBS; ++u) step(cb, u);
+            for (int b = 0; b < ROWS / 2; ++b) {
+                float p0, p1;
+                unpack2(p[b], p0, p1);
+                const __half2 h = __floats2half2_rn(p0, p1);
+                const float2 hf = __half22float2(h);
+                unsigned long long rest = p[b];
+                ffma2(rest, pack2(hf.x, hf.y), pack2(-1.0f, -1.0f));
+                unpack2(rest, p0, p1);
+                const __half2 l = __floats2half2_rn(p0, p1);
+                hi[b] = *reinterpret_cast<const unsigned*>(&h);
+                lo[b] = *reinterpret_cast<const unsigned*>(&l);
+            }
+            if (TWO) {
+                sts_v4(bbuf + 16u * lane, make_uint4(hi[0], hi[1], hi[ROWS / 2 - 2], hi[ROWS / 2 - 1]));
+                sts_v4(bbuf + 512u + 16u * lane, make_uint4(lo[0], lo[1], lo[ROWS / 2 - 2], lo[ROWS / 2 - 1]));
             } else {
-                const int nsub = (valid + SLM - 1) / SLM;
-#pragma unroll 1
-                for (int u = 0; u < nsub; ++u) step(cb, u);
+                sts_v4(bbuf + 16u * lane, make_uint4(hi[0], hi[1], lo[0], lo[1]));
             }
             __syncwarp();
-            cur = cur + 1 == (unsigned)D ? 0u : cur + 1;
-#pragma unroll
-            for (int d = 0; d + 1 < D; ++d) cols[d] = cols[d + 1];
-            cols[D - 1] = col_after;
         }
+        // ---- the product
+        unsigned bh[4], bl[4];
+        ldsm_x4_trans(bbuf + 16u * lane, bh);
+        if (TWO) ldsm_x4_trans(bbuf + 512u + 16u * lane, bl);
+#pragma unroll
+        for (int ks = 0; ks < 2; ++ks) {
+            unsigned c[SP][4];
+            Layout::load(st, ll, ks, c);
+#pragma unroll
+            for (int s = 0; s < SP; ++s) mma_group<TWO>(acc[s], c[s], bh + 2 * ks, bl + 2 * ks);
+        }
+        __syncwarp();
+        rc = rc + kStageBytes == D * kStageBytes ? 0u : rc + kStageBytes;
     }
     cp_async_wait<0>();
 
-    // warp -> CTA: reduce-scatter over the block slots, per batch row
+    // ---- the warps' sums meet in shared memory
+    {
+        float inv[2] = {0.0f, 0.0f};   // 2^24 / c of the rows in columns 2*t4 and 2*t4 + 1
 #pragma unroll
-    for (int b = 0; b < ROWS; ++b) {
-        float accf[16];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) unpack2(acc[b][i], accf[2 * i], accf[2 * i + 1]);
-        float t8[8], t4[4], keep[4];
-        halve<16>(accf, t8, lane, 16);
-        halve<8>(t8, t4, lane, 8);
-        uncumulate(t4);
-        if (LM == 8) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) keep[i] = t4[i];
-        } else {
-            float t2[2];
-            halve<4>(t4, t2, lane, 4);
-            keep[0] = t2[0];
-            keep[1] = t2[1];
+        for (int b = 0; b < ROWS / 2; ++b) {
+            float s0, s1;
+            unpack2(scale[b], s0, s1);
+            if ((t4 & (ROWS / 2 - 1)) == b) {
+                inv[0] = 0x1p24f * power_of_two_inverse(s0);
+                inv[1] = 0x1p24f * power_of_two_inverse(s1);
+            }
         }
 #pragma unroll
-        for (int i = 0; i < KEEP; ++i) {
-            const int ai = mslot * KEEP + i;  // accumulator index = word*8 + nibble
-            const int cw = ai >> 3, e2 = ai & 7;
-            const int row = (BITS == 4) ? 8 * mh + 4 * cw + (e2 >> 1) + (e2 & 1) * (G / 2)
-                                        : 4 * mh + (e2 >> 1) + (G / 4) * (2 * (e2 & 1) + cw);
-            sm.red[warp][b][row] = keep[i] * 0x1p56f;
-        }
-        float z = zl[b];
+        for (int s = 0; s < SP; ++s) {
+            mma_uncumulate(acc[s]);
+            if (TWO) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-        if (lane == 0) sm.red_z[warp][b] = z;
+                for (int i = 0; i < 16; ++i) {
+                    const int type = i >> 2, c = i & 3;
+                    sm.red[warp][2 * t4 + (c & 1)][Layout::row(s, type, c, g)] = acc[s][type][c] * inv[c & 1];
+                }
+            } else {
+                // columns b and b + 4 are the hi and lo sums of row b: lanes t4 and t4 ^ 2 exchange one half of the
+                // tiles each and add
+                const bool upper = t4 >= 2;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int type = i >> 2, c = i & 3;   // kept: types 0, 1 by t4 < 2, types 2, 3 by the others
+                    const float keep = upper ? acc[s][type + 2][c] : acc[s][type][c], send = upper ? acc[s][type][c] : acc[s][type + 2][c];
+                    const float v = keep + __shfl_xor_sync(0xffffffffu, send, 2);
+                    sm.red[warp][2 * (t4 & 1) + (c & 1)][Layout::row(s, type, c, g) + (upper ? 1 : 0)] = v * inv[c & 1];
+                }
+            }
+        }
+#pragma unroll
+        for (int b = 0; b < ROWS; ++b) {
+            float zz[2];
+            unpack2(zl[b >> 1], zz[0], zz[1]);
+            float z = zz[b & 1];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+            if (lane == 0) sm.red_z[warp][b] = z;
+        }
     }
     __syncthreads();
-
-    // CTA -> block-row
-    float* mine = partials + ((size_t)r * kSmallMaxSplit + s) * kSmallRows * (G + 1);
-    for (int i = tid; i < ROWS * (G + 1); i += kSmallThreads) {
-        const int b = i / (G + 1), j = i % (G + 1);
+    // every output of the CTA by one thread, in warp order; the sums stay in warp 0's slot
+    if (tid < ROWS) {
+        float z = 0.0f;
+#pragma unroll
+        for (int w = 0; w < kSmallWarps; ++w) z += sm.red_z[w][tid];
+        sm.sum_z[tid] = z;
+    }
+#pragma unroll
+    for (int q = 0; q < ROWS * G / kSmallThreads; ++q) {
+        const int o = q * kSmallThreads + tid, b = o / G, j = o % G;
         float v = 0.0f;
 #pragma unroll
-        for (int w = 0; w < kSmallWarps; ++w) v += (j < G) ? sm.red[w][b][j] : sm.red_z[w][b];
-        if (S == 1) {
-            // the only CTA of its block-row: keep the sums in place (warp 0's slot; every element has one writer)
-            if (j < G) sm.red[0][b][j] = v;
-            else sm.red_z[0][b] = v;
-        } else {
-            __stcg(mine + i, v);
-        }
+        for (int w = 0; w < kSmallWarps; ++w) v += sm.red[w][b][j];
+        sm.red[0][b][j] = v;
     }
-    if (S == 1) {
+    // ---- the CTAs' sums: CTA s finishes the s-th of S parts of the block-row's outputs, in CTA order
+    if (S > 1) {
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    } else {
         __syncthreads();
-        for (int i = tid; i < batch * G; i += kSmallThreads) {
-            const int b = i / G, j = i % G;
-            Y[(size_t)b * ldy + (size_t)r * G + j] = __float2half_rn(sm.red[0][b][j] + sm.red_z[0][b]);
-        }
-        return;
     }
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) sm.last = (atomicAdd(counters + r, 1) == S - 1) ? 1 : 0;
-    __syncthreads();
-    if (!sm.last) return;
-    __threadfence();
-    const float* rowp = partials + (size_t)r * kSmallMaxSplit * kSmallRows * (G + 1);
-    for (int i = tid; i < batch * G; i += kSmallThreads) {
-        const int b = i / G, j = i % G;
+    const int outs = a.batch * G, from = outs * split / S, to = outs * (split + 1) / S;
+    for (int o = from + tid; o < to; o += kSmallThreads) {
+        const int b = o / G, j = o % G;
         float v = 0.0f, z = 0.0f;
-        for (int q = 0; q < S; ++q) {
-            v += __ldcg(rowp + ((size_t)q * kSmallRows + b) * (G + 1) + j);
-            z += __ldcg(rowp + ((size_t)q * kSmallRows + b) * (G + 1) + G);
+        if (S == 1) {
+            v = sm.red[0][b][j];
+            z = sm.sum_z[b];
+        } else {
+            const unsigned av = smem_u32(&sm.red[0][b][j]), az = smem_u32(&sm.sum_z[b]);
+#pragma unroll
+            for (int q = 0; q < kSmallMaxSplit; ++q) {
+                if (q < S) {
+                    v += ld_cluster_f32(cluster_map(av, (unsigned)q));
+                    z += ld_cluster_f32(cluster_map(az, (unsigned)q));
+                }
+            }
         }
-        Y[(size_t)b * ldy + (size_t)r * G + j] = __float2half_rn(v + z);
+        a.Y[(size_t)b * a.ldy + (size_t)r * G + j] = __float2half_rn(v + z);
     }
-    if (tid == 0) counters[r] = 0;   // ready for the next call
+    if (S > 1) {   // nobody leaves while another CTA may still be reading its sums
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
 }
 
+// Workspace: one word per block-row (zero, kept for callers that look at it), then the gathered x: 16 bytes per list
+// entry at most, and the chunk a warp may read past the end.  Never less than 64 KB.
 inline size_t small_header_bytes(int R) { return (((size_t)R * 4 + 255) / 256) * 256; }
 inline size_t small_workspace_bytes(const Format& f)
 {
-    return small_header_bytes(f.R) + (size_t)f.R * kSmallMaxSplit * kSmallRows * (size_t)(f.group + 1) * sizeof(float);
+    const size_t need = small_header_bytes(f.R) + ((size_t)f.n + kSmallChunk) * 16;
+    return need < 65536 ? 65536 : need;
 }
 
-// Slices per block-row: the grid runs in waves of `per_sm` CTAs per SM; a CTA costs a fixed part (set-up,
-// reduction, the exchange of partial sums) plus its share of the list.  Pick the split with the lowest
-// estimate; ties go to the smaller one.
-static int small_split(int R, int n, int sms, int per_sm)
+// CTAs per block-row.  All of them should be resident at once (two per SM): a second wave costs more than the idle slots
+// of a first one (28672 x 4096, 4 rows: 17.4 us on 224 CTAs, 23.6 on 448).  From R = 100 up the split that this leaves,
+// two, puts two half block-rows on the busiest SMs where one whole block-row runs as fast and needs no exchange
+// (14336 x 4096, 8 rows dense: 12.3 against 14.4 us).  Below, as many as fit: 4096 x 14336, 8 rows dense 33.9 / 20.1 /
+// 16.0 / 13.4 us on 1 / 2 / 4 / 8; 8192 x 28672, 4 rows dense 51.6 / 28.6 / 26.9 us on 1 / 2 / 4; but never less than
+// one chunk per warp.
+static int small_split(const Format& f, int sms)
 {
-    const double slots = (double)per_sm * sms;
-    int best = 1;
-    double best_t = 0.0;
-    for (int S = 1; S <= kSmallMaxSplit; ++S) {
-        const double waves = (double)((long long)((R * (double)S + slots - 1) / slots));
-        const double t = waves * (4.0 + 1.5 * (double)n / (256.0 * S));
-        if (S == 1 || t < best_t - 1e-9) {
-            best = S;
-            best_t = t;
-        }
+    int S = f.R >= 100 ? 1 : (kSmallCtasPerSm * sms) / f.R;
+    const int most = (f.n + 255) / 256;
+    if (S > most) S = most;
+    if (S > kSmallMaxSplit) S = kSmallMaxSplit;
+    return S < 1 ? 1 : S;
+}
+
+// The records of the dense product when it cannot read X with 16-byte copies: REC values per column.
+template <int REC>
+__global__ void __launch_bounds__(256) gather_rows_kernel(const unsigned short* __restrict__ X, int ldx, int batch, int n, unsigned short* __restrict__ gathered)
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int k = blockIdx.x * 256 + threadIdx.x;
+    if (k >= n) return;
+    unsigned rec[REC / 2];
+#pragma unroll
+    for (int b = 0; b < REC; b += 2) {
+        const unsigned lo = b < batch ? __ldg(X + (size_t)b * ldx + k) : 0u;
+        const unsigned hi = b + 1 < batch ? __ldg(X + (size_t)(b + 1) * ldx + k) : 0u;
+        rec[b / 2] = lo | (hi << 16);
     }
-    return best;
+    if (REC == 8) *reinterpret_cast<uint4*>(gathered + (size_t)k * 8) = make_uint4(rec[0], rec[1], rec[REC / 2 - 2], rec[REC / 2 - 1]);
+    else *reinterpret_cast<uint2*>(gathered + (size_t)k * 4) = make_uint2(rec[0], rec[1]);
 }
 
-template <int G, int BITS, int ROWS>
-static spqt_status launch_small_rows(const Format& f, const void* codes, const void* meta, const __half* X, int ldx,
-                                     int nb, const int32_t* idx, const int32_t* count, __half* Y, int ldy,
-                                     void* workspace, cudaStream_t s)
+static spqt_status launch_gather_rows(const __half* X, int ldx, int batch, int n, void* gathered, cudaStream_t s)
 {
-    auto kernel = gemm_small_kernel<G, BITS, ROWS>;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((n + 255) / 256));
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = g_no_pdl ? 0 : 1;
+    const cudaError_t err = cudaLaunchKernelEx(&cfg, batch <= 4 ? gather_rows_kernel<4> : gather_rows_kernel<8>, reinterpret_cast<const unsigned short*>(X), ldx, batch, n,
+                                               static_cast<unsigned short*>(gathered));
+    count_launch();
+    return (err == cudaSuccess && cudaGetLastError() == cudaSuccess) ? SPQT_OK : SPQT_ERR_CUDA;
+}
+
+template <int G, int BITS, int ROWS, bool DIRECT>
+static spqt_status launch_small(const Format& f, SmallArgs a, cudaStream_t s)
+{
+    auto kernel = gemm_small_kernel<G, BITS, ROWS, DIRECT>;
     static bool configured[64] = {};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return SPQT_ERR_CUDA;
@@ -348,38 +447,32 @@ static spqt_status launch_small_rows(const Format& f, const void* codes, const v
     }
     const int sms = sm_count();
     if (sms <= 0) return SPQT_ERR_CUDA;
+    const int S = small_split(f, sms);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(small_split(f.R, f.n, sms, small_ctas_per_sm(ROWS)), f.R);
+    cfg.gridDim = dim3(S, f.R);
     cfg.blockDim = dim3(kSmallThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = S;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = g_no_pdl ? 0 : 1;
-    int* counters = static_cast<int*>(workspace);
-    float* partials = reinterpret_cast<float*>(static_cast<char*>(workspace) + small_header_bytes(f.R));
-    const cudaError_t err = cudaLaunchKernelEx(&cfg, kernel, static_cast<const uint8_t*>(codes),
-                                               static_cast<const unsigned*>(meta), f.n, X, ldx, nb, idx, count,
-                                               Y, ldy, partials, counters);
+    cfg.numAttrs = g_no_pdl ? 1 : 2;
+    const cudaError_t err = cudaLaunchKernelEx(&cfg, kernel, a);
     count_launch();
     return (err == cudaSuccess && cudaGetLastError() == cudaSuccess) ? SPQT_OK : SPQT_ERR_CUDA;
 }
 
 template <int G, int BITS>
-static spqt_status launch_small(const Format& f, const void* codes, const void* meta, const __half* X, int ldx,
-                                int batch, const int32_t* idx, const int32_t* count, __half* Y, int ldy,
-                                void* workspace, cudaStream_t s)
+static spqt_status launch_small_format(const Format& f, const SmallArgs& a, bool direct, cudaStream_t s)
 {
-    for (int b0 = 0; b0 < batch; b0 += kSmallRows) {
-        const int nb = batch - b0 < kSmallRows ? batch - b0 : kSmallRows;
-        const spqt_status st =
-            nb <= 2 ? launch_small_rows<G, BITS, 2>(f, codes, meta, X + (size_t)b0 * ldx, ldx, nb, idx, count, Y + (size_t)b0 * ldy, ldy, workspace, s)
-                    : launch_small_rows<G, BITS, 4>(f, codes, meta, X + (size_t)b0 * ldx, ldx, nb, idx, count, Y + (size_t)b0 * ldy, ldy, workspace, s);
-        if (st != SPQT_OK) return st;
-    }
-    return SPQT_OK;
+    // up to four rows: (hi, lo) side by side in the eight columns, half the matrix instructions
+    if (a.batch <= 4) return direct ? launch_small<G, BITS, 4, true>(f, a, s) : launch_small<G, BITS, 4, false>(f, a, s);
+    return direct ? launch_small<G, BITS, 8, true>(f, a, s) : launch_small<G, BITS, 8, false>(f, a, s);
 }
 
 static spqt_status small_entry(const void* codes, const void* meta, int m, int n, int bits, int group,
@@ -400,17 +493,31 @@ static spqt_status small_entry(const void* codes, const void* meta, int m, int n
     if (!dense && n > 65535) return SPQT_ERR_UNSUPPORTED;  // the index collection keeps 64 flag bits per lane
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const __half* Xh = static_cast<const __half*>(X);
-    if (!dense) {
-        const spqt_status st2 = launch_sparsify_rows(Xh, ldx, batch, n, t, idx, count, s);
-        if (st2 != SPQT_OK) return st2;
+    char* const ws = static_cast<char*>(workspace);
+    SmallArgs a = {};
+    a.codes = static_cast<const uint8_t*>(codes);
+    a.meta = static_cast<const unsigned*>(meta);
+    a.n = n;
+    a.ldx = ldx;
+    a.batch = batch;
+    a.Y = static_cast<__half*>(Y);
+    a.ldy = ldy;
+    const bool direct = dense && (n & 7) == 0 && (ldx & 7) == 0 && aligned(X, 16);
+    if (direct) {
+        a.x = reinterpret_cast<const uint8_t*>(Xh);
+    } else {
+        void* const gathered = ws + small_header_bytes(f.R);
+        st = dense ? launch_gather_rows(Xh, ldx, batch, n, gathered, s)
+                   : launch_sparsify_rows(Xh, ldx, batch, n, t, idx, count, gathered, s);
+        if (st != SPQT_OK) return st;
+        a.x = static_cast<const uint8_t*>(gathered);
+        a.idx = dense ? nullptr : idx;
+        a.count = count;
     }
-    const int32_t* li = dense ? nullptr : idx;
-    const int32_t* lc = dense ? nullptr : count;
-    __half* Yh = static_cast<__half*>(Y);
-    if (bits == 4 && group == 128) return launch_small<128, 4>(f, codes, meta, Xh, ldx, batch, li, lc, Yh, ldy, workspace, s);
-    if (bits == 4 && group == 64) return launch_small<64, 4>(f, codes, meta, Xh, ldx, batch, li, lc, Yh, ldy, workspace, s);
-    if (bits == 3 && group == 128) return launch_small<128, 3>(f, codes, meta, Xh, ldx, batch, li, lc, Yh, ldy, workspace, s);
-    return launch_small<64, 3>(f, codes, meta, Xh, ldx, batch, li, lc, Yh, ldy, workspace, s);
+    if (bits == 4 && group == 128) return launch_small_format<128, 4>(f, a, direct, s);
+    if (bits == 4 && group == 64) return launch_small_format<64, 4>(f, a, direct, s);
+    if (bits == 3 && group == 128) return launch_small_format<128, 3>(f, a, direct, s);
+    return launch_small_format<64, 3>(f, a, direct, s);
 }
 
 }  // namespace spqt

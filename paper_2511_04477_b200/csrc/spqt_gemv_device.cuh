@@ -126,6 +126,12 @@ __device__ __forceinline__ void cp_async_16(unsigned smem_dst, const void* gmem_
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_dst), "l"(gmem_src) : "memory");
 }
+// the same with no more than `left` 2-byte values read, zeros after them
+__device__ __forceinline__ void cp_async_16_left(unsigned smem_dst, const void* gmem_src, int left)
+{
+    const int bytes = left >= 8 ? 16 : (left <= 0 ? 0 : 2 * left);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_dst), "l"(gmem_src), "r"(bytes) : "memory");
+}
 // the same, asking L2 to fetch no more than the 64 bytes around the address
 __device__ __forceinline__ void cp_async_16_l2_64(unsigned smem_dst, const void* gmem_src)
 {
@@ -226,6 +232,12 @@ __device__ __forceinline__ unsigned cluster_map(unsigned smem_addr, unsigned ran
 __device__ __forceinline__ void st_cluster_f32(unsigned addr, float v)
 {
     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+__device__ __forceinline__ float ld_cluster_f32(unsigned addr)
+{
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+    return v;
 }
 __device__ __forceinline__ void mbar_arrive_cluster(unsigned remote_bar)
 {

@@ -6,11 +6,8 @@
 //   sparsify_kernel (one row, any n): each warp owns a contiguous segment of x, counts its active entries
 //     with __ballot_sync/__popc (the loads of eight groups of 32 entries in flight together), the 32 warp
 //     totals are scanned in shared memory, and each warp then writes its indices at its base offset.
-//   sparsify_rows_kernel (the small batch, n < 2^16: "active in at least one of B rows"; one CTA, or a
-//     cluster of 8 CTAs from n = 6144 up): 16-byte loads,
-//     all of a piece's loads in flight together (with B rows, loads that wait for one another cost a round
-//     trip each); compaction by warp scans.  For a single row it measured no faster than the kernel above
-//     (2.7 against 2.3 us at n = 4096, 5.9 against 5.2 us at n = 14336), which therefore keeps that job.
+//   sparsify_rows_kernel (the small batch, n < 2^16: "active in at least one of B rows"): a cluster of 8 CTAs, which
+//     also gathers the rows' values of the listed columns.
 // The output order is ascending by construction (no atomics, no arrival order).
 #include "spqt_common.cuh"
 
@@ -167,178 +164,119 @@ sparsify_cluster_kernel(const __half* __restrict__ x, int n, float t, int32_t* _
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// Lane l of a warp holds the 8 columns 256*piece + 8*l .. + 7 of each of the warp's pieces (a warp owns up
-// to 8 consecutive pieces of 256 columns: n < 2^16); every row's 8 values arrive with one 16-byte load (plain
-// 2-byte loads at a ragged end or when X is not aligned for it), and a piece's loads are all issued before
-// the first compare, so that they share one round trip.  Then the usual compaction: totals per warp, a scan
-// over the warps, and every lane writes its own active columns behind those of the lanes before it.
-// CLUSTER: the same on a thread-block cluster of 8 CTAs of 8 warps (the 64 warps own consecutive runs of
-// pieces; warp totals are exchanged through distributed shared memory as in sparsify_cluster_kernel).
-template <bool CLUSTER>
-__global__ void __launch_bounds__(CLUSTER ? kClusterWarps * 32 : 1024)
-sparsify_rows_kernel(const __half* __restrict__ X, int ldx, int batch, int n, float t,
-                     int32_t* __restrict__ idx, int32_t* __restrict__ count)
+// "Active in at least one of `batch` rows" (n < 2^16): a thread-block cluster of 8 CTAs of 16 warps; every warp owns a
+// run of groups of 32 columns, lane l column l of each group.  Behind every index goes the record the product reads
+// instead of X: the rows' values of that column, REC of them (4 or 8; zero past the batch), so that X is gathered once
+// per call and not once per block-row.  Up to kKeepGroups groups per warp (n <= 16384) the values stay in registers
+// between the counting and the writing pass.  What bounds it is latency (launch, one round trip, two cluster
+// barriers), so the columns are spread over as many lanes as a cluster has: neighbouring lanes then write
+// neighbouring list positions.  (8 columns per lane and scattered record stores took 5.0 us at n = 4096 and 4 rows.)
+constexpr int kRowsWarps = 16;
+constexpr int kKeepGroups = 4;
+
+template <int REC>
+__global__ void __launch_bounds__(kRowsWarps * 32)
+sparsify_rows_kernel(const unsigned short* __restrict__ X, int ldx, int batch, int n, float t,
+                     int32_t* __restrict__ idx, int32_t* __restrict__ count, unsigned short* __restrict__ gathered)
 {
-    __shared__ int warp_total[32];
-    __shared__ int warp_base[32];
-    const int lane = threadIdx.x & 31, cta_warp = threadIdx.x >> 5;
-    unsigned rank = 0;
-    if (CLUSTER) asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-    const int warp = CLUSTER ? (int)rank * kClusterWarps + cta_warp : cta_warp;   // among all the warps at work
-    constexpr int kAllWarps = CLUSTER ? kClusterCtas * kClusterWarps : 32;
+    __shared__ int warp_total[kRowsWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned rank, nctas;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(nctas));
+    // |x| > t as integers: magnitude bits above those of the largest fp16 value not above t (-1 if t < 0: everything is;
+    // infinity if t is NaN or +inf: nothing is), and not a NaN
+    const int thr = (t != t) ? 0x7c00 : (t < 0.0f ? -1 : (int)__half_as_ushort(__float2half_rd(t)));
+    const int groups = (n + (int)nctas * kRowsWarps * 32 - 1) / ((int)nctas * kRowsWarps * 32);
+    const int first = ((int)rank * kRowsWarps + warp) * groups * 32 + lane;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int pieces = (n + 255) >> 8;
-    const int pp = (pieces + kAllWarps - 1) / kAllWarps;   // pieces per warp, at most 8
-    const bool vec_ok = (reinterpret_cast<uintptr_t>(X) & 15) == 0 && (ldx & 7) == 0;
-    const unsigned short* Xs = reinterpret_cast<const unsigned short*>(X);
-    // the largest fp16 value not above t (any negative value if t < 0: everything but NaN is active; +inf if t
-    // is NaN or +inf: nothing is): |x| > t  <=>  |x| > that value, compared in fp16, two entries at a time
-    const __half thr_h = (t != t) ? __ushort_as_half((unsigned short)0x7c00)
-                                  : (t < 0.0f ? __float2half_rn(-1.0f) : __float2half_rd(t));
-    const __half2 thr_h2 = __half2half2(thr_h);
 
-    unsigned long long flags = 0ull;                   // byte j: activity bits of the lane's 8 columns of piece j
-#pragma unroll 1
-    for (int j = 0; j < pp; ++j) {
-        const int k0 = (warp * pp + j) * 256 + lane * 8;
-        const bool have = k0 < n;
-        uint4 v[8];
+    unsigned short v[kKeepGroups][REC];
+    auto load = [&](int g0) {      // groups g0 .. g0 + 3, all loads in flight together
 #pragma unroll
-        for (int b = 0; b < 8; ++b) {
-            v[b] = make_uint4(0u, 0u, 0u, 0u);
-            if (have && b < batch) {
-                const size_t off = (size_t)b * ldx + k0;
-                if (vec_ok && k0 + 8 <= n) {
-                    v[b] = __ldg(reinterpret_cast<const uint4*>(Xs + off));
-                } else {
-                    unsigned short h[8];
+        for (int j = 0; j < kKeepGroups; ++j) {
+            const int k = min(first + (g0 + j) * 32, n - 1);
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) h[e] = (k0 + e < n) ? __ldg(Xs + off + e) : (unsigned short)0;
-                    v[b] = make_uint4(h[0] | ((unsigned)h[1] << 16), h[2] | ((unsigned)h[3] << 16),
-                                      h[4] | ((unsigned)h[5] << 16), h[6] | ((unsigned)h[7] << 16));
-                }
+            for (int b = 0; b < REC; ++b) v[j][b] = (g0 + j < groups && b < batch) ? __ldg(X + (size_t)b * ldx + k) : (unsigned short)0;
+        }
+    };
+    auto active = [&](int g0, int j) -> bool {
+        bool on = false;
+#pragma unroll
+        for (int b = 0; b < REC; ++b)
+            on |= b < batch && (unsigned)((int)(v[j][b] & 0x7fff) - thr - 1) < (unsigned)(0x7c00 - thr);
+        return on && g0 + j < groups && first + (g0 + j) * 32 < n;
+    };
+    int total = 0;
+    for (int g0 = 0; g0 < groups; g0 += kKeepGroups) {
+        load(g0);
+#pragma unroll
+        for (int j = 0; j < kKeepGroups; ++j) total += __popc(__ballot_sync(0xffffffffu, active(g0, j)));
+    }
+    if (lane == 0) warp_total[warp] = total;
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    // lane l adds up the totals of warps l, l + 32, .. of the cluster
+    int below = 0, all = 0;
+    const int me = (int)rank * kRowsWarps + warp;
+#pragma unroll 4
+    for (int w = lane; w < (int)nctas * kRowsWarps; w += 32) {
+        unsigned remote;
+        const unsigned local = static_cast<unsigned>(__cvta_generic_to_shared(&warp_total[w % kRowsWarps]));
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"((unsigned)(w / kRowsWarps)));
+        int c;
+        asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(c) : "r"(remote) : "memory");
+        below += (w < me) ? c : 0;
+        all += c;
+    }
+    int base = __reduce_add_sync(0xffffffffu, below);
+    all = __reduce_add_sync(0xffffffffu, all);
+    // nobody leaves while another CTA may still be reading its table: arrive now, wait at the end
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    if (me == 0 && lane == 0) *count = all;
+    for (int g0 = 0; g0 < groups; g0 += kKeepGroups) {
+        if (groups > kKeepGroups) load(g0);
+#pragma unroll
+        for (int j = 0; j < kKeepGroups; ++j) {
+            const bool on = active(g0, j);
+            const unsigned mask = __ballot_sync(0xffffffffu, on);
+            const int pos = base + __popc(mask & ((1u << lane) - 1u));
+            if (on) {
+                idx[pos] = first + (g0 + j) * 32;
+                unsigned rec[REC / 2];
+#pragma unroll
+                for (int b = 0; b < REC / 2; ++b) rec[b] = v[j][2 * b] | ((unsigned)v[j][2 * b + 1] << 16);
+                if (REC == 8) *reinterpret_cast<uint4*>(gathered + (size_t)pos * 8) = make_uint4(rec[0], rec[1], rec[REC / 2 - 2], rec[REC / 2 - 1]);
+                else *reinterpret_cast<uint2*>(gathered + (size_t)pos * 4) = make_uint2(rec[0], rec[1]);
             }
+            base += __popc(mask);
         }
-        unsigned m8 = 0;
-#pragma unroll
-        for (int b = 0; b < 8; ++b) {
-            if (b < batch) {   // (uniform)
-                const unsigned wds[4] = {v[b].x, v[b].y, v[b].z, v[b].w};
-#pragma unroll
-                for (int e2 = 0; e2 < 4; ++e2) {
-                    const unsigned ab = wds[e2] & 0x7fff7fffu;
-                    const unsigned gt = __hgt2_mask(*reinterpret_cast<const __half2*>(&ab), thr_h2);   // false for NaN
-                    m8 |= ((gt & 1u) | ((gt >> 15) & 2u)) << (2 * e2);
-                }
-            }
-        }
-        // columns past n do not exist (with a negative threshold their zeros would count)
-        const int left = n - k0;
-        if (left < 8) m8 &= (left <= 0) ? 0u : ((1u << left) - 1u);
-        flags |= (unsigned long long)m8 << (8 * j);
     }
-    int total = __popcll(flags);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
-    int base;
-    if (CLUSTER) {
-        if (lane == 0) warp_total[cta_warp] = total;
-        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-        int below = 0, all = 0;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int w = lane + 32 * h;   // lane l looks up the totals of warps l and l + 32 of the cluster
-            unsigned remote;
-            const unsigned local = static_cast<unsigned>(__cvta_generic_to_shared(&warp_total[w % kClusterWarps]));
-            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"((unsigned)(w / kClusterWarps)));
-            int v;
-            asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(remote) : "memory");
-            below += (w < warp) ? v : 0;
-            all += v;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            below += __shfl_xor_sync(0xffffffffu, below, o);
-            all += __shfl_xor_sync(0xffffffffu, all, o);
-        }
-        if (warp == 0 && lane == 0) *count = all;
-        base = below;
-    } else {
-        if (lane == 0) warp_total[warp] = total;
-        __syncthreads();
-        if (warp == 0) {
-            int v = warp_total[lane], incl = v;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                int up = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += up;
-            }
-            warp_base[lane] = incl - v;
-            if (lane == 31) *count = incl;
-        }
-        __syncthreads();
-        base = warp_base[warp];
-    }
-    for (int j = 0; j < pp; ++j) {
-        const unsigned m8 = (unsigned)(flags >> (8 * j)) & 0xffu;
-        const int c8 = __popc(m8);
-        int incl = c8;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int up = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += up;
-        }
-        int pos = base + incl - c8;
-        const int col0 = (warp * pp + j) * 256 + lane * 8;
-        // one predicated store per column (a divergent branch per column costs far more than the store)
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const unsigned on = (m8 >> e) & 1u;
-            asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p st.global.u32 [%1], %2;\n\t}" ::"r"(on), "l"(idx + pos), "r"(col0 + e)
-                         : "memory");
-            pos += (int)on;
-        }
-        base += __shfl_sync(0xffffffffu, incl, 31);
-    }
-    if (CLUSTER) {   // nobody leaves while another CTA may still be reading its table
-        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    }
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-
-// One launch of sparsify_rows_kernel: the columns that are active in at least one of `batch` rows (n < 2^16).
+// One launch of sparsify_rows_kernel: the columns that are active in at least one of `batch` rows (n < 2^16), and
+// their x values in records of 4 (batch <= 4) or 8 fp16 values.
 spqt_status launch_sparsify_rows(const __half* X, int ldx, int batch, int n, float t, int32_t* idx, int32_t* count,
-                                 cudaStream_t stream)
+                                 void* gathered, cudaStream_t stream)
 {
+    auto kernel = batch <= 4 ? sparsify_rows_kernel<4> : sparsify_rows_kernel<8>;
     cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = kClusterCtas;
-    attr[1].val.clusterDim.y = 1;
-    attr[1].val.clusterDim.z = 1;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kClusterCtas;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.stream = stream;
-    // from a few thousand columns on, the cluster of 8 CTAs (falls back to the single CTA if it cannot be launched)
-    if (n > 6144) {
-        cfg.gridDim = dim3(kClusterCtas);
-        cfg.blockDim = dim3(kClusterWarps * 32);
-        cfg.attrs = g_no_pdl ? attr + 1 : attr;
-        cfg.numAttrs = g_no_pdl ? 1 : 2;
-        if (cudaLaunchKernelEx(&cfg, sparsify_rows_kernel<true>, X, ldx, batch, n, t, idx, count) == cudaSuccess) {
-            count_launch();
-            return cudaGetLastError() == cudaSuccess ? SPQT_OK : SPQT_ERR_CUDA;
-        }
-        (void)cudaGetLastError();
-    }
-    cfg.gridDim = dim3(1);
-    cfg.blockDim = dim3(1024);
+    cfg.gridDim = dim3(kClusterCtas);
+    cfg.blockDim = dim3(kRowsWarps * 32);
     cfg.attrs = attr;
-    cfg.numAttrs = g_no_pdl ? 0 : 1;
-    const cudaError_t err = cudaLaunchKernelEx(&cfg, sparsify_rows_kernel<false>, X, ldx, batch, n, t, idx, count);
+    cfg.numAttrs = g_no_pdl ? 1 : 2;
+    const cudaError_t err = cudaLaunchKernelEx(&cfg, kernel, reinterpret_cast<const unsigned short*>(X), ldx, batch, n, t, idx, count,
+                                               static_cast<unsigned short*>(gathered));
     count_launch();
     return (err == cudaSuccess && cudaGetLastError() == cudaSuccess) ? SPQT_OK : SPQT_ERR_CUDA;
 }
