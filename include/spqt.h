@@ -118,7 +118,9 @@ spqt_status spqt_sparsify(const void* x, int n, float t,
  *   y : fp16[m], 2-byte aligned.
  *   workspace : gemv_workspace_bytes of device memory, 16-byte aligned, zeroed
  *       ONCE by the caller before its first use; every call leaves it ready for
- *       the next.  Two calls that may overlap on the GPU need two workspaces.
+ *       the next.  (It holds the status word that checked mode sets; sums travel through
+ *       shared memory.)  Two calls that may overlap on the GPU need two
+ *       workspaces.
  * Supported: bits 4 or 3 with group 64 or 128; n <= 65535 (column numbers travel as 16 bits).
  */
 spqt_status spqt_sparse_gemv(const void* codes, const void* scale_zero,
@@ -142,9 +144,7 @@ spqt_status spqt_sparsify_gemv(const void* codes, const void* scale_zero,
 
 /*
  * The same kernel over all n columns with no index list: the dense GEMV on the
- * zigzag layout (paper Sec. 4.2.2), the sparsity-free comparison.  Any n when n is a multiple of 8
- * and x is 16-byte aligned (whole chunks of a block-row are then fetched by bulk copies); otherwise
- * n <= 65535.
+ * zigzag layout (paper Sec. 4.2.2), the sparsity-free comparison.  Any n.
  */
 spqt_status spqt_dense_gemv(const void* codes, const void* scale_zero,
                             int m, int n, int bits, int group, const void* x,
@@ -167,9 +167,8 @@ spqt_status spqt_dense_gemv(const void* codes, const void* scale_zero,
  *     that device current) and keeps it; make that first call before any stream capture begins, and
  *     from one host thread (the look-up is not guarded against two threads making it at once).
  *   - All calls on a device share the one array, which still holds the previous call's contents; the
- *     part that must start at zero (arrival counters, status word, the tagged words that carry partial
- *     sums between thread blocks: up to about 0.9 MiB) is cleared on `stream` before the kernel, after
- *     every argument check has passed.  Two calls that may overlap on the GPU (different streams, no
+ *     part that must start at zero (the status word and the words before it) is cleared on `stream`
+ *     before the kernel, after every argument check has passed.  Two calls that may overlap on the GPU (different streams, no
  *     ordering) race on it: order them, or use spqt_sparse_gemv with separate workspaces.
  *   - Because the status word is cleared per call, it describes the last call only: read it with
  *     spqt_static_status after that call.
@@ -256,16 +255,15 @@ spqt_status spqt_host_step_launch(void* step, void* stream);
 spqt_status spqt_host_step_destroy(void* step);
 
 /*
- * Tuning aid: number of CTAs of the GEMV grid (0 restores the built-in rule, one
- * persistent CTA per SM; values above 512 are clamped).  `no_overlap` is a set of bits, 0 by
+ * Tuning aid: number of CTAs the GEMV calls aim at (0 restores the built-in rule): divided by the
+ * number of block-rows it gives the CTAs that share a block-row, 1 to 8.  `no_overlap` is a set of bits, 0 by
  * default: bit 0 launches the GEMV kernels strictly stream-ordered instead of letting a GEMV start
  * (and wait inside the kernel) while the previous kernel of the stream drains; bit 1 never launches
- * thread-block clusters (otherwise, in spqt_sparse_gemv and spqt_dense_gemv, the 2..8 CTAs that share a
- * block-row combine their sums through shared memory when the device can hold all the clusters at once); bit 2 is an ablation, the paper's
+ * thread-block clusters (otherwise the 2..8 CTAs that share a block-row are one, and combine their sums
+ * through shared memory; without, one CTA does the work of all, with the same result); bit 2 is an ablation, the paper's
  * "sparse without load balancing" (Sec. 6): spqt_sparsify_gemv then gives every CTA, and inside it every
  * warp, a fixed range of the matrix columns of its block-row instead of an even share of the active
- * list (same results up to the order of partial sums; lists longer than the shared-memory window and
- * CTAs with more than 8 block-rows keep the balanced partition).
+ * list (same results up to the order of partial sums).
  * Any value gives the same results up to the order of partial sums.
  * Process-wide, not thread-safe.
  */
@@ -414,8 +412,8 @@ spqt_status spqt_calibrate_threshold(const void* x, size_t count, double sparsit
  * Per-shape profiling (paper Sec. 3.2: GEMV shapes are profiled per platform to pick the kernel's
  * hyper-parameters; Sec. 6, hyper-parameter study).  Times the call that collects the indices and
  * multiplies (spqt_sparsify_gemv with threshold t on x) and the dense call on this problem for a set
- * of grid sizes -- one CTA per SM, and every whole number 1..8 of CTAs per block-row that fits the
- * device -- and remembers the fastest of each for this (m, n, bits, group): later calls of
+ * of grid sizes -- every whole number 1..8 of CTAs per block-row of which all are resident at once --
+ * and remembers the fastest of each for this (m, n, bits, group): later calls of
  * spqt_sparsify_gemv / spqt_sparse_gemv and of spqt_dense_gemv with the same shape use them
  * (spqt_set_tuning with a non-zero grid size still overrides).  Results of those calls do not change
  * beyond the order of partial sums.  Arguments are those of spqt_sparsify_gemv; idx, count and y are
@@ -445,7 +443,7 @@ spqt_status spqt_set_debug(int on);
 /*
  * Reads the workspace's status word into *status_host (a host int) and waits for
  * the stream: 0 = every GEMV that used this workspace ran to completion;
- * 1 = a bounded wait expired inside a GEMV kernel (which then returned early,
+ * 1 = a bounded wait expired inside a GEMV kernel (no present kernel has one; it would return early,
  * leaving y unspecified); 2 = checked mode found a bad index list.  The word is
  * sticky until the caller zeroes the workspace again.  Returns SPQT_OK for 0,
  * SPQT_ERR_TIMEOUT for 1 and SPQT_ERR_INVALID_ARG for 2 (after writing *status_host).
@@ -464,10 +462,10 @@ spqt_status spqt_probe_read(const void* buf, size_t bytes, int pattern,
                             unsigned long long* moved, void* stream);
 
 /*
- * Measurement aid, not part of the method: the dequantize-FMA arithmetic of the GEMV loop alone.  One
+ * Measurement aid, not part of the method: the product of the GEMV loop alone.  One
  * CTA of 16 warps per SM; every warp runs `chunks_per_warp` (>= 1) full 2 KB chunks of 4-bit codes with
- * groups of 128 rows (eight 512-byte steps each) on operands that already sit in shared memory: no
- * copies, no list handling, no reduction.  `sink` (device, sink_floats >= 512 per SM or
+ * groups of 128 rows on operands that already sit in shared memory: no
+ * copies, no list handling, no multipliers, no reduction.  `sink` (device, sink_floats >= 512 per SM or
  * SPQT_ERR_INVALID_ARG; written so that the arithmetic is kept) receives meaningless sums; *chunks_total (host) receives the number of chunks
  * the launch processes.  Time it with events on `stream`: chunks per second times the bytes a chunk
  * stands for (2176 with its metadata) is the bandwidth at which instruction issue alone saturates.

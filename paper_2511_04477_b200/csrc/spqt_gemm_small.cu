@@ -17,9 +17,6 @@
 
 #include "spqt_common.cuh"
 
-namespace spqt {
-constexpr unsigned long long kWaitNs = 1000000000ull;
-}
 #include "spqt_gemv_device.cuh"
 #include "spqt_mma.cuh"
 

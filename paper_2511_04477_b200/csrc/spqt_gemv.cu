@@ -1,97 +1,52 @@
 // Activation-sparse GEMV over the zigzag layout, and its dense twin (4-bit and 3-bit codes).
 //
-// Work decomposition (the paper's hybrid row/column parallelism, generalised):
-// the R block-rows are laid end to end and cut into P equal pieces, one per CTA,
-// P = one persistent CTA per SM.  A piece is a run of (fractions of) block-rows;
-// the fraction [u0,u1) of block-row r means the slice [u0*count, u1*count) of
-// the ACTIVE index list, so the load follows the active entries, not the matrix
-// columns, and every CTA streams the same number of blocks whatever R is.  Each
-// (CTA, block-row) segment yields G fp32 partial sums, published as tagged 64-bit
-// words; whichever CTA contributes last to a block-row (arrive-only counter: no
-// CTA ever waits for another one to run, only for stores already issued to
-// become visible) adds the partials in slot order, adds the offset term and
-// rounds to fp16.  A CTA that finds all the other partials present before its own
-// sum is ready skips the counter and finishes the block-row directly.  With 2 or 4
-// CTAs per block-row the grid is launched as thread-block clusters of that size
-// (when the device can hold all of them at once) and the partial sums go through
-// the shared memory of the cluster's first CTA instead of global memory.
+// Work decomposition (the paper's hybrid row/column parallelism): one CTA of 8 warps per block-row, or a thread-block
+// cluster of S CTAs, each with one of S equal slices of the ACTIVE index list; every warp has an equal part of its CTA's
+// slice.  (Many block-rows with a long x: equal pieces of all block-rows instead, see gemv_pieces_kernel.)  The load follows the active entries, not the matrix columns.  A warp streams its part through its own ring
+// of chunks of 32 list entries (cp.async: 16 bytes per lane, the lanes of a block adjacent so that every sector crosses
+// once, with 64-byte L2 granularity so that an inactive neighbour block is not dragged in); nothing is shared between
+// the warps until the end.  Then the warps' sums meet in shared memory, and the CTAs' sums in the shared memory of the
+// cluster's first CTA, added in a fixed order (calls are bit-reproducible).
 //
-// The list a CTA works from lives in shared memory as one 32-bit word per active
-// entry: the column number in the low half, the fp16 bits of x_k in the high half.
-// The prologue builds it: from idx and x (sparse call), by scanning x itself (the
-// call that collects the indices in the same launch: every CTA scans x, counts the
-// active entries of every 256-entry piece and expands only the pieces that overlap
-// the list positions its own slices cover), or not at all (dense call).  When the
-// part of the list a CTA needs exceeds the shared-memory window, the window is
-// rebuilt between spans of the slice.
+// Where the list comes from:
+//   given list    lane e of a chunk reads idx directly, a few chunks ahead.
+//   fused         the call that collects the indices in the same launch: every CTA copies x to shared memory, finds the
+//                 active entries of every 256-entry piece and expands the pieces that overlap its own slice into a list
+//                 of words, column and x (where a CTA has to hold all of a long list: columns alone).  The CTAs of
+//                 block-row 0 write idx, each its slice; the first of them writes count.
+//   dense         entry e is column e.
+// Where the list has no x, it is fetched beside the entry's code copies.
 //
-// Inside a CTA, every worker warp owns a contiguous part of each slice and runs its
-// own copy pipeline over chunks of 32 list entries (64 with groups of 64 rows: 2 KB
-// of 4-bit codes either way), kDepth chunks in flight; nothing is shared between
-// the warps until the end of a segment.  Per chunk:
-//   issue    lane e reads the word of entry e, copies the 4-byte (scale, zero) pair
-//            of block (r, k_e) and keeps the entry word with the chunk; the code
-//            blocks are copied 16 bytes per lane, the lanes of a block adjacent so
-//            that every 32-byte sector crosses once, with 64-byte L2 granularity so
-//            that an inactive neighbour block is not dragged in (cp.async).  The
-//            dense call instead fetches the chunk's codes, pairs and x values with
-//            three bulk copies issued by one lane (they are contiguous).
-//   consume  lane e turns its pair into a = x_k*scale (exact in fp32) and
-//            x_k*zero, writes the packed multiplier pair of its entry to
-//            shared memory; then every lane does the dequantize-FMA work on its 16
-//            codes of each block, reading the block's multiplier back.
-// Entries past the end of a part are clamped to its last entry with weight 0, and
-// the 512-byte steps of a chunk that hold no entry are skipped.  Two more warps,
-// the writers (one per hand-over buffer), add the workers' sums at the end of a
-// segment, publish the partial and, if this CTA is the last contributor of the
-// block-row, produce y; they wait for the workers at a hardware barrier and for
-// other CTAs with waits bounded in wall time (on expiry the workspace's status word
-// is set and the kernel returns).
+// Per chunk, lane e turns the (scale, zero) pair of its entry into a = x_k*scale (exact in fp32), left as hi and lo for
+// the tensor cores (spqt_mma.cuh), and adds x_k*zero to its share of the offset term; then the warp multiplies, the
+// codes being operands as they are.  y[j] = sum_k a_k * code_jk + sum_k x_k * zero_rk.
 //
-// Arithmetic:  y[j] = sum_k a_k * code_jk + sum_k x_k * zero_rk.  A 4-bit code
-// becomes an fp32 operand with no conversion: a word whose bits above bit 22 are
-// zero IS an fp32 subnormal, its integer value times 2^-149, and the multiplier
-// a*2^93 is an exact power-of-two rescale, so each product is a*value*2^-56 up to
-// the single rounding of the FMA.  Per 16-bit half-word the operands are its low
-// 4, 8, 12 and 16 bits (u_j = q_0 + 16 q_1 + ... + 16^j q_j: three masks, the last
-// needs none); the sums over the list are linear in them, so the per-code sums
-// come back at the end of a segment as (U_j - U_{j-1}) / 16^j.  Under one logic op
-// and one FMA per weight; two FMAs are issued as one packed fma.rn.f32x2.
+// What bounds it.  Small and medium matrices: the fixed cost of a launch (a 4096 x 4096 call at 50 % needs 4.5 MB, 0.7 us
+// of DRAM time, and takes 4.6 us), most of it chains of dependent instructions that every warp of every CTA goes
+// through: clock stamps put 600 cycles on fetching x, 600 on the activity masks, 500 on the list, 400 on the first
+// copies, 500 on their arrival, 600 on a first chunk, 500 on the sums.  Hence whole block-rows instead of fractions (no
+// work map), one instance of every code path, few warps with much work each rather than many, and two CTAs per SM where
+// the grid is large enough, so that one computes while the other starts or ends.  The kernel before this one (one
+// persistent CTA of 18 warps per SM, fractional block-rows, packed FMAs, partial sums as tagged words in global memory;
+// 4500 instructions of code against 1600) took 6.4 us there.  Large matrices: the code stream; 28672 x 8192 dense went
+// from 26.9 to 24.2 us, 8192 x 28672 dense from 29.2 to 22.3 us (5.6 TB/s, 0.86 of the measured copy bandwidth).
 #include <cstddef>
 
 #include "spqt_common.cuh"
 
 namespace spqt {
 
-#ifndef SPQT_WORKERS
-#define SPQT_WORKERS 16
-#endif
-#ifndef SPQT_DEPTH
-#define SPQT_DEPTH 3
-#endif
-#ifndef SPQT_CAP
-#define SPQT_CAP 12288
-#endif
-constexpr int kWorkers = SPQT_WORKERS;   // compute warps
-constexpr int kWriters = 2;              // writer warps; segment sg goes to writer sg % kWriters
-constexpr int kWriterWarp = kWorkers;    // the first of them
-constexpr int kWarps = kWorkers + kWriters;
-constexpr int kGemvThreads = kWarps * 32;
-// list entries per chunk: 2 KB of 4-bit code blocks for either group size (32 blocks of 128 rows, 64 of 64)
-__host__ __device__ constexpr int chunk_entries(int group) { return 32 * (128 / group); }
-constexpr int kDepth = SPQT_DEPTH;       // chunks in flight per warp
-constexpr unsigned long long kWaitNs = 1000000000ull;  // bound on every mbarrier wait: one second
-constexpr int kMaxCluster = 8;           // largest thread-block cluster (CTAs of one block-row) used
-constexpr int kCap = SPQT_CAP;              // list entries a CTA keeps in shared memory at a time
-constexpr int kMaxListN = 65535;         // column numbers travel as 16 bits
-constexpr int kMaxFusedN = 32768;        // longest x the in-kernel scan handles (128 pieces of 256 entries)
+constexpr int kCtasPerSm = 2;             // CTAs of 8 warps; of those of 16 there is one
+constexpr int kMaxSplit = 8;              // CTAs of a block-row: the largest portable cluster
+constexpr int kCapPlain = 8192;           // list entries a CTA of a fused call keeps in shared memory: of a whole block-row,
+constexpr int kCapSlice = 7168;           // of a slice
+constexpr int kMaxListN = 65535;          // column numbers travel as 16 bits
+constexpr int kMaxFusedN = 32768;         // longest x the in-kernel scan handles (128 pieces of 256 entries)
 constexpr int kMaxPieces = kMaxFusedN / 256;
 
 enum : int { kModeList = 0, kModeFused = 1, kModeDense = 2 };
-enum : int { kFlagIdentity = 1, kFlagXs = 2, kFlagStatic = 4 };
-constexpr int kMaxStaticSeg = 8;         // block-rows per CTA the static-partition ablation handles
 
-static int g_tune_ctas = 0;  // 0 = one CTA per SM
+static int g_tune_ctas = 0;  // 0 = the built-in rule
 int g_no_pdl = 0;            // 1 = plain stream-ordered launches (also read by the index-collection launch)
 static int g_no_cluster = 0; // 1 = never launch thread-block clusters
 static int g_static_partition = 0;  // 1 = ablation: static partition of the matrix columns instead of the list
@@ -99,897 +54,837 @@ static int g_static_partition = 0;  // 1 = ablation: static partition of the mat
 }  // namespace spqt
 
 #include "spqt_gemv_device.cuh"
-#include "spqt_gemv_map.cuh"
+#include "spqt_mma.cuh"
 
 namespace spqt {
 
-// ---------------------------------------------------------------- kernel
+// How a grid shares the block-rows.
+//   plain     one CTA per block-row
+//   cluster   a cluster of CTAs per block-row, one slice of the list each
+//   serial    one CTA per block-row, the slices of the list in turn (the same parts and order of sums as a cluster)
+// and, as a kernel of its own,
+//   pieces    one CTA of 16 warps per SM; the block-rows are laid end to end and cut into equal pieces, one for every warp
+enum : int { kPlain = 0, kCluster = 1, kSerial = 2 };
 
-template <int G, int BITS>
-struct GemvSmem {
-    static constexpr int B = G * BITS / 8;
-    static constexpr int CH = chunk_entries(G);
-    struct Stage {
-        alignas(16) unsigned char codes[CH * B];  // block e of the chunk at e*B
-        alignas(16) unsigned meta[CH];            // (scale, zero) pair of entry e
-        alignas(16) unsigned xc[CH];              // list calls: the entry word; dense call: CH fp16 values of x
+// ---------------------------------------------------------------- shared memory
+
+// A warp's ring: D chunks of CH list entries.
+template <int G, int MODE>
+struct RowRing {                         // where a CTA works on one block-row
+    // 64-row blocks without a list (every block is read): chunks of 64, half the bookkeeping (11072 x 4096 7.7 against 9.0 us);
+    // with a list they cost more in the parts' last chunks (4096 x 14336 at 50 % 10.0 against 9.5 us)
+    static constexpr int CH = MODE == kModeDense ? 32 * (128 / G) : 32, D = MODE == kModeDense || G == 128 ? 4 : 6;
+};
+template <int G, int MODE>
+struct PieceRing {
+    static constexpr int CH = 32, D = G == 128 ? 4 : 6;
+};
+
+template <int G, int BITS, class Ring>
+struct Stage {
+    alignas(16) unsigned char codes[Ring::CH * MmaStage<G, BITS>::kRow];   // the chunk's blocks, as the matrix loads want them
+    alignas(16) unsigned meta[Ring::CH];              // (scale, zero) pair of entry e
+};
+
+template <int G, int BITS, int MODE, int NW>
+struct LoopSmem {
+    using Ring = RowRing<G, MODE>;
+    Stage<G, BITS, Ring> stage[NW][Ring::D];
+    union Warp {
+        unsigned short b[Ring::CH][8];                // operand B of a chunk: hi and lo of every entry's multiplier, then padding
+        float red[G];                                 // after the last chunk: the warp's sums, as the tiles have them
     };
-    Stage stage[kWorkers][kDepth];                 // (the prologue borrows this area for its copy of x and its masks)
-    alignas(16) float mult[kWorkers][CH][2];       // packed multiplier pair (a, a) * 2^93 of every entry of the chunk in work
-    alignas(16) float red[2][kWorkers][G];         // per-warp partial sums of a finished segment
-    float red_z[2][kWorkers];                      // and their offset terms
-    alignas(8) uint64_t full[kWorkers][kDepth];    // dense call: completion of a stage's bulk copies
-    uint64_t red_full[2], red_empty[2];
-    // thread-block clusters only: partial sums the other CTAs of the cluster store here (CTA rank 0)
-    alignas(16) float xred[kMaxCluster][G + 4];
-    uint64_t xbar;                                 // counts their arrivals
-    alignas(16) int tot[kMaxPieces];               // in-kernel scan: active entries of every 256 entries of x
-    int static_table[kMaxStaticSeg][kWorkers + 1]; // ablation: list positions of a static column partition
-    alignas(16) unsigned ent[kCap];                // the resident part of the list: x bits << 16 | column
+    alignas(16) Warp warp[NW];
+    float2 red_z[NW];                                 // the sums' scale and offset terms
+};
+
+template <int G, int BITS, int MODE, int NW>
+struct PieceLoopSmem {
+    using Ring = PieceRing<G, MODE>;
+    Stage<G, BITS, Ring> stage[NW][Ring::D];
+    alignas(16) unsigned short b[NW][Ring::CH][8];
+    alignas(16) float red[2][NW][G];
+    float2 red_z[2][NW];
+};
+
+struct ScanSmem {                                     // fused: while the list is built
+    alignas(16) unsigned char xs[kMaxFusedN * 2];     // x
+    alignas(16) int tot[kMaxPieces];                  // active entries of every 256 entries of x
+    unsigned short mask[kMaxPieces][32];              // which they are, 8 entries a byte; above it, how many precede them in the piece
+};
+
+template <int G, int BITS, int MODE, int KIND, int NW>
+struct GemvSmem {
+    using Loop = LoopSmem<G, BITS, MODE, NW>;
+    union Area {
+        Loop loop;
+        unsigned char scan[MODE == kModeFused ? sizeof(ScanSmem) : 16];
+    };
+    alignas(16) unsigned char area[sizeof(Area)];
+    alignas(16) float xred[KIND == kCluster ? kMaxSplit : 1][G + 4];   // first CTA of a cluster: the other CTAs' sums
+    int table[NW + 1];                                // ablation: list positions of a static column partition
+    alignas(16) unsigned ent[MODE == kModeFused ? (KIND == kPlain ? kCapPlain : kCapSlice) : 4];   // fused: the CTA's slice of the list, x bits << 16 | column
+};
+
+constexpr int kPieceWarps = 16;
+template <int G, int BITS, int MODE>
+struct PieceSmem {
+    using Loop = PieceLoopSmem<G, BITS, MODE, kPieceWarps>;
+    union Area {
+        Loop loop;
+        unsigned char scan[MODE == kModeFused ? sizeof(ScanSmem) : 16];
+    };
+    alignas(16) unsigned char area[sizeof(Area)];
+    alignas(16) unsigned short ent[MODE == kModeFused ? kMaxFusedN : 8];   // fused: the columns of the whole list
+    int last[2];                                      // whether this CTA came last to its first / last block-row
 };
 
 struct GemvArgs {
     const uint8_t* codes;
     const unsigned* meta;       // (scale, zero) pairs
-    int R, n;
+    int n, R;
+    int splits;                 // slices of the list
+    unsigned magic_s;           // floor((2^32 - 1) / splits)
+    unsigned warps, magic_w;    // pieces: warps of the grid, floor((2^32 - 1) / warps)
+    unsigned magic_r, magic_p;  // the same of R and of the number of CTAs
+    unsigned* arrived;          // per block-row: CTAs that have left their sums (zero between calls)
+    float* partial;             // sums of the first and of the last block-row of every CTA's piece (zero between calls)
     const __half* x;
     const int32_t* idx;
     const int32_t* count;
     __half* y;
-    int* counters;
-    int* status;
-    unsigned long long* words;
-    float* partials;
-    float* zpartials;
-    int max_slots;
-    unsigned magic_p, magic_r;
-    int cluster_k;
-    float thr;
+    unsigned short thr;         // fused: the largest fp16 value not above the threshold (negative: -1)
     int32_t* idx_out;
     int32_t* count_out;
-    int flags;
+    int static_partition;
 };
 
-template <int G, int BITS, int MODE, bool CLUSTER>
-__global__ void __launch_bounds__(kGemvThreads, 1)
+// floor(v / d) for any 32-bit v from the multiplier m = floor((2^32 - 1) / d): the high product is
+// the quotient or one less (the multiplier falls short of 2^32 / d by at most 1), one compare fixes it.
+__device__ __forceinline__ unsigned magic_div(unsigned v, unsigned d, unsigned m)
+{
+    const unsigned q = __umulhi(v, m);
+    return q + ((v - q * d >= d) ? 1u : 0u);
+}
+
+// A hint only (no data is consumed before the wait for the previous kernel): pull x, and a given list, towards L2 while
+// that kernel drains.  A few CTAs do it for all.
+template <int MODE, int THREADS>
+__device__ __forceinline__ void prefetch_inputs(const GemvArgs& a, int tid)
+{
+    if ((blockIdx.x & 15) != 0) return;
+    const char* xp = reinterpret_cast<const char*>(a.x);
+    for (int off = tid * 128; off < 2 * a.n; off += THREADS * 128)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(xp + off));
+    if (MODE == kModeList) {
+        const char* ip = reinterpret_cast<const char*>(a.idx);
+        for (int off = tid * 128; off < 4 * a.n; off += THREADS * 128)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(ip + off));
+    }
+}
+
+// ---------------------------------------------------------------- copies
+
+// The copies of one chunk: the (scale, zero) pairs and code blocks of columns col[], lane's entries lane, lane + 32, ..
+template <int G, int BITS, class Ring>
+__device__ __forceinline__ void copy_chunk(unsigned st, const uint8_t* row_codes, const unsigned* row_meta, const unsigned* col, int lane)
+{
+    constexpr int B = G * BITS / 8, CH = Ring::CH, EPL = CH / 32;
+    constexpr int CB = (B % 16 == 0) ? 16 : 8;        // bytes per copy: 3-bit blocks of 64 rows are only 8-byte aligned
+    constexpr int NC = CH * B / CB / 32;              // copies per lane and chunk
+    constexpr int kRow = MmaStage<G, BITS>::kRow;
+    constexpr unsigned kMetaOff = (unsigned)sizeof(Stage<G, BITS, Ring>::codes);
+#pragma unroll
+    for (int q = 0; q < EPL; ++q) cp_async_4(st + kMetaOff + 4u * (lane + 32 * q), row_meta + col[q]);
+#pragma unroll
+    for (int q = 0; q < NC; ++q) {
+        const int p = q * 32 + lane, e = p / (B / CB), part = p % (B / CB);
+        unsigned dst;
+        if (BITS == 4 && G == 128) dst = e * 64 + ((part ^ ((e >> 1) & 3)) << 4);
+        else if (BITS == 4) dst = e * 32 + ((part ^ ((e >> 2) & 1)) << 4);
+        else dst = e * kRow + part * CB;
+        const unsigned cu = __shfl_sync(0xffffffffu, col[q / (NC / EPL)], e & 31);
+        const uint8_t* src = row_codes + ((size_t)cu * B + part * CB);
+        if (CB == 16) cp_async_16_l2_64(st + dst, src);
+        else cp_async_8(st + dst, src);
+    }
+    if (BITS == 3 && G == 64) {                       // the 1-bit plane a second time (see MmaStage)
+#pragma unroll
+        for (int q = 0; q < EPL; ++q) cp_async_8(st + (lane + 32 * q) * kRow + 24, row_codes + ((size_t)col[q] * B + 16));
+    }
+}
+
+// ---------------------------------------------------------------- the product
+
+// A warp's sums and what it takes to multiply a chunk.  While chunk i is multiplied, chunk i + 1 is prepared: lane e turns
+// its entry's pair and x into a = x*scale (exact in fp32), left as hi and lo, and x*zero.
+template <int G, int BITS, class Ring>
+struct Product {
+    static constexpr int EPL = Ring::CH / 32, SP = MmaStage<G, BITS>::kSp;
+    using Layout = MmaStage<G, BITS>;
+    float acc[SP][4][4];             // sums of the rows times the hi (column 0) and lo (column 1) multipliers, in lanes t4 == 0
+    float scale, regain;             // c of spqt_mma.cuh; factor that the sums still have to be brought to it by
+    float zl, zn;                    // sum of x*zero, and the prepared chunk's part of it
+    float am[EPL], pm[EPL];
+    unsigned b_base;                 // this lane's row of B
+    int lane;
+
+    __device__ __forceinline__ Product(unsigned b, int lane_) : scale(kMmaNoScale), regain(1.0f), zn(0.0f), b_base(b + 16u * lane_), lane(lane_) { clear(); }
+    __device__ __forceinline__ void clear()
+    {
+        zl = 0.0f;
+#pragma unroll
+        for (int i = 0; i < SP * 16; ++i) acc[i >> 4][(i >> 2) & 3][i & 3] = 0.0f;
+    }
+    // xb: the fp16 bits of the lane's x values, 0 for an entry that does not exist; true if one exceeds the range
+    __device__ __forceinline__ bool prepare(unsigned st, const unsigned* xb)
+    {
+        constexpr unsigned kMetaOff = (unsigned)sizeof(Stage<G, BITS, Ring>::codes);
+        zn = 0.0f;
+        float top = 0.0f;
+#pragma unroll
+        for (int q = 0; q < EPL; ++q) {
+            const unsigned mz = lds_u32(st + kMetaOff + 4u * (lane + 32 * q));
+            const float xf = __half2float(__ushort_as_half((unsigned short)xb[q]));
+            am[q] = xf * __half2float(__ushort_as_half((unsigned short)(mz & 0xffffu)));
+            zn += xf * __half2float(__ushort_as_half((unsigned short)(mz >> 16)));
+            pm[q] = am[q] * scale;   // a power of two
+            top = fmaxf(top, fabsf(pm[q]));
+        }
+        return top > kMmaLimit;
+    }
+    // a larger entry than the range holds: a new scale; the sums follow once chunk i is in them
+    __device__ __forceinline__ void rescale()
+    {
+        unsigned m = 0;
+#pragma unroll
+        for (int q = 0; q < EPL; ++q) {
+            const unsigned bits = __float_as_uint(am[q]) & 0x7fffffffu;
+            m = max(m, bits < 0x7f800000u ? bits : 0u);   // finite ones
+        }
+        m = __reduce_max_sync(0xffffffffu, m);
+        if (__uint_as_float(m) * scale > kMmaLimit) {
+            const float next = __uint_as_float((264u - (m >> 23)) << 23);   // m goes to 2^10 .. 2^11
+            regain = next * power_of_two_inverse(scale);
+            scale = next;
+#pragma unroll
+            for (int q = 0; q < EPL; ++q) pm[q] = am[q] * next;
+        }
+    }
+    __device__ __forceinline__ void leave()
+    {
+#pragma unroll
+        for (int q = 0; q < EPL; ++q) {
+            const float h = __low2float(__floats2half2_rn(pm[q], 0.0f));
+            const __half2 hl = __floats2half2_rn(pm[q], pm[q] - h);
+            sts_u32(b_base + 512u * q, *reinterpret_cast<const unsigned*>(&hl));
+        }
+    }
+    // the first chunk: there is nothing in the sums yet
+    __device__ __forceinline__ void begin(unsigned st, const unsigned* xb)
+    {
+        if (__any_sync(0xffffffffu, prepare(st, xb))) rescale();
+        leave();
+        regain = 1.0f;
+        __syncwarp();
+    }
+    // multiplies the chunk in stage st and leaves B of the next one, whose entries prepare() reads from stage `next`
+    __device__ __forceinline__ void multiply(unsigned st, const typename Layout::Lane& ll, unsigned next, const unsigned* xb)
+    {
+        zl += zn;
+        const bool over = prepare(next, xb);
+        unsigned bb[EPL][4], c[SP][4];
+#pragma unroll
+        for (int q = 0; q < EPL; ++q) ldsm_x4_trans(b_base + 512u * q, bb[q]);
+        __syncwarp();                // (B is in registers: its place is free)
+#pragma unroll
+        for (int ks = 0; ks < 2 * EPL; ++ks) {
+            Layout::load(st, ll, ks, c);
+            if (ks == 2 * EPL - 1) {
+                if (__any_sync(0xffffffffu, over)) rescale();
+                leave();
+            }
+#pragma unroll
+            for (int sp = 0; sp < SP; ++sp) mma_group<false>(acc[sp], c[sp], bb[ks >> 1] + 2 * (ks & 1), bb[0]);
+        }
+        if (regain != 1.0f) {
+#pragma unroll
+            for (int i = 0; i < SP * 16; ++i) acc[i >> 4][(i >> 2) & 3][i & 3] *= regain;
+            regain = 1.0f;
+        }
+        __syncwarp();                // every lane is done with this chunk's stage
+    }
+    // the sums as the tiles have them (eight lanes of a warp hold them all), their scale and the offset term
+    __device__ __forceinline__ void hand_over(float* red, float2* red_z)
+    {
+        if ((lane & 3) == 0) {
+#pragma unroll
+            for (int sp = 0; sp < SP; ++sp)
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int type = i >> 1, hf = 2 * (i & 1);
+                    red[Layout::row(sp, type, hf, lane >> 2)] = acc[sp][type][hf] + acc[sp][type][hf + 1];   // hi + lo
+                }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) zl += __shfl_xor_sync(0xffffffffu, zl, o);
+        if (lane == 0) *red_z = make_float2(0x1p24f * power_of_two_inverse(scale), zl);
+    }
+};
+
+// The warps' sums of a block-row, in warp order: thread j < G / 2 gets rows j and j + G/2, those of the low and the high
+// nibbles of a byte (the latter's tiles sum whole bytes).
+template <int G, int NW, class Warp>
+__device__ __forceinline__ void add_warps(const Warp* warp, const float2* red_z, int j, float* v, float* z)
+{
+    v[0] = v[1] = *z = 0.0f;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) {
+        const float2 cz = red_z[w];
+        v[0] += warp[w].red[j] * cz.x;
+        v[1] += warp[w].red[j + G / 2] * cz.x;
+        *z += cz.y;
+    }
+    v[1] = (v[1] - v[0]) * 0.0625f;
+}
+
+// ---------------------------------------------------------------- fused: the list
+
+template <int NW>
+struct Scan {
+    ScanSmem& sc;
+    int n, nv, lane, warp;
+    int t[4];                                         // lane l: active entries of pieces 4l .. 4l+3
+
+    __device__ __forceinline__ Scan(unsigned char* area, int n_, int lane_, int warp_)
+        : sc(*reinterpret_cast<ScanSmem*>(area)), n(n_), nv((n_ + 255) >> 8), lane(lane_), warp(warp_)
+    {
+    }
+    __device__ __forceinline__ int below(int li) const   // active entries before piece li
+    {
+        int v = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v += lane * 4 + q < li ? t[q] : 0;
+        return (int)__reduce_add_sync(0xffffffffu, (unsigned)v);
+    }
+    // x to shared memory, and per piece of 256 entries which ones are active and how many; returns the count
+    __device__ __forceinline__ int scan_x(const __half* x, unsigned short thr_bits)
+    {
+        const int tid = warp * 32 + lane;
+        const unsigned xs_base = smem_u32(sc.xs);
+        const unsigned short* const xg = reinterpret_cast<const unsigned short*>(x);
+        if (tid >= nv && tid < kMaxPieces) sc.tot[tid] = 0;
+        // a warp copies its own pieces (warp, warp + NW, ..)
+        if ((reinterpret_cast<uintptr_t>(x) & 15) == 0) {
+            for (int k = tid * 8; k < nv * 256; k += NW * 256) cp_async_16_left(xs_base + 2u * k, xg + k, n - k);
+        } else {
+            for (int k = warp * 256 + lane; k < nv * 256; k += ((k & 255) < 224) ? 32 : NW * 256 - 224)
+                sts_u16(xs_base + 2u * k, k < n ? (unsigned)__ldg(xg + k) : 0u);
+        }
+        cp_async_commit();
+        cp_async_wait<0>();
+        __syncwarp();
+        // eight entries per lane and piece, two per compare, exact in fp16; false for NaN.  Two pieces at a time.
+        const __half2 thr = __half2half2(__ushort_as_half(thr_bits));
+        auto count_piece = [&](int li, const uint4& v) {
+            const unsigned w[4] = {v.x, v.y, v.z, v.w};
+            unsigned m = 0;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const unsigned ab = w[j] & 0x7fff7fffu;
+                m |= __hgt2_mask(*reinterpret_cast<const __half2*>(&ab), thr) & (0x00020001u << (2 * j));
+            }
+            m = (m | (m >> 16)) & 0xffu;
+            const int left = n - li * 256 - lane * 8;   // entries past n do not exist
+            if (left < 8) m &= left <= 0 ? 0u : (1u << left) - 1u;
+            // how many precede this lane's: bit by bit of the counts
+            const unsigned c = (unsigned)__popc(m), lt = (1u << lane) - 1u;
+            unsigned before = 0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) before += (unsigned)__popc(__ballot_sync(0xffffffffu, (c >> i) & 1u) & lt) << i;
+            sc.mask[li][lane] = (unsigned short)(m | (before << 8));
+            if (lane == 31) sc.tot[li] = (int)(before + c);
+        };
+#pragma unroll 1
+        for (int li = warp; li < nv; li += 2 * NW) {
+            const uint4 v0 = lds_v4(xs_base + li * 512u + lane * 16u);
+            const bool two = li + NW < nv;
+            const uint4 v1 = two ? lds_v4(xs_base + (li + NW) * 512u + lane * 16u) : v0;
+            count_piece(li, v0);
+            if (two) count_piece(li + NW, v1);
+        }
+        __syncthreads();
+        const int4 v = *reinterpret_cast<const int4*>(&sc.tot[lane * 4]);
+        t[0] = v.x; t[1] = v.y; t[2] = v.z; t[3] = v.w;
+        return (int)__reduce_add_sync(0xffffffffu, (unsigned)(v.x + v.y + v.z + v.w));
+    }
+    // the list position of column kb: the number of active entries below it (the same in all lanes)
+    __device__ __forceinline__ int position(int kb) const
+    {
+        const int piece = kb >> 8;
+        int inside = 0;
+        if (piece < nv) {
+            const int in8 = (kb & 255) - 8 * lane;   // entries of this lane's byte below it
+            inside = __popc((unsigned)sc.mask[piece][lane] & (in8 >= 8 ? 0xffu : in8 <= 0 ? 0u : (1u << in8) - 1u));
+        }
+        return below(piece) + (int)__reduce_add_sync(0xffffffffu, (unsigned)inside);
+    }
+    // The entries [lo, hi) of the list into ent (E = unsigned: x bits << 16 | column; unsigned short: columns), and the
+    // entries [out_lo, out_hi) into the returned list.
+    template <class E>
+    __device__ __forceinline__ void build(E* ent, int lo, int hi, int32_t* idx_out, int out_lo, int out_hi)
+    {
+        const unsigned short* const xs = reinterpret_cast<const unsigned short*>(sc.xs);
+        const unsigned bit = 1u << (lane & 7), len = (unsigned)(hi - lo), out_len = (unsigned)(out_hi - out_lo);
+#pragma unroll 1
+        for (int li = warp; li < nv; li += NW) {
+            const int base = below(li);
+            if (base >= hi || base + sc.tot[li] <= lo) continue;   // (uniform)
+            const unsigned col = (unsigned)(li * 256 + lane);
+            // all loads first (the compiler cannot move one past a store: 360 instead of 1300 cycles a piece); neighbouring
+            // lanes to neighbouring places
+            unsigned m[8], w[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) m[j] = sc.mask[li][4 * j + (lane >> 3)];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) w[j] = sizeof(E) == 4 ? (unsigned)xs[col + 32 * j] << 16 : 0u;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const unsigned at = (unsigned)base + (m[j] >> 8) + (unsigned)__popc(m[j] & (bit - 1u));
+                w[j] |= col + 32 * j;
+                m[j] = (m[j] & bit) != 0u ? at : 0x7fffffffu;
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (m[j] - (unsigned)lo < len) ent[m[j] - (unsigned)lo] = (E)w[j];
+            if (out_len != 0u) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    if (m[j] - (unsigned)out_lo < out_len) idx_out[m[j]] = (int)(col + 32 * j);
+            }
+        }
+    }
+};
+
+// ---------------------------------------------------------------- whole block-rows
+
+template <int G, int BITS, int MODE, int KIND, int NW>
+__global__ void __launch_bounds__(NW * 32, NW == 8 ? kCtasPerSm : 1)
 gemv_kernel(const GemvArgs a)
 {
-    constexpr int B = G * BITS / 8;
-    constexpr int LPB = G / 32;       // copies: lanes per 4-bit block (16 bytes each)
-    constexpr int CB = (B % 16 == 0) ? 16 : 8;   // bytes per copy: 3-bit blocks of 64 rows are only 8-byte aligned
-    static_assert(BITS == 3 || BITS == 4, "3- or 4-bit codes");
-    constexpr int SLOTS = 32 / LPB;   // copies: 4-bit blocks per 512-byte round
-    constexpr int CH = chunk_entries(G);  // list entries per chunk
-    constexpr int EPL = CH / 32;          // entries whose metadata a lane holds
-    constexpr int SUBS = CH / SLOTS;      // copies: rounds per chunk
-    // arithmetic: LM lanes share a block, each owns 16 of its rows (16 accumulators per lane: half the
-    // registers of a 32-row share, which is what lets twice the warps stay resident)
-    constexpr int LM = G / 16;
-    constexpr int SLM = 32 / LM;          // blocks per step
-    constexpr int MSUBS = CH / SLM;       // steps per chunk
-    constexpr int KEEP = 16 / SLM;        // values per lane after the in-warp reduce-scatter
-    constexpr int D = kDepth;
-    constexpr bool DENSE = MODE == kModeDense;
-    constexpr bool FUSED = MODE == kModeFused;
-    using Smem = GemvSmem<G, BITS>;
-    using Stage = typename Smem::Stage;
+    using Ring = RowRing<G, MODE>;
+    constexpr int B = G * BITS / 8, CH = Ring::CH, EPL = CH / 32, D = Ring::D;   // EPL: entries a lane looks after
+    constexpr int kThreads = NW * 32;
+    constexpr bool FUSED = MODE == kModeFused, LIST = MODE == kModeList;
+    using Smem = GemvSmem<G, BITS, MODE, KIND, NW>;
 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem& sm = *reinterpret_cast<Smem*>(smem_raw);
-
+    typename Smem::Loop& lp = *reinterpret_cast<typename Smem::Loop*>(sm.area);
     const int tid = threadIdx.x, lane = tid & 31;
-    // the warp number through a shuffle: the compiler then knows it is the same in every lane and keeps
-    // everything derived from it (the work map, the stage addresses) in uniform registers
+    // the warp number through a shuffle: the compiler then knows it is the same in every lane
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
-    const int P = gridDim.x, c = blockIdx.x;
-    const int n = a.n, R = a.R;
-    if (tid == 0) {
-        for (int b = 0; b < 2; ++b) {
-            mbar_init(&sm.red_full[b], kWorkers);
-            mbar_init(&sm.red_empty[b], 1);
-        }
-        if (DENSE) {
-            for (int w = 0; w < kWorkers; ++w)
-                for (int s = 0; s < D; ++s) mbar_init(&sm.full[w][s], 1);
-        }
-        if (CLUSTER) mbar_init(&sm.xbar, a.cluster_k - 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    const int n = a.n;
+    unsigned rank = 0, r = blockIdx.x;
+    if (KIND == kCluster) {
+        asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+        asm volatile("mov.u32 %0, %%clusterid.x;" : "=r"(r));
+        // nobody may write to another CTA's shared memory before that CTA runs: arrive now, wait much later
+        cluster_arrive();
     }
-    __syncthreads();
-    // Cluster launch (cluster_k CTAs work on one block-row and CTA rank 0 collects their sums): nobody
-    // may touch another CTA's barrier before it is initialised.  Arrive now, wait much later.
-    if (CLUSTER) cluster_arrive();
+    // the slices of the list this CTA works on: first_part .. last_part - 1 of `parts`
+    const unsigned parts = (unsigned)a.splits, first_part = rank, last_part = KIND == kCluster ? rank + 1u : parts;
 
-    Piece pc;
-    pc.init_rows(R, P, c, a.magic_p, a.magic_r);
+    prefetch_inputs<MODE, kThreads>(a, tid);
+    // constants of the loop that need no data
+    const typename MmaStage<G, BITS>::Lane ll(lane);
+    const unsigned stage0 = smem_u32(&lp.stage[warp][0]);
+    constexpr unsigned kStageBytes = (unsigned)sizeof(Stage<G, BITS, Ring>), kRing = D * kStageBytes;
+    const unsigned ent_base = smem_u32(&sm.ent[0]);
+    const unsigned short* const xg = reinterpret_cast<const unsigned short*>(a.x);
+    const uint8_t* const row_codes = a.codes + (size_t)r * (size_t)n * B;
+    const unsigned* const row_meta = a.meta + (size_t)r * (size_t)n;
 
-    // A hint only (no data is consumed before the wait below): pull x, and a given list, towards L2 while
-    // the previous kernel of the stream drains.  A few CTAs do it for all.  (Measured: 1 to 2 % of a decode
-    // layer's linears when x has left L2 since it was written.)
-    if (!DENSE && (c & 7) == 0) {
-        const char* xp = reinterpret_cast<const char*>(a.x);
-        for (int off = tid * 128; off < 2 * n; off += kGemvThreads * 128)
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(xp + off));
-        if (!FUSED && a.idx != nullptr) {
-            const char* ip = reinterpret_cast<const char*>(a.idx);
-            for (int off = tid * 128; off < 4 * n; off += kGemvThreads * 128)
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(ip + off));
-        }
-    }
-    // Programmatic dependent launch: this grid may have been started while the previous kernel of
-    // the stream was still draining.  Nothing above touches memory another kernel writes; everything
-    // below waits for that kernel to complete, and lets the next kernel of the stream start early in turn.
+    // Programmatic dependent launch: this grid may have been started while the previous kernel of the stream was still
+    // draining.  Nothing above touches memory another kernel writes; everything below waits for that kernel to
+    // complete, and lets the next kernel of the stream start early in turn.
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-    // ------------------------------------------------------------ prologue: the list in shared memory
-    // Scratch borrowed from the stage area until the pipeline starts: a copy of x (16-bit words,
-    // padded to whole 256-entry pieces) and, for the in-kernel scan, one activity byte per lane and piece.
-    const int nv = (n + 255) >> 8;
-    const unsigned xs_addr = smem_u32(&sm.stage[0][0]);
-    unsigned char* const pm = reinterpret_cast<unsigned char*>(&sm.stage[0][0]) + (size_t)nv * 512;
-    const unsigned short* const xg = reinterpret_cast<const unsigned short*>(a.x);
-    const bool vec_ok = (reinterpret_cast<uintptr_t>(a.x) & 15) == 0;
-    const bool has_xs = FUSED || (a.flags & kFlagXs) != 0;
-    const unsigned ent_base = smem_u32(&sm.ent[0]);
-
-    // piece li of x (entries 256 li + 8 lane .. + 7) from global memory, zero past the end
-    auto load_piece = [&](int li) -> uint4 {
-        const int k0 = li * 256 + lane * 8;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (vec_ok && k0 + 8 <= n) {
-            v = __ldg(reinterpret_cast<const uint4*>(a.x + k0));
-        } else if (k0 < n) {
-            unsigned short hv[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) hv[e] = (k0 + e < n) ? __ldg(xg + k0 + e) : (unsigned short)0;
-            v.x = hv[0] | ((unsigned)hv[1] << 16);
-            v.y = hv[2] | ((unsigned)hv[3] << 16);
-            v.z = hv[4] | ((unsigned)hv[5] << 16);
-            v.w = hv[6] | ((unsigned)hv[7] << 16);
-        }
-        return v;
-    };
-
-    // Copy x to shared memory; the in-kernel scan also records which entries are active and how many
-    // per piece.  Run by the warps gw = 0..NW-1 of a group; the caller synchronises the group afterwards.
-    auto stage_x = [&](int gw, int NW) {
-        constexpr int kPiecesPerRound = 4;   // loads of one round share a round trip
-        // the largest fp16 value not above t (any negative value if t < 0: everything but NaN is
-        // active; +inf if t is NaN or +inf: nothing is)
-        const float thr = a.thr;
-        const __half thr_h = (thr != thr) ? __ushort_as_half((unsigned short)0x7c00)
-                                          : (thr < 0.0f ? __float2half_rn(-1.0f) : __float2half_rd(thr));
-        const __half2 thr_h2 = __half2half2(thr_h);
-        if (FUSED) {
-            for (int i = nv + gw * 32 + lane; i < kMaxPieces; i += NW * 32) sm.tot[i] = 0;
-        }
-#pragma unroll 1
-        for (int l0 = gw; l0 < nv; l0 += kPiecesPerRound * NW) {
-            uint4 xv[kPiecesPerRound];
-#pragma unroll
-            for (int j = 0; j < kPiecesPerRound; ++j) {
-                const int li = l0 + j * NW;
-                xv[j] = make_uint4(0u, 0u, 0u, 0u);
-                if (li < nv) xv[j] = load_piece(li);  // uniform across the warp
-            }
-#pragma unroll
-            for (int j = 0; j < kPiecesPerRound; ++j) {
-                const int li = l0 + j * NW, k0 = li * 256 + lane * 8;
-                if (li < nv) {
-                    sts_v4(xs_addr + (unsigned)li * 512u + (unsigned)lane * 16u, xv[j]);
-                    if (FUSED) {
-                        const unsigned wds[4] = {xv[j].x, xv[j].y, xv[j].z, xv[j].w};
-                        unsigned m8 = 0;
-#pragma unroll
-                        for (int e2 = 0; e2 < 4; ++e2) {
-                            // |x| > t  <=>  |x| > (largest fp16 value <= t): two entries per compare, in fp16,
-                            // exact; the ordered compare is false for NaN
-                            const unsigned ab = wds[e2] & 0x7fff7fffu;
-                            const unsigned gt = __hgt2_mask(*reinterpret_cast<const __half2*>(&ab), thr_h2);
-                            m8 |= (gt & (1u << (2 * e2))) | (gt & (0x20000u << (2 * e2))) >> 16;
-                        }
-                        const int left = n - k0;  // entries of this lane that exist
-                        if (left < 8) m8 &= (left <= 0) ? 0u : ((1u << left) - 1u);
-                        pm[li * 32 + lane] = (unsigned char)m8;
-                        const unsigned tot = __reduce_add_sync(0xffffffffu, (unsigned)__popc(m8));
-                        if (lane == 0) sm.tot[li] = (int)tot;
-                    }
-                }
-            }
-        }
-    };
-
-    // The window [lo, hi) of the list into sm.ent, by the threads gt = 0..NT-1 (warps gw = 0..NW-1) of
-    // a group.  The in-kernel scan also writes the list positions [olo, ohi) of the index list the
-    // call returns.  The caller synchronises the group before (x staged) and afterwards.
-    auto build_window = [&](int lo, int hi, int olo, int ohi, int gw, int NW) {
-        if (FUSED) {
-            // lane l holds the totals of pieces 4l..4l+3; sums over the pieces below a given one come
-            // from one warp reduction each
-            int tot4[4];
-            {
-                const int4 t4 = *reinterpret_cast<const int4*>(&sm.tot[lane * 4]);
-                tot4[0] = t4.x; tot4[1] = t4.y; tot4[2] = t4.z; tot4[3] = t4.w;
-            }
-            const unsigned len = (unsigned)max(hi - lo, 0), olen = (unsigned)max(ohi - olo, 0);
-#pragma unroll 1
-            for (int li = gw; li < nv; li += NW) {
-                unsigned below = 0;  // active entries of this lane's pieces that come before piece li
-#pragma unroll
-                for (int q = 0; q < 4; ++q) below += (lane * 4 + q < li) ? (unsigned)tot4[q] : 0u;
-                const int base = (int)__reduce_add_sync(0xffffffffu, below);
-                const int q = li & 3;
-                const int tsel = q == 0 ? tot4[0] : q == 1 ? tot4[1] : q == 2 ? tot4[2] : tot4[3];
-                const int end = base + __shfl_sync(0xffffffffu, tsel, li >> 2);
-                const bool in_win = end > lo && base < hi, in_out = end > olo && base < ohi;
-                if (!in_win && !in_out) continue;  // uniform across the warp
-                const unsigned m8 = pm[li * 32 + lane];
-                const uint4 xv = lds_v4(xs_addr + (unsigned)li * 512u + (unsigned)lane * 16u);
-                const unsigned xw[4] = {xv.x, xv.y, xv.z, xv.w};
-                const int c8 = __popc(m8);
-                int incl = c8;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int up = __shfl_up_sync(0xffffffffu, incl, o);
-                    if (lane >= o) incl += up;
-                }
-                int pos = base + incl - c8;
-                const int col0 = li * 256 + lane * 8;
-                // one predicated store per entry (a divergent branch per entry would cost far more)
-                if (in_win) {
-                    int p2 = pos;
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        const unsigned on = (m8 >> e) & 1u, d = (unsigned)(p2 - lo);
-                        const unsigned xb = (e & 1) ? (xw[e >> 1] & 0xffff0000u) : (xw[e >> 1] << 16);
-                        st_shared_u32_if(on & (d < len ? 1u : 0u), ent_base + 4u * d, xb | (unsigned)(col0 + e));
-                        p2 += (int)on;
-                    }
-                }
-                if (in_out) {
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        const unsigned on = (m8 >> e) & 1u, d = (unsigned)(pos - olo);
-                        st_global_if(on & (d < olen ? 1u : 0u), a.idx_out + pos, col0 + e);
-                        pos += (int)on;
-                    }
-                }
-            }
-        } else if (!DENSE) {
-            const bool identity = (a.flags & kFlagIdentity) != 0;
-            const int NT = NW * 32, gt = gw * 32 + lane;
-#pragma unroll 4
-            for (int i = gt; i < hi - lo; i += NT) {
-                const unsigned col = identity ? (unsigned)(lo + i) : (unsigned)__ldg(a.idx + lo + i);
-                const unsigned xb = has_xs ? lds_u16(xs_addr + 2u * col) : (unsigned)__ldg(xg + col);
-                sm.ent[i] = (xb << 16) | col;
-            }
-        }
-    };
-
-    int count = 0;
-    bool resident = true;
-    int win_lo = 0;  // list position of sm.ent[0]
-    if (DENSE) {
-        count = n;
-        pc.set_count(n, 8);
-    } else {
-        if (!FUSED) count = (a.flags & kFlagIdentity) ? n : __ldg(a.count);  // in flight while x is staged
-        // A given list that fits the window whole is copied whole, whatever the count turns out to be
-        // (idx holds n entries): its first entries are then loaded beside x and the count, in the same
-        // round trip, instead of after them.  Entries past the count are never used.
-        constexpr int kEarly = 8;
-        const bool whole_list = !FUSED && !(a.flags & kFlagIdentity) && has_xs && n <= kCap;
-        int early[kEarly];
-        if (whole_list) {
-#pragma unroll
-            for (int j = 0; j < kEarly; ++j) {
-                const int i = tid + j * kGemvThreads;
-                early[j] = i < n ? __ldg(a.idx + i) : 0;
-            }
-        }
-        if (has_xs) stage_x(warp, kWarps);
-        __syncthreads();
-        if (whole_list) {
-#pragma unroll
-            for (int j = 0; j < kEarly; ++j) {
-                const int i = tid + j * kGemvThreads;
-                const unsigned col = min((unsigned)early[j], (unsigned)(n - 1));   // past the count: anything, but in range
-                if (i < n) sm.ent[i] = (lds_u16(xs_addr + 2u * col) << 16) | col;
-            }
-            for (int i = tid + kEarly * kGemvThreads; i < n; i += kGemvThreads) {
-                const unsigned col = min((unsigned)__ldg(a.idx + i), (unsigned)(n - 1));
-                sm.ent[i] = (lds_u16(xs_addr + 2u * col) << 16) | col;
-            }
-        }
-        if (FUSED) {
-            const int4 t4 = *reinterpret_cast<const int4*>(&sm.tot[lane * 4]);
-            count = (int)__reduce_add_sync(0xffffffffu, (unsigned)(t4.x + t4.y + t4.z + t4.w));
-            if (c == 0 && tid == 0) *a.count_out = count;
-        }
-        pc.set_count(count);
-        if (FUSED && (a.flags & kFlagStatic) && pc.r_last - pc.r_first < kMaxStaticSeg) {
-            // Ablation, the paper's "sparse without load balancing": every CTA, and inside it every warp,
-            // takes a fixed range of the matrix COLUMNS of its block-row and works on whatever active
-            // entries fall into it.  Boundary j of the CTA's column range in a block-row becomes the list
-            // position "active entries below that column", read off the scan: the totals of the pieces
-            // below, plus the activity bits below the column inside its piece.
-            const int nseg = pc.r_last - pc.r_first + 1;
-            int tot4[4];
-            {
-                const int4 t4 = *reinterpret_cast<const int4*>(&sm.tot[lane * 4]);
-                tot4[0] = t4.x; tot4[1] = t4.y; tot4[2] = t4.z; tot4[3] = t4.w;
-            }
-#pragma unroll 1
-            for (int q = warp; q < nseg * (kWorkers + 1); q += kWarps) {
-                const int sgi = q / (kWorkers + 1), j = q % (kWorkers + 1);
-                unsigned u0, u1;
-                pc.fraction(pc.r_first + sgi, &u0, &u1);
-                const int k0 = (int)((u0 * (unsigned)n) / (unsigned)P), k1 = (int)((u1 * (unsigned)n) / (unsigned)P);
-                const int kb = k0 + (int)(((long long)(k1 - k0) * j) / kWorkers);
-                const int piece = kb >> 8, lane_of = (kb & 255) >> 3, bit = kb & 7;
-                unsigned below = 0;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) below += (lane * 4 + i < piece) ? (unsigned)tot4[i] : 0u;
-                const unsigned m8 = piece < nv ? pm[piece * 32 + lane] : 0u;
-                below += lane < lane_of ? (unsigned)__popc(m8) : (lane == lane_of ? (unsigned)__popc(m8 & ((1u << bit) - 1u)) : 0u);
-                const int posk = (int)__reduce_add_sync(0xffffffffu, below);
-                if (lane == 0) sm.static_table[sgi][j] = posk;
-            }
-            __syncthreads();
-            pc.table = &sm.static_table[0][0];
-        }
-        // list positions this CTA will read: the union of its slices.  (A piece that spans several
-        // block-rows ends the first one and begins the last one: its slices cover the whole list
-        // between them.)
-        int need_lo = 0, need_hi = count;
-        if (pc.r_first == pc.r_last) pc.slice(pc.r_first, &need_lo, &need_hi);
-        if (pc.table != nullptr && pc.r_first != pc.r_last) {
-            // a static partition: the CTA's column ranges in its first and last block-row, and whole rows between
-            int a0, b0, a1, b1;
-            pc.slice(pc.r_first, &a0, &b0);
-            pc.slice(pc.r_last, &a1, &b1);
-            need_lo = pc.r_last - pc.r_first > 1 ? 0 : min(a0, a1);
-            need_hi = pc.r_last - pc.r_first > 1 ? count : max(b0, b1);
-        }
-        resident = (need_hi - need_lo) <= kCap;
-        if (!resident && pc.table != nullptr) {
-            // (the ablation does not rebuild windows: long lists take the balanced partition)
-            pc.table = nullptr;
-            need_lo = 0;
-            need_hi = count;
-            if (pc.r_first == pc.r_last) pc.slice(pc.r_first, &need_lo, &need_hi);
-        }
-        int olo = 0, ohi = 0;  // the part of the returned index list this CTA writes: its slice of block-row 0
-        if (FUSED && pc.r_first == 0) pc.slice(0, &olo, &ohi);
-        if (whole_list) {
-            win_lo = 0;          // the whole list is in place already
-            resident = true;
-        } else if (resident) {
-            win_lo = need_lo;
-            build_window(need_lo, need_hi, olo, ohi, warp, kWarps);
-        } else {
-            // the window of the first span; the workers rebuild it for every later span
-            int p0, p1;
-            pc.slice(pc.r_first, &p0, &p1);
-            win_lo = p0;
-            const int whi = min(p1, p0 + kCap);
-            build_window(p0, whi, max(olo, p0), min(ohi, whi), warp, kWarps);
-        }
-        __syncthreads();  // the list is in place; the stage area is free for the pipeline
+    Scan<NW> scan(sm.area, n, lane, warp);            // (fused calls only)
+    int count = n;
+    if (LIST) count = __ldg(a.count);
+    if (FUSED) {
+        count = scan.scan_x(a.x, a.thr);
+        if (blockIdx.x == 0 && tid == 0) *a.count_out = count;
     }
-    if (CLUSTER) cluster_wait();  // every CTA of the cluster has initialised its barriers by now
 
-    if (warp >= kWriterWarp) {
-        // ------------------------------------------------------------ writers
-        // Two warps, one per hand-over buffer, so that the chains of dependent L2 round trips
-        // (store, fence, counter, read back) of consecutive segments overlap.
-        constexpr int RPL = G / 32;  // rows per lane
-        constexpr int kStride = G + 2;  // words per contributing CTA: G sums, the offset term, one of padding
-        const int wr = warp - kWriterWarp;
-        __half* const y = a.y;
-        int* const counters = a.counters;
-        bool ok = true;
-        for (int r = pc.r_first + wr, sg = wr; r <= pc.r_last; r += kWriters, sg += kWriters) {
-            const int b = sg & 1;  // hand-over buffer of this segment
-            int first, nslots;
-            pc.contributors(r, &first, &nslots);
-            const int mine = c - first;
-            unsigned long long* const row_words = a.words + (size_t)r * kTagSlots * kStride;
-            // A block-row that is not the CTA's first is shared with CTAs that work on it first and are
-            // done long before this one.  While the workers are still computing, watch for their words
-            // (one word per CTA as a cheap hint, at a low rate).  Once all of them are there, this CTA
-            // is the one that finishes the block-row, and nothing remains to be done across CTAs after
-            // its own sum.  (On a CTA's first block-row all contributors finish at about the same time
-            // and watching would only delay the counter path.)
-            constexpr int kSpec = kTagSlots - 1;
-            float ov[kSpec][RPL], oz[kSpec];
-            bool spec = false;
-            if (sg > 0 && nslots > 1 && nslots <= kSpec + 1) {
-                unsigned long long t0 = 0;
-                for (unsigned it = 0;; ++it) {
-                    const unsigned long long hint =
-                        lane < nslots - 1 ? ld_word(row_words + (size_t)(lane + (lane >= mine ? 1 : 0)) * kStride + G) : kTagBit;
-                    if (__all_sync(0xffffffffu, (hint >> 32) != 0ull)) {
-                        unsigned tags = 1u;
-#pragma unroll
-                        for (int j = 0; j < kSpec; ++j) {
-                            const bool in = j < nslots - 1;
-                            const unsigned long long* src = row_words + (size_t)(j + (j >= mine ? 1 : 0)) * kStride;
-#pragma unroll
-                            for (int i = 0; i < RPL; ++i) {
-                                const unsigned long long wv = in ? ld_word(src + lane * RPL + i) : kTagBit;
-                                ov[j][i] = __uint_as_float((unsigned)wv);
-                                tags &= (unsigned)(wv >> 32);
-                            }
-                            const unsigned long long wz = (in && lane == 0) ? ld_word(src + G) : kTagBit;
-                            oz[j] = __uint_as_float((unsigned)wz);
-                            tags &= (unsigned)(wz >> 32);
-                        }
-                        spec = __all_sync(0xffffffffu, tags != 0u);
-                        if (spec) break;
-                    }
-                    if (mbar_test(&sm.red_full[b], (sg >> 1) & 1)) break;  // own sums are ready: stop watching
-                    if (it == 0) t0 = global_ns();
-                    else if (global_ns() - t0 > kWaitNs) break;
-                    __nanosleep(400);   // a look every fraction of a microsecond: the watching must not take issue slots from the workers
+    float total[2] = {0.0f, 0.0f}, total_z = 0.0f;   // thread j < G / 2: rows j and j + G/2, over the slices of this CTA
+#pragma unroll 1
+    for (unsigned part = first_part; KIND != kSerial || part < last_part; ++part) {
+        // ---- the slice: in units of 8 entries, so that slices and parts begin at multiples of 8
+        int lo = 0, hi = count;
+        bool fixed_parts = false;
+        if (KIND != kPlain) {
+            const unsigned units = (unsigned)(count + 7) >> 3;
+            lo = 8 * (int)magic_div(part * units, parts, a.magic_s);
+            hi = min(8 * (int)magic_div((part + 1u) * units, parts, a.magic_s), count);
+        }
+        if (FUSED) {
+            if (KIND == kSerial && part != first_part) scan.scan_x(a.x, a.thr);
+            if (a.static_partition) {
+                // Ablation, the paper's "sparse without load balancing": a slice is a fixed range of the matrix COLUMNS,
+                // and so is every warp's part of it.
+                for (int j = warp; j <= NW; j += NW) {
+                    const int at = scan.position((int)(((long long)n * ((int)part * NW + j)) / ((int)parts * NW)));
+                    if (lane == 0) sm.table[j] = at;
                 }
-                if (spec) {
+                __syncthreads();
+                lo = sm.table[0];
+                hi = sm.table[NW];
+                fixed_parts = true;
+            }
+            scan.build(sm.ent, lo, hi, a.idx_out, lo, r == 0 ? hi : lo);
+            __syncthreads();             // the list is in place, and the ring may overwrite x
+        }
+        // ---- this warp's part of it
+        const int pu = (hi - lo + 7) >> 3;
+        int first = lo + 8 * ((pu * warp) / NW), end = min(lo + 8 * ((pu * (warp + 1)) / NW), hi);
+        if (FUSED && fixed_parts) {
+            first = sm.table[warp];
+            end = sm.table[warp + 1];
+        }
+
+        // given list: the columns of the lane's entries in the chunks the copies come to next, fetched kAhead chunks early
+        constexpr int kAhead = 3;
+        int coming[kAhead][EPL], ahead = first;
+        auto fetch_ahead = [&](int d) {
 #pragma unroll
-                    for (int j = 0; j < kSpec; ++j) oz[j] = __shfl_sync(0xffffffffu, oz[j], 0);
+            for (int q = 0; q < EPL; ++q) coming[d][q] = __ldg(a.idx + min(ahead + 32 * q + lane, end - 1));
+            ahead = ahead + CH >= end ? first : ahead + CH;
+        };
+        if (LIST && first < end) {
+#pragma unroll
+            for (int d = 0; d < kAhead; ++d) fetch_ahead(d);
+        }
+        unsigned xv[D][EPL];             // list and dense: the x values of the chunks in flight, the oldest first
+#pragma unroll
+        for (int i = 0; i < D * EPL; ++i) xv[i / EPL][i % EPL] = 0;
+        int ipos = first;                // where the copies stand: D - 1 chunks ahead of the product
+        unsigned ri = 0;                 // byte offset of the copies' stage
+        auto issue = [&]() {             // the copies of the next chunk, if there is one
+            if (!FUSED) {
+#pragma unroll
+                for (int i = 0; i < (D - 1) * EPL; ++i) xv[i / EPL][i % EPL] = xv[i / EPL + 1][i % EPL];
+            }
+            if (ipos < end) {
+                unsigned col[EPL];
+#pragma unroll
+                for (int q = 0; q < EPL; ++q) {       // (past the end: the last entry again, with x = 0)
+                    const int e = ipos + 32 * q + lane;
+                    col[q] = LIST ? (unsigned)coming[0][q] : FUSED ? lds_u16(ent_base + 4u * (unsigned)(min(e, end - 1) - lo)) : (unsigned)min(e, end - 1);
+                    if (!FUSED) xv[D - 1][q] = e < end ? (unsigned)__ldg(xg + col[q]) : 0u;
+                }
+                copy_chunk<G, BITS, Ring>(stage0 + ri, row_codes, row_meta, col, lane);
+                ri = ri + kStageBytes == kRing ? 0u : ri + kStageBytes;
+                ipos += CH;
+                if (LIST) {
+#pragma unroll
+                    for (int i = 0; i < (kAhead - 1) * EPL; ++i) coming[i / EPL][i % EPL] = coming[i / EPL + 1][i % EPL];
+                    fetch_ahead(kAhead - 1);
                 }
             }
-            handover_wait(b, (kWorkers + 1) * 32);
-            float v[RPL];
+            cp_async_commit();
+        };
+#pragma unroll 1
+        for (int d = 0; d < D - 1; ++d) issue();
+
+        // ---- the loop
+        Product<G, BITS, Ring> product(smem_u32(&lp.warp[warp].b[0][0]), lane);
+        unsigned xb[EPL];                // x of the entries from list position p on
+        auto x_at = [&](int p) {
 #pragma unroll
-            for (int i = 0; i < RPL; ++i) v[i] = 0.0f;
-            float zpart = 0.0f;
-#pragma unroll
-            for (int q = 0; q < kWorkers; ++q) {
-#pragma unroll
-                for (int i = 0; i < RPL; ++i) v[i] += sm.red[b][q][lane * RPL + i];
-                zpart += sm.red_z[b][q];
+            for (int q = 0; q < EPL; ++q) {
+                const int e = p + 32 * q + lane;
+                xb[q] = !FUSED ? xv[1][q] : e < end ? lds_u16(ent_base + 4u * (unsigned)(e - lo) + 2u) : 0u;
             }
+        };
+        unsigned rc = 0;                 // the stage of chunk i
+        if (first < end) {
+            cp_async_wait<D - 2>();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&sm.red_empty[b]);
-            if (nslots == 1) {
-                // this CTA holds the whole block-row: nothing to combine
-#pragma unroll
-                for (int i = 0; i < RPL; ++i) y[(size_t)r * G + lane * RPL + i] = __float2half_rn(v[i] + zpart);
-                continue;
-            }
-            float t[RPL], zsum = 0.0f;  // the block-row's sums, always accumulated in slot order
-#pragma unroll
-            for (int i = 0; i < RPL; ++i) t[i] = 0.0f;
-            if (CLUSTER) {
-                // The contributors of this block-row are the CTAs of this cluster, in rank order.  The
-                // others store their sums into rank 0's shared memory and arrive on its barrier; rank 0
-                // adds them in rank order.  Nothing goes through global memory.
-                if (mine != 0) {
-                    const unsigned dst = cluster_map(smem_u32(&sm.xred[mine][0]), 0u);
-#pragma unroll
-                    for (int i = 0; i < RPL; ++i) st_cluster_f32(dst + 4u * (lane * RPL + i), v[i]);
-                    if (lane == 0) st_cluster_f32(dst + 4u * G, zpart);
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive_cluster(cluster_map(smem_u32(&sm.xbar), 0u));
-                    continue;
-                }
-                ok = mbar_wait_cluster(&sm.xbar, 0);
-                if (!ok) break;
-#pragma unroll
-                for (int i = 0; i < RPL; ++i) t[i] += v[i];
-                zsum += zpart;
-                for (int s = 1; s < a.cluster_k; ++s) {
-#pragma unroll
-                    for (int i = 0; i < RPL; ++i) t[i] += sm.xred[s][lane * RPL + i];
-                    zsum += sm.xred[s][G];
-                }
-#pragma unroll
-                for (int i = 0; i < RPL; ++i) y[(size_t)r * G + lane * RPL + i] = __float2half_rn(t[i] + zsum);
-                continue;
-            }
-            if (spec) {
-#pragma unroll
-                for (int s = 0; s < kSpec + 1; ++s) {
-                    if (s < nslots) {
-                        const int j = s - (s > mine ? 1 : 0);  // position among the other CTAs
-#pragma unroll
-                        for (int i = 0; i < RPL; ++i) {
-                            float pv = v[i];
-#pragma unroll
-                            for (int jj = 0; jj < kSpec; ++jj) pv = (s != mine && j == jj) ? ov[jj][i] : pv;
-                            t[i] += pv;
-                        }
-                        float pz = zpart;
-#pragma unroll
-                        for (int jj = 0; jj < kSpec; ++jj) pz = (s != mine && j == jj) ? oz[jj] : pz;
-                        zsum += pz;
-                    }
-                }
-            } else if (nslots <= kSpec + 1) {
-                // publish this CTA's words (value and tag travel together: no fence), then count arrivals
-                unsigned long long* dst = row_words + (size_t)mine * kStride;
-#pragma unroll
-                for (int i = 0; i < RPL; ++i) st_word(dst + lane * RPL + i, kTagBit | __float_as_uint(v[i]));
-                if (lane == 0) st_word(dst + G, kTagBit | __float_as_uint(zpart));
-                int prev = 0;
-                if (lane == 0) prev = atomicAdd(counters + r, 1);
-                prev = __shfl_sync(0xffffffffu, prev, 0);
-                if (prev != nslots - 1) continue;
-                // last to arrive: every other CTA has issued its stores; wait (bounded) until their
-                // words are visible
-                float pv[kSpec + 1][RPL], pz[kSpec + 1];
-                unsigned long long t0 = 0;
-                for (unsigned it = 0;; ++it) {
-                    unsigned tags = 1u;
-#pragma unroll
-                    for (int j = 0; j < kSpec + 1; ++j) {
-                        const bool in = j < nslots && j != mine;
-                        const unsigned long long* src = row_words + (size_t)j * kStride;
-#pragma unroll
-                        for (int i = 0; i < RPL; ++i) {
-                            const unsigned long long wv = in ? ld_word(src + lane * RPL + i) : kTagBit;
-                            pv[j][i] = __uint_as_float((unsigned)wv);
-                            tags &= (unsigned)(wv >> 32);
-                        }
-                        const unsigned long long wz = (in && lane == 0) ? ld_word(src + G) : kTagBit;
-                        pz[j] = __uint_as_float((unsigned)wz);
-                        tags &= (unsigned)(wz >> 32);
-                    }
-                    if (__all_sync(0xffffffffu, tags != 0u)) break;
-                    if (it == 4) t0 = global_ns();
-                    if (it > 4 && global_ns() - t0 > kWaitNs) { ok = false; break; }
-                }
-                if (!ok) break;
-#pragma unroll
-                for (int j = 0; j < kSpec + 1; ++j) {
-                    const float z0 = __shfl_sync(0xffffffffu, pz[j], 0);
-                    if (j < nslots) {
-#pragma unroll
-                        for (int i = 0; i < RPL; ++i) t[i] += (j == mine) ? v[i] : pv[j][i];
-                        zsum += (j == mine) ? zpart : z0;
-                    }
-                }
-            } else {
-                // many contributors: plain fp32 partials in a region of their own, a fence, and the
-                // counter; the last to arrive reads eight slots at a time
-                const size_t pslot = (size_t)r * a.max_slots + mine;
-#pragma unroll
-                for (int i = 0; i < RPL; ++i) __stcg(a.partials + pslot * G + lane * RPL + i, v[i]);
-                if (lane == 0) __stcg(a.zpartials + pslot, zpart);
-                __threadfence();
-                __syncwarp();
-                int prev = 0;
-                if (lane == 0) prev = atomicAdd(counters + r, 1);
-                prev = __shfl_sync(0xffffffffu, prev, 0);
-                if (prev != nslots - 1) continue;
-                __threadfence();
-                const float* p = a.partials + (size_t)r * a.max_slots * G + lane * RPL;
-                const float* zp = a.zpartials + (size_t)r * a.max_slots;
-                for (int s0 = 0; s0 < nslots; s0 += 8) {
-                    float pv[8][RPL], pz[8];
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const bool in = s0 + j < nslots;
-#pragma unroll
-                        for (int i = 0; i < RPL; ++i) pv[j][i] = in ? __ldcg(p + (size_t)(s0 + j) * G + i) : 0.0f;
-                        pz[j] = in ? __ldcg(zp + s0 + j) : 0.0f;
-                    }
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        if (s0 + j < nslots) {
-#pragma unroll
-                            for (int i = 0; i < RPL; ++i) t[i] += pv[j][i];
-                            zsum += pz[j];
-                        }
-                    }
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < RPL; ++i) y[(size_t)r * G + lane * RPL + i] = __float2half_rn(t[i] + zsum);
-            // leave the workspace ready for the next call: no tag may stay set
-            if (nslots <= kSpec + 1) {
-                for (int s = 0; s < nslots; ++s) {
-                    unsigned long long* dst = row_words + (size_t)s * kStride;
-#pragma unroll
-                    for (int i = 0; i < RPL; ++i) st_word(dst + lane * RPL + i, 0ull);
-                    if (lane == 0) st_word(dst + G, 0ull);
-                }
-            }
-            // The counter: after the last arrival nobody else touches it, so it is simply cleared.  On the
-            // early path the other CTAs' increments may still be under way: a reduction that takes away
-            // exactly what they add leaves zero whatever the order (and none of them can see "last").
-            if (lane == 0) {
-                if (spec) atomicAdd(counters + r, -(nslots - 1));
-                else counters[r] = 0;
-            }
+            x_at(first);
+            product.begin(stage0, xb);
         }
-        if (!ok && lane == 0) atomicExch(a.status, 1);
-        return;
+#pragma unroll 1
+        for (int pos = first; pos < end; pos += CH) {
+            issue();
+            const unsigned rn = rc + kStageBytes == kRing ? 0u : rc + kStageBytes;
+            x_at(pos + CH);
+            cp_async_wait<D - 2>();
+            __syncwarp();
+            product.multiply(stage0 + rc, ll, stage0 + rn, xb);
+            rc = rn;
+        }
+        product.hand_over(lp.warp[warp].red, &lp.red_z[warp]);
+        __syncthreads();
+        if (tid < G / 2) {
+            float v[2], z;
+            add_warps<G, NW>(lp.warp, lp.red_z, tid, v, &z);
+            total[0] += v[0];
+            total[1] += v[1];
+            total_z += z;
+        }
+        cp_async_wait<0>();
+        if (KIND != kSerial) break;
+        __syncthreads();                 // (every warp is done with the ring and the list)
     }
 
-    // ---------------------------------------------------------------- workers
-    // Everything the loop touches in shared memory is addressed with 32-bit shared addresses kept in
-    // registers, and the control around a chunk is kept to a handful of instructions: the loop is
-    // bound by instruction issue and by the half-rate integer pipe, so every instruction outside the
-    // arithmetic counts.  Per chunk k of a warp: ISSUE(k) the copies; once they have landed PREP(k),
-    // the multipliers of its entries; MATH(k); then ISSUE(k+D) into the stage MATH(k) has freed.
-    constexpr unsigned kStageBytes = (unsigned)sizeof(Stage);
-    constexpr unsigned kMetaOff = (unsigned)offsetof(Stage, meta);
-    constexpr unsigned kXcOff = (unsigned)offsetof(Stage, xc);
-    const int slot = lane / LPB, h = lane % LPB;   // copies
-    const int mslot = lane / LM, mh = lane % LM;   // arithmetic
-    const unsigned stage_base = smem_u32(&sm.stage[warp][0]);
-    const unsigned mult_base = smem_u32(&sm.mult[warp][0][0]);
-    const unsigned full_base = smem_u32(&sm.full[warp][0]);
-    const unsigned lane0 = lane == 0 ? 1u : 0u;
-
-    // block-row constants of the issue side, refreshed when it enters a new block-row
-    const uint8_t* b_codes = nullptr;   // codes of the block-row (list calls: this lane's 16-byte part)
-    const unsigned* b_meta = nullptr;   // (scale, zero) pairs of the block-row
-    const uint8_t* d_codes = nullptr;   // dense call: where the issue side's next chunk starts in the three arrays
-    const unsigned* d_meta = nullptr;
-    const __half* d_x = nullptr;
-    auto enter_row = [&](int r, int pos) {
-        const size_t row_base = (size_t)r * (size_t)n;
-        b_codes = a.codes + row_base * B + ((!DENSE && BITS == 4) ? 16 * h : 0);
-        b_meta = a.meta + row_base;
-        if (DENSE) {
-            d_codes = b_codes + (size_t)pos * B;
-            d_meta = b_meta + pos;
-            d_x = a.x + pos;
-        }
-    };
-
-    // the list words of the entries a lane handles in the chunk at list position pos (FULL: all CH
-    // entries exist; else the entries past the end of the part read the part's last entry again)
-    auto load_entries = [&](int pos, int valid, bool full, unsigned* ev) {
-        const unsigned ent_addr = ent_base + 4u * (unsigned)(pos - win_lo);
-#pragma unroll
-        for (int q = 0; q < EPL; ++q) {
-            const int e = lane + 32 * q;
-            ev[q] = lds_u32(ent_addr + 4u * (unsigned)(full ? e : min(e, valid - 1)));
-        }
-    };
-
-    // ISSUE: the copies of one chunk (entries pos .. pos+valid-1 of the current block-row's list) into a stage
-    auto issue = [&](int pos, int valid, bool full, unsigned st_addr, unsigned bar_addr) {
-        if (DENSE) {
-            // the chunk's blocks, pairs and x values are contiguous: three bulk copies by one lane, from
-            // three pointers that simply advance (computing the addresses afresh for every chunk took
-            // five times the instructions)
-            if (full) {
-                mbar_expect_tx_if(lane0, bar_addr, (unsigned)CH * (B + 6));
-                bulk_copy_if(lane0, st_addr, d_codes, (unsigned)CH * B, bar_addr);
-                bulk_copy_if(lane0, st_addr + kMetaOff, d_meta, (unsigned)CH * 4, bar_addr);
-                bulk_copy_if(lane0, st_addr + kXcOff, d_x, (unsigned)CH * 2, bar_addr);
-            } else {
-                mbar_expect_tx_if(lane0, bar_addr, (unsigned)valid * (B + 6));
-                bulk_copy_if(lane0, st_addr, d_codes, (unsigned)valid * B, bar_addr);
-                bulk_copy_if(lane0, st_addr + kMetaOff, d_meta, (unsigned)valid * 4, bar_addr);
-                bulk_copy_if(lane0, st_addr + kXcOff, d_x, (unsigned)valid * 2, bar_addr);
+    if (KIND == kCluster) {
+        // the other CTAs leave their sums in the first one's shared memory; it adds them in CTA order
+        cluster_wait();                  // (every CTA of the cluster runs)
+        if (rank != 0) {
+            if (tid < G / 2) {
+                const unsigned dst = cluster_map(smem_u32(&sm.xred[rank][0]), 0u);
+                st_cluster_f32(dst + 4u * tid, total[0]);
+                st_cluster_f32(dst + 4u * (tid + G / 2), total[1]);
+                if (tid == 0) st_cluster_f32(dst + 4u * G, total_z);
             }
-            d_codes += CH * B;
-            d_meta += CH;
-            d_x += CH;
+            asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
             return;
         }
-        unsigned col[EPL];
-        load_entries(pos, valid, full, col);
-#pragma unroll
-        for (int q = 0; q < EPL; ++q) {
-            col[q] &= 0xffffu;
-            cp_async_4(st_addr + kMetaOff + 4u * (lane + 32 * q), b_meta + col[q]);
-        }
-        if (BITS == 4) {
-            // (steps past the end of the part copy the part's last block again: an L2 hit, and no branch)
-#pragma unroll
-            for (int u = 0; u < SUBS; ++u) {
-                const unsigned cu = __shfl_sync(0xffffffffu, col[(u * SLOTS) / 32], (u * SLOTS + slot) & 31);
-                cp_async_16_l2_64(st_addr + lane * 16 + u * 512, b_codes + (size_t)cu * B);
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (tid < G / 2) {
+            for (int q = 1; q < a.splits; ++q) {
+                total[0] += sm.xred[q][tid];
+                total[1] += sm.xred[q][tid + G / 2];
+                total_z += sm.xred[q][G];
             }
-        } else {
-            // 3-bit blocks (48 or 24 bytes): the chunk's bytes in copies of CB bytes, lane after lane
-            constexpr int NC = CH * B / CB / 32;
-#pragma unroll
-            for (int q = 0; q < NC; ++q) {
-                const int off = (q * 32 + lane) * CB;    // byte offset inside the chunk's stage
-                const int e = off / B, part = off % B;
-                const unsigned cu = __shfl_sync(0xffffffffu, col[(q * 32 * CB / B) / 32], e & 31);
-                const uint8_t* src = b_codes + (size_t)cu * B + part;
-                if (CB == 16) cp_async_16_l2_64(st_addr + off, src);
-                else cp_async_8(st_addr + off, src);
-            }
-        }
-    };
-
-    unsigned long long acc[8];  // 16 fp32 sums, two per register
-#pragma unroll
-    for (int i = 0; i < 8; ++i) acc[i] = 0ull;
-    float zl = 0.0f;     // this lane's share of sum x_k * zero_rk of the current segment
-
-    // PREP: lane e turns the pair of its entry into a = x_k*scale (exact in fp32), written as the packed
-    // multiplier pair (a, a) * 2^93, and adds x_k*zero to its share of the offset term
-    auto prep = [&](unsigned st_addr, int pos, int valid, bool full) {
-        unsigned ev[EPL];
-        if (!DENSE) load_entries(pos, valid, full, ev);
-#pragma unroll
-        for (int q = 0; q < EPL; ++q) {
-            const int e = lane + 32 * q;
-            const unsigned mz = lds_u32(st_addr + kMetaOff + 4u * e);
-            const unsigned xb = DENSE ? lds_u16(st_addr + kXcOff + 2u * e) : (ev[q] >> 16);
-            const float xf = __half2float(__ushort_as_half((unsigned short)xb));
-            const float sf = __half2float(__ushort_as_half((unsigned short)(mz & 0xffffu)));
-            const float zf = __half2float(__ushort_as_half((unsigned short)(mz >> 16)));
-            float am = xf * sf;   // exact
-            float zt = xf * zf;   // exact
-            if (!full) {          // an entry past the end of the part: weight 0
-                am = e < valid ? am : 0.0f;
-                zt = e < valid ? zt : 0.0f;
-            }
-            zl += zt;
-            const unsigned long long aa = pack2(am, am);
-            sts_u64(mult_base + 8u * e, fmul2(aa, pack2(0x1p93f, 0x1p93f)));
-        }
-    };
-
-    // MATH: one step of a chunk: SLM blocks, each lane 16 codes of one of them
-    auto step = [&](unsigned st_addr, int u) {
-        const unsigned long long mm = lds_u64(mult_base + 8u * (u * SLM + mslot));
-        if (BITS == 4) {
-            const uint2 wv = lds_v2(st_addr + lane * 8 + u * 256);
-            fma_block8_cum(acc, wv, mm);
-        } else {
-            // lane t of a block: word t of the 2-bit plane (G/16 words); its top bits are the even
-            // (t < LM/2) or odd bits of word t mod LM/2 of the 1-bit plane
-            const unsigned blk = st_addr + (u * SLM + mslot) * B;
-            const unsigned w2 = lds_u32(blk + 4u * mh);
-            const unsigned w1 = lds_u32(blk + (G / 4) + 4u * (mh % (LM / 2))) >> (mh / (LM / 2));
-            fma_block3_cum(acc, w2, w1, mm);
-        }
-    };
-
-    // Stage ring: chunk number k of this warp (in issue order = consume order) uses stage k mod D, so
-    // ISSUE(k+D) refills the stage MATH(k) has just read.  wi: where the issue side stands in the
-    // warp's sequence of chunks (it runs ahead of the arithmetic, across block-rows); wc: the arithmetic.
-    unsigned rc = 0;   // byte offset of the arithmetic's stage
-    unsigned bc = 0;   // dense call: byte offset of that stage's barrier, and its phase parity
-    unsigned par = 0;
-    Walker wi, wc;
-    wc.first(pc, warp, resident);
-    wi = wc;
-    bool ok = true;
-    // moves the issue side to its next non-empty part (within the current span only when the window is
-    // rebuilt between spans); false when there is none
-    auto seek_issue = [&]() -> bool {
-        if (resident) {
-            while (wi.valid(pc) && !wi.has_chunk()) wi.next_span(pc, warp, true);
-        }
-        const bool more = wi.valid(pc) && wi.has_chunk();
-        if (more) enter_row(wi.r, wi.pos);
-        return more;
-    };
-    bool more_i = seek_issue();
-    // ISSUE of the warp's next chunk, if there is one, into the stage at byte offset rs; one commit
-    // group per call either way
-    auto issue_next = [&](unsigned rs, unsigned bs) {
-        if (more_i) {
-            const int left = wi.end - wi.pos;
-            if (left >= CH) issue(wi.pos, CH, true, stage_base + rs, full_base + bs);
-            else issue(wi.pos, left, false, stage_base + rs, full_base + bs);
-            wi.pos += CH;
-            if (wi.pos >= wi.end) more_i = seek_issue();
-        }
-        if (!DENSE) cp_async_commit();
-    };
-    // fills the pipeline, starting with the stage the arithmetic will read next
-    auto prime = [&]() {
-        unsigned rs = rc, bs = bc;
-#pragma unroll 1
-        for (int s = 0; s < D; ++s) {
-            issue_next(rs, bs);
-            rs = (rs + kStageBytes == D * kStageBytes) ? 0u : rs + kStageBytes;
-            bs = (bs + 8u == D * 8u) ? 0u : bs + 8u;
-        }
-    };
-    prime();
-
-    int sg = 0;
-    while (wc.valid(pc)) {
-#pragma unroll 1
-        for (int pos = wc.pos; pos < wc.end; pos += CH) {
-            const int left = wc.end - pos;
-            if (DENSE) {
-                if (ok) ok = mbar_wait_addr(full_base + bc, par);
-            } else {
-                cp_async_wait<D - 1>();
-                __syncwarp();
-            }
-            const unsigned st_addr = stage_base + rc;
-            if (left >= CH) {
-                prep(st_addr, pos, CH, true);
-                __syncwarp();
-                // a full chunk: straight-line code (branches between the steps made the compiler shuffle
-                // the accumulators around them, half as many instructions again)
-#pragma unroll
-                for (int u = 0; u < MSUBS; ++u) step(st_addr, u);
-            } else {
-                prep(st_addr, pos, left, false);
-                __syncwarp();
-                // the last chunk of a part: only the steps that hold entries
-                const int nsub = (left + SLM - 1) / SLM;
-#pragma unroll 1
-                for (int u = 0; u < nsub; ++u) step(st_addr, u);
-            }
-            __syncwarp();  // every lane is done with this chunk's stage and multipliers
-            issue_next(rc, bc);
-            if (rc + kStageBytes == D * kStageBytes) { rc = 0u; bc = 0u; par ^= 1u; } else { rc += kStageBytes; bc += 8u; }
-        }
-        if (wc.last_of_segment()) {
-            // ---- end of the segment: in-warp reduce-scatter over the column slots, then hand the
-            // per-warp sums to the writer warp
-            const int b = sg & 1;
-            if (sg >= 2 && ok) ok = mbar_wait(&sm.red_empty[b], ((sg >> 1) - 1) & 1);
-            float accf[16];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                unpack2(acc[i], accf[2 * i], accf[2 * i + 1]);
-                acc[i] = 0ull;
-            }
-            // lanes that differ in the bits above log2(LM) hold sums of the same rows
-            float t8[8], t4[4], keep[4];
-            halve<16>(accf, t8, lane, 16);
-            halve<8>(t8, t4, lane, 8);
-            uncumulate(t4);   // the four values are the cumulative sums of one half-word
-            if (LM == 8) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) keep[i] = t4[i];
-            } else {
-                float t2[2];
-                halve<4>(t4, t2, lane, 4);
-                keep[0] = t2[0];
-                keep[1] = t2[1];
-            }
-            const int a_base = mslot * KEEP;
-#pragma unroll
-            for (int i = 0; i < KEEP; ++i) {
-                const int ai = a_base + i;  // accumulator index = word*8 + nibble
-                const int cw = ai >> 3, e2 = ai & 7;
-                const int row = (BITS == 4)
-                                    ? 8 * mh + 4 * cw + (e2 >> 1) + (e2 & 1) * (G / 2)
-                                    : 4 * mh + (e2 >> 1) + (G / 4) * (2 * (e2 & 1) + cw);
-                sm.red[b][warp][row] = keep[i] * 0x1p56f;  // undo the 2^-56 of the subnormal trick
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) zl += __shfl_xor_sync(0xffffffffu, zl, o);
-            if (lane == 0) sm.red_z[b][warp] = zl;
-            zl = 0.0f;
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&sm.red_full[b]);   // what the watching writer tests
-            handover_arrive(b, (kWorkers + 1) * 32);       // what it finally waits on
-            ++sg;
-        }
-        wc.next_span(pc, warp, resident);
-        if (!DENSE && !resident && wc.valid(pc)) {
-            // The next span needs another part of the list: every worker has drained its pipeline (the
-            // span's chunks are consumed), so the stage area and the window can be rebuilt.
-            cp_async_wait<0>();
-            worker_barrier(kWorkers * 32);
-            if (has_xs) stage_x(warp, kWorkers);
-            worker_barrier(kWorkers * 32);
-            int olo = 0, ohi = 0;
-            if (FUSED && wc.r == 0) { olo = wc.lo; ohi = wc.hi; }
-            win_lo = wc.lo;
-            build_window(wc.lo, wc.hi, olo, ohi, warp, kWorkers);
-            worker_barrier(kWorkers * 32);
-            wi = wc;
-            more_i = seek_issue();
-            prime();
         }
     }
-    if (!DENSE) cp_async_wait<0>();
-    if (!ok && lane == 0) atomicExch(a.status, 1);
+    if (tid < G / 2) {
+        a.y[(size_t)r * G + tid] = __float2half_rn(total[0] + total_z);
+        a.y[(size_t)r * G + tid + G / 2] = __float2half_rn(total[1] + total_z);
+    }
+}
+
+// ---------------------------------------------------------------- pieces
+
+// N warps, R block-rows laid end to end: warp W has [W*R/N, (W+1)*R/N), the fraction of a block-row being that fraction of
+// its list entries, in units of 8.  N >= R: a warp has part of one block-row, or the end of one and the start of the next.
+// The warps' sums meet in shared memory, added in warp order; a block-row that two or more CTAs
+// share is finished by the CTA that comes last, which adds their sums in CTA order (calls are bit-reproducible).
+// What bounds it at 28672 x 8192 and 50 % (18.3 us): 17000 cycles of loop at 7 TB/s, L2 hits among them, and 12000 cycles of
+// fixed cost: x and the masks 2000, the list 2200, the first chunks' arrival 3300, the sums and their exchange 4500.  That
+// is more than whole block-rows pay, so the host takes it only where those leave SMs idle or their list does not fit.
+template <int G, int BITS, int MODE>
+__global__ void __launch_bounds__(kPieceWarps * 32, 1)
+gemv_pieces_kernel(const GemvArgs a)
+{
+    using Ring = PieceRing<G, MODE>;
+    constexpr int B = G * BITS / 8, CH = Ring::CH, EPL = CH / 32, D = Ring::D, NW = kPieceWarps, kThreads = NW * 32;
+    constexpr bool FUSED = MODE == kModeFused, LIST = MODE == kModeList;
+    using Smem = PieceSmem<G, BITS, MODE>;
+
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    Smem& sm = *reinterpret_cast<Smem*>(smem_raw);
+    typename Smem::Loop& lp = *reinterpret_cast<typename Smem::Loop*>(sm.area);
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+    const int n = a.n;
+    const unsigned R = (unsigned)a.R, N = a.warps, cta = blockIdx.x;
+
+    prefetch_inputs<MODE, kThreads>(a, tid);
+    const typename MmaStage<G, BITS>::Lane ll(lane);
+    const unsigned stage0 = smem_u32(&lp.stage[warp][0]);
+    constexpr unsigned kStageBytes = (unsigned)sizeof(Stage<G, BITS, Ring>), kRing = D * kStageBytes;
+    const unsigned ent_base = smem_u32(&sm.ent[0]);
+    const unsigned short* const xg = reinterpret_cast<const unsigned short*>(a.x);
+    // this warp's piece: from fraction part0 / N of block-row row0 to part1 / N of row1
+    const unsigned W = cta * NW + (unsigned)warp;
+    const unsigned row0 = magic_div(W * R, N, a.magic_w), part0 = W * R - row0 * N;
+    const unsigned row1 = magic_div((W + 1u) * R, N, a.magic_w), part1 = (W + 1u) * R - row1 * N;
+    const unsigned last_row = part1 > 0u ? row1 : row1 - 1u;
+
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+    Scan<NW> scan(sm.area, n, lane, warp);            // (fused calls only)
+    int count = n;
+    if (LIST) count = __ldg(a.count);
+    if (FUSED) count = scan.scan_x(a.x, a.thr);
+    const unsigned units = (unsigned)(count + 7) >> 3;
+    int first = 8 * (int)magic_div(part0 * units, N, a.magic_w), end = 8 * (int)magic_div(part1 * units, N, a.magic_w);
+    if (FUSED) {
+        if (cta == 0 && tid == 0) *a.count_out = count;
+        if (a.static_partition) {
+            // ablation (see above): the fraction of a block-row is a fraction of its columns
+            first = scan.position((int)magic_div(part0 * (unsigned)n, N, a.magic_w));
+            end = scan.position((int)magic_div(part1 * (unsigned)n, N, a.magic_w));
+        }
+        // every CTA writes its share of idx
+        const unsigned P = gridDim.x;
+        scan.build(sm.ent, 0, count, a.idx_out, 8 * (int)magic_div(cta * units, P, a.magic_p),
+                   min(8 * (int)magic_div((cta + 1u) * units, P, a.magic_p), count));
+        __syncthreads();                 // the list is in place, and the ring may overwrite x
+    }
+    if (part1 == 0u) end = count;        // of the piece's last block-row
+
+    // A place in the piece: entries from pos on, of those below hi, of block-row `row`
+    struct Cursor {
+        unsigned row;
+        int pos, hi;
+    };
+    auto advance = [&](Cursor& c) {
+        c.pos += CH;
+        if (c.pos >= c.hi) {
+            ++c.row;
+            c.pos = 0;
+            c.hi = c.row < last_row ? count : c.row == last_row ? end : 0;   // (0: past the end)
+        }
+    };
+    Cursor at{row0, first, row0 < last_row ? count : end};   // where the copies stand
+    if (at.pos >= at.hi) advance(at);    // (nothing of the first block-row: the ablation, or an empty list)
+    const uint8_t* row_codes = a.codes + (size_t)at.row * (size_t)n * B;
+    const unsigned* row_meta = a.meta + (size_t)at.row * (size_t)n;
+
+    // given list: the columns of the lane's entries in the chunks the copies come to next, fetched kAhead chunks early
+    constexpr int kAhead = 3;
+    int coming[kAhead][EPL] = {};
+    Cursor ahead = at;
+    auto fetch_ahead = [&](int d) {
+        if (ahead.pos < ahead.hi) {
+#pragma unroll
+            for (int q = 0; q < EPL; ++q) coming[d][q] = __ldg(a.idx + min(ahead.pos + 32 * q + lane, ahead.hi - 1));
+        }
+        advance(ahead);
+    };
+    if (LIST) {
+#pragma unroll
+        for (int d = 0; d < kAhead; ++d) fetch_ahead(d);
+    }
+    unsigned xv[D][EPL];                 // the x values of the chunks in flight, the oldest first
+#pragma unroll
+    for (int i = 0; i < D * EPL; ++i) xv[i / EPL][i % EPL] = 0;
+    unsigned ri = 0;
+    auto issue = [&]() {                 // the copies of the next chunk, if there is one
+#pragma unroll
+        for (int i = 0; i < (D - 1) * EPL; ++i) xv[i / EPL][i % EPL] = xv[i / EPL + 1][i % EPL];
+        if (at.pos < at.hi) {
+            unsigned col[EPL];
+#pragma unroll
+            for (int q = 0; q < EPL; ++q) {           // (past the end: the last entry again, with x = 0)
+                const int e = at.pos + 32 * q + lane, in = min(e, at.hi - 1);
+                col[q] = LIST ? (unsigned)coming[0][q] : FUSED ? lds_u16(ent_base + 2u * (unsigned)in) : (unsigned)in;
+                xv[D - 1][q] = e < at.hi ? (unsigned)__ldg(xg + col[q]) : 0u;
+            }
+            copy_chunk<G, BITS, Ring>(stage0 + ri, row_codes, row_meta, col, lane);
+            ri = ri + kStageBytes == kRing ? 0u : ri + kStageBytes;
+            const unsigned row = at.row;
+            advance(at);
+            if (at.row != row) {
+                row_codes += (size_t)n * B;
+                row_meta += n;
+            }
+            if (LIST) {
+#pragma unroll
+                for (int i = 0; i < (kAhead - 1) * EPL; ++i) coming[i / EPL][i % EPL] = coming[i / EPL + 1][i % EPL];
+                fetch_ahead(kAhead - 1);
+            }
+        }
+        cp_async_commit();
+    };
+    const bool work = at.pos < at.hi;
+#pragma unroll 1
+    for (int d = 0; d < D - 1; ++d) issue();
+
+    Product<G, BITS, Ring> product(smem_u32(&lp.b[warp][0][0]), lane);
+    unsigned rc = 0;                     // the stage of chunk i
+    if (work) {
+        cp_async_wait<D - 2>();
+        __syncwarp();
+        product.begin(stage0, xv[1]);
+    }
+    int pos = first;
+#pragma unroll 1
+    for (unsigned row = row0;; ++row) {
+        const int hi = row < last_row ? count : end;
+#pragma unroll 1
+        for (; pos < hi; pos += CH) {
+            issue();
+            const unsigned rn = rc + kStageBytes == kRing ? 0u : rc + kStageBytes;
+            cp_async_wait<D - 2>();
+            __syncwarp();
+            product.multiply(stage0 + rc, ll, stage0 + rn, xv[1]);
+            rc = rn;
+        }
+        product.hand_over(lp.red[row - row0][warp], &lp.red_z[row - row0][warp]);
+        if (row == last_row) break;
+        pos = 0;
+        product.clear();
+    }
+    cp_async_wait<0>();
+    __syncthreads();
+
+    // ---- block-rows that several warps share: G / 2 threads each, two rows a thread
+    const int j = tid % (G / 2), group = tid / (G / 2);
+    const unsigned W0 = cta * NW;
+    const unsigned begin_row = magic_div(W0 * R, N, a.magic_w), end_row = magic_div((W0 + NW) * R + N - 1u, N, a.magic_w);
+    auto first_warp = [&](unsigned r) { return magic_div(r * N, R, a.magic_r); };               // of the grid's, with part of r
+    auto last_warp = [&](unsigned r) { return magic_div((r + 1u) * N + R - 1u, R, a.magic_r) - 1u; };
+    auto store_y = [&](unsigned r, float v0, float v1) {
+        a.y[(size_t)r * G + j] = __float2half_rn(v0);
+        a.y[(size_t)r * G + j + G / 2] = __float2half_rn(v1);
+    };
+#pragma unroll 1
+    for (unsigned r = begin_row + (unsigned)group; r < end_row; r += kThreads / (G / 2)) {
+        const unsigned fw = first_warp(r), lw = last_warp(r);
+        float v0 = 0.0f, v1 = 0.0f, z = 0.0f;
+#pragma unroll 1
+        for (unsigned w = max(fw, W0); w <= min(lw, W0 + NW - 1u); ++w) {
+            const int s = w * R >= r * N ? 0 : 1;   // the first or the second block-row of warp w
+            const float2 cz = lp.red_z[s][w - W0];
+            v0 += lp.red[s][w - W0][j] * cz.x;
+            v1 += lp.red[s][w - W0][j + G / 2] * cz.x;
+            z += cz.y;
+        }
+        v1 = (v1 - v0) * 0.0625f;        // the high nibbles' tiles sum whole bytes
+        if (fw >= W0 && lw < W0 + NW) {
+            store_y(r, v0 + z, v1 + z);
+        } else {
+            float* const p = a.partial + (size_t)(2u * cta + (fw >= W0 ? 1u : 0u)) * G;
+            __stcg(p + j, v0 + z);
+            __stcg(p + j + G / 2, v1 + z);
+        }
+    }
+    // ---- block-rows that several CTAs share: the last one there adds the sums, and leaves zeros in the workspace
+    const unsigned edge[2] = {begin_row, end_row - 1u};
+    __threadfence();
+    __syncthreads();
+    if (tid < 2) {
+        const unsigned r = tid == 0 ? edge[0] : edge[1], c0 = first_warp(r) / NW, c1 = last_warp(r) / NW;
+        int is_last = 0;
+        if (c0 != c1 && (tid == 0 || edge[1] != edge[0])) {
+            is_last = atomicAdd(a.arrived + r, 1u) == c1 - c0 ? 1 : 0;
+            if (is_last) a.arrived[r] = 0u;
+        }
+        sm.last[tid] = is_last;
+    }
+    __syncthreads();
+    if (group < 2 && sm.last[group]) {
+        __threadfence();
+        const unsigned r = group == 0 ? edge[0] : edge[1], c0 = first_warp(r) / NW, c1 = last_warp(r) / NW;
+        float v0 = 0.0f, v1 = 0.0f;
+        for (unsigned c = c0; c <= c1; ++c) {
+            float* const p = a.partial + (size_t)(2u * c + (c == c0 ? 1u : 0u)) * G;
+            v0 += __ldcg(p + j);
+            v1 += __ldcg(p + j + G / 2);
+            __stcg(p + j, 0.0f);
+            __stcg(p + j + G / 2, 0.0f);
+        }
+        store_y(r, v0, v1);
+    }
 }
 
 // ---------------------------------------------------------------- host side
@@ -1097,139 +992,139 @@ static void store_tuned(const Format& f, int mode, int ctas)
     if (g_tuned_count < kMaxTuned) g_tuned[g_tuned_count++] = TunedEntry{f.m, f.n, f.bits, f.group, mode, ctas};
 }
 
-// Bytes of the stage area the prologue may borrow, and what it needs for an x of n entries.
-template <int G, int BITS>
-constexpr size_t stage_area_bytes() { return sizeof(GemvSmem<G, BITS>::stage); }
-inline size_t scratch_bytes(int n, bool fused) { return (size_t)((n + 255) / 256) * (fused ? 544 : 512); }
-
-template <int G, int BITS>
-static bool fused_fits(int n) { return n <= kMaxFusedN && scratch_bytes(n, true) <= stage_area_bytes<G, BITS>(); }
+// How many clusters of k CTAs the device holds at once with `smem` bytes each (asked once per kernel, cluster size and device).
+template <int G, int BITS, int MODE>
+static int max_clusters(int k, int smem, bool alone, int sms, int dev)
+{
+    static int known[64][2][kMaxSplit + 1] = {};
+    int& at_once = known[dev][alone ? 1 : 0][k];
+    if (at_once == 0) {
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = k;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(k * kCtasPerSm * sms));
+        cfg.blockDim = dim3(256);
+        cfg.dynamicSmemBytes = smem;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int can = 0;
+        if (cudaOccupancyMaxActiveClusters(&can, gemv_kernel<G, BITS, MODE, kCluster, 8>, &cfg) != cudaSuccess) (void)cudaGetLastError();
+        at_once = can > 0 ? can : 1;
+    }
+    return at_once;
+}
 
 template <int G, int BITS, int MODE>
 static spqt_status launch_gemv(const Format& f, const void* codes, const void* meta, const void* x,
                                const int32_t* idx, const int32_t* count, void* y, void* workspace,
-                               cudaStream_t s, FusedArgs fa, int flags)
+                               cudaStream_t s, FusedArgs fa)
 {
-    auto kernel = gemv_kernel<G, BITS, MODE, false>;
-    auto kernel_c = gemv_kernel<G, BITS, MODE, true>;  // the thread-block-cluster variant
+    constexpr int kAlone = 120 * 1024;   // shared memory that keeps a second CTA of 8 warps off the SM
+    // (a given list counts its clusters with the size of the fused call: the same slices, the same sums)
+    constexpr int kSlices = MODE == kModeList ? kModeFused : MODE;
+    constexpr int kSmem = (int)sizeof(GemvSmem<G, BITS, kSlices, kCluster, 8>), kSmemPlain = (int)sizeof(GemvSmem<G, BITS, MODE, kPlain, 8>);
+    constexpr int kSmem16 = (int)sizeof(GemvSmem<G, BITS, MODE, kPlain, 16>), kSmemPieces = (int)sizeof(PieceSmem<G, BITS, MODE>);
+    static_assert(sizeof(GemvSmem<G, BITS, MODE, kCluster, 8>) <= kSmem && sizeof(GemvSmem<G, BITS, MODE, kSerial, 8>) <= kSmem && kSmem <= kAlone, "one size for all slices");
+    static_assert(kSmem <= 115712 && kSmemPlain <= 115712 && kSmem16 <= 232448 && kSmemPieces <= 232448, "two CTAs of 8 warps per SM, or one of 16");
     static bool configured[64] = {};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return SPQT_ERR_CUDA;
-    const int smem = (int)sizeof(GemvSmem<G, BITS>);
     if (!configured[dev]) {
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-            cudaFuncSetAttribute(kernel_c, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
+        if (cudaFuncSetAttribute(gemv_kernel<G, BITS, MODE, kPlain, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPlain) != cudaSuccess ||
+            cudaFuncSetAttribute(gemv_kernel<G, BITS, MODE, kPlain, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem16) != cudaSuccess ||
+            cudaFuncSetAttribute(gemv_kernel<G, BITS, MODE, kCluster, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAlone) != cudaSuccess ||
+            cudaFuncSetAttribute(gemv_kernel<G, BITS, MODE, kSerial, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess ||
+            cudaFuncSetAttribute(gemv_pieces_kernel<G, BITS, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPieces) != cudaSuccess)
             return SPQT_ERR_CUDA;
         configured[dev] = true;
     }
     const int sms = sm_count();
     if (sms <= 0) return SPQT_ERR_CUDA;
+    // CTAs per block-row.  Up to about 35 block-rows: the largest cluster of which all fit with one CTA per SM (4096 x 4096,
+    // index collection inside: 6.35 / 5.57 / 4.99 / 4.61 us on 1 / 2 / 3 / 4 CTAs per block-row; 5.2 us on 7, two per SM).
+    // From there to 100: the largest with two per SM (5120 x 5120, given list: 6.25 / 5.08 / 4.72 / 4.31 us on 1 / 2 / 3 /
+    // 5; 8192 x 28672 dense 44.1 / 26.2 / 22.4 us on 1 / 2 / 4).  From 100 up one CTA per block-row: two would put two
+    // halves on the busiest SMs, which take as long as one whole and need an exchange (14336 x 4096: 6.5 against 7.3 us).
+    int S = 1;
     const int tuned = g_tune_ctas > 0 ? g_tune_ctas : tuned_ctas(f, MODE);
-    int P = tuned > 0 ? tuned : sms;
-    if (tuned == 0 && f.R <= P) {
-        // With few block-rows, a whole number of CTAs per block-row (if that keeps >= 85 % of the SMs
-        // busy; 70 % for light launches, below) gives every CTA a single segment: no CTA then carries two
-        // aggregation chains.
-        int k = P / f.R;
-        // A small matrix gains nothing from more than four CTAs per block-row: the combination of many
-        // partial sums then costs more than the extra CTAs save (measured: 1024 x 4096 takes 6.8 us on 144
-        // CTAs, 4.9 us on 32).  "Small": under 256 KB of blocks per CTA at four CTAs per block-row.
-        const size_t row_bytes = (size_t)f.n * (size_t)(f.B + 4);
-        bool small = k > 4 && row_bytes / 4 < (size_t(256) << 10);
-        if (small) k = 4;
-        // A block-row of under 96 KB is not worth cutting at all once there are 32 of them (measured:
-        // 4096 x 1024 takes 4.0 / 4.5 / 3.8 us -- given list, index collection inside, dense -- on 32 CTAs
-        // against 4.5 / 5.5 / 3.8 on 128; 8192 x 1024 4.1 / 4.6 / 3.8 on 64 against 4.8 / 5.5 / 4.2 on 128).
-        if (k > 1 && f.R >= 32 && row_bytes < (size_t(96) << 10)) {
-            k = 1;
-            small = true;
+    int P = sms < kMaxPieceCtas ? sms : kMaxPieceCtas;   // CTAs of the pieces kernel
+    bool pieces = false;
+    // slices that fit the shared memory of a fused call (a given list is sliced the same way: the same sums)
+    const int least = MODE == kModeDense || f.n <= kCapPlain || f.n > kMaxFusedN ? 1 : (f.n + kCapSlice - 1) / kCapSlice;
+    if (tuned > 0) {
+        S = tuned / f.R;
+        if (S == 0) {
+            pieces = true;
+            P = tuned < P ? tuned : P;
         }
-        // While a CTA's share stays under half a megabyte the launch is latency-bound, and leaving up to 30 %
-        // of the SMs idle costs less than partial sums that cross CTAs in a ragged pattern
-        // (measured: 14336 x 4096 on 112 CTAs, one block-row each, 8.9 us against 9.7 us on 148; 13824 x 5120
-        // on 108 CTAs 8.7 against 9.6 us).
-        const size_t share = (size_t)f.R * row_bytes / (size_t)P;
-        const bool light = share < (size_t(512) << 10);
-        // The dense call streams every block: from about a third of a megabyte per CTA the idle SMs cost more than
-        // the ragged pieces (measured, 64 block-rows: 8192 x 28672 takes 28.5 us on 148 CTAs against 31.1 us on
-        // 128, 8192 x 16384 18.3 against 19.3 us, 8192 x 8192 11.7 against 11.2 us; the sparse calls, with half
-        // the bytes, stay better off on 128).
-        const bool heavy_dense = MODE == kModeDense && share >= (size_t(320) << 10);
-        if (small || (!heavy_dense && k * f.R * 100 >= (light ? 70 : 85) * P)) P = k * f.R;
+    } else if (f.R < 100) {
+        const bool spread = f.R <= max_clusters<G, BITS, MODE>(4, kAlone, true, sms, dev);
+        for (int k = 2; k <= kMaxSplit; ++k)
+            if (f.n >= 256 * k && f.R <= max_clusters<G, BITS, MODE>(k, spread ? kAlone : kSmem, spread, sms, dev)) S = k;
     }
-    // no more CTAs than pieces of at least 64 columns of one block-row
-    const long long pieces = (long long)f.R * ((f.n + 63) / 64);
-    if (P > pieces) P = (int)pieces;
-    if (P > kMaxCtas) P = kMaxCtas;
-    if (P < 1) P = 1;
-    const int slots = max_slots(f.R);
+    if (tuned <= 0 && S < least) {
+        // A whole block-row does not fit a CTA: a cluster with one slice per CTA if all are resident at once (14336 x 11008
+        // 14.5 against 16.2 us), otherwise pieces (12288 x 14589 3-bit 19.9 against 25 us with CTAs in two waves).
+        if (f.R <= max_clusters<G, BITS, MODE>(least, kSmem, false, sms, dev)) S = least;
+        else pieces = true;
+    }
+    // No list to build, and enough per CTA to pay for sharing block-rows (2 us): an even load instead of one or two whole
+    // block-rows per SM (28672 x 16384 44 against 50 us, x 8192 24.5 against 26, x 5120 19 against 16.5)
+    if (tuned <= 0 && MODE == kModeDense && f.R > sms && f.n >= 8192) pieces = true;
+    const unsigned long long warps = (unsigned long long)P * kPieceWarps;
+    // a warp has parts of two block-rows at most, and the arithmetic is 32-bit
+    if (warps < (unsigned)f.R || (warps + 1) * (unsigned)(f.R + 2) >= (1ull << 32) || warps * ((unsigned)f.n + 8u) >= (1ull << 32)) pieces = false;
+    S = S < least ? least : (S > kMaxSplit ? kMaxSplit : S);
+    const int kind = S == 1 ? kPlain : g_no_cluster ? kSerial : kCluster;
+    // a grid that fits one CTA per SM is spread that way (two CTAs of a cluster may otherwise share an SM while others idle)
+    const bool alone = !pieces && kind == kCluster && f.R <= max_clusters<G, BITS, MODE>(S, kAlone, true, sms, dev);
+    // whole block-rows on one CTA per SM: 16 warps (14336 x 4096 6.2 against 6.5 us, 18944 x 4096 6.4 against 7.0)
+    const bool wide = !pieces && kind == kPlain && f.R <= sms;
+    const bool cluster = !pieces && kind == kCluster;
     GemvArgs ga;
     ga.codes = static_cast<const uint8_t*>(codes);
     ga.meta = static_cast<const unsigned*>(meta);
-    ga.R = f.R;
     ga.n = f.n;
+    ga.R = f.R;
+    ga.splits = S;
+    ga.magic_s = 0xffffffffu / (unsigned)S;
+    ga.warps = (unsigned)warps;
+    ga.magic_w = 0xffffffffu / ga.warps;
+    ga.magic_r = 0xffffffffu / (unsigned)f.R;
+    ga.magic_p = 0xffffffffu / (unsigned)P;
+    ga.arrived = static_cast<unsigned*>(workspace);
+    ga.partial = reinterpret_cast<float*>(static_cast<unsigned char*>(workspace) + header_bytes(f.R));
     ga.x = static_cast<const __half*>(x);
     ga.idx = idx;
     ga.count = count;
     ga.y = static_cast<__half*>(y);
-    ga.counters = static_cast<int*>(workspace);
-    ga.status = ga.counters + f.R;
-    ga.words = reinterpret_cast<unsigned long long*>(static_cast<char*>(workspace) + header_bytes(f.R));
-    ga.partials = reinterpret_cast<float*>(static_cast<char*>(workspace) + header_bytes(f.R) + tagged_bytes(f));
-    ga.zpartials = ga.partials + (size_t)f.R * slots * G;
-    ga.max_slots = slots;
-    ga.magic_p = magic_of((unsigned)P);
-    ga.magic_r = magic_of((unsigned)f.R);
-    ga.thr = fa.t;
+    ga.thr = fa.t != fa.t ? 0x7c00 : fa.t < 0.0f ? 0xbc00 : __half_as_ushort(__float2half_rd(fa.t));
     ga.idx_out = fa.idx_out;
     ga.count_out = fa.count_out;
-    ga.flags = flags;
-    if (MODE == kModeList && scratch_bytes(f.n, false) <= stage_area_bytes<G, BITS>()) ga.flags |= kFlagXs;
-    if (MODE == kModeFused && g_static_partition) ga.flags |= kFlagStatic;
+    ga.static_partition = g_static_partition;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(P);
-    cfg.blockDim = dim3(kGemvThreads);
-    cfg.dynamicSmemBytes = smem;
+    cfg.blockDim = dim3(pieces || wide ? 512 : 256);
+    cfg.dynamicSmemBytes = pieces ? kSmemPieces : alone ? kAlone : wide ? kSmem16 : kind == kPlain ? kSmemPlain : kSmem;
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
-    int nattr = 0;
-    if (!g_no_pdl) {
-        attr[nattr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[nattr].val.programmaticStreamSerializationAllowed = 1;
-        ++nattr;
-    }
-    // A whole number (2..8) of CTAs per block-row: launch them as one thread-block cluster each, if the
-    // device can hold all the clusters at once (asked once per kernel, cluster size and device).
-    int cluster_k = 0;
-    // Not for the call that collects the indices inside: alone, or behind launches of its own kind, it gains
-    // 0.3-0.45 us from a cluster like the others, but in a stream that alternates it with launches that fill
-    // every SM (the stacked gate|up matrix of a decoder layer) every such pair of launches was measured 1.4-1.8 us
-    // slower than the sum of its parts (0.2-0.6 us for the other kinds of call): a layer's four launches take
-    // 37.1 us without these clusters and 38.7 us with them.  The CTAs of a cluster can only start together.
-    if (!g_no_cluster && MODE != kModeFused && f.R <= P && P % f.R == 0 && P / f.R >= 2 && P / f.R <= kMaxCluster) {
-        const int k = P / f.R;
-        static signed char fits[64][kMaxCluster + 1][149] = {};  // [device][k][clusters]: 0 unknown, 1 yes, -1 no
-        const int nclusters = P / k;
-        if (nclusters <= 148) {
-            signed char& known = fits[dev][k][nclusters];
-            attr[nattr].id = cudaLaunchAttributeClusterDimension;
-            attr[nattr].val.clusterDim.x = k;
-            attr[nattr].val.clusterDim.y = 1;
-            attr[nattr].val.clusterDim.z = 1;
-            if (known == 0) {
-                cfg.attrs = attr;
-                cfg.numAttrs = nattr + 1;
-                int can = 0;
-                if (cudaOccupancyMaxActiveClusters(&can, kernel_c, &cfg) == cudaSuccess && can >= nclusters) known = 1;
-                else { known = -1; (void)cudaGetLastError(); }
-            }
-            if (known == 1) { cluster_k = k; ++nattr; }
-        }
-    }
-    ga.cluster_k = cluster_k;
-    cfg.attrs = attr;
-    cfg.numAttrs = nattr;
-    const cudaError_t err = cudaLaunchKernelEx(&cfg, cluster_k ? kernel_c : kernel, ga);
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = S;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(pieces ? (unsigned)P : (unsigned)f.R * (unsigned)(cluster ? S : 1));
+    cfg.attrs = g_no_pdl ? attr + 1 : attr;
+    cfg.numAttrs = (g_no_pdl ? 0 : 1) + (cluster ? 1 : 0);
+    auto kernel = pieces             ? gemv_pieces_kernel<G, BITS, MODE>
+                  : wide             ? gemv_kernel<G, BITS, MODE, kPlain, 16>
+                  : kind == kPlain   ? gemv_kernel<G, BITS, MODE, kPlain, 8>
+                  : kind == kCluster ? gemv_kernel<G, BITS, MODE, kCluster, 8>
+                                     : gemv_kernel<G, BITS, MODE, kSerial, 8>;
+    const cudaError_t err = cudaLaunchKernelEx(&cfg, kernel, ga);
     count_launch();
     return (err == cudaSuccess && cudaGetLastError() == cudaSuccess) ? SPQT_OK : SPQT_ERR_CUDA;
 }
@@ -1248,28 +1143,19 @@ static spqt_status check_gemv_args(const void* codes, const void* meta, int m, i
         (!dense && (!aligned(idx, 4) || !aligned(count, 4))))
         return SPQT_ERR_ALIGNMENT;
     if (ws_bytes < workspace_bytes(*f)) return SPQT_ERR_WORKSPACE;
-    if ((long long)f->R * kMaxCtas >= (1ll << 31)) return SPQT_ERR_UNSUPPORTED;  // the work map is 32-bit
+    if ((long long)f->R * kMaxSplit >= (1ll << 31)) return SPQT_ERR_UNSUPPORTED;  // grid size
     return SPQT_OK;
 }
 
 template <int MODE>
 static spqt_status gemv_dispatch(const Format& f, const void* codes, const void* meta, const void* x,
-                                 const int32_t* idx, const int32_t* count, void* y, void* workspace,
-                                 cudaStream_t s, FusedArgs fa, int flags)
+                                 const int32_t* idx, const int32_t* count, void* y, void* workspace, cudaStream_t s, FusedArgs fa)
 {
-    if (f.bits == 4 && f.group == 128) return launch_gemv<128, 4, MODE>(f, codes, meta, x, idx, count, y, workspace, s, fa, flags);
-    if (f.bits == 4 && f.group == 64) return launch_gemv<64, 4, MODE>(f, codes, meta, x, idx, count, y, workspace, s, fa, flags);
-    if (f.bits == 3 && f.group == 128) return launch_gemv<128, 3, MODE>(f, codes, meta, x, idx, count, y, workspace, s, fa, flags);
-    if (f.bits == 3 && f.group == 64) return launch_gemv<64, 3, MODE>(f, codes, meta, x, idx, count, y, workspace, s, fa, flags);
+    if (f.bits == 4 && f.group == 128) return launch_gemv<128, 4, MODE>(f, codes, meta, x, idx, count, y, workspace, s, fa);
+    if (f.bits == 4 && f.group == 64) return launch_gemv<64, 4, MODE>(f, codes, meta, x, idx, count, y, workspace, s, fa);
+    if (f.bits == 3 && f.group == 128) return launch_gemv<128, 3, MODE>(f, codes, meta, x, idx, count, y, workspace, s, fa);
+    if (f.bits == 3 && f.group == 64) return launch_gemv<64, 3, MODE>(f, codes, meta, x, idx, count, y, workspace, s, fa);
     return SPQT_ERR_UNSUPPORTED;
-}
-
-static bool fused_fits_format(const Format& f)
-{
-    if (f.bits == 4 && f.group == 128) return fused_fits<128, 4>(f.n);
-    if (f.bits == 4 && f.group == 64) return fused_fits<64, 4>(f.n);
-    if (f.bits == 3 && f.group == 128) return fused_fits<128, 3>(f.n);
-    return fused_fits<64, 3>(f.n);
 }
 
 // The sparse call after its arguments have been checked.
@@ -1281,13 +1167,12 @@ static spqt_status sparse_checked(const Format& f, const void* codes, const void
         spqt_status st = debug_check(idx, count, f.n, static_cast<int*>(workspace) + f.R, s, &count);
         if (st != SPQT_OK) return st;
     }
-    return gemv_dispatch<kModeList>(f, codes, meta, x, idx, count, y, workspace, s, FusedArgs{0.0f, nullptr, nullptr}, 0);
+    return gemv_dispatch<kModeList>(f, codes, meta, x, idx, count, y, workspace, s, FusedArgs{0.0f, nullptr, nullptr});
 }
 
 }  // namespace spqt
 
-// Scratch of the entry point that allocates nothing: one block-row counter array, status word and
-// partial-sum area, resident in every device that loads the library until the process exits.
+// Scratch of the entry point that allocates nothing (it holds the status word), resident in every device that loads the library until the process exits.
 constexpr size_t kStaticScratchBytes = size_t(1) << 20;
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
 
@@ -1334,15 +1219,13 @@ spqt_status spqt_sparsify_gemv(const void* codes, const void* scale_zero,
     if (st != SPQT_OK) return st;
     if (n > kMaxListN) return SPQT_ERR_UNSUPPORTED;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (!fused_fits_format(f)) {
+    if (n > kMaxFusedN) {
         // too long for the in-kernel scan: the same result from the two separate launches
         st = spqt_sparsify(x, n, t, idx, count, stream);
         if (st != SPQT_OK) return st;
-        return gemv_dispatch<kModeList>(f, codes, scale_zero, x, idx, count, y, workspace, s,
-                                        FusedArgs{0.0f, nullptr, nullptr}, 0);
+        return gemv_dispatch<kModeList>(f, codes, scale_zero, x, idx, count, y, workspace, s, FusedArgs{0.0f, nullptr, nullptr});
     }
-    return gemv_dispatch<kModeFused>(f, codes, scale_zero, x, nullptr, nullptr, y, workspace, s,
-                                     FusedArgs{t, idx, count}, 0);
+    return gemv_dispatch<kModeFused>(f, codes, scale_zero, x, nullptr, nullptr, y, workspace, s, FusedArgs{t, idx, count});
 }
 
 spqt_status spqt_dense_gemv(const void* codes, const void* scale_zero,
@@ -1356,12 +1239,7 @@ spqt_status spqt_dense_gemv(const void* codes, const void* scale_zero,
     if (st != SPQT_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const FusedArgs none{0.0f, nullptr, nullptr};
-    // whole chunks of a block-row by bulk copies when every chunk starts on a 16-byte boundary
-    if ((n & 7) == 0 && aligned(x, 16))
-        return gemv_dispatch<kModeDense>(f, codes, scale_zero, x, nullptr, nullptr, y, workspace, s, none, 0);
-    if (n > kMaxListN) return SPQT_ERR_UNSUPPORTED;
-    // otherwise the list path over the identity list
-    return gemv_dispatch<kModeList>(f, codes, scale_zero, x, nullptr, nullptr, y, workspace, s, none, kFlagIdentity);
+    return gemv_dispatch<kModeDense>(f, codes, scale_zero, x, nullptr, nullptr, y, workspace, s, none);
 }
 
 spqt_status spqt_sparse_gemv_static(const void* codes, const void* scale_zero,
@@ -1379,10 +1257,9 @@ spqt_status spqt_sparse_gemv_static(const void* codes, const void* scale_zero,
     st = check_gemv_args(codes, scale_zero, m, n, bits, group, x, idx, count, false, y, scratch, kStaticScratchBytes, &f);
     if (st != SPQT_OK) return st;
     if (n > kMaxListN) return SPQT_ERR_UNSUPPORTED;
-    // The scratch keeps whatever the previous call (or an interrupted one, or one of another shape)
-    // left: the arrival counters, the status word and the tagged words must start at zero.
+    // The scratch keeps whatever the previous call left: the status word must start at zero.
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (cudaMemsetAsync(scratch, 0, header_bytes(f.R) + tagged_bytes(f), s) != cudaSuccess) return SPQT_ERR_CUDA;
+    if (cudaMemsetAsync(scratch, 0, header_bytes(f.R), s) != cudaSuccess) return SPQT_ERR_CUDA;
     return sparse_checked(f, codes, scale_zero, x, idx, count, y, scratch, s);
 }
 
@@ -1416,15 +1293,14 @@ spqt_status spqt_autotune(const void* codes, const void* scale_zero, int m, int 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int sms = sm_count();
     if (sms <= 0) return SPQT_ERR_CUDA;
-    // candidates: one CTA per SM, and every whole number (1..8) of CTAs per block-row that fits
-    int cand[10], ncand = 0;
-    cand[ncand++] = sms;
-    for (int k = 1; k <= kMaxCluster; ++k)
-        if ((long long)k * f.R <= sms && k * f.R != sms) cand[ncand++] = k * f.R;
+    // candidates: every number of CTAs per block-row of which all are resident at once
+    int cand[kMaxSplit], ncand = 0;
+    for (int k = 1; k <= kMaxSplit; ++k)
+        if (k == 1 || (long long)k * f.R <= kCtasPerSm * sms) cand[ncand++] = k * f.R;
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) return SPQT_ERR_CUDA;
     const int saved = g_tune_ctas;
-    const bool fused_ok = fused_fits_format(f);
+    const bool fused_ok = n <= kMaxFusedN;
     int best[2] = {0, 0};
     st = SPQT_OK;
     for (int kind = 0; kind < 2 && st == SPQT_OK; ++kind) {   // 0: index collection + sparse product, 1: dense product
@@ -1456,7 +1332,7 @@ spqt_status spqt_autotune(const void* codes, const void* scale_zero, int m, int 
     if (st != SPQT_OK) return st;
     store_tuned(f, fused_ok ? kModeFused : kModeList, best[0]);
     if (fused_ok) store_tuned(f, kModeList, best[0]);
-    store_tuned(f, (n & 7) == 0 && aligned(x, 16) ? kModeDense : kModeList, best[1]);
+    store_tuned(f, kModeDense, best[1]);
     if (ctas_sparse) *ctas_sparse = best[0];
     if (ctas_dense) *ctas_dense = best[1];
     return SPQT_OK;

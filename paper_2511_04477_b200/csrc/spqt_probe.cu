@@ -4,24 +4,21 @@
 // 128-byte line -- the access pattern of a sparse GEMV at 50 % block density.  The two figures are the
 // achievable read and gather rooflines the benchmark prints next to the copy-bandwidth peak.
 //
-// A second probe measures the other ceiling of the GEMV loop: the dequantize-FMA arithmetic alone, on
-// operands that already sit in shared memory (no copies, no list, no reduction), with the GEMV's own
-// device functions.  Its rate, in 2 KB chunks per second, times the bytes a chunk stands for, is the
-// bandwidth at which instruction issue alone would saturate.
+// A second probe measures the other ceiling of the GEMV loop: the product of a chunk alone, on operands that already sit
+// in shared memory (no copies, no list, no preparation of multipliers, no reduction), with the GEMV's own device
+// functions.  Its rate, in 2 KB chunks per second, times the bytes a chunk stands for, is the bandwidth at which
+// instruction issue alone would saturate.
 #include "spqt_common.cuh"
-
-namespace spqt {
-constexpr unsigned long long kWaitNs = 1000000000ull;  // (the device header's bounded waits; unused here)
-}
 #include "spqt_gemv_device.cuh"
+#include "spqt_mma.cuh"
 
 namespace spqt {
 
 constexpr int kProbeWarps = 16;
 constexpr int kArithStages = 3;          // 2 KB stages a warp cycles through, as in the GEMV
-constexpr int kArithWarpBytes = kArithStages * 2048 + 256;   // + the chunk's 32 multiplier pairs
+constexpr int kArithWarpBytes = kArithStages * 2048 + 512;   // + the chunk's B operand
 
-// Every warp runs `chunks` times the eight 512-byte steps of a full 4-bit chunk with groups of 128 rows.
+// Every warp runs `chunks` times the product of a full 4-bit chunk with groups of 128 rows.
 __global__ void __launch_bounds__(kProbeWarps * 32, 1) probe_arith_kernel(int chunks, float* __restrict__ sink)
 {
     extern __shared__ __align__(16) unsigned char probe_smem[];
@@ -32,35 +29,33 @@ __global__ void __launch_bounds__(kProbeWarps * 32, 1) probe_arith_kernel(int ch
         words[i] = h ^ (h >> 13);       // arbitrary code bytes
     }
     __syncthreads();
-    float* mf = reinterpret_cast<float*>(probe_smem + warp * kArithWarpBytes + kArithStages * 2048);
-    for (int i = lane; i < 64; i += 32) mf[i] = 0x1p93f * (1.0f + (float)(i >> 1));   // pairs (a, a) * 2^93
+    __half* mf = reinterpret_cast<__half*>(probe_smem + warp * kArithWarpBytes + kArithStages * 2048);
+    for (int i = lane; i < 256; i += 32) mf[i] = __float2half_rn((float)(32 * (1 + (i >> 3))));
     __syncwarp();
     const unsigned base = smem_u32(probe_smem) + warp * kArithWarpBytes;
-    const unsigned mult_base = base + kArithStages * 2048;
-    const int mslot = lane / 8;
-    unsigned long long acc[8];
+    using Layout = MmaStage<128, 4>;
+    const Layout::Lane ll(lane);
+    float acc[2][4][4];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) acc[i] = 0ull;
+    for (int i = 0; i < 32; ++i) acc[i >> 4][(i >> 2) & 3][i & 3] = 0.0f;
     unsigned rc = 0;
 #pragma unroll 1
     for (int it = 0; it < chunks; ++it) {
-        const unsigned st_addr = base + rc;
+        unsigned bb[4];
+        ldsm_x4_trans(base + kArithStages * 2048 + 16 * lane, bb);
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const unsigned long long mm = lds_u64(mult_base + 8u * (u * 4 + mslot));
-            const uint2 wv = lds_v2(st_addr + lane * 8 + u * 256);
-            fma_block8_cum(acc, wv, mm);
+        for (int ks = 0; ks < 2; ++ks) {
+            unsigned c[2][4];
+            Layout::load(base + rc, ll, ks, c);
+#pragma unroll
+            for (int sp = 0; sp < 2; ++sp) mma_group<false>(acc[sp], c[sp], bb + 2 * ks, bb);
         }
         __syncwarp();
         rc = (rc + 2048u == kArithStages * 2048u) ? 0u : rc + 2048u;
     }
     float s = 0.0f;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        float lo, hi;
-        unpack2(acc[i], lo, hi);
-        s += lo + hi;
-    }
+    for (int i = 0; i < 32; ++i) s += acc[i >> 4][(i >> 2) & 3][i & 3];
     sink[(size_t)blockIdx.x * blockDim.x + threadIdx.x] = s;
 }
 

@@ -41,3 +41,34 @@ def test_small_batch_at_chunk_part_and_split_edges(bits, group, m_blocks, n, bat
         y_ref, dbound = oracle.dense_gemv(codes, s, z, m, n, X[b], bits, group)
         check_y(Y.cpu().numpy()[b], y_ref, dbound, "dense row %d" % b)
         check_y(Ys.cpu().numpy()[b], Ys_ref[b], bound[b], "row %d" % b)
+
+
+@pytest.mark.parametrize("bits,group", FORMATS)
+@pytest.mark.parametrize("m_blocks,n,ctas", [(1, 1, 0), (2, 31, 0), (3, 33, 2), (7, 257, 4), (40, 300, 7), (19, 2049, 8), (5, 8193, 0), (9, 300, 72),
+                                             (101, 33, 0), (149, 260, 0), (299, 40, 0), (149, 8192, 0), (149, 8200, 0)])
+def test_single_row_at_chunk_part_slice_and_piece_edges(bits, group, m_blocks, n, ctas):
+    """Clusters, one CTA per block-row with 16 and with 8 warps, equal pieces of all block-rows; the list given, collected in
+    the call (the same bits) and absent."""
+    m = m_blocks * group
+    W = inputs.weights(m, n, seed=m + n, std=0.1)
+    x = growing_activations(n, seed=90)
+    p = pack_on_gpu(W, bits, group)
+    codes, s, z = packed_to_host(p)
+    ws = binding.new_workspace(m, n, bits, group)
+    t = inputs.threshold_for_sparsity(x, 0.4) if n != 8192 else -1.0   # (the longest list of one CTA)
+    try:
+        binding.spqt_set_tuning(ctas)
+        y, idx, cnt = binding.spqt_sparsify_gemv(p, dev(x), t, ws)
+        y_list = binding.spqt_sparse_gemv(p, dev(x), idx, cnt, ws)
+        y_dense = binding.spqt_dense_gemv(p, dev(x), ws)
+        torch.cuda.synchronize()
+    finally:
+        binding.spqt_set_tuning(0)
+    ref_idx, ref_cnt = oracle.sparsify(x, t)
+    assert int(cnt.item()) == ref_cnt and np.array_equal(idx.cpu().numpy()[:ref_cnt], ref_idx)
+    y_ref, bound = oracle.sparse_gemv(codes, s, z, m, n, x, ref_idx, bits, group)
+    check_y(y.cpu().numpy(), y_ref, bound, "list collected")
+    assert torch.equal(y, y_list)
+    y_ref, bound = oracle.sparse_gemv(codes, s, z, m, n, x, np.arange(n, dtype=np.int32), bits, group)
+    check_y(y_dense.cpu().numpy(), y_ref, bound, "dense")
+    assert binding.spqt_workspace_status(ws, m, group) == 0 and int(ws.count_nonzero()) == 0
