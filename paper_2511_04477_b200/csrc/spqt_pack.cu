@@ -2,176 +2,195 @@
 // zigzag block layout (groups run down G rows of one column; blocks stored
 // row-major over (block-row, column)), plus the inverse of the layout step.
 #include "spqt_common.cuh"
+#include "spqt_quantize.cuh"
 
 namespace spqt {
 
-constexpr int kPackCols = 32;     // columns of one block-row handled by a CTA
-constexpr int kPackThreads = 256; // 8 warps, 4 columns each
+constexpr int kPackThreads = 128;  // 4 warps, 16 to 64 columns each
 
-// One CTA stages a G x 32 tile of W in shared memory with row-contiguous
-// (coalesced) reads, then each warp quantizes four columns.  Lane l of a warp
-// owns rows l, l+32, ... of the column.
+// One column by a warp, lane l owning rows l, l+32, ..: anything goes (not-a-number, infinities, a scale so small that
+// its rounding lets codes exceed the range).
 template <int G, int BITS>
-__global__ void __launch_bounds__(kPackThreads)
-pack_kernel(const __half* __restrict__ W, int n, int ldw,
-            uint8_t* __restrict__ codes, __half2* __restrict__ scale_zero)
+__device__ __noinline__ void convert_column(const __half* __restrict__ col, int ldw, int lane, uint8_t* __restrict__ q_sm, uint8_t* __restrict__ out, __half2* scale_zero)
 {
-    constexpr int B = G * BITS / 8;
-    constexpr int QMAX = (1 << BITS) - 1;
-    constexpr int PER_LANE = G / 32;
-    __shared__ __align__(16) __half tile[G][kPackCols + 2];
-    __shared__ uint8_t q_sm[kPackThreads / 32][G];
-
-    const int r = blockIdx.y;
-    const int k0 = blockIdx.x * kPackCols;
-    const int tid = threadIdx.x;
-
-    // Stage the tile.  A row of the tile is 64 bytes: four 16-byte loads when W, ldw and the tile allow
-    // it (the usual case), else one 2-byte load per weight.
-    const bool vec = (reinterpret_cast<uintptr_t>(W) & 15) == 0 && (ldw & 7) == 0 && k0 + kPackCols <= n;
-    if (vec) {
-        static_assert(kPackCols == 32 && ((kPackCols + 2) * 2) % 4 == 0, "tile rows are copied as 32-bit words");
-        for (int e = tid; e < G * 4; e += kPackThreads) {
-            const int i = e >> 2, part = e & 3;
-            const uint4 v = __ldg(reinterpret_cast<const uint4*>(W + (size_t)(r * G + i) * ldw + k0) + part);
-            unsigned* dst = reinterpret_cast<unsigned*>(&tile[i][part * 8]);  // rows start on a 4-byte boundary
-            dst[0] = v.x; dst[1] = v.y; dst[2] = v.z; dst[3] = v.w;
-        }
-    } else {
-        for (int e = tid; e < G * kPackCols; e += kPackThreads) {
-            int i = e / kPackCols, c = e % kPackCols;
-            int k = k0 + c;
-            tile[i][c] = (k < n) ? W[(size_t)(r * G + i) * ldw + k] : __float2half(0.0f);
-        }
+    constexpr int PER_LANE = G / 32, B = G * BITS / 8, QMAX = (1 << BITS) - 1;
+    float w[PER_LANE];
+    float lo = INFINITY, hi = -INFINITY;
+#pragma unroll
+    for (int u = 0; u < PER_LANE; ++u) {
+        w[u] = __half2float(col[(size_t)(lane + 32 * u) * ldw]);
+        lo = fminf(lo, w[u]);
+        hi = fmaxf(hi, w[u]);
     }
-    __syncthreads();
-
-    const int warp = tid / 32, lane = tid % 32;
-    for (int cc = 0; cc < kPackCols / (kPackThreads / 32); ++cc) {
-        const int c = warp * (kPackCols / (kPackThreads / 32)) + cc;
-        const int k = k0 + c;
-        if (k >= n) break;  // uniform across the warp
-        float w[PER_LANE];
-        float lo = INFINITY, hi = -INFINITY;
 #pragma unroll
-        for (int u = 0; u < PER_LANE; ++u) {
-            w[u] = __half2float(tile[lane + 32 * u][c]);
-            lo = fminf(lo, w[u]);
-            hi = fmaxf(hi, w[u]);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-            hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-        }
-        // a zero extreme of either sign counts as +0.0 (x + (+0.0) is x, except that -0.0 becomes +0.0)
-        lo = __fadd_rn(lo, 0.0f);
-        hi = __fadd_rn(hi, 0.0f);
-        // scale = fp16((max - min) / qmax): one IEEE subtract, one IEEE divide, RN-even
-        const float s32 = __fdiv_rn(__fsub_rn(hi, lo), (float)QMAX);
-        const __half sh = __float2half_rn(s32);
-        const float sf = __half2float(sh);
-        // w - lo >= 0 exactly, so the rounded quotient needs no lower clamp; round-to-nearest-even
-        // conversion and one integer min give the code
-        int code[PER_LANE];
-#pragma unroll
-        for (int u = 0; u < PER_LANE; ++u)
-            code[u] = (sf != 0.0f) ? min(__float2int_rn(__fdiv_rn(__fsub_rn(w[u], lo), sf)), QMAX) : 0;
-        const size_t blk = (size_t)r * n + k;
-        uint8_t* out = codes + blk * B;
-        if (BITS == 4) {
-            // lane l owns rows l, l+32, ...: byte i pairs rows i and i + G/2, both of the same lane
-#pragma unroll
-            for (int u = 0; u < PER_LANE / 2; ++u)
-                out[lane + 32 * u] = (uint8_t)(code[u] | (code[u + PER_LANE / 2] << 4));
-        } else {
-#pragma unroll
-            for (int u = 0; u < PER_LANE; ++u) q_sm[warp][lane + 32 * u] = (uint8_t)code[u];
-            __syncwarp();
-            for (int b = lane; b < B; b += 32) {
-                unsigned v = 0;
-                if (b < G / 4) {
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) v |= (q_sm[warp][b + u * (G / 4)] & 3u) << (2 * u);
-                } else {
-                    const int j = b - G / 4;
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) v |= ((q_sm[warp][j + u * (G / 8)] >> 2) & 1u) << u;
-                }
-                out[b] = (uint8_t)v;
-            }
-        }
-        if (lane == 0) scale_zero[blk] = __halves2half2(sh, __float2half_rn(lo));  // exact: lo is an fp16 value
-        __syncwarp();
+    for (int o = 16; o > 0; o >>= 1) {
+        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
     }
-}
-
-// 4-bit codes, one THREAD per column: a CTA stages a G x 128 tile with 16-byte loads, then thread c
-// walks down column c twice (min/max, then codes), so that nothing crosses lanes and the per-column
-// work (scale, offset, stores) is done by all lanes at once.  A thread writes its block with 16-byte
-// stores.  Same arithmetic as pack_kernel, bit for bit.  Used for G = 64 when W, ldw and n allow the
-// vector loads.
-constexpr int kPack4Cols = 128;
-
-template <int G>
-__global__ void __launch_bounds__(kPack4Cols)
-pack4_kernel(const __half* __restrict__ W, int n, int ldw,
-             uint8_t* __restrict__ codes, __half2* __restrict__ scale_zero)
-{
-    constexpr int B = G / 2;
-    constexpr int QMAX = 15;
-    constexpr int kStride = kPack4Cols + 8;  // halves per tile row: keeps rows 16-byte aligned
-    __shared__ __align__(16) __half tile[G][kStride];
-
-    const int r = blockIdx.y;
-    const int k0 = blockIdx.x * kPack4Cols;
-    const int tid = threadIdx.x;
-    const int cols = min(kPack4Cols, n - k0);  // a multiple of 8 (the host checks n)
-
-    // 16 chunks of 8 halves per tile row
-    for (int e = tid; e < G * (kPack4Cols / 8); e += kPack4Cols) {
-        const int i = e / (kPack4Cols / 8), part = e % (kPack4Cols / 8);
-        if (part * 8 < cols)
-            *reinterpret_cast<uint4*>(&tile[i][part * 8]) =
-                __ldg(reinterpret_cast<const uint4*>(W + (size_t)(r * G + i) * ldw + k0) + part);
-    }
-    __syncthreads();
-    if (tid >= cols) return;
-
-    // minimum and maximum of the column: exact in fp16
-    __half lo_h = tile[0][tid], hi_h = lo_h;
-#pragma unroll 8
-    for (int i = 1; i < G; ++i) {
-        const __half v = tile[i][tid];
-        lo_h = __hmin(lo_h, v);
-        hi_h = __hmax(hi_h, v);
-    }
-    // a zero extreme of either sign counts as +0.0
-    const float lo = __fadd_rn(__half2float(lo_h), 0.0f), hi = __fadd_rn(__half2float(hi_h), 0.0f);
-    // scale = fp16((max - min) / qmax): one IEEE subtract, one IEEE divide, RN-even
+    lo = __fadd_rn(lo, 0.0f);
+    hi = __fadd_rn(hi, 0.0f);
     const __half sh = __float2half_rn(__fdiv_rn(__fsub_rn(hi, lo), (float)QMAX));
     const float sf = __half2float(sh);
-    const size_t blk = (size_t)r * n + k0 + tid;
-    uint4* out = reinterpret_cast<uint4*>(codes + blk * B);
-    // byte i = code of row i | code of row i + G/2 << 4; sixteen bytes per store
-#pragma unroll 1
-    for (int q = 0; q < B / 16; ++q) {
-        unsigned wds[4] = {0u, 0u, 0u, 0u};
+    __syncwarp();
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            const int i = q * 16 + j;
-            const float a = __half2float(tile[i][tid]), b = __half2float(tile[i + G / 2][tid]);
-            int ca = 0, cb = 0;
-            if (sf != 0.0f) {
-                // w - lo >= 0 exactly: no lower clamp; round-to-nearest-even conversion and one integer min
-                ca = min(__float2int_rn(__fdiv_rn(__fsub_rn(a, lo), sf)), QMAX);
-                cb = min(__float2int_rn(__fdiv_rn(__fsub_rn(b, lo), sf)), QMAX);
-            }
-            wds[j >> 2] |= (unsigned)(ca | (cb << 4)) << (8 * (j & 3));
+    for (int u = 0; u < PER_LANE; ++u)
+        q_sm[lane + 32 * u] = (uint8_t)((sf != 0.0f) ? min(__float2int_rn(__fdiv_rn(__fsub_rn(w[u], lo), sf)), QMAX) : 0);
+    __syncwarp();
+    for (int b = lane; b < B; b += 32) {
+        unsigned v = 0;
+        if (BITS == 4) {
+            v = q_sm[b] | (q_sm[b + G / 2] << 4);
+        } else if (b < G / 4) {
+            for (int u = 0; u < 4; ++u) v |= (q_sm[b + u * (G / 4)] & 3u) << (2 * u);
+        } else {
+            for (int u = 0; u < 8; ++u) v |= ((q_sm[b - G / 4 + u * (G / 8)] >> 2) & 1u) << u;
         }
-        out[q] = make_uint4(wds[0], wds[1], wds[2], wds[3]);
+        out[b] = (uint8_t)v;
     }
-    scale_zero[blk] = __halves2half2(sh, __float2half_rn(lo));
+    if (lane == 0) *scale_zero = __halves2half2(sh, __float2half_rn(lo));
+}
+
+// A thread converts 64 rows of NC columns in registers (so that W is read once, up to 8 KB in flight per warp), two fp32
+// operations per instruction: two neighbouring columns when W can be read by the word, else one and neighbouring rows.  With
+// G = 128 two lanes share a column: of every 16 rows lane half h has those from 8h on.  The codes of a warp's blocks meet in
+// shared memory and leave in 16-byte pieces, neighbouring lanes to neighbouring places.
+//
+// Bound by memory: 28672 x 8192 to 4 bits, 595 MB.  With an IEEE division per weight (about 20 instructions) and one
+// column per warp or thread it took 344 us, now 128 us (4.65 TB/s); with all 128 rows of a group in one thread's
+// registers (12 warps per SM) 161 us.
+template <int G, int BITS, int NC>
+__global__ void __launch_bounds__(kPackThreads, NC == 2 ? 5 : 6)
+pack_kernel(const __half* W, int n, int ldw, uint8_t* codes, __half2* scale_zero)
+{
+    constexpr int B = G * BITS / 8, Q = (1 << BITS) - 1, H = G / 64, kCols = 32 * NC / H;
+    constexpr int CB = B % 16 == 0 ? 16 : 8;         // bytes per piece of a block
+    constexpr int kPieces = B / CB;                  // of a block
+    __shared__ __align__(16) unsigned char out_sm[kPackThreads / 32][kCols * B];
+
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, h = lane / (32 / H), column = NC * (lane % (32 / H));
+    const int r = blockIdx.y;
+    const int k0 = (blockIdx.x * (kPackThreads / 32) + warp) * kCols, k = k0 + column;
+    if (k0 >= n) return;
+    unsigned char* const mine = out_sm[warp];
+    // place of byte b of the warp's blocks: 16-byte pieces so that lanes 128 or 64 bytes apart hit different banks
+    auto place = [](int b) { return CB == 16 ? ((b >> 4) ^ ((b >> 7) & 7)) * 16 + (b & 15) : b; };
+
+    const __half* const src = W + ((size_t)r * G + 8 * h) * ldw + k;
+    const bool on = k < n;               // (NC = 2: n is even)
+    // rows (G/8)*u + 8h + j, u and j in 0..7.  NC = 2: the two columns of one; NC = 1: j and j + 1
+    __half2 v[32 * NC];
+#pragma unroll
+    for (int i = 0; i < 32 * NC; ++i) {
+        const int row = (G / 8) * (i / (4 * NC)) + (i % (4 * NC)) * (NC == 2 ? 1 : 2);
+        if (NC == 2) {
+            const unsigned u = on ? __ldcs(reinterpret_cast<const unsigned*>(src + (size_t)row * ldw)) : 0u;
+            v[i] = *reinterpret_cast<const __half2*>(&u);
+        } else {
+            v[i] = __halves2half2(on ? src[(size_t)row * ldw] : __half(0.0f), on ? src[(size_t)(row + 1) * ldw] : __half(0.0f));
+            if ((i & 7) == 7) asm volatile("" ::: "memory");   // (not all halves in registers of their own before they are paired)
+        }
+    }
+    // minimum and maximum: exact in fp16 (the maximum is not-a-number if any weight is)
+    __half2 lo2 = v[0], hi2 = v[0];
+#pragma unroll
+    for (int i = 1; i < 32 * NC; ++i) {
+        lo2 = __hmin2(lo2, v[i]);
+        hi2 = __hmax2_nan(hi2, v[i]);
+    }
+    if (H == 2) {
+        lo2 = __hmin2(lo2, __shfl_xor_sync(0xffffffffu, lo2, 16));
+        hi2 = __hmax2_nan(hi2, __shfl_xor_sync(0xffffffffu, hi2, 16));
+    }
+    if (NC == 1) {
+        lo2 = __hmin2(lo2, __lowhigh2highlow(lo2));
+        hi2 = __hmax2_nan(hi2, __lowhigh2highlow(hi2));
+    }
+    // a zero extreme of either sign counts as +0.0 (x + (+0.0) is x, except that -0.0 becomes +0.0)
+    const float2 lo = make_float2(__fadd_rn(__low2float(lo2), 0.0f), __fadd_rn(__high2float(lo2), 0.0f));
+    const float2 hi = make_float2(__fadd_rn(__low2float(hi2), 0.0f), __fadd_rn(__high2float(hi2), 0.0f));
+    // scale = fp16((max - min) / qmax): one IEEE subtract, one IEEE divide, RN-even
+    const __half s0 = __float2half_rn(__fdiv_rn(__fsub_rn(hi.x, lo.x), (float)Q));
+    const __half s1 = NC == 2 ? __float2half_rn(__fdiv_rn(__fsub_rn(hi.y, lo.y), (float)Q)) : s0;
+    const Divisor2 by(make_float2(__half2float(s0), __half2float(s1)));
+    // (false for not-a-number: hi has it if any weight is; for infinities; if codes may exceed the range)
+    const bool plain[2] = {__fsub_rn(hi.x, lo.x) * by.inv.x <= (float)Q + 0.25f, __fsub_rn(hi.y, lo.y) * by.inv.y <= (float)Q + 0.25f};
+    const float2 minus_lo = make_float2(-lo.x, -lo.y);
+    // the codes of four rows from j = jj of u on, a byte each, of every column
+    auto four = [&](int u, int jj, unsigned* w) {
+        float2 t[2 * NC];
+#pragma unroll
+        for (int j = 0; j < 2 * NC; ++j) t[j] = round_to_low_bits(by.quotient(add2(__half22float2(v[(8 * u + jj) * NC / 2 + j]), minus_lo)));
+        if (NC == 2) {
+            w[0] = four_bytes(t[0].x, t[1].x, t[2 * NC - 2].x, t[2 * NC - 1].x) & (0x01010101u * Q);
+            w[NC - 1] = four_bytes(t[0].y, t[1].y, t[2 * NC - 2].y, t[2 * NC - 1].y) & (0x01010101u * Q);
+        } else {
+            w[0] = four_bytes(t[0].x, t[0].y, t[1].x, t[1].y) & (0x01010101u * Q);
+        }
+    };
+    auto put = [&](int c, int byte, const unsigned* w) { *reinterpret_cast<uint2*>(mine + place((column + c) * B + byte + 8 * h)) = make_uint2(w[0], w[1]); };
+    if (BITS == 4) {
+        // byte i: rows i and i + G/2
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            unsigned o[NC][2];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                unsigned l[NC], t[NC];
+                four(u, 4 * q, l);
+                four(u + 4, 4 * q, t);
+#pragma unroll
+                for (int c = 0; c < NC; ++c) o[c][q] = l[c] | (t[c] << 4);
+            }
+#pragma unroll
+            for (int c = 0; c < NC; ++c) put(c, (G / 8) * u, o[c]);
+        }
+    } else {
+        // byte b < G/4: the low two bits of rows b + (G/4)*u; byte G/4 + j: the third of rows j + (G/8)*u
+        unsigned top[NC][2] = {}, low[NC][2][2] = {};
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                unsigned l[NC];
+                four(u, 4 * q, l);
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    top[c][q] |= ((l[c] >> 2) & 0x01010101u) << u;
+                    low[c][u & 1][q] |= (l[c] & 0x03030303u) << (2 * (u >> 1));
+                }
+            }
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            put(c, 0, low[c][0]);
+            put(c, G / 8, low[c][1]);
+            put(c, G / 4, top[c]);
+        }
+    }
+    const size_t blk = (size_t)r * n + k;
+    if (on && h == 0) {
+        scale_zero[blk] = __halves2half2(s0, __float2half_rn(lo.x));                    // exact: lo is an fp16 value
+        if (NC == 2) scale_zero[blk + 1] = __halves2half2(s1, __float2half_rn(lo.y));
+    }
+    __syncwarp();
+    unsigned char* const dst = codes + ((size_t)r * n + k0) * B;
+    const int pieces = min(kCols, n - k0) * kPieces;
+#pragma unroll
+    for (int c = lane; c < kCols * kPieces; c += 32) {
+        if (c >= pieces) break;
+        if (CB == 16) *reinterpret_cast<uint4*>(dst + c * 16) = *reinterpret_cast<const uint4*>(mine + place(c * 16));
+        else *reinterpret_cast<uint2*>(dst + c * 8) = *reinterpret_cast<const uint2*>(mine + place(c * 8));
+    }
+    // the other columns once more
+#pragma unroll 1
+    for (int half = 0; half < NC; ++half) {
+        unsigned again = __ballot_sync(0xffffffffu, on && h == 0 && !(half == 0 ? plain[0] : plain[1]));
+        __syncwarp();
+        while (again != 0u) {
+            const int c = NC * (__ffs((int)again) - 1) + half;
+            again &= again - 1u;
+            convert_column<G, BITS>(W + (size_t)r * G * ldw + k0 + c, ldw, lane, mine, dst + c * B, scale_zero + (size_t)r * n + k0 + c);
+        }
+    }
 }
 
 // One thread per weight: read its code out of the zigzag buffer.
@@ -199,20 +218,12 @@ template <int G, int BITS>
 static spqt_status launch_pack(const Format& f, const void* W, int ldw, void* codes, void* scale_zero,
                                cudaStream_t s)
 {
-    // (with G = 128 its 34 KB tile per 128 threads leaves too few warps per SM to hide the division
-    // chains, and the warp-per-column kernel below is faster)
-    if (BITS == 4 && G == 64 && (reinterpret_cast<uintptr_t>(W) & 15) == 0 && (ldw & 7) == 0 && (f.n & 7) == 0) {
-        dim3 grid4((f.n + kPack4Cols - 1) / kPack4Cols, f.R);
-        pack4_kernel<G><<<grid4, kPack4Cols, 0, s>>>(
-            static_cast<const __half*>(W), f.n, ldw, static_cast<uint8_t*>(codes),
-            static_cast<__half2*>(scale_zero));
-        count_launch();
-        return cudaGetLastError() == cudaSuccess ? SPQT_OK : SPQT_ERR_CUDA;
-    }
-    dim3 grid((f.n + kPackCols - 1) / kPackCols, f.R);
-    pack_kernel<G, BITS><<<grid, kPackThreads, 0, s>>>(
-        static_cast<const __half*>(W), f.n, ldw, static_cast<uint8_t*>(codes),
-        static_cast<__half2*>(scale_zero));
+    const bool pairs = (reinterpret_cast<uintptr_t>(W) & 3) == 0 && ((ldw | f.n) & 1) == 0;   // of columns, as words
+    const int cols = kPackThreads * (pairs ? 2 : 1) * 64 / G;
+    const dim3 grid((f.n + cols - 1) / cols, f.R);
+    auto kernel = pairs ? pack_kernel<G, BITS, 2> : pack_kernel<G, BITS, 1>;
+    kernel<<<grid, kPackThreads, 0, s>>>(static_cast<const __half*>(W), f.n, ldw, static_cast<uint8_t*>(codes),
+                                         static_cast<__half2*>(scale_zero));
     count_launch();
     return cudaGetLastError() == cudaSuccess ? SPQT_OK : SPQT_ERR_CUDA;
 }

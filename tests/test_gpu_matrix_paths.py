@@ -1,4 +1,4 @@
-"""Edges of the kernels that multiply on tensor cores, against the fp64 oracle."""
+"""Edges of the kernels that multiply on tensor cores, against the fp64 oracle, and of the conversion that feeds them."""
 import numpy as np
 import pytest
 import torch
@@ -72,3 +72,30 @@ def test_single_row_at_chunk_part_slice_and_piece_edges(bits, group, m_blocks, n
     y_ref, bound = oracle.sparse_gemv(codes, s, z, m, n, x, np.arange(n, dtype=np.int32), bits, group)
     check_y(y_dense.cpu().numpy(), y_ref, bound, "dense")
     assert binding.spqt_workspace_status(ws, m, group) == 0 and int(ws.count_nonzero()) == 0
+
+
+@pytest.mark.parametrize("bits,group", FORMATS)
+@pytest.mark.parametrize("m_blocks,n,pad,shift", [(1, 1, 0, 0), (2, 16, 2, 0), (1, 66, 0, 0), (3, 130, 2, 2), (2, 258, 2, 1), (2, 257, 0, 0), (1, 31, 3, 0)])
+def test_conversion_at_the_edges_of_tiles_and_alignments(bits, group, m_blocks, n, pad, shift):
+    """Pairs of columns as words, single columns, bytes equal to the oracle's: quotients in the middle between two codes, groups
+    over many orders of magnitude, constant ones, scales that are subnormal or round to zero."""
+    m = m_blocks * group
+    rng = np.random.Generator(np.random.PCG64(m * 1000 + n + bits))
+    W = (rng.standard_normal((m, n)) * 10.0 ** rng.uniform(-6, 3, n)).astype(np.float16)
+    qmax = (1 << bits) - 1
+    ties = rng.integers(0, 2 * qmax + 1, (m, n)) * 0.5   # multiples of half the scale
+    ties[::group // 2] = 0.0
+    ties[1::group // 2] = qmax
+    pick = rng.integers(0, 4, n)
+    W = np.where(pick == 1, (ties * 2.0 ** rng.integers(-12, 5, n)).astype(np.float16), W)
+    W = np.where(pick == 2, (W * np.logspace(-3, 0, m)[:, None]).astype(np.float16), W)
+    W[:, n // 2] = W[0, n // 2]
+    buf = torch.zeros(shift + m * (n + pad), dtype=torch.float16, device="cuda")
+    Wd = buf[shift:].view(m, n + pad)[:, :n]
+    Wd.copy_(dev(np.ascontiguousarray(W)))
+    p = binding.spqt_pack(Wd, bits, group)
+    codes, s, z = packed_to_host(p)
+    ref_codes, ref_s, ref_z = oracle.pack(W, bits, group)
+    assert np.array_equal(np.asarray(codes).reshape(-1), np.asarray(ref_codes).reshape(-1))
+    assert np.array_equal(s.view(np.uint16).reshape(-1), ref_s.view(np.uint16).reshape(-1))
+    assert np.array_equal(z.view(np.uint16).reshape(-1), ref_z.view(np.uint16).reshape(-1))
