@@ -15,8 +15,7 @@
 // first code and of both codes together; per byte of single bits its low 1, 2, .. 8 bits: the cumulative form of
 // the main kernel) and takes the differences at the end.
 //
-//   kq_pack_kernel   a CTA stages a 256 x 32 tile of W; a warp quantizes four columns, lane l owning rows
-//                    l, l+32, .. (one row of every block).
+//   kq_pack_kernel   a thread converts two columns, a warp 64.
 //   kq_gemv_kernel   grid (S, R): CTA (s, r) takes the s-th of S slices of the index list (or of all
 //                    columns) for block-row r; its 8 warps take the slice's chunks of 16 entries in turn,
 //                    two record buffers per warp (cp.async: a record is one contiguous gather of 144 bytes,
@@ -31,6 +30,7 @@
 #include "spqt_common.cuh"
 
 #include "spqt_gemv_device.cuh"
+#include "spqt_quantize.cuh"
 
 namespace spqt {
 
@@ -42,7 +42,6 @@ constexpr int kKqWarps = 8;
 constexpr int kKqThreads = kKqWarps * 32;
 constexpr int kKqChunk = 16;        // list entries per chunk
 constexpr int kKqMaxSplit = 32;     // slices per block-row at most
-constexpr int kKqPackCols = 32;
 
 // ---------------------------------------------------------------- conversion
 //   per block i:      lo_i = min(min_j w_j, 0),  step_i = (max_j w_j - lo_i) / 15,  neg_i = 0 - lo_i
@@ -51,97 +50,153 @@ constexpr int kKqPackCols = 32;
 //                     sc_i = min(rint(step_i / d), 63),  m_i = min(rint(neg_i / dmin), 63)   (0 if the divisor is 0)
 //   per weight:       q_j = clamp(rint((w_j + dmin*m_i) / (d*sc_i)), 0, 15)                   (0 if d*sc_i == 0)
 // (15 = 2^BITS - 1 for 4-bit codes; 3 and 255 for the other widths)
-template <int BITS>
-__global__ void __launch_bounds__(256)
-kq_pack_kernel(const __half* __restrict__ W, int n, int ldw, uint8_t* __restrict__ records)
+// A thread converts two neighbouring columns, two fp32 operations per instruction, reading W twice (the second time from
+// L2): for the ranges of the blocks, then 4 rows of all eight blocks at a time for the codes.  Both are loops: unrolled over
+// all 256 rows the code has 150 KB, and the warps wait for it (14336 x 4096 to 4 bits 141 against 82 us; with an IEEE division per
+// weight and a column per warp 229 us).  The records of a warp's 64 columns meet in shared memory, a word of padding after
+// each against bank conflicts.
+constexpr int kKqPackWarps = 2;
+template <int BITS, bool VEC>
+__global__ void __launch_bounds__(kKqPackWarps * 32, 8)
+kq_pack_kernel(const __half* W, int n, int ldw, uint8_t* records)
 {
-    constexpr int kTop = (1 << BITS) - 1, NCB = kq_code_bytes(BITS), REC = kq_rec_bytes(BITS);
-    __shared__ __align__(16) __half tile[kKqG][kKqPackCols + 2];
-    const int r = blockIdx.y, k0 = blockIdx.x * kKqPackCols, tid = threadIdx.x;
-    for (int e = tid; e < kKqG * kKqPackCols; e += 256) {
-        const int i = e / kKqPackCols, c = e % kKqPackCols, k = k0 + c;
-        tile[i][c] = (k < n) ? W[(size_t)(r * kKqG + i) * ldw + k] : __float2half(0.0f);
+    constexpr int kTop = (1 << BITS) - 1, NCB = kq_code_bytes(BITS), REC = kq_rec_bytes(BITS), RW = REC / 4;
+    __shared__ unsigned rec_sm[kKqPackWarps][64 * (RW + 1)];
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int r = blockIdx.y, k0 = (blockIdx.x * kKqPackWarps + warp) * 64, k = k0 + 2 * lane;
+    if (k0 >= n) return;
+    unsigned* const mine = rec_sm[warp];
+    const bool on0 = k < n, on1 = k + 1 < n;
+    const __half* const src = W + (size_t)r * kKqG * ldw + k;
+    auto load = [&](int i) -> __half2 {
+        if (VEC) {                       // (n is even)
+            const unsigned u = on0 ? *reinterpret_cast<const unsigned*>(src + (size_t)i * ldw) : 0u;
+            return *reinterpret_cast<const __half2*>(&u);
+        }
+        return __halves2half2(on0 ? src[(size_t)i * ldw] : __half(0.0f), on1 ? src[(size_t)i * ldw + 1] : __half(0.0f));
+    };
+    // ---- ranges: exact in fp16
+#pragma unroll 1
+    for (int u = 0; u < 8; ++u) {
+        __half2 lo2 = load(32 * u), hi2 = lo2;
+#pragma unroll
+        for (int j = 1; j < 32; ++j) {
+            const __half2 v = load(32 * u + j);
+            lo2 = __hmin2(lo2, v);
+            hi2 = __hmax2(hi2, v);
+        }
+        mine[(2 * u) * 32 + lane] = *reinterpret_cast<const unsigned*>(&lo2);
+        mine[(2 * u + 1) * 32 + lane] = *reinterpret_cast<const unsigned*>(&hi2);
     }
-    __syncthreads();
-    const int warp = tid >> 5, lane = tid & 31;
-    for (int cc = 0; cc < 4; ++cc) {
-        const int c = warp * 4 + cc, k = k0 + c;
-        if (k >= n) break;  // uniform across the warp
-        float w[8], step[8], neg[8];
-        float step_max = 0.0f, neg_max = 0.0f;
+    float2 step[8], neg[8], step_max = make_float2(0.0f, 0.0f), neg_max = make_float2(0.0f, 0.0f);
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            w[u] = __half2float(tile[lane + 32 * u][c]);  // row lane of block u
-            float lo = w[u], hi = w[u];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-                hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-            }
+    for (int u = 0; u < 8; ++u) {
+        const unsigned l = mine[(2 * u) * 32 + lane], h = mine[(2 * u + 1) * 32 + lane];
+        const float2 lo = __half22float2(*reinterpret_cast<const __half2*>(&l)), hi = __half22float2(*reinterpret_cast<const __half2*>(&h));
+        auto range = [&](float lo, float hi, float& st, float& ng) {
             lo = __fadd_rn(fminf(lo, 0.0f), 0.0f);  // a zero of either sign counts as +0.0
             hi = __fadd_rn(hi, 0.0f);
-            step[u] = __fdiv_rn(__fsub_rn(hi, lo), (float)kTop);
-            neg[u] = __fsub_rn(0.0f, lo);           // (0 - 0 is +0.0)
-            step_max = fmaxf(step_max, step[u]);
-            neg_max = fmaxf(neg_max, neg[u]);
-        }
-        const __half dh = __float2half_rn(__fdiv_rn(step_max, 63.0f));
-        const __half mh = __float2half_rn(__fdiv_rn(neg_max, 63.0f));
-        const float df = __half2float(dh), dminf = __half2float(mh);
-        unsigned sc[8], mn[8];
-        int q[8];
+            st = __fdiv_rn(__fsub_rn(hi, lo), (float)kTop);
+            ng = __fsub_rn(0.0f, lo);
+        };
+        range(lo.x, hi.x, step[u].x, neg[u].x);
+        range(lo.y, hi.y, step[u].y, neg[u].y);
+        step_max = make_float2(fmaxf(step_max.x, step[u].x), fmaxf(step_max.y, step[u].y));
+        neg_max = make_float2(fmaxf(neg_max.x, neg[u].x), fmaxf(neg_max.y, neg[u].y));
+    }
+    __syncwarp();                        // (the records take the place of the ranges)
+    // ---- scales and minima
+    const __half2 dh = __halves2half2(__float2half_rn(__fdiv_rn(step_max.x, 63.0f)), __float2half_rn(__fdiv_rn(step_max.y, 63.0f)));
+    const __half2 mh = __halves2half2(__float2half_rn(__fdiv_rn(neg_max.x, 63.0f)), __float2half_rn(__fdiv_rn(neg_max.y, 63.0f)));
+    const float2 df = __half22float2(dh), dminf = __half22float2(mh);
+    const Divisor2 by_d(df), by_dmin(dminf);
+    auto limited = [](float2 v, float top) { return make_float2(fminf(fmaxf(v.x, 0.0f), top), fminf(fmaxf(v.y, 0.0f), top)); };   // (0 for not-a-number)
+    unsigned long long f64[2] = {0ull, 0ull};   // fields 0..9 and the low 4 bits of field 10
+    unsigned f32[2] = {0u, 0u};                 // bits 64..95
+    float2 offset[8];
+    Divisor2 by[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            sc[u] = (df != 0.0f) ? (unsigned)min(__float2int_rn(__fdiv_rn(step[u], df)), 63) : 0u;
-            mn[u] = (dminf != 0.0f) ? (unsigned)min(__float2int_rn(__fdiv_rn(neg[u], dminf)), 63) : 0u;
-            const float se = __fmul_rn(df, (float)sc[u]), oe = __fmul_rn(dminf, (float)mn[u]);
-            q[u] = (se != 0.0f) ? max(0, min(__float2int_rn(__fdiv_rn(__fadd_rn(w[u], oe), se)), kTop)) : 0;
-        }
-        uint8_t* rec = records + ((size_t)r * n + k) * REC;
-        // this lane holds the codes of rows lane + 32u
-        if (BITS == 4) {            // byte i = code of row i | code of row i + 128 << 4
+    for (int u = 0; u < 8; ++u) {
+        float2 ns = limited(by_d.quotient(step[u]), 63.0f), nm = limited(by_dmin.quotient(neg[u]), 63.0f);
+        ns = make_float2(rintf(ns.x), rintf(ns.y));
+        nm = make_float2(rintf(nm.x), rintf(nm.y));
+        offset[u] = make_float2(__fmul_rn(dminf.x, nm.x), __fmul_rn(dminf.y, nm.y));
+        by[u] = Divisor2(make_float2(__fmul_rn(df.x, ns.x), __fmul_rn(df.y, ns.y)));
+        const unsigned sc[2] = {(unsigned)ns.x, (unsigned)ns.y}, mn[2] = {(unsigned)nm.x, (unsigned)nm.y};
 #pragma unroll
-            for (int u = 0; u < 4; ++u) rec[lane + 32 * u] = (uint8_t)(q[u] | (q[u + 4] << 4));
-        } else if (BITS == 8) {     // byte i = code of row i
-#pragma unroll
-            for (int u = 0; u < 8; ++u) rec[lane + 32 * u] = (uint8_t)q[u];
-        } else if (BITS == 5 || BITS == 6) {
-            // the low four bits like 4-bit codes, then the high bits: one per row, bit j % 8 of byte j / 8 (the
-            // 32 rows lane + 32u of all lanes are one 32-bit word), or two per row arranged like 2-bit codes
-#pragma unroll
-            for (int u = 0; u < 4; ++u) rec[lane + 32 * u] = (uint8_t)((q[u] & 15) | ((q[u + 4] & 15) << 4));
-            if (BITS == 5) {
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const unsigned bal = __ballot_sync(0xffffffffu, (q[u] >> 4) & 1);
-                    if (lane == 0) reinterpret_cast<unsigned*>(rec + 128)[u] = bal;
-                }
-            } else {
-#pragma unroll
-                for (int u = 0; u < 2; ++u)
-                    rec[128 + lane + 32 * u] = (uint8_t)((q[u] >> 4) | ((q[u + 2] >> 4) << 2) | ((q[u + 4] >> 4) << 4) | ((q[u + 6] >> 4) << 6));
-            }
-        } else {                    // byte i = codes of rows i, i + 64, i + 128, i + 192, two bits each
-#pragma unroll
-            for (int u = 0; u < 2; ++u) rec[lane + 32 * u] = (uint8_t)(q[u] | (q[u + 2] << 2) | (q[u + 4] << 4) | (q[u + 6] << 6));
-        }
-        if (lane == 0) {
-            unsigned long long lo64 = 0ull;  // fields 0..9 and the low 4 bits of field 10
-            unsigned hi32 = 0u;              // bits 64..95
-#pragma unroll
-            for (int f = 0; f < 16; ++f) {
-                const unsigned long long v = (f < 8) ? sc[f] : mn[f - 8];
-                const int b = 6 * f;
-                if (b < 64) lo64 |= v << b;
-                if (b + 6 > 64) hi32 |= (b >= 64) ? (unsigned)(v << (b - 64)) : (unsigned)(v >> (64 - b));
-            }
-            unsigned* tail = reinterpret_cast<unsigned*>(rec + NCB);  // records start on 16-byte boundaries
-            tail[0] = (unsigned)lo64;
-            tail[1] = (unsigned)(lo64 >> 32);
-            tail[2] = hi32;
-            tail[3] = (unsigned)__half_as_ushort(dh) | ((unsigned)__half_as_ushort(mh) << 16);
+        for (int c = 0; c < 2; ++c) {
+            f64[c] |= (unsigned long long)sc[c] << (6 * u);
+            const int b = 6 * (u + 8);
+            if (b < 64) f64[c] |= (unsigned long long)mn[c] << b;
+            if (b >= 64) f32[c] |= mn[c] << (b - 64);
+            else if (b + 6 > 64) f32[c] |= mn[c] >> (64 - b);
         }
     }
+    // ---- codes
+    unsigned* const rec[2] = {mine + (2 * lane) * (RW + 1), mine + (2 * lane + 1) * (RW + 1)};
+    unsigned bits5[2][BITS == 5 ? 8 : 1] = {};
+#pragma unroll 1
+    for (int i = 0; i < 8; ++i) {
+        unsigned L[2][8];                // codes of rows 32u + 4i .. + 3, a byte each
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            float2 t[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                t[j] = round_to_low_bits(limited(by[u].quotient(add2(__half22float2(load(32 * u + 4 * i + j)), offset[u])), (float)kTop));
+            L[0][u] = four_bytes(t[0].x, t[1].x, t[2].x, t[3].x);
+            L[1][u] = four_bytes(t[0].y, t[1].y, t[2].y, t[3].y);
+        }
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            if (BITS == 8) {             // byte i = code of row i
+#pragma unroll
+                for (int u = 0; u < 8; ++u) rec[c][8 * u + i] = L[c][u];
+            } else if (BITS == 2) {      // byte i = codes of rows i, i + 64, i + 128, i + 192
+#pragma unroll
+                for (int u = 0; u < 2; ++u) rec[c][8 * u + i] = L[c][u] | (L[c][u + 2] << 2) | (L[c][u + 4] << 4) | (L[c][u + 6] << 6);
+            } else {                     // byte i = low four bits of rows i and i + 128, then the high bits
+#pragma unroll
+                for (int u = 0; u < 4; ++u) rec[c][8 * u + i] = (L[c][u] & 0x0f0f0f0fu) | ((L[c][u + 4] & 0x0f0f0f0fu) << 4);
+                if (BITS == 6) {         // two per row, arranged like 2-bit codes
+#pragma unroll
+                    for (int u = 0; u < 2; ++u)
+                        rec[c][32 + 8 * u + i] = ((L[c][u] >> 4) & 0x03030303u) | ((L[c][u + 2] >> 2) & 0x0c0c0c0cu) | (L[c][u + 4] & 0x30303030u) | ((L[c][u + 6] << 2) & 0xc0c0c0c0u);
+                }
+                if (BITS == 5) {         // one per row, bit j % 8 of byte j / 8: four bytes' bits meet in the product's top
+#pragma unroll
+                    for (int u = 0; u < 8; ++u)
+                        bits5[c][BITS == 5 ? u : 0] |= (((((L[c][u] >> 4) & 0x01010101u) * 0x01020408u) >> 24) & 15u) << (4 * i);
+                }
+            }
+        }
+    }
+    const unsigned dl = *reinterpret_cast<const unsigned*>(&dh), ml = *reinterpret_cast<const unsigned*>(&mh);
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        if (BITS == 5) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) rec[c][32 + u] = bits5[c][BITS == 5 ? u : 0];
+        }
+        rec[c][NCB / 4] = (unsigned)f64[c];
+        rec[c][NCB / 4 + 1] = (unsigned)(f64[c] >> 32);
+        rec[c][NCB / 4 + 2] = f32[c];
+        rec[c][NCB / 4 + 3] = __byte_perm(dl, ml, c == 0 ? 0x5410 : 0x7632);
+    }
+    __syncwarp();
+    unsigned* const dst = reinterpret_cast<unsigned*>(records + ((size_t)r * n + k0) * REC);
+    const int words = min(64, n - k0) * RW;
+#pragma unroll 4
+    for (int w = lane; w < words; w += 32) dst[w] = mine[w + w / RW];
+}
+
+template <int BITS>
+static void launch_kq_pack(const __half* W, int m, int n, int ldw, uint8_t* records, cudaStream_t s)
+{
+    const dim3 grid((n + kKqPackWarps * 64 - 1) / (kKqPackWarps * 64), m / kKqG);
+    const bool vec = aligned(W, 4) && ((ldw | n) & 1) == 0;   // pairs of columns as words
+    auto kernel = vec ? kq_pack_kernel<BITS, true> : kq_pack_kernel<BITS, false>;
+    kernel<<<grid, kKqPackWarps * 32, 0, s>>>(W, n, ldw, records);
 }
 
 // ---------------------------------------------------------------- GEMV
@@ -517,15 +572,14 @@ spqt_status spqt_kqw_pack(const void* W, int m, int n, int ldw, int bits, void* 
     if (!kq_bits_ok(bits)) return SPQT_ERR_UNSUPPORTED;
     if (ldw < n) return SPQT_ERR_INVALID_ARG;
     if (!spqt::aligned(W, 2) || !spqt::aligned(records, 16)) return SPQT_ERR_ALIGNMENT;
-    const dim3 grid((n + spqt::kKqPackCols - 1) / spqt::kKqPackCols, m / spqt::kKqG);
     const cudaStream_t st_ = static_cast<cudaStream_t>(stream);
     const __half* w = static_cast<const __half*>(W);
     uint8_t* rec = static_cast<uint8_t*>(records);
-    if (bits == 2) spqt::kq_pack_kernel<2><<<grid, 256, 0, st_>>>(w, n, ldw, rec);
-    else if (bits == 4) spqt::kq_pack_kernel<4><<<grid, 256, 0, st_>>>(w, n, ldw, rec);
-    else if (bits == 5) spqt::kq_pack_kernel<5><<<grid, 256, 0, st_>>>(w, n, ldw, rec);
-    else if (bits == 6) spqt::kq_pack_kernel<6><<<grid, 256, 0, st_>>>(w, n, ldw, rec);
-    else spqt::kq_pack_kernel<8><<<grid, 256, 0, st_>>>(w, n, ldw, rec);
+    if (bits == 2) spqt::launch_kq_pack<2>(w, m, n, ldw, rec, st_);
+    else if (bits == 4) spqt::launch_kq_pack<4>(w, m, n, ldw, rec, st_);
+    else if (bits == 5) spqt::launch_kq_pack<5>(w, m, n, ldw, rec, st_);
+    else if (bits == 6) spqt::launch_kq_pack<6>(w, m, n, ldw, rec, st_);
+    else spqt::launch_kq_pack<8>(w, m, n, ldw, rec, st_);
     spqt::count_launch();
     return cudaGetLastError() == cudaSuccess ? SPQT_OK : SPQT_ERR_CUDA;
 }

@@ -99,3 +99,21 @@ def test_conversion_at_the_edges_of_tiles_and_alignments(bits, group, m_blocks, 
     assert np.array_equal(np.asarray(codes).reshape(-1), np.asarray(ref_codes).reshape(-1))
     assert np.array_equal(s.view(np.uint16).reshape(-1), ref_s.view(np.uint16).reshape(-1))
     assert np.array_equal(z.view(np.uint16).reshape(-1), ref_z.view(np.uint16).reshape(-1))
+
+
+@pytest.mark.parametrize("bits", [2, 4, 5, 6, 8])
+@pytest.mark.parametrize("m_blocks,n,pad,shift", [(1, 1, 0, 0), (2, 64, 2, 0), (1, 66, 0, 0), (2, 130, 2, 1), (2, 129, 0, 0), (1, 31, 3, 0)])
+def test_two_level_conversion_at_the_edges_of_tiles_and_alignments(bits, m_blocks, n, pad, shift):
+    """As above; blocks of one sign, of zeros, and of very different sizes in one superblock."""
+    m = 256 * m_blocks
+    rng = np.random.Generator(np.random.PCG64(m * 1000 + n + bits))
+    W = rng.standard_normal((m, n)) * 10.0 ** rng.uniform(-4, 2, n) * np.repeat(10.0 ** rng.uniform(-2, 0, (m // 32, n)), 32, axis=0)
+    pick = rng.integers(0, 5, n)
+    W = np.where(pick == 1, np.abs(W), np.where(pick == 2, -np.abs(W), np.where(pick == 3, np.round(W * 8) / 8, W))).astype(np.float16)
+    W[32:64, n // 2] = 0.0
+    buf = torch.zeros(shift + m * (n + pad), dtype=torch.float16, device="cuda")
+    Wd = buf[shift:].view(m, n + pad)[:, :n]
+    Wd.copy_(dev(np.ascontiguousarray(W)))
+    got = binding.spqt_kqw_pack(Wd, bits).records.cpu().numpy()
+    want = oracle.kq_pack(*oracle.kq_quantize(W, bits=bits), bits=bits)
+    assert np.array_equal(got, np.asarray(want).reshape(-1))
