@@ -10,26 +10,21 @@
 // 8; 2^BITS - 1 replaces 15 in the rule and only the code bytes of a record change -- 8 bits: byte i = q_i (256
 // bytes, records of 272); 2 bits: byte i = q_i | q_{i+64} << 2 | q_{i+128} << 4 | q_{i+192} << 6 (64 bytes,
 // records of 80); 5 and 6 bits: the low four bits as 4-bit codes, then a plane of the high bits q >> 4, one per
-// row (bit j%8 of byte j/8) or two per row arranged like 2-bit codes (records of 176 and 208).  The arithmetic of
-// the 2- and 8-bit codes and of the high planes sums cumulative values (per 16-bit half-word the value of its
-// first code and of both codes together; per byte of single bits its low 1, 2, .. 8 bits: the cumulative form of
-// the main kernel) and takes the differences at the end.
+// row (bit j%8 of byte j/8) or two per row arranged like 2-bit codes (records of 176 and 208).
 //
 //   kq_pack_kernel   a thread converts two columns, a warp 64.
-//   kq_gemv_kernel   grid (S, R): CTA (s, r) takes the s-th of S slices of the index list (or of all
-//                    columns) for block-row r; its 8 warps take the slice's chunks of 16 entries in turn,
-//                    two record buffers per warp (cp.async: a record is one contiguous gather of 144 bytes,
-//                    metadata included).  Lanes e and e+16 decode the fields of entry e and write the packed
-//                    multiplier pairs of its four lane groups; lane t of a 16-lane half owns rows 8t..8t+7
-//                    and 128+8t..128+8t+7 of the entry's superblock (blocks t/4 and 4+t/4: one multiplier
-//                    pair covers both).  Conversion-free dequantization as in the main kernel.  Partial
-//                    sums: warp -> CTA (shared memory) -> block-row (fp32 partials in the workspace,
-//                    arrive-only counter, the last CTA adds them in slice order: bit-reproducible).
+//   kq_gemv_kernel   one CTA or a cluster of S CTAs per block-row, 8 or 16 warps each; every warp has an equal part of the
+//                    list (or of all columns) and streams it through its own ring of chunks of 16 records (cp.async: a
+//                    record is one contiguous gather, metadata included).  The product on tensor cores (spqt_mma.cuh):
+//                    records are an odd number of 16-byte pieces, so that ldmatrix.trans reads them as they lie; the
+//                    eight columns of B are hi and lo of the multipliers of four blocks, a second set those of the other
+//                    four.  Sums: warps through shared memory, CTAs through the cluster's, in a fixed order.
 #include <cstddef>
 
 #include "spqt_common.cuh"
 
 #include "spqt_gemv_device.cuh"
+#include "spqt_mma.cuh"
 #include "spqt_quantize.cuh"
 
 namespace spqt {
@@ -37,11 +32,10 @@ namespace spqt {
 constexpr int kKqG = 256;           // rows of a superblock
 __host__ __device__ constexpr int kq_code_bytes(int bits) { return kKqG * bits / 8; }
 __host__ __device__ constexpr int kq_rec_bytes(int bits) { return kq_code_bytes(bits) + 16; }
-__host__ __device__ constexpr int kq_ctas_per_sm(int bits) { return bits >= 5 ? 2 : 3; }   // (registers of a second accumulator set; shared memory of the record buffers)
-constexpr int kKqWarps = 8;
-constexpr int kKqThreads = kKqWarps * 32;
 constexpr int kKqChunk = 16;        // list entries per chunk
-constexpr int kKqMaxSplit = 32;     // slices per block-row at most
+// CTAs of a block-row: the largest portable cluster, twice that with one CTA of 16 warps per SM
+__host__ __device__ constexpr int kq_max_cluster(int warps) { return warps; }
+constexpr int kKqMaxSplit = 32;     // (of the workspace's size)
 
 // ---------------------------------------------------------------- conversion
 //   per block i:      lo_i = min(min_j w_j, 0),  step_i = (max_j w_j - lo_i) / 15,  neg_i = 0 - lo_i
@@ -201,296 +195,305 @@ static void launch_kq_pack(const __half* W, int m, int n, int ldw, uint8_t* reco
 
 // ---------------------------------------------------------------- GEMV
 
-template <int BITS>
+__host__ __device__ constexpr int kq_depth(int bits) { return bits == 2 ? 6 : bits <= 5 ? 4 : 3; }   // chunks in a warp's ring: 7.7 to 13 KB
+
+template <int BITS, int NW>
 struct KqSmem {
-    alignas(16) unsigned char rec[kKqWarps][2][kKqChunk * kq_rec_bytes(BITS)];  // two record buffers per warp
-    alignas(16) float mult[kKqWarps][kKqChunk][4][4];               // per entry and lane group: two packed multiplier pairs
-    alignas(16) float red[kKqWarps][kKqG];
-    float red_z[kKqWarps][8];
-    int last;
+    struct Loop {
+        alignas(16) unsigned char rec[NW][kq_depth(BITS)][kKqChunk * kq_rec_bytes(BITS)];
+        alignas(16) unsigned short b[NW][32][8];      // operand B of a chunk: row e of set s (blocks 4s .. 4s+3) at 16s + e, hi and lo of each block
+    };
+    struct Sums {
+        float red[NW][kKqG];
+        float red_z[NW][8];
+    };
+    union Area {
+        unsigned char loop[sizeof(Loop)];
+        unsigned char sums[sizeof(Sums)];
+    };
+    alignas(16) unsigned char area[sizeof(Area)];
+    alignas(16) float xred[kq_max_cluster(NW) - 1][kKqG];   // first CTA of a cluster: the other CTAs' sums
 };
 
-// 6-bit field f of the 96-bit string w0 | w1 << 32 | w2 << 64
-__device__ __forceinline__ unsigned kq_field(unsigned w0, unsigned w1, unsigned w2, int f)
+// The rotation that brings bit `from` of both halves to bit `to`.
+__device__ __forceinline__ unsigned kq_rotate(unsigned v, int from, int to) { return __funnelshift_r(v, v, from - to); }
+
+// acc[2*blk + o]: sums of rows 32*blk + 16*half + 2g + o, half = register / 2, over the 16 entries in stage st; columns
+// 2*(blk % 4) and the next of B set blk / 4 are the block's multipliers.  What the sums are multiples of: kq_unit.
+template <int BITS>
+__device__ __forceinline__ void kq_multiply(float (*acc)[4], unsigned st, int lane, const unsigned* bb)
 {
-    const int b = 6 * f, word = b >> 5;
-    const unsigned lo = word == 0 ? w0 : (word == 1 ? w1 : w2);
-    const unsigned hi = word == 0 ? w1 : (word == 1 ? w2 : 0u);
-    return __funnelshift_r(lo, hi, b & 31) & 63u;
+    constexpr int REC = kq_rec_bytes(BITS), NCB = kq_code_bytes(BITS), kGroups = BITS == 8 ? 8 : BITS == 2 ? 2 : 4;
+    // records are an odd number of 16-byte pieces: the eight rows of a matrix lie in different banks
+    const unsigned addr = st + (unsigned)((((lane >> 4) << 3) + (lane & 7)) * REC + ((lane >> 3) & 1) * 16);
+    const int g = lane >> 2, t4 = lane & 3;
+    auto product = [&](int blk, int o, const unsigned* a) { mma_16816(acc[2 * blk + o], a[0], a[1], a[2], a[3], bb[2 * (blk >> 2)], bb[2 * (blk >> 2) + 1]); };
+    unsigned p[2][4];
+    if (BITS == 6) {
+        ldsm_x4_trans(addr + 128u, p[0]);
+        ldsm_x4_trans(addr + 160u, p[1]);
+    }
+#pragma unroll
+    for (int i = 0; i < kGroups; ++i) {
+        unsigned c[4], d[4], a[4];
+        ldsm_x4_trans(addr + 32u * i, c);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) d[q] = __byte_perm(c[q], 0u, 0x4341);   // the odd bytes
+#pragma unroll
+        for (int o = 0; o < 2; ++o) {
+            const unsigned* const s = o ? d : c;
+            if (BITS == 8) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) a[q] = o ? s[q] : s[q] & 0x00ff00ffu;
+                product(i, o, a);
+            } else if (BITS == 2) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) a[q] = s[q] & (0x00030003u << (2 * j));
+                    product(2 * j + i, o, a);
+                }
+            } else {
+                unsigned hl[4], hh[4];               // the high bits of blocks i and i + 4, at bits 4 and 8 up
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    hl[q] = hh[q] = 0u;
+                    if (BITS == 6) {
+                        const unsigned w = p[i & 1][q], v = (o ? __byte_perm(w, 0u, 0x4341) : w) << (4 - 2 * (i >> 1));
+                        hl[q] = v & 0x00300030u;
+                        hh[q] = v & 0x03000300u;
+                    }
+                    if (BITS == 5) {
+                        // bit row of the blocks' words of entries 2t and 2t + 1 (+ 8): the halves of one word
+                        const unsigned e = st + (unsigned)((2 * t4 + 8 * (q >> 1)) * REC + 128 + 4 * i);
+                        const unsigned sel = (q & 1) ? 0x7632u : 0x5410u;
+                        const unsigned u0 = __byte_perm(lds_u32(e), lds_u32(e + REC), sel), u4 = __byte_perm(lds_u32(e + 16u), lds_u32(e + REC + 16u), sel);
+                        hl[q] = kq_rotate(u0, 2 * g + o, 4) & 0x00100010u;
+                        hh[q] = kq_rotate(u4, 2 * g + o, 8) & 0x01000100u;
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) a[q] = (s[q] & 0x000f000fu) | hl[q];
+                product(i, o, a);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) a[q] = (s[q] & 0x00f000f0u) | hh[q];
+                product(i + 4, o, a);
+            }
+        }
+    }
+}
+__host__ __device__ constexpr float kq_unit(int bits, int blk)
+{
+    return bits == 8 ? 1.0f : bits == 2 ? (blk < 2 ? 1.0f : blk < 4 ? 0.25f : blk < 6 ? 0.0625f : 0.015625f) : (blk < 4 ? 1.0f : 0.0625f);
 }
 
 // idx == nullptr: the dense product (the list is 0, 1, .., n-1 and count is n).
-template <int BITS>
-__global__ void __launch_bounds__(kKqThreads, kq_ctas_per_sm(BITS))
-kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* __restrict__ x,
-               const int32_t* __restrict__ idx, const int32_t* __restrict__ count_ptr,
-               __half* __restrict__ y, float* __restrict__ partials, int* __restrict__ counters)
+template <int BITS, bool LIST, int NW>
+__global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1)
+kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* __restrict__ x, const int32_t* __restrict__ idx,
+               const int32_t* __restrict__ count_ptr, __half* __restrict__ y, int splits)
 {
-    constexpr int CH = kKqChunk, G = kKqG;
-    constexpr int REC = kq_rec_bytes(BITS), NCB = kq_code_bytes(BITS), PPR = REC / 16;
-    constexpr int NP = CH * REC / 16;            // 16-byte pieces of a chunk
-    constexpr int NC = (NP + 31) / 32;           // copies per lane and chunk
-    extern __shared__ __align__(16) unsigned char kq_raw[];
-    KqSmem<BITS>& sm = *reinterpret_cast<KqSmem<BITS>*>(kq_raw);
-    const int tid = threadIdx.x, lane = tid & 31;
-    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
-    const int s = blockIdx.x, S = gridDim.x, r = blockIdx.y;
-    const int half = lane >> 4, t = lane & 15;   // arithmetic: entry of the step, rows 8t.. and 128+8t..
+    constexpr int REC = kq_rec_bytes(BITS), NCB = kq_code_bytes(BITS), PPR = REC / 16, CH = kKqChunk, D = kq_depth(BITS);
+    constexpr int kPieces = CH * PPR, NC = (kPieces + 31) / 32;
+    using Smem = KqSmem<BITS, NW>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    Smem& sm = *reinterpret_cast<Smem*>(smem_raw);
+    typename Smem::Loop& lp = *reinterpret_cast<typename Smem::Loop*>(sm.area);
+    typename Smem::Sums& su = *reinterpret_cast<typename Smem::Sums*>(sm.area);
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+    const int e = lane & 15;
+    const unsigned S = (unsigned)splits, rank = blockIdx.x % S, r = blockIdx.x / S;
+    if (S > 1) cluster_arrive();         // nobody may write to another CTA's shared memory before that CTA runs
+
+    const unsigned stage0 = smem_u32(&lp.rec[warp][0][0]);
+    constexpr unsigned kStageBytes = CH * REC, kRing = D * kStageBytes;
+    const unsigned b_base = smem_u32(&lp.b[warp][0][0]) + 16u * lane;
+    const uint8_t* const row = records + (size_t)r * (size_t)n * REC;
+    const unsigned short* const xg = reinterpret_cast<const unsigned short*>(x);
 
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-    const int count = idx ? __ldg(count_ptr) : n;
-    const int lo = (int)(((long long)s * count) / S), hi = (int)(((long long)(s + 1) * count) / S);
-    const uint8_t* row_rec = records + (size_t)r * (size_t)n * REC;
-    const unsigned rbuf = smem_u32(&sm.rec[warp][0][0]);
-    const unsigned mbuf = smem_u32(&sm.mult[warp][0][0][0]);
-    constexpr unsigned kBufBytes = CH * REC;
-    const unsigned short* xb = reinterpret_cast<const unsigned short*>(x);
+    const int count = LIST ? __ldg(count_ptr) : n;
+    // this warp's part of the list, in units of 8 entries
+    const unsigned units = (unsigned)(count + 7) >> 3, parts = S * NW, part = rank * NW + (unsigned)warp;
+    const int first = 8 * (int)((unsigned long long)units * part / parts);
+    const int end = min(8 * (int)((unsigned long long)units * (part + 1u) / parts), count);
 
-    unsigned long long acc[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) acc[i] = 0ull;
-    constexpr bool kHigh = BITS == 5 || BITS == 6;   // a second plane with the bits above the low four
-    unsigned long long acch[kHigh ? 8 : 1];          // its sums (cumulative, see the step), same rows as acc
-#pragma unroll
-    for (int i = 0; i < (kHigh ? 8 : 1); ++i) acch[i] = 0ull;
-    float zl[4] = {0.0f, 0.0f, 0.0f, 0.0f};      // x*dmin*m of blocks 4*half .. 4*half+3
-
-    // column of the entry lanes e and e+16 hold in the chunk at list position pos (past the end: the last entry again)
-    auto column_at = [&](int pos) -> int {
-        const int e = min(pos + t, hi - 1);
-        return idx ? __ldg(idx + e) : e;
+    constexpr int kAhead = 3;
+    int coming[kAhead], ahead = first;   // list: the columns of the chunks the copies come to next
+    auto fetch_ahead = [&](int d) {
+        coming[d] = __ldg(idx + min(ahead + e, end - 1));
+        ahead = ahead + CH >= end ? first : ahead + CH;
     };
-    auto copy_records = [&](int col, unsigned dst) {
+    if (LIST && first < end) {
 #pragma unroll
-        for (int q = 0; q < NC; ++q) {
-            const int p = q * 32 + lane;
-            const int e = p / PPR, part = p - PPR * e;
-            const int cu = __shfl_sync(0xffffffffu, col, e & 15);
-            if (p < NP) cp_async_16_l2_64(dst + (unsigned)(e * REC + part * 16), row_rec + (size_t)cu * REC + part * 16);
+        for (int d = 0; d < kAhead; ++d) fetch_ahead(d);
+    }
+    unsigned xv[D];                      // the x values of the chunks in flight, the oldest first
+#pragma unroll
+    for (int i = 0; i < D; ++i) xv[i] = 0;
+    int ipos = first;
+    unsigned ri = 0;
+    auto issue = [&]() {                 // the copies of the next chunk, if there is one
+#pragma unroll
+        for (int i = 0; i < D - 1; ++i) xv[i] = xv[i + 1];
+        xv[D - 1] = 0u;
+        if (ipos < end) {                // (past the end: the last entry again, with x = 0)
+            const unsigned col = LIST ? (unsigned)coming[0] : (unsigned)min(ipos + e, end - 1);
+            if (ipos + e < end) xv[D - 1] = (unsigned)__ldg(xg + col);
+#pragma unroll
+            for (int q = 0; q < NC; ++q) {
+                const int p = q * 32 + lane;
+                const unsigned cu = __shfl_sync(0xffffffffu, col, (p / PPR) & 15);
+                if (kPieces % 32 == 0 || p < kPieces) cp_async_16_l2_64(stage0 + ri + 16u * p, row + ((size_t)cu * REC + (p % PPR) * 16));
+            }
+            ri = ri + kStageBytes == kRing ? 0u : ri + kStageBytes;
+            ipos += CH;
+            if (LIST) {
+#pragma unroll
+                for (int i = 0; i < kAhead - 1; ++i) coming[i] = coming[i + 1];
+                fetch_ahead(kAhead - 1);
+            }
         }
         cp_async_commit();
     };
-
-    const int first = lo + warp * CH, stride = kKqWarps * CH;
-    if (first < hi) {
-        int col = column_at(first);
-        copy_records(col, rbuf);
-        int col_next = first + stride < hi ? column_at(first + stride) : 0;
-        unsigned short xv = (first + t < hi) ? __ldg(xb + col) : (unsigned short)0;
-        unsigned cur = 0;
-        for (int pos = first; pos < hi; pos += stride) {
-            const bool more = pos + stride < hi;
-            if (more) copy_records(col_next, rbuf + (cur == 0u ? kBufBytes : 0u));
-            else cp_async_commit();
-            const int col_after = pos + 2 * stride < hi ? column_at(pos + 2 * stride) : 0;
-            const unsigned short xv_next = (more && pos + stride + t < hi) ? __ldg(xb + col_next) : (unsigned short)0;
-            cp_async_wait<1>();   // this chunk's records have landed (the next chunk's may still fly)
-            __syncwarp();
-            // lanes e and e+16: the fields of entry e -> multiplier pairs of lane groups 2*half, 2*half+1 and
-            // the offset terms of blocks 4*half .. 4*half+3
-            {
-                const unsigned ra = rbuf + cur + (unsigned)(t * REC) + (unsigned)NCB;
-                const uint4 tail = lds_v4(ra);
-                const float xf = __half2float(__ushort_as_half(xv));
-                const float df = __half2float(__ushort_as_half((unsigned short)(tail.w & 0xffffu)));
-                const float dminf = __half2float(__ushort_as_half((unsigned short)(tail.w >> 16)));
-#pragma unroll
-                for (int g2 = 0; g2 < 2; ++g2) {
-                    const int sb = 2 * half + g2;   // lane group: rows of blocks sb (low nibbles) and sb + 4 (high nibbles)
-                    const float a_lo = xf * (df * (float)kq_field(tail.x, tail.y, tail.z, sb));       // d*sc is exact
-                    const float a_hi = xf * (df * (float)kq_field(tail.x, tail.y, tail.z, sb + 4));
-                    if (BITS == 4 || kHigh)
-                        sts_pairs(mbuf + 16u * (unsigned)(t * 4 + sb), pack2(a_lo * 0x1p93f, a_hi * 0x1p89f),
-                                  pack2(a_lo * 0x1p85f, a_hi * 0x1p81f));
-                    else   // one pair: the high rows' codes sit in the same bytes (2 bits, four bits up) or in bytes of their own (8 bits)
-                        sts_u64(mbuf + 16u * (unsigned)(t * 4 + sb), pack2(a_lo * 0x1p93f, a_hi * (BITS == 2 ? 0x1p89f : 0x1p93f)));
-                }
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    zl[i] += xf * (dminf * (float)kq_field(tail.x, tail.y, tail.z, 8 + 4 * half + i));
-            }
-            __syncwarp();
-            const int valid = min(CH, hi - pos);
-            const unsigned cb = rbuf + cur;
-            auto step = [&](int u) {
-                const unsigned e = (unsigned)(2 * u + half);
-                if (BITS == 4 || kHigh) {
-                    const uint2 wv = lds_v2(cb + e * REC + (unsigned)t * 8u);
-                    unsigned long long m01, m23;
-                    lds_pairs(mbuf + 16u * (e * 4u + (unsigned)(t >> 2)), m01, m23);
-                    fma_block8(acc, wv, m01, m23);     // the low four bits of every code
-                    if (BITS == 6) {
-                        // the high two bits, 16 times the weight: a plane laid out like 2-bit codes, summed the same way
-                        const unsigned long long mh = fmul2(m01, pack2(16.0f, 16.0f));
-                        const uint2 hv = lds_v2(cb + e * REC + 128u + (unsigned)(t & 7) * 8u);
-                        const int sh = 2 * (t >> 3);
-#pragma unroll
-                        for (int k = 0; k < 2; ++k) {
-                            const unsigned w = (k ? hv.y : hv.x) >> sh, v = w >> 16;
-                            ffma2(acch[4 * k + 0], pack2(__uint_as_float(w & 0x03u), __uint_as_float(w & 0x30u)), mh);
-                            ffma2(acch[4 * k + 1], pack2(__uint_as_float(w & 0x0303u), __uint_as_float(w & 0x3030u)), mh);
-                            ffma2(acch[4 * k + 2], pack2(__uint_as_float(v & 0x03u), __uint_as_float(v & 0x30u)), mh);
-                            ffma2(acch[4 * k + 3], pack2(__uint_as_float(v & 0x0303u), __uint_as_float(v & 0x3030u)), mh);
-                        }
-                    } else if (BITS == 5) {
-                        // the fifth bit of rows 8t.. and 128+8t..: one byte each; position b sums the byte's low b+1 bits
-                        const unsigned long long mh = fmul2(m01, pack2(16.0f, 256.0f));   // (a_lo, a_hi) * 16 * 2^93
-                        unsigned lb, hb;
-                        asm volatile("ld.shared.u8 %0, [%1];" : "=r"(lb) : "r"(cb + e * REC + 128u + (unsigned)t) : "memory");
-                        asm volatile("ld.shared.u8 %0, [%1];" : "=r"(hb) : "r"(cb + e * REC + 144u + (unsigned)t) : "memory");
-#pragma unroll
-                        for (int b = 0; b < 8; ++b) {
-                            const unsigned mk = (2u << b) - 1u;
-                            ffma2(acch[b], pack2(__uint_as_float(lb & mk), __uint_as_float(hb & mk)), mh);
-                        }
-                    }
-                    return;
-                }
-                // 2 and 8 bits: per 16-bit half-word the value of its first byte's code and the value of both
-                // codes together (second code times 256) are summed; the second code's sum is their difference
-                const unsigned long long mm = lds_u64(mbuf + 16u * (e * 4u + (unsigned)(t >> 2)));
-                if (BITS == 8) {
-                    const uint2 lw = lds_v2(cb + e * REC + (unsigned)t * 8u);           // rows 8t .. 8t+7
-                    const uint2 hw = lds_v2(cb + e * REC + 128u + (unsigned)t * 8u);    // rows 128+8t ..
-#pragma unroll
-                    for (int k = 0; k < 2; ++k) {
-                        const unsigned l = k ? lw.y : lw.x, h = k ? hw.y : hw.x, lv = l >> 16, hv = h >> 16;
-                        ffma2(acc[4 * k + 0], pack2(__uint_as_float(l & 0xffu), __uint_as_float(h & 0xffu)), mm);
-                        ffma2(acc[4 * k + 1], pack2(__uint_as_float(l & 0xffffu), __uint_as_float(h & 0xffffu)), mm);
-                        ffma2(acc[4 * k + 2], pack2(__uint_as_float(lv & 0xffu), __uint_as_float(hv & 0xffu)), mm);
-                        ffma2(acc[4 * k + 3], pack2(__uint_as_float(lv), __uint_as_float(hv)), mm);
-                    }
-                } else {
-                    // byte i holds rows i, i+64, i+128, i+192: lanes 0..7 use fields 0 and 2 of bytes 8t.., lanes
-                    // 8..15 fields 1 and 3 of bytes 8(t-8)..
-                    const uint2 wv = lds_v2(cb + e * REC + (unsigned)(t & 7) * 8u);
-                    const int sh = 2 * (t >> 3);
-#pragma unroll
-                    for (int k = 0; k < 2; ++k) {
-                        const unsigned w = (k ? wv.y : wv.x) >> sh, v = w >> 16;
-                        ffma2(acc[4 * k + 0], pack2(__uint_as_float(w & 0x03u), __uint_as_float(w & 0x30u)), mm);
-                        ffma2(acc[4 * k + 1], pack2(__uint_as_float(w & 0x0303u), __uint_as_float(w & 0x3030u)), mm);
-                        ffma2(acc[4 * k + 2], pack2(__uint_as_float(v & 0x03u), __uint_as_float(v & 0x30u)), mm);
-                        ffma2(acc[4 * k + 3], pack2(__uint_as_float(v & 0x0303u), __uint_as_float(v & 0x3030u)), mm);
-                    }
-                }
-            };
-            if (valid == CH) {
-#pragma unroll
-                for (int u = 0; u < CH / 2; ++u) step(u);   // a full chunk: straight-line code
-            } else {
-                const int nsub = (valid + 1) >> 1;
 #pragma unroll 1
-                for (int u = 0; u < nsub; ++u) step(u);
-            }
-            __syncwarp();
-            cur = (cur == 0u) ? kBufBytes : 0u;
-            col = col_next;
-            col_next = col_after;
-            xv = xv_next;
+    for (int d = 0; d < D - 1; ++d) issue();
+
+    // While chunk i is multiplied, chunk i + 1 is prepared: lane 16s + e decodes the fields of blocks 4s .. 4s+3 of entry e,
+    // a = x*(d*sc) (d*sc exact in fp32) left as hi and lo, and x*(dmin*m).
+    float acc[16][4];
+#pragma unroll
+    for (int i = 0; i < 64; ++i) acc[i >> 2][i & 3] = 0.0f;
+    float scale = kMmaNoScale, regain = 1.0f, zl[4] = {0.0f, 0.0f, 0.0f, 0.0f}, zn[4] = {0.0f, 0.0f, 0.0f, 0.0f}, am[4], pm[4];
+    auto prepare = [&](unsigned st, unsigned xb) -> bool {
+        const uint4 f = lds_v4(st + (unsigned)(e * REC + NCB));
+        const unsigned sc = lane < 16 ? f.x : __funnelshift_r(f.x, f.y, 24), mn = lane < 16 ? __funnelshift_r(f.y, f.z, 16) : f.z >> 8;
+        const float xf = __half2float(__ushort_as_half((unsigned short)xb));
+        const float df = __half2float(__ushort_as_half((unsigned short)(f.w & 0xffffu))), mf = __half2float(__ushort_as_half((unsigned short)(f.w >> 16)));
+        float top = 0.0f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float s = __uint_as_float(((sc >> (6 * j)) & 63u) | 0x4b000000u) - 8388608.0f;   // the integers as floats
+            const float m = __uint_as_float(((mn >> (6 * j)) & 63u) | 0x4b000000u) - 8388608.0f;
+            am[j] = xf * (df * s);
+            zn[j] = xf * (mf * m);
+            pm[j] = am[j] * scale;       // a power of two
+            top = fmaxf(top, fabsf(pm[j]));
         }
+        return top > kMmaLimit;
+    };
+    // a larger entry than the range holds: a new scale; the sums follow once chunk i is in them
+    auto rescale = [&]() {
+        unsigned m = 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const unsigned bits = __float_as_uint(am[j]) & 0x7fffffffu;
+            m = max(m, bits < 0x7f800000u ? bits : 0u);   // finite ones
+        }
+        m = __reduce_max_sync(0xffffffffu, m);
+        if (__uint_as_float(m) * scale > kMmaLimit) {
+            const float next = __uint_as_float((264u - (m >> 23)) << 23);   // m goes to 2^10 .. 2^11
+            regain = next * power_of_two_inverse(scale);
+            scale = next;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) pm[j] = am[j] * next;
+        }
+    };
+    auto leave = [&]() {
+        unsigned w[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float h = __low2float(__floats2half2_rn(pm[j], 0.0f));
+            const __half2 hl = __floats2half2_rn(pm[j], pm[j] - h);
+            w[j] = *reinterpret_cast<const unsigned*>(&hl);
+        }
+        sts_v4(b_base, make_uint4(w[0], w[1], w[2], w[3]));
+    };
+    unsigned rc = 0;
+    if (first < end) {
+        cp_async_wait<D - 2>();
+        __syncwarp();
+        if (__any_sync(0xffffffffu, prepare(stage0, xv[1]))) rescale();
+        leave();
+        regain = 1.0f;                   // (there is nothing in the sums yet)
+        __syncwarp();
+    }
+#pragma unroll 1
+    for (int pos = first; pos < end; pos += CH) {
+        issue();
+        const unsigned rn = rc + kStageBytes == kRing ? 0u : rc + kStageBytes;
+        cp_async_wait<D - 2>();
+        __syncwarp();
+        unsigned bb[4];
+        ldsm_x4_trans(b_base, bb);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) zl[j] += zn[j];
+        const bool over = prepare(stage0 + rn, xv[1]);
+        __syncwarp();                    // (B is in registers: its place is free)
+        kq_multiply<BITS>(acc, stage0 + rc, lane, bb);
+        if (__any_sync(0xffffffffu, over)) rescale();
+        leave();
+        if (regain != 1.0f) {
+#pragma unroll
+            for (int i = 0; i < 64; ++i) acc[i >> 2][i & 3] *= regain;
+            regain = 1.0f;
+        }
+        __syncwarp();                    // every lane is done with this chunk's stage
+        rc = rn;
     }
     cp_async_wait<0>();
+    __syncthreads();                     // (the sums take the place of the rings)
 
-    // warp -> CTA.  acc[b] = (row 8t+b, row 128+8t+b) of the entries this half-warp handled
-    {
-        float lo_rows[8], hi_rows[8];
+    // ---- sums: lane (g, t4) has those of blocks t4 and t4 + 4
+    const float unit = 0x1p24f * power_of_two_inverse(scale);
+    const int g = lane >> 2, t4 = lane & 3;
 #pragma unroll
-        for (int b = 0; b < 8; ++b) {
-            unpack2(acc[b], lo_rows[b], hi_rows[b]);
-            lo_rows[b] += __shfl_xor_sync(0xffffffffu, lo_rows[b], 16);
-            hi_rows[b] += __shfl_xor_sync(0xffffffffu, hi_rows[b], 16);
-        }
-        if (kHigh) {
-            float lh[8], hh[8];
+    for (int blk = 0; blk < 8; ++blk)
+        if ((blk & 3) == t4) {
 #pragma unroll
-            for (int b = 0; b < 8; ++b) {
-                unpack2(acch[b], lh[b], hh[b]);
-                lh[b] += __shfl_xor_sync(0xffffffffu, lh[b], 16);
-                hh[b] += __shfl_xor_sync(0xffffffffu, hh[b], 16);
-            }
-            if (BITS == 6) {      // pairs, as for 2-bit codes
-#pragma unroll
-                for (int b = 1; b < 8; b += 2) {
-                    lh[b] = (lh[b] - lh[b - 1]) * 0x1p-8f;
-                    hh[b] = (hh[b] - hh[b - 1]) * 0x1p-8f;
-                }
-            } else {              // a chain over the eight bits of a byte
-#pragma unroll
-                for (int b = 7; b > 0; --b) {
-                    lh[b] = (lh[b] - lh[b - 1]) * (1.0f / (float)(1 << b));
-                    hh[b] = (hh[b] - hh[b - 1]) * (1.0f / (float)(1 << b));
-                }
-            }
-#pragma unroll
-            for (int b = 0; b < 8; ++b) {
-                lo_rows[b] += lh[b];
-                hi_rows[b] += hh[b];
-            }
-        } else if (BITS != 4) {   // odd positions hold (first code + 256 * second code) of a half-word
-#pragma unroll
-            for (int b = 1; b < 8; b += 2) {
-                lo_rows[b] = (lo_rows[b] - lo_rows[b - 1]) * 0x1p-8f;
-                hi_rows[b] = (hi_rows[b] - hi_rows[b - 1]) * 0x1p-8f;
-            }
-        }
-        if (half == 0) {
-#pragma unroll
-            for (int b = 0; b < 8; ++b) {
-                sm.red[warp][8 * t + b] = lo_rows[b] * 0x1p56f;
-                sm.red[warp][128 + 8 * t + b] = hi_rows[b] * 0x1p56f;
+            for (int i = 0; i < 4; ++i) {
+                const int o = i & 1, half = i >> 1;
+                su.red[warp][32 * blk + 16 * half + 2 * g + o] = (acc[2 * blk + o][2 * half] + acc[2 * blk + o][2 * half + 1]) * (unit * kq_unit(BITS, blk));   // hi + lo
             }
         }
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            float z = zl[i];
+    for (int j = 0; j < 4; ++j) {
 #pragma unroll
-            for (int o = 8; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-            if (t == 0) sm.red_z[warp][4 * half + i] = z;
-        }
+        for (int o = 8; o > 0; o >>= 1) zl[j] += __shfl_xor_sync(0xffffffffu, zl[j], o);
+        if (e == 0) su.red_z[warp][(lane >> 4) * 4 + j] = zl[j];
     }
     __syncthreads();
-
-    // CTA -> block-row: G sums and 8 offset terms
-    float* mine = partials + ((size_t)r * kKqMaxSplit + s) * (G + 8);
-    for (int i = tid; i < G + 8; i += kKqThreads) {
-        float v = 0.0f;
+    float total = 0.0f;                  // thread j < 256: row j
+    if (tid < kKqG) {
+        float z = 0.0f;
 #pragma unroll
-        for (int w = 0; w < kKqWarps; ++w) v += (i < G) ? sm.red[w][i] : sm.red_z[w][i - G];
-        if (S == 1) {
-            if (i < G) sm.red[0][i] = v;    // (warp 0's slot; every element has one writer)
-            else sm.red_z[0][i - G] = v;
-        } else {
-            __stcg(mine + i, v);
+        for (int w = 0; w < NW; ++w) {
+            total += su.red[w][tid];
+            z += su.red_z[w][tid >> 5];
         }
+        total -= z;
     }
-    if (S == 1) {
-        __syncthreads();
-        for (int j = tid; j < G; j += kKqThreads) y[(size_t)r * G + j] = __float2half_rn(sm.red[0][j] - sm.red_z[0][j >> 5]);
-        return;
-    }
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) sm.last = (atomicAdd(counters + r, 1) == S - 1) ? 1 : 0;
-    __syncthreads();
-    if (!sm.last) return;
-    __threadfence();
-    const float* rowp = partials + (size_t)r * kKqMaxSplit * (G + 8);
-    for (int j = tid; j < G; j += kKqThreads) {
-        float v = 0.0f, z = 0.0f;
-        for (int q = 0; q < S; ++q) {
-            v += __ldcg(rowp + (size_t)q * (G + 8) + j);
-            z += __ldcg(rowp + (size_t)q * (G + 8) + G + (j >> 5));
+    if (S > 1) {
+        // the other CTAs leave their sums in the first one's shared memory; it adds them in CTA order
+        cluster_wait();                  // (every CTA of the cluster runs)
+        if (rank != 0) {
+            if (tid < kKqG) st_cluster_f32(cluster_map(smem_u32(&sm.xred[rank - 1][0]), 0u) + 4u * tid, total);
+            asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+            return;
         }
-        y[(size_t)r * G + j] = __float2half_rn(v - z);
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (tid < kKqG)
+            for (unsigned q = 1; q < S; ++q) total += sm.xred[q - 1][tid];
     }
-    if (tid == 0) counters[r] = 0;   // ready for the next call
+    if (tid < kKqG) y[(size_t)r * kKqG + tid] = __float2half_rn(total);
 }
 
 // ---------------------------------------------------------------- host side
 
+// (sums travel through shared memory; the sizes are those callers know)
 inline size_t kq_header_bytes(int R) { return (((size_t)R * 4 + 255) / 256) * 256; }
 inline size_t kq_workspace_bytes(int R) { return kq_header_bytes(R) + (size_t)R * kKqMaxSplit * (kKqG + 8) * sizeof(float); }
 
@@ -500,6 +503,86 @@ static spqt_status kq_shape(int m, int n)
     if (m % kKqG != 0) return SPQT_ERR_UNSUPPORTED;
     if (m / kKqG > 65535) return SPQT_ERR_UNSUPPORTED;
     return SPQT_OK;
+}
+
+// How many clusters of k CTAs the device holds at once with `smem` bytes each (asked once per kernel, cluster size and device).
+template <int BITS, bool LIST, int NW>
+static int kq_max_clusters(int k, int smem, bool alone, int sms, int dev)
+{
+    static int known[64][2][kq_max_cluster(NW) + 1] = {};
+    int& at_once = known[dev][alone ? 1 : 0][k];
+    if (at_once == 0) {
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = k;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(k * 2 * sms));
+        cfg.blockDim = dim3(NW * 32);
+        cfg.dynamicSmemBytes = smem;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int can = 0;
+        if (cudaOccupancyMaxActiveClusters(&can, kq_gemv_kernel<BITS, LIST, NW>, &cfg) != cudaSuccess) (void)cudaGetLastError();
+        at_once = can > 0 ? can : 1;
+    }
+    return at_once;
+}
+
+template <int BITS, bool LIST>
+static spqt_status kq_launch_mode(const void* records, int R, int n, const void* x, const int32_t* idx, const int32_t* count, void* y, cudaStream_t s)
+{
+    constexpr int kAlone = 120 * 1024;   // shared memory that keeps a second CTA of 8 warps off the SM
+    constexpr int kSmem = (int)sizeof(KqSmem<BITS, 8>), kSmem16 = (int)sizeof(KqSmem<BITS, 16>);
+    static_assert(kSmem <= 115712 && kSmem16 <= 232448, "two CTAs of 8 warps per SM, or one of 16");
+    static bool configured[64] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return SPQT_ERR_CUDA;
+    if (!configured[dev]) {
+        if (cudaFuncSetAttribute(kq_gemv_kernel<BITS, LIST, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAlone) != cudaSuccess ||
+            cudaFuncSetAttribute(kq_gemv_kernel<BITS, LIST, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem16) != cudaSuccess ||
+            cudaFuncSetAttribute(kq_gemv_kernel<BITS, LIST, 16>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+            return SPQT_ERR_CUDA;
+        configured[dev] = true;
+    }
+    const int sms = sm_count();
+    if (sms <= 0) return SPQT_ERR_CUDA;
+    // CTAs per block-row: the rule of the one-level format's kernel (the same structure), and with few block-rows of a long x
+    // clusters of up to 16 CTAs of 16 warps, so that more SMs fetch (dense 1024 x 28672 to 8 bits, 31 MB: 21.0 us on 32 CTAs
+    // of 8 warps)
+    int S = 1;
+    bool alone = false, wide = R >= 100 && R <= sms;
+    if (R < 100) {
+        alone = R <= kq_max_clusters<BITS, LIST, 8>(4, kAlone, true, sms, dev);
+        for (int k = 2; k <= kq_max_cluster(8); ++k)
+            if (n >= 128 * k && R <= kq_max_clusters<BITS, LIST, 8>(k, alone ? kAlone : kSmem, alone, sms, dev)) S = k;
+        alone = alone || R <= kq_max_clusters<BITS, LIST, 8>(S, kAlone, true, sms, dev);
+        if (alone && n >= 1024 * S) {
+            wide = R <= kq_max_clusters<BITS, LIST, 16>(S, kSmem16, true, sms, dev);
+            for (int k = S + 1; wide && k <= kq_max_cluster(16); ++k)
+                if (n >= 1024 * k && R <= kq_max_clusters<BITS, LIST, 16>(k, kSmem16, true, sms, dev)) S = k;
+        }
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)S * (unsigned)R);
+    cfg.blockDim = dim3(wide ? 512 : 256);
+    cfg.dynamicSmemBytes = wide ? kSmem16 : alone ? kAlone : kSmem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = S;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = g_no_pdl ? attr + 1 : attr;
+    cfg.numAttrs = (g_no_pdl ? 0 : 1) + (S > 1 ? 1 : 0);
+    auto kernel = wide ? kq_gemv_kernel<BITS, LIST, 16> : kq_gemv_kernel<BITS, LIST, 8>;
+    const cudaError_t err = cudaLaunchKernelEx(&cfg, kernel, static_cast<const uint8_t*>(records), n, static_cast<const __half*>(x), idx, count,
+                                               static_cast<__half*>(y), S);
+    count_launch();
+    return (err == cudaSuccess && cudaGetLastError() == cudaSuccess) ? SPQT_OK : SPQT_ERR_CUDA;
 }
 
 template <int BITS>
@@ -514,38 +597,8 @@ static spqt_status kq_launch(const void* records, int m, int n, const void* x, c
         return SPQT_ERR_ALIGNMENT;
     const int R = m / kKqG;
     if (ws_bytes < kq_workspace_bytes(R)) return SPQT_ERR_WORKSPACE;
-    static bool configured[64] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return SPQT_ERR_CUDA;
-    const int smem = (int)sizeof(KqSmem<BITS>);
-    if (!configured[dev]) {
-        if (cudaFuncSetAttribute(kq_gemv_kernel<BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return SPQT_ERR_CUDA;
-        configured[dev] = true;
-    }
-    const int sms = sm_count();
-    if (sms <= 0) return SPQT_ERR_CUDA;
-    // slices per block-row: fill the resident CTAs of every SM once; never less than a chunk per warp
-    int S = (kq_ctas_per_sm(BITS) * sms) / R;
-    const int by_work = n / (kKqChunk * kKqWarps);
-    if (S > by_work) S = by_work;
-    if (S > kKqMaxSplit) S = kKqMaxSplit;
-    if (S < 1) S = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(S, R);
-    cfg.blockDim = dim3(kKqThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = static_cast<cudaStream_t>(stream);
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = g_no_pdl ? 0 : 1;
-    int* counters = static_cast<int*>(workspace);
-    float* partials = reinterpret_cast<float*>(static_cast<char*>(workspace) + kq_header_bytes(R));
-    const cudaError_t err = cudaLaunchKernelEx(&cfg, kq_gemv_kernel<BITS>, static_cast<const uint8_t*>(records), n,
-                                               static_cast<const __half*>(x), idx, count, static_cast<__half*>(y), partials, counters);
-    count_launch();
-    return (err == cudaSuccess && cudaGetLastError() == cudaSuccess) ? SPQT_OK : SPQT_ERR_CUDA;
+    const cudaStream_t s = static_cast<cudaStream_t>(stream);
+    return idx ? kq_launch_mode<BITS, true>(records, R, n, x, idx, count, y, s) : kq_launch_mode<BITS, false>(records, R, n, x, idx, count, y, s);
 }
 
 }  // namespace spqt

@@ -117,3 +117,27 @@ def test_two_level_conversion_at_the_edges_of_tiles_and_alignments(bits, m_block
     got = binding.spqt_kqw_pack(Wd, bits).records.cpu().numpy()
     want = oracle.kq_pack(*oracle.kq_quantize(W, bits=bits), bits=bits)
     assert np.array_equal(got, np.asarray(want).reshape(-1))
+
+
+@pytest.mark.parametrize("bits", [2, 4, 5, 6, 8])
+@pytest.mark.parametrize("m_blocks,n", [(1, 1), (2, 17), (1, 2049), (20, 300), (37, 1030), (60, 264), (101, 129), (149, 40)])
+def test_two_level_products_at_chunk_part_and_cluster_edges(bits, m_blocks, n):
+    m = 256 * m_blocks
+    W = inputs.weights(m, n, seed=m + n, std=0.1)
+    x = growing_activations(n, seed=91)
+    parts = oracle.kq_quantize(W, bits=bits)
+    p = binding.spqt_kqw_pack(dev(W), bits)
+    ws = binding.new_kq_workspace(p)
+    t = inputs.threshold_for_sparsity(x, 0.4)
+    xd = dev(x)
+    idx, cnt = binding.spqt_sparsify(xd, t)
+    y = binding.spqt_kqw_sparse_gemv(p, xd, idx, cnt, ws)
+    again = binding.spqt_kqw_sparse_gemv(p, xd, idx, cnt, ws)
+    y_dense = binding.spqt_kqw_dense_gemv(p, xd, ws)
+    torch.cuda.synchronize()
+    ref_idx, _ = oracle.sparsify(x, t)
+    y_ref, bound = oracle.kq_gemv(*parts, x, ref_idx)
+    check_y(y.cpu().numpy(), y_ref, bound, "sparse")
+    assert torch.equal(y, again)
+    y_ref, bound = oracle.kq_gemv(*parts, x)
+    check_y(y_dense.cpu().numpy(), y_ref, bound, "dense")
