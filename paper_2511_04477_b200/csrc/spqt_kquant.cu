@@ -19,6 +19,11 @@
 //                    records are an odd number of 16-byte pieces, so that ldmatrix.trans reads them as they lie; the
 //                    eight columns of B are hi and lo of the multipliers of four blocks, a second set those of the other
 //                    four.  Sums: warps through shared memory, CTAs through the cluster's, in a fixed order.
+//                    What bounds it: the fixed cost of the call and of the list's launch before it, then latency: 12 to 16
+//                    warps per SM with 2 to 5 chunks in flight each.  28672 x 4096 to 4 bits at 50 %, list included, takes
+//                    15.9 us (19.4 with packed FMAs, partial sums in global memory and chunks dealt in turn), 8192 x 8192
+//                    to 6 bits dense 16.6 us (20.4; 55 MB), 28672 x 4096 to 2 bits dense 17.3 us (24.7).
+//                    A multiplier x*(d*sc) is rounded to fp32 and goes in as two fp16 values, which keep 24 bits of it.
 #include <cstddef>
 
 #include "spqt_common.cuh"
@@ -33,9 +38,8 @@ constexpr int kKqG = 256;           // rows of a superblock
 __host__ __device__ constexpr int kq_code_bytes(int bits) { return kKqG * bits / 8; }
 __host__ __device__ constexpr int kq_rec_bytes(int bits) { return kq_code_bytes(bits) + 16; }
 constexpr int kKqChunk = 16;        // list entries per chunk
-// CTAs of a block-row: the largest portable cluster, twice that with one CTA of 16 warps per SM
-__host__ __device__ constexpr int kq_max_cluster(int warps) { return warps; }
-constexpr int kKqMaxSplit = 32;     // (of the workspace's size)
+constexpr int kKqMaxCluster = 8;    // the largest portable cluster
+constexpr int kKqMaxSplit = 32;     // clusters of a block-row at most (the workspace's size)
 
 // ---------------------------------------------------------------- conversion
 //   per block i:      lo_i = min(min_j w_j, 0),  step_i = (max_j w_j - lo_i) / 15,  neg_i = 0 - lo_i
@@ -206,13 +210,14 @@ struct KqSmem {
     struct Sums {
         float red[NW][kKqG];
         float red_z[NW][8];
+        int last;                                     // whether this cluster came last to the block-row
     };
     union Area {
         unsigned char loop[sizeof(Loop)];
         unsigned char sums[sizeof(Sums)];
     };
     alignas(16) unsigned char area[sizeof(Area)];
-    alignas(16) float xred[kq_max_cluster(NW) - 1][kKqG];   // first CTA of a cluster: the other CTAs' sums
+    alignas(16) float xred[kKqMaxCluster - 1][kKqG];   // first CTA of a cluster: the other CTAs' sums
 };
 
 // The rotation that brings bit `from` of both halves to bit `to`.
@@ -291,7 +296,7 @@ __host__ __device__ constexpr float kq_unit(int bits, int blk)
 template <int BITS, bool LIST, int NW>
 __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1)
 kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* __restrict__ x, const int32_t* __restrict__ idx,
-               const int32_t* __restrict__ count_ptr, __half* __restrict__ y, int splits)
+               const int32_t* __restrict__ count_ptr, __half* __restrict__ y, int splits, int clusters, unsigned* arrived, float* partial)
 {
     constexpr int REC = kq_rec_bytes(BITS), NCB = kq_code_bytes(BITS), PPR = REC / 16, CH = kKqChunk, D = kq_depth(BITS);
     constexpr int kPieces = CH * PPR, NC = (kPieces + 31) / 32;
@@ -302,7 +307,7 @@ kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* __restr
     typename Smem::Sums& su = *reinterpret_cast<typename Smem::Sums*>(sm.area);
     const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     const int e = lane & 15;
-    const unsigned S = (unsigned)splits, rank = blockIdx.x % S, r = blockIdx.x / S;
+    const unsigned S = (unsigned)splits, T = (unsigned)clusters, rank = blockIdx.x % S, cluster = blockIdx.x / S, r = cluster / T;
     if (S > 1) cluster_arrive();         // nobody may write to another CTA's shared memory before that CTA runs
 
     const unsigned stage0 = smem_u32(&lp.rec[warp][0][0]);
@@ -316,7 +321,7 @@ kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* __restr
 
     const int count = LIST ? __ldg(count_ptr) : n;
     // this warp's part of the list, in units of 8 entries
-    const unsigned units = (unsigned)(count + 7) >> 3, parts = S * NW, part = rank * NW + (unsigned)warp;
+    const unsigned units = (unsigned)(count + 7) >> 3, parts = T * S * NW, part = ((cluster - r * T) * S + rank) * NW + (unsigned)warp;
     const int first = 8 * (int)((unsigned long long)units * part / parts);
     const int end = min(8 * (int)((unsigned long long)units * (part + 1u) / parts), count);
 
@@ -488,12 +493,29 @@ kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* __restr
         if (tid < kKqG)
             for (unsigned q = 1; q < S; ++q) total += sm.xred[q - 1][tid];
     }
+    if (T > 1) {
+        // the cluster that comes last to the block-row adds the clusters' sums in order, and leaves the counter at zero
+        float* const row_sums = partial + (size_t)r * T * kKqG;
+        if (tid < kKqG) __stcg(row_sums + (cluster - r * T) * kKqG + tid, total);
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) {
+            su.last = atomicAdd(arrived + r, 1u) == T - 1u;
+            if (su.last) arrived[r] = 0u;
+        }
+        __syncthreads();
+        if (!su.last) return;
+        __threadfence();
+        if (tid < kKqG) {
+            total = 0.0f;
+            for (unsigned t = 0; t < T; ++t) total += __ldcg(row_sums + t * kKqG + tid);
+        }
+    }
     if (tid < kKqG) y[(size_t)r * kKqG + tid] = __float2half_rn(total);
 }
 
 // ---------------------------------------------------------------- host side
 
-// (sums travel through shared memory; the sizes are those callers know)
 inline size_t kq_header_bytes(int R) { return (((size_t)R * 4 + 255) / 256) * 256; }
 inline size_t kq_workspace_bytes(int R) { return kq_header_bytes(R) + (size_t)R * kKqMaxSplit * (kKqG + 8) * sizeof(float); }
 
@@ -509,7 +531,7 @@ static spqt_status kq_shape(int m, int n)
 template <int BITS, bool LIST, int NW>
 static int kq_max_clusters(int k, int smem, bool alone, int sms, int dev)
 {
-    static int known[64][2][kq_max_cluster(NW) + 1] = {};
+    static int known[64][2][kKqMaxCluster + 1] = {};
     int& at_once = known[dev][alone ? 1 : 0][k];
     if (at_once == 0) {
         cudaLaunchAttribute attr[1];
@@ -531,7 +553,7 @@ static int kq_max_clusters(int k, int smem, bool alone, int sms, int dev)
 }
 
 template <int BITS, bool LIST>
-static spqt_status kq_launch_mode(const void* records, int R, int n, const void* x, const int32_t* idx, const int32_t* count, void* y, cudaStream_t s)
+static spqt_status kq_launch_mode(const void* records, int R, int n, const void* x, const int32_t* idx, const int32_t* count, void* y, void* workspace, cudaStream_t s)
 {
     constexpr int kAlone = 120 * 1024;   // shared memory that keeps a second CTA of 8 warps off the SM
     constexpr int kSmem = (int)sizeof(KqSmem<BITS, 8>), kSmem16 = (int)sizeof(KqSmem<BITS, 16>);
@@ -541,31 +563,36 @@ static spqt_status kq_launch_mode(const void* records, int R, int n, const void*
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return SPQT_ERR_CUDA;
     if (!configured[dev]) {
         if (cudaFuncSetAttribute(kq_gemv_kernel<BITS, LIST, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAlone) != cudaSuccess ||
-            cudaFuncSetAttribute(kq_gemv_kernel<BITS, LIST, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem16) != cudaSuccess ||
-            cudaFuncSetAttribute(kq_gemv_kernel<BITS, LIST, 16>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+            cudaFuncSetAttribute(kq_gemv_kernel<BITS, LIST, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem16) != cudaSuccess)
             return SPQT_ERR_CUDA;
         configured[dev] = true;
     }
     const int sms = sm_count();
     if (sms <= 0) return SPQT_ERR_CUDA;
-    // CTAs per block-row: the rule of the one-level format's kernel (the same structure), and with few block-rows of a long x
-    // clusters of up to 16 CTAs of 16 warps, so that more SMs fetch (dense 1024 x 28672 to 8 bits, 31 MB: 21.0 us on 32 CTAs
-    // of 8 warps)
-    int S = 1;
+    // CTAs per block-row: the rule of the one-level format's kernel (the same structure).  With few block-rows of a long x
+    // several clusters of 4 CTAs of 16 warps, so that more SMs fetch, if that are half as many CTAs again (the sums of a
+    // block-row then meet in global memory, 1.5 us: dense 1024 x 28672 to 8 bits, 31 MB, took 21.0 us on 32 CTAs of 8 warps).
+    int S = 1, T = 1;
     bool alone = false, wide = R >= 100 && R <= sms;
     if (R < 100) {
         alone = R <= kq_max_clusters<BITS, LIST, 8>(4, kAlone, true, sms, dev);
-        for (int k = 2; k <= kq_max_cluster(8); ++k)
+        for (int k = 2; k <= kKqMaxCluster; ++k)
             if (n >= 128 * k && R <= kq_max_clusters<BITS, LIST, 8>(k, alone ? kAlone : kSmem, alone, sms, dev)) S = k;
         alone = alone || R <= kq_max_clusters<BITS, LIST, 8>(S, kAlone, true, sms, dev);
         if (alone && n >= 1024 * S) {
             wide = R <= kq_max_clusters<BITS, LIST, 16>(S, kSmem16, true, sms, dev);
-            for (int k = S + 1; wide && k <= kq_max_cluster(16); ++k)
-                if (n >= 1024 * k && R <= kq_max_clusters<BITS, LIST, 16>(k, kSmem16, true, sms, dev)) S = k;
+            int t = kq_max_clusters<BITS, LIST, 16>(4, kSmem16, true, sms, dev) / R;
+            t = t < n / 2048 ? t : n / 2048;
+            t = t < kKqMaxSplit ? t : kKqMaxSplit;
+            if (8 * t >= 3 * S) {
+                S = 4;
+                T = t;
+                wide = true;
+            }
         }
     }
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)S * (unsigned)R);
+    cfg.gridDim = dim3((unsigned)S * (unsigned)T * (unsigned)R);
     cfg.blockDim = dim3(wide ? 512 : 256);
     cfg.dynamicSmemBytes = wide ? kSmem16 : alone ? kAlone : kSmem;
     cfg.stream = s;
@@ -580,7 +607,8 @@ static spqt_status kq_launch_mode(const void* records, int R, int n, const void*
     cfg.numAttrs = (g_no_pdl ? 0 : 1) + (S > 1 ? 1 : 0);
     auto kernel = wide ? kq_gemv_kernel<BITS, LIST, 16> : kq_gemv_kernel<BITS, LIST, 8>;
     const cudaError_t err = cudaLaunchKernelEx(&cfg, kernel, static_cast<const uint8_t*>(records), n, static_cast<const __half*>(x), idx, count,
-                                               static_cast<__half*>(y), S);
+                                               static_cast<__half*>(y), S, T, static_cast<unsigned*>(workspace),
+                                               reinterpret_cast<float*>(static_cast<char*>(workspace) + kq_header_bytes(R)));
     count_launch();
     return (err == cudaSuccess && cudaGetLastError() == cudaSuccess) ? SPQT_OK : SPQT_ERR_CUDA;
 }
@@ -598,7 +626,7 @@ static spqt_status kq_launch(const void* records, int m, int n, const void* x, c
     const int R = m / kKqG;
     if (ws_bytes < kq_workspace_bytes(R)) return SPQT_ERR_WORKSPACE;
     const cudaStream_t s = static_cast<cudaStream_t>(stream);
-    return idx ? kq_launch_mode<BITS, true>(records, R, n, x, idx, count, y, s) : kq_launch_mode<BITS, false>(records, R, n, x, idx, count, y, s);
+    return idx ? kq_launch_mode<BITS, true>(records, R, n, x, idx, count, y, workspace, s) : kq_launch_mode<BITS, false>(records, R, n, x, idx, count, y, workspace, s);
 }
 
 }  // namespace spqt

@@ -120,7 +120,7 @@ def test_two_level_conversion_at_the_edges_of_tiles_and_alignments(bits, m_block
 
 
 @pytest.mark.parametrize("bits", [2, 4, 5, 6, 8])
-@pytest.mark.parametrize("m_blocks,n", [(1, 1), (2, 17), (1, 2049), (20, 300), (37, 1030), (60, 264), (101, 129), (149, 40)])
+@pytest.mark.parametrize("m_blocks,n", [(1, 1), (2, 17), (1, 2049), (20, 300), (37, 1030), (60, 264), (101, 129), (149, 40), (3, 16421)])
 def test_two_level_products_at_chunk_part_and_cluster_edges(bits, m_blocks, n):
     m = 256 * m_blocks
     W = inputs.weights(m, n, seed=m + n, std=0.1)
