@@ -1026,9 +1026,10 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
     // (a given list counts its clusters with the size of the fused call: the same slices, the same sums)
     constexpr int kSlices = MODE == kModeList ? kModeFused : MODE;
     constexpr int kSmem = (int)sizeof(GemvSmem<G, BITS, kSlices, kCluster, 8>), kSmemPlain = (int)sizeof(GemvSmem<G, BITS, MODE, kPlain, 8>);
-    constexpr int kSmem16 = (int)sizeof(GemvSmem<G, BITS, MODE, kPlain, 16>), kSmemPieces = (int)sizeof(PieceSmem<G, BITS, MODE>);
+    constexpr int kSmem16 = (int)sizeof(GemvSmem<G, BITS, MODE, kPlain, 16>), kSmemSlice16 = (int)sizeof(GemvSmem<G, BITS, MODE, kCluster, 16>);
+    constexpr int kSmemPieces = (int)sizeof(PieceSmem<G, BITS, MODE>);
     static_assert(sizeof(GemvSmem<G, BITS, MODE, kCluster, 8>) <= kSmem && sizeof(GemvSmem<G, BITS, MODE, kSerial, 8>) <= kSmem && kSmem <= kAlone, "one size for all slices");
-    static_assert(kSmem <= 115712 && kSmemPlain <= 115712 && kSmem16 <= 232448 && kSmemPieces <= 232448, "two CTAs of 8 warps per SM, or one of 16");
+    static_assert(kSmem <= 115712 && kSmemPlain <= 115712 && kSmem16 <= 232448 && kSmemSlice16 <= 232448 && kSmemPieces <= 232448, "two CTAs of 8 warps per SM, or one of 16");
     static bool configured[64] = {};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return SPQT_ERR_CUDA;
@@ -1036,6 +1037,8 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
         if (cudaFuncSetAttribute(gemv_kernel<G, BITS, MODE, kPlain, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPlain) != cudaSuccess ||
             cudaFuncSetAttribute(gemv_kernel<G, BITS, MODE, kPlain, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem16) != cudaSuccess ||
             cudaFuncSetAttribute(gemv_kernel<G, BITS, MODE, kCluster, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAlone) != cudaSuccess ||
+            cudaFuncSetAttribute(gemv_kernel<G, BITS, MODE, kCluster, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemSlice16) != cudaSuccess ||
+            cudaFuncSetAttribute(gemv_kernel<G, BITS, MODE, kSerial, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemSlice16) != cudaSuccess ||
             cudaFuncSetAttribute(gemv_kernel<G, BITS, MODE, kSerial, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess ||
             cudaFuncSetAttribute(gemv_pieces_kernel<G, BITS, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPieces) != cudaSuccess)
             return SPQT_ERR_CUDA;
@@ -1071,16 +1074,26 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
         if (f.R <= max_clusters<G, BITS, MODE>(least, kSmem, false, sms, dev)) S = least;
         else pieces = true;
     }
-    // No list to build, and enough per CTA to pay for sharing block-rows (2 us): an even load instead of one or two whole
-    // block-rows per SM (28672 x 16384 44 against 50 us, x 8192 24.5 against 26, x 5120 19 against 16.5)
-    if (tuned <= 0 && MODE == kModeDense && f.R > sms && f.n >= 8192) pieces = true;
+    // More block-rows than SMs: some SMs have two whole block-rows, the others one.  An even load instead pays for sharing
+    // block-rows (2 us) when the excess is small and x long.  Sparse, 50 %, whole against pieces: 20224 x 6615 13.8 / 13.75 us
+    // (at 28 % 17.6 / 16.8), x 8192 16.2 / 15.7; 22016 x 8192 16.3 / 16.3; 25600 x 8192 16.9 / 17.5; 20224 x 5120 11.3 / 12.5.
+    // 24-byte blocks gain more (10624 x 8192 18.5 / 14.2, x 4096 9.4 / 10.2).  Dense (no list to build in every CTA): 22016 x
+    // 6144 17.7 / 16.2, x 4096 12.7 / 13.2, 28672 x 7168 22 / 22.5, x 16384 50 / 44.
+    if (tuned <= 0 && f.R > sms) {
+        const int excess = f.R - sms;
+        if (MODE == kModeDense) pieces = pieces || f.n >= 8192 || 64 * excess <= f.n - 4096;
+        else if (f.n >= 6144) pieces = pieces || (BITS == 3 && G == 64 ? 4 * excess <= sms : 170 * excess <= f.n - 4096);
+    }
     const unsigned long long warps = (unsigned long long)P * kPieceWarps;
     // a warp has parts of two block-rows at most, and the arithmetic is 32-bit
     if (warps < (unsigned)f.R || (warps + 1) * (unsigned)(f.R + 2) >= (1ull << 32) || warps * ((unsigned)f.n + 8u) >= (1ull << 32)) pieces = false;
     S = S < least ? least : (S > kMaxSplit ? kMaxSplit : S);
     const int kind = S == 1 ? kPlain : g_no_cluster ? kSerial : kCluster;
     // a grid that fits one CTA per SM is spread that way (two CTAs of a cluster may otherwise share an SM while others idle)
-    const bool alone = !pieces && kind == kCluster && f.R <= max_clusters<G, BITS, MODE>(S, kAlone, true, sms, dev);
+    const bool alone = !pieces && S > 1 && f.R <= max_clusters<G, BITS, MODE>(S, kAlone, true, sms, dev);
+    // a long x: 16 warps, for the scan and for the loop (4096 x 14336 at 50 % 8.1 against 8.5 us, dense 7.7 against 8.6; 3072 x
+    // 28672 11.5 against 13.0; at n = 4096 and for 3-bit codes no faster)
+    const bool wide_slices = alone && BITS == 4 && f.n >= 8192;
     // whole block-rows on one CTA per SM: 16 warps (14336 x 4096 6.2 against 6.5 us, 18944 x 4096 6.4 against 7.0)
     const bool wide = !pieces && kind == kPlain && f.R <= sms;
     const bool cluster = !pieces && kind == kCluster;
@@ -1106,8 +1119,8 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
     ga.count_out = fa.count_out;
     ga.static_partition = g_static_partition;
     cudaLaunchConfig_t cfg = {};
-    cfg.blockDim = dim3(pieces || wide ? 512 : 256);
-    cfg.dynamicSmemBytes = pieces ? kSmemPieces : alone ? kAlone : wide ? kSmem16 : kind == kPlain ? kSmemPlain : kSmem;
+    cfg.blockDim = dim3(pieces || wide || wide_slices ? 512 : 256);
+    cfg.dynamicSmemBytes = pieces ? kSmemPieces : wide_slices ? kSmemSlice16 : alone && cluster ? kAlone : wide ? kSmem16 : kind == kPlain ? kSmemPlain : kSmem;
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1122,7 +1135,8 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
     auto kernel = pieces             ? gemv_pieces_kernel<G, BITS, MODE>
                   : wide             ? gemv_kernel<G, BITS, MODE, kPlain, 16>
                   : kind == kPlain   ? gemv_kernel<G, BITS, MODE, kPlain, 8>
-                  : kind == kCluster ? gemv_kernel<G, BITS, MODE, kCluster, 8>
+                  : kind == kCluster ? (wide_slices ? gemv_kernel<G, BITS, MODE, kCluster, 16> : gemv_kernel<G, BITS, MODE, kCluster, 8>)
+                  : wide_slices      ? gemv_kernel<G, BITS, MODE, kSerial, 16>
                                      : gemv_kernel<G, BITS, MODE, kSerial, 8>;
     const cudaError_t err = cudaLaunchKernelEx(&cfg, kernel, ga);
     count_launch();

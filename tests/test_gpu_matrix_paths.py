@@ -45,7 +45,7 @@ def test_small_batch_at_chunk_part_and_split_edges(bits, group, m_blocks, n, bat
 
 @pytest.mark.parametrize("bits,group", FORMATS)
 @pytest.mark.parametrize("m_blocks,n,ctas", [(1, 1, 0), (2, 31, 0), (3, 33, 2), (7, 257, 4), (40, 300, 7), (19, 2049, 8), (5, 8193, 0), (9, 300, 72),
-                                             (101, 33, 0), (149, 260, 0), (299, 40, 0), (149, 8192, 0), (149, 8200, 0)])
+                                             (101, 33, 0), (149, 260, 0), (299, 40, 0), (149, 8191, 0), (200, 8192, 0), (149, 8200, 0), (3, 8200, 0)])
 def test_single_row_at_chunk_part_slice_and_piece_edges(bits, group, m_blocks, n, ctas):
     """Clusters, one CTA per block-row with 16 and with 8 warps, equal pieces of all block-rows; the list given, collected in
     the call (the same bits) and absent."""
