@@ -75,9 +75,12 @@ struct RowRing {                         // where a CTA works on one block-row
     // with a list they cost more in the parts' last chunks (4096 x 14336 at 50 % 10.0 against 9.5 us)
     static constexpr int CH = MODE == kModeDense ? 32 * (128 / G) : 32, D = MODE == kModeDense || G == 128 ? 4 : 6;
 };
-template <int G, int MODE>
-struct PieceRing {
-    static constexpr int CH = 32, D = G == 128 ? 4 : 6;
+template <int G, int BITS, int MODE>
+struct PieceRing {                       // the CTA keeps the whole list as well
+    // 64-row blocks: chunks of 64 (dense 28672 x 8192 4 bits 25.6 against 27.3 us, 3 bits 31.9 against 36.9), but not for
+    // lists of 24-byte blocks (24.1 against 31.4 us: fewer copies in flight)
+    static constexpr bool kShort = BITS == 3 && G == 64 && MODE != kModeDense;
+    static constexpr int CH = kShort ? 32 : 32 * (128 / G), D = G == 128 ? 4 : kShort ? 6 : 3;
 };
 
 template <int G, int BITS, class Ring>
@@ -100,7 +103,7 @@ struct LoopSmem {
 
 template <int G, int BITS, int MODE, int NW>
 struct PieceLoopSmem {
-    using Ring = PieceRing<G, MODE>;
+    using Ring = PieceRing<G, BITS, MODE>;
     Stage<G, BITS, Ring> stage[NW][Ring::D];
     alignas(16) unsigned short b[NW][Ring::CH][8];
     alignas(16) float red[2][NW][G];
@@ -682,7 +685,7 @@ template <int G, int BITS, int MODE>
 __global__ void __launch_bounds__(kPieceWarps * 32, 1)
 gemv_pieces_kernel(const GemvArgs a)
 {
-    using Ring = PieceRing<G, MODE>;
+    using Ring = PieceRing<G, BITS, MODE>;
     constexpr int B = G * BITS / 8, CH = Ring::CH, EPL = CH / 32, D = Ring::D, NW = kPieceWarps, kThreads = NW * 32;
     constexpr bool FUSED = MODE == kModeFused, LIST = MODE == kModeList;
     using Smem = PieceSmem<G, BITS, MODE>;
@@ -1071,18 +1074,21 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
     if (tuned <= 0 && S < least) {
         // A whole block-row does not fit a CTA: a cluster with one slice per CTA if all are resident at once (14336 x 11008
         // 14.5 against 16.2 us), otherwise pieces (12288 x 14589 3-bit 19.9 against 25 us with CTAs in two waves).
-        if (f.R <= max_clusters<G, BITS, MODE>(least, kSmem, false, sms, dev)) S = least;
+        // (24-byte blocks: pieces; 6400 x 14336 took 18.8 us in clusters)
+        if (!(BITS == 3 && G == 64) && f.R <= max_clusters<G, BITS, MODE>(least, kSmem, false, sms, dev)) S = least;
         else pieces = true;
     }
     // More block-rows than SMs: some SMs have two whole block-rows, the others one.  An even load instead pays for sharing
     // block-rows (2 us) when the excess is small and x long.  Sparse, 50 %, whole against pieces: 20224 x 6615 13.8 / 13.75 us
     // (at 28 % 17.6 / 16.8), x 8192 16.2 / 15.7; 22016 x 8192 16.3 / 16.3; 25600 x 8192 16.9 / 17.5; 20224 x 5120 11.3 / 12.5.
-    // 24-byte blocks gain more (10624 x 8192 18.5 / 14.2, x 4096 9.4 / 10.2).  Dense (no list to build in every CTA): 22016 x
+    // The same goes for block-rows a little above a second wave of CTAs (64-row groups, 28672 x 8192 25.0 / 24.3).  24-byte
+    // blocks gain more (28672 x 8192 34.8 / 23.9, x 4096 20.0 / 15.6; 10624 x 8192 18.5 / 14.2, x 4096 9.4 / 10.2).  Dense (no list to build in every CTA): 22016 x
     // 6144 17.7 / 16.2, x 4096 12.7 / 13.2, 28672 x 7168 22 / 22.5, x 16384 50 / 44.
     if (tuned <= 0 && f.R > sms) {
         const int excess = f.R - sms;
         if (MODE == kModeDense) pieces = pieces || f.n >= 8192 || 64 * excess <= f.n - 4096;
-        else if (f.n >= 6144) pieces = pieces || (BITS == 3 && G == 64 ? 4 * excess <= sms : 170 * excess <= f.n - 4096);
+        else if (BITS == 3 && G == 64) pieces = pieces || f.n >= 6144 || (f.n >= 4096 && f.R > 2 * sms);
+        else if (f.n >= 6144) pieces = pieces || 170 * excess <= f.n - 4096 || (f.R > 2 * sms && f.R <= 3 * sms + sms / 4);
     }
     const unsigned long long warps = (unsigned long long)P * kPieceWarps;
     // a warp has parts of two block-rows at most, and the arithmetic is 32-bit
