@@ -244,7 +244,7 @@ gemm_small_kernel(const SmallArgs a)
 #pragma unroll
             for (int b = 0; b < ROWS / 2; ++b) {
                 float p0, p1;
-                unpack2(p[b], p0, p1);
+                unpack2(to_halves2(p[b]), p0, p1);
                 const __half2 h = __floats2half2_rn(p0, p1);
                 const float2 hf = __half22float2(h);
                 unsigned long long rest = p[b];
@@ -266,12 +266,18 @@ gemm_small_kernel(const SmallArgs a)
         unsigned bh[4], bl[4];
         ldsm_x4_trans(bbuf + 16u * lane, bh);
         if (TWO) ldsm_x4_trans(bbuf + 512u + 16u * lane, bl);
+        unsigned c[2][SP][4];
 #pragma unroll
         for (int ks = 0; ks < 2; ++ks) {
-            unsigned c[SP][4];
-            Layout::load(st, ll, ks, c);
+            Layout::load(st, ll, ks, c[ks]);
+            if (!TWO) {
 #pragma unroll
-            for (int s = 0; s < SP; ++s) mma_group<TWO>(acc[s], c[s], bh + 2 * ks, bl + 2 * ks);
+                for (int s = 0; s < SP; ++s) mma_group(acc[s], c[ks][s], bh + 2 * ks);
+            }
+        }
+        if (TWO) {
+#pragma unroll
+            for (int s = 0; s < SP; ++s) mma_group_two(acc[s], c[0][s], c[1][s], bh, bl);
         }
         __syncwarp();
         rc = rc + kStageBytes == D * kStageBytes ? 0u : rc + kStageBytes;

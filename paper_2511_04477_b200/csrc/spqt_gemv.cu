@@ -278,8 +278,8 @@ struct Product {
     {
 #pragma unroll
         for (int q = 0; q < EPL; ++q) {
-            const float h = __low2float(__floats2half2_rn(pm[q], 0.0f));
-            const __half2 hl = __floats2half2_rn(pm[q], pm[q] - h);
+            const float h = __low2float(__floats2half2_rn(to_halves(pm[q]), 0.0f));
+            const __half2 hl = __floats2half2_rn(h, pm[q] - h);
             sts_u32(b_base + 512u * q, *reinterpret_cast<const unsigned*>(&hl));
         }
     }
@@ -308,7 +308,7 @@ struct Product {
                 leave();
             }
 #pragma unroll
-            for (int sp = 0; sp < SP; ++sp) mma_group<false>(acc[sp], c[sp], bb[ks >> 1] + 2 * (ks & 1), bb[0]);
+            for (int sp = 0; sp < SP; ++sp) mma_group(acc[sp], c[sp], bb[ks >> 1] + 2 * (ks & 1));
         }
         if (regain != 1.0f) {
 #pragma unroll
@@ -336,7 +336,7 @@ struct Product {
 };
 
 // The warps' sums of a block-row, in warp order: thread j < G / 2 gets rows j and j + G/2, those of the low and the high
-// nibbles of a byte (the latter's tiles sum whole bytes).
+// nibbles of byte j (the latter's tiles sum 16 times the nibble of even bytes and the whole of odd ones).
 template <int G, int NW, class Warp>
 __device__ __forceinline__ void add_warps(const Warp* warp, const float2* red_z, int j, float* v, float* z)
 {
@@ -348,7 +348,7 @@ __device__ __forceinline__ void add_warps(const Warp* warp, const float2* red_z,
         v[1] += warp[w].red[j + G / 2] * cz.x;
         *z += cz.y;
     }
-    v[1] = (v[1] - v[0]) * 0.0625f;
+    v[1] = (v[1] - ((j & 1) ? v[0] : 0.0f)) * 0.0625f;
 }
 
 // ---------------------------------------------------------------- fused: the list
@@ -852,7 +852,7 @@ gemv_pieces_kernel(const GemvArgs a)
             v1 += lp.red[s][w - W0][j + G / 2] * cz.x;
             z += cz.y;
         }
-        v1 = (v1 - v0) * 0.0625f;        // the high nibbles' tiles sum whole bytes
+        v1 = (v1 - ((j & 1) ? v0 : 0.0f)) * 0.0625f;   // (see add_warps)
         if (fw >= W0 && lw < W0 + NW) {
             store_y(r, v0 + z, v1 + z);
         } else {

@@ -218,6 +218,14 @@ __device__ __forceinline__ void fma_block8(unsigned long long* acc, const uint2&
     fma_word(acc + 4, w.y, m01, m23);
 }
 
+// a + b on both lanes
+__device__ __forceinline__ unsigned long long fadd2(unsigned long long a, unsigned long long b)
+{
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
 // One step of a butterfly reduce-scatter: lanes that differ in bit `bit` hold
 // partial sums of the same rows; each keeps one half of its N values and
 // receives the partner's partials of that half.

@@ -23,7 +23,8 @@
 //                    warps per SM with 2 to 5 chunks in flight each.  28672 x 4096 to 4 bits at 50 %, list included, takes
 //                    15.9 us (19.4 with packed FMAs, partial sums in global memory and chunks dealt in turn), 8192 x 8192
 //                    to 6 bits dense 16.6 us (20.4; 55 MB), 28672 x 4096 to 2 bits dense 17.3 us (24.7).
-//                    A multiplier x*(d*sc) is rounded to fp32 and goes in as two fp16 values, which keep 24 bits of it.
+//                    A multiplier x*(d*sc) is rounded to fp32 and goes in as two fp16 values, off by 2^-24 of the warp's
+//                    largest at most (spqt_mma.cuh; multiples of 1/2 cost 0.6 to 2.6 %: 28672 x 8192 dense to 4 bits 34.5 -> 35.4 us).
 #include <cstddef>
 
 #include "spqt_common.cuh"
@@ -410,8 +411,8 @@ kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* __restr
         unsigned w[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const float h = __low2float(__floats2half2_rn(pm[j], 0.0f));
-            const __half2 hl = __floats2half2_rn(pm[j], pm[j] - h);
+            const float h = __low2float(__floats2half2_rn(to_halves(pm[j]), 0.0f));
+            const __half2 hl = __floats2half2_rn(h, pm[j] - h);
             w[j] = *reinterpret_cast<const unsigned*>(&hl);
         }
         sts_v4(b_base, make_uint4(w[0], w[1], w[2], w[3]));

@@ -7,10 +7,17 @@
 // ldmatrix.trans delivers from blocks that lie row after row in shared memory: one register then holds bytes
 // (2g, 2g+1) of entries 2t and 2t+1, i.e. four codes of each, and four operations make four operands of it.
 //
-// a = x*scale has up to 22 significant bits.  It goes in as two fp16 values, hi = fp16(a*c) and lo = fp16(a*c - hi),
-// c a power of two that every warp keeps per batch row so that its largest |a*c| so far lies in 2^10 .. 2^15: hi + lo
-// is then a*c exactly, or to 2^-36 of the largest entry, far below the fp32 accumulation.  When an entry exceeds the
-// range, the sums are rescaled (a power of two: exact) and c changes.
+// a = x*scale has up to 22 significant bits.  It goes in as two fp16 values: hi = a*c rounded to a multiple of 1/2 and to
+// fp16, lo = fp16(a*c - hi), c a power of two that every warp keeps per batch row so that its largest |a*c| so far lies in
+// 2^10 .. 2^15.  hi + lo is a*c, or off by 2^-14 at most (2^-24 of the largest entry).  When an entry exceeds the range, the
+// sums are rescaled (a power of two: exact) and c changes.
+// Why multiples of 1/2: the instruction brings its 16 products and the sum to one exponent, the largest, and keeps 25 bits
+// below it (measured).  A subnormal operand counts there with the exponent of the smallest normal number, 2^-14, though its
+// leading bit is up to ten places lower: a code's product may then reach past the 25 bits and is cut.  hi < 2^15 in
+// multiples of 1/2 makes the largest exponent 2^0 and every product a multiple of 2^-25: nothing is cut, and the sums of hi are
+// exact up to 24 bits.  What lo's products lose is 2^-11 of that; hi and lo have sums of their own.  With hi = fp16(a*c) 1.7 % of
+// the dense call's y were not the fp16 nearest to the exact value (2.2 % of a batch's), now 0.33 %, as with fp32 FMAs in
+// sequence (0.32 %; sixty shapes between 512 x 256 and 16384 x 28672); 8192 x 28672 dense 22.3 us either way.
 //
 // Per chunk of 32 entries x 128 rows the arithmetic is 84 warp instructions (4 ldmatrix, 64 masks and byte
 // permutations, 16 mma) where the packed-FMA form takes 218 for one row and 64 more for every further one.
@@ -21,6 +28,13 @@ namespace spqt {
 // c of a warp that has seen nothing but zeros: any entry exceeds the range
 constexpr float kMmaNoScale = 0x1p100f;
 constexpr float kMmaLimit = 32768.0f;
+
+// v rounded to a multiple of 1/2, |v| < 2^21; two of them
+__device__ __forceinline__ float to_halves(float v) { return __fsub_rn(__fadd_rn(v, 6291456.0f), 6291456.0f); }
+__device__ __forceinline__ unsigned long long to_halves2(unsigned long long v)
+{
+    return fadd2(fadd2(v, pack2(6291456.0f, 6291456.0f)), pack2(-6291456.0f, -6291456.0f));
+}
 
 // 1 / c of a power of two between 2^-100 and 2^100, exactly
 __device__ __forceinline__ float power_of_two_inverse(float c) { return __uint_as_float((254u << 23) - __float_as_uint(c)); }
@@ -115,32 +129,56 @@ struct MmaStage {
     }
 };
 
-// The four tiles of one group: acc[type] += the operand of that type times B.  type 0 / 2: the low nibbles of the even /
-// odd bytes; 1 / 3: the whole even / odd bytes (low + 16 * high, still a subnormal: one operation less than the high
-// nibble alone, whose sum is recovered at the end as (byte - low) / 16).  TWO: B comes as hi and lo.
-template <bool TWO>
-__device__ __forceinline__ void mma_group(float (*acc)[4], const unsigned* c, const unsigned* bh, const unsigned* bl)
+// The four tiles of 16 entries and 64 rows: type 0 / 2 the low nibbles of the even / odd bytes, 1 the high nibbles of the
+// even ones (in place: 16 times the code), 3 the whole odd bytes (one operation less than their high nibbles, whose sum is
+// recovered at the end as (byte - low) / 16).
+struct MmaTiles {
+    unsigned a[4][4];
+    __device__ __forceinline__ explicit MmaTiles(const unsigned* c)
+    {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            a[0][i] = c[i] & 0x000f000fu;
+            a[1][i] = c[i] & 0x00f000f0u;
+            a[3][i] = __byte_perm(c[i], 0u, 0x4341);
+            a[2][i] = a[3][i] & 0x000f000fu;
+        }
+    }
+};
+
+// acc[type] += the operands of that type times B
+__device__ __forceinline__ void mma_group(float (*acc)[4], const unsigned* c, const unsigned* b)
 {
-    constexpr unsigned kLow = 0x000f000fu, kByte = 0x00ff00ffu;
-    unsigned d[4];
+    const MmaTiles t(c);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) d[i] = __byte_perm(c[i], 0u, 0x4341);   // the odd bytes
+    for (int type = 0; type < 4; ++type) mma_16816(acc[type], t.a[type][0], t.a[type][1], t.a[type][2], t.a[type][3], b[0], b[1]);
+}
+
+// The same over 32 entries (c0, then c1) for a B in two sets, hi and lo, whose sums share registers.  A sum that holds lo parts
+// would lose them when the next hi product of a low nibble sets the exponent, so the 32 entries are summed from zero, hi
+// before lo, and then added in fp32.  (Straight into the sums: 1.5 % of y not the nearest fp16 instead of 0.33 %; 28672 x 8192
+// with 8 rows dense 37.6 against 40.4 us.  Sums of lo in registers of their own: 41.3 us.)
+__device__ __forceinline__ void mma_group_two(float (*acc)[4], const unsigned* c0, const unsigned* c1, const unsigned* bh, const unsigned* bl)
+{
+    const MmaTiles t0(c0), t1(c1);
 #pragma unroll
-    for (int h = 0; h < (TWO ? 2 : 1); ++h) {
-        const unsigned b0 = h ? bl[0] : bh[0], b1 = h ? bl[1] : bh[1];
-        mma_16816(acc[0], c[0] & kLow, c[1] & kLow, c[2] & kLow, c[3] & kLow, b0, b1);
-        mma_16816(acc[1], c[0] & kByte, c[1] & kByte, c[2] & kByte, c[3] & kByte, b0, b1);
-        mma_16816(acc[2], d[0] & kLow, d[1] & kLow, d[2] & kLow, d[3] & kLow, b0, b1);
-        mma_16816(acc[3], d[0], d[1], d[2], d[3], b0, b1);
+    for (int type = 0; type < 4; ++type) {
+        float d[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        mma_16816(d, t0.a[type][0], t0.a[type][1], t0.a[type][2], t0.a[type][3], bh[0], bh[1]);
+        mma_16816(d, t1.a[type][0], t1.a[type][1], t1.a[type][2], t1.a[type][3], bh[2], bh[3]);
+        mma_16816(d, t0.a[type][0], t0.a[type][1], t0.a[type][2], t0.a[type][3], bl[0], bl[1]);
+        mma_16816(d, t1.a[type][0], t1.a[type][1], t1.a[type][2], t1.a[type][3], bl[2], bl[3]);
+#pragma unroll
+        for (int i = 0; i < 4; i += 2) unpack2(fadd2(pack2(acc[type][i], acc[type][i + 1]), pack2(d[i], d[i + 1])), acc[type][i], acc[type][i + 1]);
     }
 }
 
-// The sums of a group as the sums of its codes (see mma_group)
+// The sums of a group as the sums of its codes (see MmaTiles)
 __device__ __forceinline__ void mma_uncumulate(float (*acc)[4])
 {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        acc[1][i] = (acc[1][i] - acc[0][i]) * 0.0625f;
+        acc[1][i] *= 0.0625f;
         acc[3][i] = (acc[3][i] - acc[2][i]) * 0.0625f;
     }
 }

@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(kProbeWarps * 32, 1) probe_arith_kernel(int ch
             unsigned c[2][4];
             Layout::load(base + rc, ll, ks, c);
 #pragma unroll
-            for (int sp = 0; sp < 2; ++sp) mma_group<false>(acc[sp], c[sp], bb + 2 * ks, bb);
+            for (int sp = 0; sp < 2; ++sp) mma_group(acc[sp], c[sp], bb + 2 * ks);
         }
         __syncwarp();
         rc = (rc + 2048u == kArithStages * 2048u) ? 0u : rc + 2048u;

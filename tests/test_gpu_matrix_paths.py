@@ -43,6 +43,49 @@ def test_small_batch_at_chunk_part_and_split_edges(bits, group, m_blocks, n, bat
         check_y(Ys.cpu().numpy()[b], Ys_ref[b], bound[b], "row %d" % b)
 
 
+def share_not_nearest(y, exact):
+    """Share of the outputs that are not the fp16 nearest to the exact value.  A value lands on the other side of a rounding
+    boundary with a probability of its error before the rounding over the spacing of fp16: the mean error in those units."""
+    return float(np.mean(y.view(np.uint16) != exact.astype(np.float16).view(np.uint16)))
+
+
+# fp32 FMAs in sequence leave 0.3 % on these inputs (an error of 2^-25 of the partial sum per step, n / 32 steps per warp at
+# most, |y| about n^-1/2 of the sum of the magnitudes); multipliers cut by the alignment of the tensor core's products
+# 1.0 to 4 %.  The bound is three times the former; the count of a share of 0.3 % of 8192 has a deviation of 0.06 %.
+NOT_NEAREST = 0.0075
+
+
+@pytest.mark.parametrize("bits,group,n", [(4, 128, 602), (4, 64, 1490), (3, 128, 543), (3, 64, 293), (4, 128, 4100)])
+def test_sums_are_as_exact_as_fp32(bits, group, n):
+    m, batch = 8192, 8
+    W = inputs.weights(m, n, seed=n)
+    X = np.stack([inputs.activations(n, seed=40 + b) for b in range(batch)])
+    X[1::2, ::97] *= 20
+    p = pack_on_gpu(W, bits, group)
+    codes, s, z = packed_to_host(p)
+    Xd = dev(X)
+    small = binding.new_gemm_small_workspace(p)
+    rows = [oracle.dense_gemv(codes, s, z, m, n, X[b], bits, group)[0] for b in range(batch)]
+    for b in (0, 1):
+        y = binding.spqt_dense_gemv(p, Xd[b].contiguous(), binding.new_workspace(m, n, bits, group)).cpu().numpy()
+        assert share_not_nearest(y, rows[b]) < NOT_NEAREST, "one row, %d" % b
+    for rows_at_once in (4, 8):
+        Y = binding.spqt_dense_gemm_small(p, Xd[:rows_at_once], small).cpu().numpy()
+        assert share_not_nearest(Y, np.stack(rows[:rows_at_once])) < NOT_NEAREST, "%d rows" % rows_at_once
+
+
+# (0.17 to 0.27 % with fp32 FMAs in sequence: multipliers cut by the alignment leave 0.5 to 0.7 %)
+@pytest.mark.parametrize("bits,n", [(2, 700), (4, 300)])
+def test_two_level_sums_are_as_exact_as_fp32(bits, n):
+    m = 8192
+    W = inputs.weights(m, n, seed=n)
+    x = inputs.activations(n, seed=50)
+    y_ref, _ = oracle.kq_gemv(*oracle.kq_quantize(W, bits=bits), x)
+    p = binding.spqt_kqw_pack(dev(W), bits)
+    y = binding.spqt_kqw_dense_gemv(p, dev(x), binding.new_kq_workspace(p)).cpu().numpy()
+    assert share_not_nearest(y, y_ref) < 0.004
+
+
 @pytest.mark.parametrize("bits,group", FORMATS)
 @pytest.mark.parametrize("m_blocks,n,ctas", [(1, 1, 0), (2, 31, 0), (3, 33, 2), (7, 257, 4), (40, 300, 7), (19, 2049, 8), (5, 8193, 0), (9, 300, 72),
                                              (101, 33, 0), (149, 260, 0), (299, 40, 0), (149, 8191, 0), (200, 8192, 0), (149, 8200, 0), (3, 8200, 0)])
