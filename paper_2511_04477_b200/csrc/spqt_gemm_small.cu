@@ -171,6 +171,7 @@ gemm_small_kernel(const SmallArgs a)
 #pragma unroll 1
     for (int d = 0; d < D - 1; ++d) issue();
 
+    bool empty = true;            // nothing in the sums yet
 #pragma unroll 1
     for (; pos < end; pos += CH) {
         issue();
@@ -215,6 +216,7 @@ gemm_small_kernel(const SmallArgs a)
             }
             if (__any_sync(0xffffffffu, top > kMmaLimit)) {
                 // a larger entry than the range holds: new scales for the rows concerned
+                float factor[2] = {1.0f, 1.0f};   // of the lane's columns
 #pragma unroll
                 for (int b = 0; b < ROWS / 2; ++b) {
                     float av[2], sv[2], fv[2] = {1.0f, 1.0f};
@@ -225,7 +227,7 @@ gemm_small_kernel(const SmallArgs a)
                         const unsigned bits = __float_as_uint(av[j]) & 0x7fffffffu;
                         const unsigned m = __reduce_max_sync(0xffffffffu, bits < 0x7f800000u ? bits : 0u);   // finite ones
                         if (__uint_as_float(m) * sv[j] > kMmaLimit) {
-                            const float next = __uint_as_float((264u - (m >> 23)) << 23);   // m goes to 2^10 .. 2^11
+                            const float next = __uint_as_float((266u - (m >> 23)) << 23);   // m goes to 2^12 .. 2^13
                             fv[j] = next * power_of_two_inverse(sv[j]);
                             sv[j] = next;
                         }
@@ -233,11 +235,25 @@ gemm_small_kernel(const SmallArgs a)
                     scale[b] = pack2(sv[0], sv[1]);
                     p[b] = fmul2(am[b], scale[b]);
                     if ((t4 & (ROWS / 2 - 1)) == b) {   // the lane's columns are rows 2b and 2b + 1
-#pragma unroll
-                        for (int s = 0; s < SP; ++s)
-#pragma unroll
-                            for (int i = 0; i < 16; ++i) acc[s][i >> 2][i & 3] *= fv[i & 1];
+                        factor[0] = fv[0];
+                        factor[1] = fv[1];
                     }
+                }
+                if (!empty) {
+#pragma unroll
+                    for (int s = 0; s < SP; ++s)
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) {
+                            float& v = acc[s][i >> 2][i & 3];
+                            if (TWO) {
+                                v *= factor[i & 1];
+                            } else {   // lanes t4 < 2 have the sums of hi, t4 ^ 2 those of lo
+                                float hi = v, rest = 0.0f;
+                                rescale_sums(hi, rest, factor[i & 1]);
+                                rest = __shfl_xor_sync(0xffffffffu, rest, 2);
+                                v = t4 < 2 ? hi : v * factor[i & 1] + rest;
+                            }
+                        }
                 }
             }
             unsigned hi[ROWS / 2], lo[ROWS / 2];
@@ -279,6 +295,7 @@ gemm_small_kernel(const SmallArgs a)
 #pragma unroll
             for (int s = 0; s < SP; ++s) mma_group_two(acc[s], c[0][s], c[1][s], bh, bl);
         }
+        empty = false;
         __syncwarp();
         rc = rc + kStageBytes == D * kStageBytes ? 0u : rc + kStageBytes;
     }

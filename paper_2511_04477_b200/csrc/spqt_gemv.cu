@@ -267,7 +267,7 @@ struct Product {
         }
         m = __reduce_max_sync(0xffffffffu, m);
         if (__uint_as_float(m) * scale > kMmaLimit) {
-            const float next = __uint_as_float((264u - (m >> 23)) << 23);   // m goes to 2^10 .. 2^11
+            const float next = __uint_as_float((266u - (m >> 23)) << 23);   // m goes to 2^12 .. 2^13
             regain = next * power_of_two_inverse(scale);
             scale = next;
 #pragma unroll
@@ -312,7 +312,10 @@ struct Product {
         }
         if (regain != 1.0f) {
 #pragma unroll
-            for (int i = 0; i < SP * 16; ++i) acc[i >> 4][(i >> 2) & 3][i & 3] *= regain;
+            for (int i = 0; i < SP * 8; ++i) {
+                float* const a = &acc[i >> 3][(i >> 1) & 3][2 * (i & 1)];
+                rescale_sums(a[0], a[1], regain);
+            }
             regain = 1.0f;
         }
         __syncwarp();                // every lane is done with this chunk's stage
@@ -576,9 +579,9 @@ gemv_kernel(const GemvArgs a)
         int ipos = first;                // where the copies stand: D - 1 chunks ahead of the product
         unsigned ri = 0;                 // byte offset of the copies' stage
         auto issue = [&]() {             // the copies of the next chunk, if there is one
-            if (!FUSED) {
+            if (!FUSED) {                // (0 past the end: what the stages hold there must not change the scale)
 #pragma unroll
-                for (int i = 0; i < (D - 1) * EPL; ++i) xv[i / EPL][i % EPL] = xv[i / EPL + 1][i % EPL];
+                for (int i = 0; i < D * EPL; ++i) xv[i / EPL][i % EPL] = i < (D - 1) * EPL ? xv[(i / EPL + 1) % D][i % EPL] : 0u;
             }
             if (ipos < end) {
                 unsigned col[EPL];
@@ -773,7 +776,7 @@ gemv_pieces_kernel(const GemvArgs a)
     unsigned ri = 0;
     auto issue = [&]() {                 // the copies of the next chunk, if there is one
 #pragma unroll
-        for (int i = 0; i < (D - 1) * EPL; ++i) xv[i / EPL][i % EPL] = xv[i / EPL + 1][i % EPL];
+        for (int i = 0; i < D * EPL; ++i) xv[i / EPL][i % EPL] = i < (D - 1) * EPL ? xv[(i / EPL + 1) % D][i % EPL] : 0u;   // (0 past the end)
         if (at.pos < at.hi) {
             unsigned col[EPL];
 #pragma unroll

@@ -23,8 +23,8 @@
 //                    warps per SM with 2 to 5 chunks in flight each.  28672 x 4096 to 4 bits at 50 %, list included, takes
 //                    15.9 us (19.4 with packed FMAs, partial sums in global memory and chunks dealt in turn), 8192 x 8192
 //                    to 6 bits dense 16.6 us (20.4; 55 MB), 28672 x 4096 to 2 bits dense 17.3 us (24.7).
-//                    A multiplier x*(d*sc) is rounded to fp32 and goes in as two fp16 values, off by 2^-24 of the warp's
-//                    largest at most (spqt_mma.cuh; multiples of 1/2 cost 0.6 to 2.6 %: 28672 x 8192 dense to 4 bits 34.5 -> 35.4 us).
+//                    A multiplier x*(d*sc) is rounded to fp32 and goes in as two fp16 values, off by 2^-26 of the warp's
+//                    largest at most (spqt_mma.cuh; their rounding and rescaling cost 2 to 3 %: 28672 x 8192 dense to 4 bits 34.4 -> 35.4 us).
 #include <cstddef>
 
 #include "spqt_common.cuh"
@@ -400,7 +400,7 @@ kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* __restr
         }
         m = __reduce_max_sync(0xffffffffu, m);
         if (__uint_as_float(m) * scale > kMmaLimit) {
-            const float next = __uint_as_float((264u - (m >> 23)) << 23);   // m goes to 2^10 .. 2^11
+            const float next = __uint_as_float((266u - (m >> 23)) << 23);   // m goes to 2^12 .. 2^13
             regain = next * power_of_two_inverse(scale);
             scale = next;
 #pragma unroll
@@ -443,7 +443,7 @@ kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* __restr
         leave();
         if (regain != 1.0f) {
 #pragma unroll
-            for (int i = 0; i < 64; ++i) acc[i >> 2][i & 3] *= regain;
+            for (int i = 0; i < 32; ++i) rescale_sums(acc[i >> 1][2 * (i & 1)], acc[i >> 1][2 * (i & 1) + 1], regain);
             regain = 1.0f;
         }
         __syncwarp();                    // every lane is done with this chunk's stage

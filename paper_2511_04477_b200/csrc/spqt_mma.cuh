@@ -9,15 +9,16 @@
 //
 // a = x*scale has up to 22 significant bits.  It goes in as two fp16 values: hi = a*c rounded to a multiple of 1/2 and to
 // fp16, lo = fp16(a*c - hi), c a power of two that every warp keeps per batch row so that its largest |a*c| so far lies in
-// 2^10 .. 2^15.  hi + lo is a*c, or off by 2^-14 at most (2^-24 of the largest entry).  When an entry exceeds the range, the
-// sums are rescaled (a power of two: exact) and c changes.
+// 2^12 .. 2^15.  hi + lo is a*c, or off by 2^-14 at most (2^-26 of the largest entry).  When an entry exceeds the range, c
+// changes and the sums are rescaled.
 // Why multiples of 1/2: the instruction brings its 16 products and the sum to one exponent, the largest, and keeps 25 bits
 // below it (measured).  A subnormal operand counts there with the exponent of the smallest normal number, 2^-14, though its
 // leading bit is up to ten places lower: a code's product may then reach past the 25 bits and is cut.  hi < 2^15 in
 // multiples of 1/2 makes the largest exponent 2^0 and every product a multiple of 2^-25: nothing is cut, and the sums of hi are
-// exact up to 24 bits.  What lo's products lose is 2^-11 of that; hi and lo have sums of their own.  With hi = fp16(a*c) 1.7 % of
-// the dense call's y were not the fp16 nearest to the exact value (2.2 % of a batch's), now 0.33 %, as with fp32 FMAs in
-// sequence (0.32 %; sixty shapes between 512 x 256 and 16384 x 28672); 8192 x 28672 dense 22.3 us either way.
+// exact up to 24 bits.  What lo's products lose is 2^-11 of that; hi and lo have sums of their own.  Share of y that is not the
+// fp16 nearest to the exact value, 200 shapes between 512 x 256 and 16384 x 28672, half of them with outliers: with
+// hi = fp16(a*c) 1.8 % of the dense call's and 2.4 % of a batch's, now 0.27 and 0.31 %; with fp32 FMAs in sequence 0.34 and
+// 0.33 %.  8192 x 28672 dense takes 22.3 us either way.  (Largest |a*c| from 2^10 up: 0.33 % with outliers.)
 //
 // Per chunk of 32 entries x 128 rows the arithmetic is 84 warp instructions (4 ldmatrix, 64 masks and byte
 // permutations, 16 mma) where the packed-FMA form takes 218 for one row and 64 more for every further one.
@@ -50,6 +51,15 @@ __device__ __forceinline__ void ldsm_x2_trans(unsigned addr, unsigned* r)
 {
     asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(addr) : "memory");
 }
+// The sums of hi and lo multipliers, when c changes by the factor f: what the new hi sum has below 2^-25 goes to lo's, or the
+// next instruction would cut it off.  (From 1/4 up the new sum has no such bits; .375 rounds smaller ones.)
+__device__ __forceinline__ void rescale_sums(float& hi, float& lo, float f)
+{
+    const float h = hi * f;
+    hi = __fsub_rn(__fadd_rn(h, 0.375f), 0.375f);
+    lo = lo * f + (h - hi);
+}
+
 // c[0..3] += A (16 x 16) * B (16 x 8), fp32 sums
 __device__ __forceinline__ void mma_16816(float* c, unsigned a0, unsigned a1, unsigned a2, unsigned a3, unsigned b0, unsigned b1)
 {

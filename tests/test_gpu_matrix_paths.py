@@ -49,18 +49,19 @@ def share_not_nearest(y, exact):
     return float(np.mean(y.view(np.uint16) != exact.astype(np.float16).view(np.uint16)))
 
 
-# fp32 FMAs in sequence leave 0.3 % on these inputs (an error of 2^-25 of the partial sum per step, n / 32 steps per warp at
-# most, |y| about n^-1/2 of the sum of the magnitudes); multipliers cut by the alignment of the tensor core's products
-# 1.0 to 4 %.  The bound is three times the former; the count of a share of 0.3 % of 8192 has a deviation of 0.06 %.
-NOT_NEAREST = 0.0075
+# fp32 FMAs in sequence leave 0.2 to 0.5 % on such inputs, multipliers cut by the alignment of the tensor core's products 1 to
+# 5 %, sums cut when the scale changes 0.8 % (the last case).  The bound is twice the mean of the first; a share of 0.3 % of
+# 8192 values has a deviation of 0.06 %.
+NOT_NEAREST = 0.006
 
 
-@pytest.mark.parametrize("bits,group,n", [(4, 128, 602), (4, 64, 1490), (3, 128, 543), (3, 64, 293), (4, 128, 4100)])
+@pytest.mark.parametrize("bits,group,n", [(4, 128, 602), (4, 64, 1490), (3, 128, 543), (3, 64, 293), (4, 128, 4100), (3, 128, 9000)])
 def test_sums_are_as_exact_as_fp32(bits, group, n):
     m, batch = 8192, 8
     W = inputs.weights(m, n, seed=n)
     X = np.stack([inputs.activations(n, seed=40 + b) for b in range(batch)])
-    X[1::2, ::97] *= 20
+    for b in range(1, batch, 2):   # outliers: the scale of the multipliers changes along the list
+        X[b, np.random.Generator(np.random.PCG64(b)).random(n) < 0.01] *= 20
     p = pack_on_gpu(W, bits, group)
     codes, s, z = packed_to_host(p)
     Xd = dev(X)
