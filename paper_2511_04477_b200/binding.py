@@ -426,11 +426,11 @@ def spqt_kqw_pack(W: torch.Tensor, bits: int, stream=None) -> KqPacked:
 
 def spqt_kqw_sparse_gemv(p: KqPacked, x: torch.Tensor, idx: torch.Tensor, count: torch.Tensor, workspace: torch.Tensor,
                          y: torch.Tensor = None, stream=None) -> torch.Tensor:
-    return native().kqw_gemv(p, x, idx, count, workspace, y, stream, "spqt_kqw_sparse_gemv")
+    return native().kqw_sparse_gemv(p, x, idx, count, workspace, y, stream, "spqt_kqw_sparse_gemv")
 
 
 def spqt_kqw_dense_gemv(p: KqPacked, x: torch.Tensor, workspace: torch.Tensor, y: torch.Tensor = None, stream=None) -> torch.Tensor:
-    return native().kqw_gemv(p, x, None, None, workspace, y, stream, "spqt_kqw_dense_gemv")
+    return native().kqw_dense_gemv(p, x, workspace, y, stream, "spqt_kqw_dense_gemv")
 
 
 def new_kq_workspace(p: KqPacked) -> torch.Tensor:
@@ -441,11 +441,11 @@ def new_kq_workspace(p: KqPacked) -> torch.Tensor:
 
 def spqt_kq_sparse_gemv(p: KqPacked, x: torch.Tensor, idx: torch.Tensor, count: torch.Tensor, workspace: torch.Tensor,
                         y: torch.Tensor = None, stream=None) -> torch.Tensor:
-    return native().kqw_gemv(p, x, idx, count, workspace, y, stream, "spqt_kq_sparse_gemv")
+    return native().kqw_sparse_gemv(p, x, idx, count, workspace, y, stream, "spqt_kq_sparse_gemv")
 
 
 def spqt_kq_dense_gemv(p: KqPacked, x: torch.Tensor, workspace: torch.Tensor, y: torch.Tensor = None, stream=None) -> torch.Tensor:
-    return native().kqw_gemv(p, x, None, None, workspace, y, stream, "spqt_kq_dense_gemv")
+    return native().kqw_dense_gemv(p, x, workspace, y, stream, "spqt_kq_dense_gemv")
 
 
 def spqt_rowwise_thresholded_gemv(p: RowwisePacked, x: torch.Tensor, t: float, y: torch.Tensor = None, stream=None) -> torch.Tensor:

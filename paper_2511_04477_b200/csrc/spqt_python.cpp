@@ -317,33 +317,38 @@ PyObject* dense_gemm_small(PyObject*, Args a, Py_ssize_t na)
     });
 }
 
-// (p, x, idx, count, workspace, y, stream, where) -> y; idx and count None: over all columns
+// list: (p, x, idx, count, workspace, y, stream, where) -> y; over all columns: without idx and count
+template <bool LIST>
 PyObject* kqw_gemv(PyObject*, Args a, Py_ssize_t na)
 {
     return guarded([&]() -> PyObject* {
-        need_args(na, 8);
+        need_args(na, LIST ? 8 : 6);
         PyObject* p = a[0];
+        const Args rest = a + (LIST ? 4 : 2);   // workspace, y, stream, where
         const void* records = tensor_attr(p, g_names.records, at::kByte, "records").data_ptr();
         const int m = int_attr(p, g_names.m), n = int_attr(p, g_names.n), bits = int_attr(p, g_names.bits);
         const at::Tensor& x = tensor_of(a[1], at::kHalf, "x");
-        at::Tensor y = given_or_empty(a[5], {m}, at::kHalf, "y", x);
-        const at::Tensor& ws = tensor_of(a[4], at::kByte, "workspace");
-        void* s = stream_of(a[6]);
-        const char* where = PyUnicode_AsUTF8(a[7]);
+        at::Tensor y = given_or_empty(rest[1], {m}, at::kHalf, "y", x);
+        const at::Tensor& ws = tensor_of(rest[0], at::kByte, "workspace");
+        void* s = stream_of(rest[2]);
+        const char* where = PyUnicode_AsUTF8(rest[3]);
         if (!where) throw Raised();
-        if (a[2] == Py_None && a[3] == Py_None) {
-            call(where, [&] { return spqt_kqw_dense_gemv(records, m, n, bits, x.data_ptr(), y.data_ptr(), ws.data_ptr(), (size_t)ws.numel(), s); });
-        } else {
+        if (LIST) {
             const at::Tensor& idx = tensor_of(a[2], at::kInt, "idx");
             const at::Tensor& count = tensor_of(a[3], at::kInt, "count");
             call(where, [&] {
                 return spqt_kqw_sparse_gemv(records, m, n, bits, x.data_ptr(), (const int32_t*)idx.data_ptr(), (const int32_t*)count.data_ptr(),
                                             y.data_ptr(), ws.data_ptr(), (size_t)ws.numel(), s);
             });
+        } else {
+            call(where, [&] { return spqt_kqw_dense_gemv(records, m, n, bits, x.data_ptr(), y.data_ptr(), ws.data_ptr(), (size_t)ws.numel(), s); });
         }
-        return hand_back(a[5], y);
+        return hand_back(rest[1], y);
     });
 }
+
+constexpr auto kqw_sparse_gemv = kqw_gemv<true>;
+constexpr auto kqw_dense_gemv = kqw_gemv<false>;
 
 const at::Tensor& weights_of(PyObject* o)
 {
@@ -411,7 +416,7 @@ PyObject* set_error(PyObject*, PyObject* cls)
 #define SPQT_METHOD(f) {#f, (PyCFunction)(void (*)(void))f, METH_FASTCALL, nullptr}
 PyMethodDef g_methods[] = {
     SPQT_METHOD(sparsify), SPQT_METHOD(sparse_gemv), SPQT_METHOD(sparsify_gemv), SPQT_METHOD(dense_gemv),
-    SPQT_METHOD(sparse_gemm_small), SPQT_METHOD(dense_gemm_small), SPQT_METHOD(kqw_gemv), SPQT_METHOD(pack),
+    SPQT_METHOD(sparse_gemm_small), SPQT_METHOD(dense_gemm_small), SPQT_METHOD(kqw_sparse_gemv), SPQT_METHOD(kqw_dense_gemv), SPQT_METHOD(pack),
     SPQT_METHOD(kqw_pack), SPQT_METHOD(host_step_launch),
     {"set_error", set_error, METH_O, nullptr},
     {nullptr, nullptr, 0, nullptr},

@@ -185,3 +185,15 @@ def test_two_level_products_at_chunk_part_and_cluster_edges(bits, m_blocks, n):
     assert torch.equal(y, again)
     y_ref, bound = oracle.kq_gemv(*parts, x)
     check_y(y_dense.cpu().numpy(), y_ref, bound, "dense")
+
+
+def test_two_level_sparse_product_refuses_a_missing_list():
+    p = binding.spqt_kqw_pack(dev(inputs.weights(256, 64, seed=3)), 4)
+    x, ws = dev(inputs.activations(64, seed=4)), binding.new_kq_workspace(p)
+    idx, cnt = binding.spqt_sparsify(x, 0.5)
+    before = binding.spqt_launch_count()
+    for product in (binding.spqt_kqw_sparse_gemv, binding.spqt_kq_sparse_gemv):
+        for i, c in ((None, None), (idx, None), (None, cnt)):
+            with pytest.raises(TypeError):
+                product(p, x, i, c, ws)
+    assert binding.spqt_launch_count() == before
