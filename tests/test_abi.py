@@ -142,3 +142,14 @@ def test_host_step_refuses_bad_arguments_without_touching_the_device(L):
     assert L.spqt_host_step_create(ctypes.c_void_p(16), 1, None) == 1
     assert L.spqt_host_step_launch(None, None) == 1
     assert L.spqt_host_step_destroy(None) == 1
+
+
+def test_the_tolerance_check_of_the_gpu_tests_refuses_not_a_number():
+    import numpy as np
+    from gpu_util import check_y
+    ref, bound = np.array([1.0, 2.0]), np.array([10.0, 10.0])
+    check_y(np.array([1.0, 2.0], dtype=np.float16), ref, bound)
+    for bad in (np.nan, np.inf):
+        with pytest.raises(AssertionError):
+            check_y(np.array([1.0, bad], dtype=np.float16), ref, bound)
+    check_y(np.array([1.0, np.nan], dtype=np.float16), np.array([1.0, np.inf]), np.array([10.0, np.inf]))
