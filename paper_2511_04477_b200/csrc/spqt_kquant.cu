@@ -495,7 +495,8 @@ kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* __restr
             for (unsigned q = 1; q < S; ++q) total += sm.xred[q - 1][tid];
     }
     if (T > 1) {
-        // the cluster that comes last to the block-row adds the clusters' sums in order, and leaves the counter at zero
+        // The cluster that comes last to the block-row adds the clusters' sums in order, and leaves the counter and the sums at
+        // zero: calls of another shape may have counters where this one has sums.
         float* const row_sums = partial + (size_t)r * T * kKqG;
         if (tid < kKqG) __stcg(row_sums + (cluster - r * T) * kKqG + tid, total);
         __threadfence();
@@ -510,6 +511,7 @@ kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* __restr
         if (tid < kKqG) {
             total = 0.0f;
             for (unsigned t = 0; t < T; ++t) total += __ldcg(row_sums + t * kKqG + tid);
+            for (unsigned t = 0; t < T; ++t) __stcg(row_sums + t * kKqG + tid, 0.0f);   // (a loop of its own: the loads go together)
         }
     }
     if (tid < kKqG) y[(size_t)r * kKqG + tid] = __float2half_rn(total);

@@ -197,3 +197,15 @@ def test_two_level_sparse_product_refuses_a_missing_list():
             with pytest.raises(TypeError):
                 product(p, x, i, c, ws)
     assert binding.spqt_launch_count() == before
+
+
+@pytest.mark.parametrize("bits,m_blocks,n", [(8, 1, 16384), (4, 3, 16421), (2, 4, 28672)])
+def test_two_level_products_leave_the_workspace_zero(bits, m_blocks, n):
+    """Several clusters of a block-row: their sums lie where a shape with more block-rows has its counters."""
+    p = binding.spqt_kqw_pack(dev(inputs.weights(256 * m_blocks, n, seed=n)), bits)
+    x, ws = dev(inputs.activations(n, seed=5)), binding.new_kq_workspace(p)
+    idx, cnt = binding.spqt_sparsify(x, 0.5)
+    for _ in range(2):
+        y, y_dense = binding.spqt_kqw_sparse_gemv(p, x, idx, cnt, ws), binding.spqt_kqw_dense_gemv(p, x, ws)
+        assert int(ws.count_nonzero()) == 0
+    assert torch.equal(y, binding.spqt_kqw_sparse_gemv(p, x, idx, cnt, ws)) and torch.equal(y_dense, binding.spqt_kqw_dense_gemv(p, x, ws))
