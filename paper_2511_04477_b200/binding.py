@@ -12,13 +12,13 @@ from __future__ import annotations
 import ctypes
 import importlib.util
 import os
+import sysconfig
 from dataclasses import dataclass
 
 import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libspqt.so")
-NATIVE_PATH = os.path.join(_HERE, "_native.so")
 
 EXPORTS = (
     "spqt_status_string", "spqt_version", "spqt_packed_sizes", "spqt_pack", "spqt_unpack",
@@ -107,14 +107,21 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+def native_path() -> str:
+    """Where the native marshalling for this Python and this PyTorch lies.  It uses both ABIs (of PyTorch internal functions
+    too), so the name carries the versions: after an upgrade it is missing, which says so, and not loaded by another one."""
+    return os.path.join(_HERE, "_native.%s.torch-%s.so" % (sysconfig.get_config_var("SOABI"), torch.__version__))
+
+
 def native():
     """The native marshalling of the per-token calls (``csrc/spqt_python.cpp``), loaded once."""
     global _native
     if _native is None:
         lib()
-        spec = importlib.util.spec_from_file_location(__package__ + "._native", NATIVE_PATH) if os.path.exists(NATIVE_PATH) else None
-        if spec is None:
-            raise RuntimeError("_native.so is missing: build it with `python -m paper_2511_04477_b200.build`")
+        path = native_path()
+        if not os.path.exists(path):
+            raise RuntimeError("%s is missing: build it with `python -m paper_2511_04477_b200.build`" % os.path.basename(path))
+        spec = importlib.util.spec_from_file_location(__package__ + "._native", path)
         module = importlib.util.module_from_spec(spec)
         spec.loader.exec_module(module)
         module.set_error(SpqtError)

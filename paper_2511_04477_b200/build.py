@@ -1,4 +1,4 @@
-"""Build the C-ABI library ``libspqt.so`` in-tree with nvcc for sm_100a, and ``_native.so``, the Python
+"""Build the C-ABI library ``libspqt.so`` in-tree with nvcc for sm_100a, and ``_native.<Python>.<PyTorch>.so``, the Python
 marshalling of its per-token calls (``csrc/spqt_python.cpp``), with g++ against PyTorch's headers.
 
     python -m paper_2511_04477_b200.build [--force] [--verbose]
@@ -16,7 +16,6 @@ import sys
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
 LIB_PATH = os.path.join(_HERE, "libspqt.so")
-NATIVE_PATH = os.path.join(_HERE, "_native.so")
 NATIVE_SOURCE = os.path.join(CSRC, "spqt_python.cpp")
 HEADER = os.path.join(os.path.dirname(_HERE), "include", "spqt.h")
 
@@ -47,7 +46,7 @@ def _run(cmd, tmp: str, target: str, verbose: bool) -> None:
     os.replace(tmp, target)
 
 
-def _build_native(verbose: bool) -> None:
+def _build_native(target: str, verbose: bool) -> None:
     import sysconfig
 
     import torch
@@ -57,14 +56,14 @@ def _build_native(verbose: bool) -> None:
     cuda = cpp_extension.CUDA_HOME or "/usr/local/cuda"
     includes = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
                 os.path.join(cuda, "include"), sysconfig.get_paths()["include"]]
-    tmp = NATIVE_PATH + ".%d.tmp" % os.getpid()
+    tmp = target + ".%d.tmp" % os.getpid()
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
            "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI)]
     for d in includes:
         cmd += ["-isystem", d]
     cmd += [NATIVE_SOURCE, "-o", tmp, "-L" + _HERE, "-l:libspqt.so", "-Wl,-rpath,$ORIGIN",
             "-L" + os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cuda", "-ltorch_cpu", "-lc10_cuda", "-lc10"]
-    _run(cmd, tmp, NATIVE_PATH, verbose)
+    _run(cmd, tmp, target, verbose)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -72,8 +71,11 @@ def build(force: bool = False, verbose: bool = False) -> str:
         tmp = LIB_PATH + ".%d.tmp" % os.getpid()
         _run([os.environ.get("NVCC", "nvcc")] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-o", tmp] + sources(),
              tmp, LIB_PATH, verbose)
-    if force or _stale(NATIVE_PATH, [NATIVE_SOURCE, HEADER]):
-        _build_native(verbose)
+    from .binding import native_path
+
+    native = native_path()
+    if force or _stale(native, [NATIVE_SOURCE, HEADER]):
+        _build_native(native, verbose)
     return LIB_PATH
 
 

@@ -153,3 +153,14 @@ def test_the_tolerance_check_of_the_gpu_tests_refuses_not_a_number():
         with pytest.raises(AssertionError):
             check_y(np.array([1.0, bad], dtype=np.float16), ref, bound)
     check_y(np.array([1.0, np.nan], dtype=np.float16), np.array([1.0, np.inf]), np.array([10.0, np.inf]))
+
+
+def test_the_native_marshalling_of_another_pytorch_is_not_loaded(L, monkeypatch):
+    built = binding.native_path()
+    assert os.path.exists(built)
+    monkeypatch.setattr(binding, "_native", None)
+    monkeypatch.setattr(binding.torch, "__version__", "0.0.0+none")
+    assert binding.native_path() != built
+    assert build._stale(binding.native_path(), [build.NATIVE_SOURCE, build.HEADER])
+    with pytest.raises(RuntimeError, match="build it"):
+        binding.native()
