@@ -1052,11 +1052,11 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
     }
     const int sms = sm_count();
     if (sms <= 0) return SPQT_ERR_CUDA;
-    // CTAs per block-row.  Up to about 35 block-rows: the largest cluster of which all fit with one CTA per SM (4096 x 4096,
-    // index collection inside: 6.35 / 5.57 / 4.99 / 4.61 us on 1 / 2 / 3 / 4 CTAs per block-row; 5.2 us on 7, two per SM).
-    // From there to 100: the largest with two per SM (5120 x 5120, given list: 6.25 / 5.08 / 4.72 / 4.31 us on 1 / 2 / 3 /
-    // 5; 8192 x 28672 dense 44.1 / 26.2 / 22.4 us on 1 / 2 / 4).  From 100 up one CTA per block-row: two would put two
-    // halves on the busiest SMs, which take as long as one whole and need an exchange (14336 x 4096: 6.5 against 7.3 us).
+    // CTAs per block-row: the largest cluster of which all are resident at once with one CTA per SM (4096 x 4096, index
+    // collection inside: 6.35 / 5.57 / 4.99 / 4.61 us on 1 / 2 / 3 / 4 CTAs per block-row; 5.2 us on 7, two per SM); where that
+    // is no cluster, or one of two and five or more fit with two CTAs per SM, the largest with two per SM (9728 x 4096 6.65 us
+    // on 1, 6.57 on 3; 6144 x 14336 10.8 on 2, 10.7 on 5); else one CTA (11776 x 4096 6.8 us, 7.4 on 2, 9.0 on 3).  A CTA has
+    // 512 columns of the matrix at least, 1024 where two share an SM (2304 x 1024 of 64-row groups, dense: 3.4 us on 4, 2.6 on 1).
     int S = 1;
     const int tuned = g_tune_ctas > 0 ? g_tune_ctas : tuned_ctas(f, MODE);
     int P = sms < kMaxPieceCtas ? sms : kMaxPieceCtas;   // CTAs of the pieces kernel
@@ -1069,29 +1069,51 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
             pieces = true;
             P = tuned < P ? tuned : P;
         }
-    } else if (f.R < 100) {
-        const bool spread = f.R <= max_clusters<G, BITS, MODE>(4, kAlone, true, sms, dev);
-        for (int k = 2; k <= kMaxSplit; ++k)
-            if (f.n >= 256 * k && f.R <= max_clusters<G, BITS, MODE>(k, spread ? kAlone : kSmem, spread, sms, dev)) S = k;
-    }
-    if (tuned <= 0 && S < least) {
-        // A whole block-row does not fit a CTA: a cluster with one slice per CTA if all are resident at once (14336 x 11008
-        // 14.5 against 16.2 us), otherwise pieces (12288 x 14589 3-bit 19.9 against 25 us with CTAs in two waves).
-        // (24-byte blocks: pieces; 6400 x 14336 took 18.8 us in clusters)
-        if (!(BITS == 3 && G == 64) && f.R <= max_clusters<G, BITS, MODE>(least, kSmem, false, sms, dev)) S = least;
-        else pieces = true;
-    }
-    // More block-rows than SMs: some SMs have two whole block-rows, the others one.  An even load instead pays for sharing
-    // block-rows (2 us) when the excess is small and x long.  Sparse, 50 %, whole against pieces: 20224 x 6615 13.8 / 13.75 us
-    // (at 28 % 17.6 / 16.8), x 8192 16.2 / 15.7; 22016 x 8192 16.3 / 16.3; 25600 x 8192 16.9 / 17.5; 20224 x 5120 11.3 / 12.5.
-    // The same goes for block-rows a little above a second wave of CTAs (64-row groups, 28672 x 8192 25.0 / 24.3).  24-byte
-    // blocks gain more (28672 x 8192 34.8 / 23.9, x 4096 20.0 / 15.6; 10624 x 8192 18.5 / 14.2, x 4096 9.4 / 10.2).  Dense (no list to build in every CTA): 22016 x
-    // 6144 17.7 / 16.2, x 4096 12.7 / 13.2, 28672 x 7168 22 / 22.5, x 16384 50 / 44.
-    if (tuned <= 0 && f.R > sms) {
-        const int excess = f.R - sms;
-        if (MODE == kModeDense) pieces = pieces || f.n >= 8192 || 64 * excess <= f.n - 4096;
-        else if (BITS == 3 && G == 64) pieces = pieces || f.n >= 6144 || (f.n >= 4096 && f.R > 2 * sms);
-        else if (f.n >= 6144) pieces = pieces || 170 * excess <= f.n - 4096 || (f.R > 2 * sms && f.R <= 3 * sms + sms / 4);
+    } else {
+        // "all resident" with a margin: the previous launch's CTAs leave SM by SM, and the CTAs of a cluster need places on
+        // neighbouring SMs at the same time, in odd numbers above all (7168 x 8192 on 5, of which the device holds 56: 11.1 us
+        // against 8.3 on 4 and 8.1 on 2; 11776 x 8192 on 3, of 93: 13.0 against 10.1 on 1; 4096 x 4096 on 4, of 33: no loss)
+        auto resident = [&](int k, bool per_sm) {
+            const int most = max_clusters<G, BITS, MODE>(k, per_sm ? kAlone : kSmem, per_sm, sms, dev);
+            return (k & (k - 1)) == 0 ? f.R < most : 25 * f.R <= 24 * most;
+        };
+        int one = 1, two = 1;            // CTAs per block-row with one and with two CTAs per SM
+        for (int k = 2; k <= kMaxSplit; ++k) {
+            if (f.n >= 512 * k && resident(k, true)) one = k;
+            if (k > 2 && f.n >= 1024 * k && resident(k, false)) two = k;
+        }
+        S = one == 1 || (one == 2 && two >= 5) ? two : one;
+        if (S < least) {
+            // A whole block-row does not fit a CTA: clusters of more, smaller slices if all are resident at once (14336 x 11008
+            // on 2 14.5 against 16.2 us), otherwise pieces (12288 x 14589 3-bit 19.9 against 25 us with CTAs in two waves).
+            if (two >= least) S = two;
+            else if (!(BITS == 3 && G == 64) && resident(least, false)) S = least;
+            else pieces = true;
+        }
+        // (24-byte blocks: pieces rather than clusters of no more than the least; 5120 x 20480 19.6 against 17.7 us)
+        if (BITS == 3 && G == 64 && least >= 3 && S <= least) pieces = true;
+        // One CTA per block-row: in the last round of block-rows some SMs have none, or one where they could run two.  Equal
+        // pieces of all block-rows pay for sharing block-rows instead (2 us): worth it where what those SMs could do meanwhile,
+        // in weights, is enough.  The lines are where the two times cross, between 149 and 640 block-rows and n = 2048 and
+        // 20480 (pieces against whole, us):
+        //   dense, 4 bits   66 to 77 M: 128-row groups 150 x 4096 11.9 / 12.6, 190 x 4096 14.1 / 13.3, 96 x 14336 19.7 / 21.0;
+        //                   64-row groups 224 x 8192 15.9 / 14.4, 224 x 16384 27.7 / 29.1
+        //   dense, 3 bits   36 to 51 M: 173 x 4096 14.3 / 15.5, 256 x 4096 18.3 / 16.7, 96 x 11008 17.6 / 20.2
+        //   sparse          4 bits 112 M (149 x 6144 12.3 / 12.7, 173 x 6144 13.2 / 12.8; nearer to it the list's length
+        //                   decides: 173 x 8192 at 25 % 18.6 / 21.4, at 65 % 13.0 / 12.9), 3 bits 96 M, 24-byte blocks 28 M
+        //                   (173 x 4096 9.6 / 9.9) and always from n = 6144 on
+        // Above two rounds whole block-rows run one after the other on few SMs: pieces from n = 2048 on (dense, 4 bits: 320 x 4096
+        // 18.4 / 22.3; 64-row groups from 4096), and from 3072 on for lists (300 x 4096 13.6 / 15.1; 64-row groups of 4 bits from
+        // 6144: 300 x 4096 12.0 / 12.4, but 12.9 / 11.6 with the list given).
+        if (S == 1 && !pieces) {
+            const long long idle = (long long)((sms - f.R % sms) % sms) * G * f.n;
+            if (MODE == kModeDense) {
+                pieces = idle >= (BITS == 4 ? 68000000ll : 42000000ll) || (BITS == 4 && f.R > 2 * sms && G * f.n >= 1 << 18);
+            } else if (f.R > sms) {
+                pieces = idle >= (BITS == 4 ? 112000000ll : G == 128 ? 96000000ll : 28000000ll) || (BITS == 3 && G == 64 && f.n >= 6144) ||
+                         (f.R > 2 * sms && f.n >= (BITS == 4 && G == 64 ? 6144 : 3072));
+            }
+        }
     }
     const unsigned long long warps = (unsigned long long)P * kPieceWarps;
     // a warp has parts of two block-rows at most, and the arithmetic is 32-bit

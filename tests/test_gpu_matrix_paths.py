@@ -209,3 +209,30 @@ def test_two_level_products_leave_the_workspace_zero(bits, m_blocks, n):
         y, y_dense = binding.spqt_kqw_sparse_gemv(p, x, idx, cnt, ws), binding.spqt_kqw_dense_gemv(p, x, ws)
         assert int(ws.count_nonzero()) == 0
     assert torch.equal(y, binding.spqt_kqw_sparse_gemv(p, x, idx, cnt, ws)) and torch.equal(y_dense, binding.spqt_kqw_dense_gemv(p, x, ws))
+
+
+@pytest.mark.parametrize("bits,group,m_blocks,n", [(4, 128, 92, 9505), (4, 64, 95, 20049), (3, 128, 90, 5665), (3, 64, 92, 11720), (4, 128, 301, 2048),
+                                                   (3, 64, 150, 4501), (3, 128, 298, 3072)])
+def test_pieces_where_the_last_round_of_block_rows_leaves_sms_idle(bits, group, m_blocks, n):
+    """Equal pieces with fewer block-rows than SMs (a block-row's sums come from up to three CTAs) and with little more than one
+    or two rounds of them; each just above its line."""
+    m = m_blocks * group
+    rng = np.random.Generator(np.random.PCG64(m + n))
+    sizes = binding.spqt_packed_sizes(m, n, bits, group)
+    codes = rng.integers(0, 256, sizes.codes_bytes, dtype=np.uint8)
+    pairs = np.stack([rng.uniform(0.001, 0.01, m_blocks * n), rng.uniform(-0.1, 0.0, m_blocks * n)], axis=1).astype(np.float16)
+    p = binding.Packed(dev(codes), dev(pairs.reshape(-1)), m, n, bits, group)
+    s, z = (np.ascontiguousarray(pairs[:, i]).reshape(m_blocks, n) for i in (0, 1))
+    x = growing_activations(n, seed=92)
+    ws = binding.new_workspace(m, n, bits, group)
+    t = inputs.threshold_for_sparsity(x, 0.4)
+    y, idx, cnt = binding.spqt_sparsify_gemv(p, dev(x), t, ws)
+    y_list = binding.spqt_sparse_gemv(p, dev(x), idx, cnt, ws)
+    y_dense = binding.spqt_dense_gemv(p, dev(x), ws)
+    again = binding.spqt_dense_gemv(p, dev(x), ws)
+    ref_idx, ref_cnt = oracle.sparsify(x, t)
+    assert int(cnt.item()) == ref_cnt and np.array_equal(idx.cpu().numpy()[:ref_cnt], ref_idx)
+    check_y(y.cpu().numpy(), *oracle.sparse_gemv(codes, s, z, m, n, x, ref_idx, bits, group), "list collected")
+    assert torch.equal(y, y_list) and torch.equal(y_dense, again)
+    check_y(y_dense.cpu().numpy(), *oracle.dense_gemv(codes, s, z, m, n, x, bits, group), "dense")
+    assert int(ws.count_nonzero()) == 0
