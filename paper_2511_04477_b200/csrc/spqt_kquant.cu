@@ -572,26 +572,33 @@ static spqt_status kq_launch_mode(const void* records, int R, int n, const void*
     }
     const int sms = sm_count();
     if (sms <= 0) return SPQT_ERR_CUDA;
-    // CTAs per block-row: the rule of the one-level format's kernel (the same structure).  With few block-rows of a long x
-    // several clusters of 4 CTAs of 16 warps, so that more SMs fetch, if that are half as many CTAs again (the sums of a
-    // block-row then meet in global memory, 1.5 us: dense 1024 x 28672 to 8 bits, 31 MB, took 21.0 us on 32 CTAs of 8 warps).
-    int S = 1, T = 1;
-    bool alone = false, wide = R >= 100 && R <= sms;
-    if (R < 100) {
-        alone = R <= kq_max_clusters<BITS, LIST, 8>(4, kAlone, true, sms, dev);
-        for (int k = 2; k <= kKqMaxCluster; ++k)
-            if (n >= 128 * k && R <= kq_max_clusters<BITS, LIST, 8>(k, alone ? kAlone : kSmem, alone, sms, dev)) S = k;
-        alone = alone || R <= kq_max_clusters<BITS, LIST, 8>(S, kAlone, true, sms, dev);
-        if (alone && n >= 1024 * S) {
-            wide = R <= kq_max_clusters<BITS, LIST, 16>(S, kSmem16, true, sms, dev);
-            int t = kq_max_clusters<BITS, LIST, 16>(4, kSmem16, true, sms, dev) / R;
-            t = t < n / 2048 ? t : n / 2048;
-            t = t < kKqMaxSplit ? t : kKqMaxSplit;
-            if (8 * t >= 3 * S) {
-                S = 4;
-                T = t;
-                wide = true;
-            }
+    // CTAs per block-row: the rule of the one-level format's kernel (launch_gemv: the same structure), with 128 columns to a CTA
+    // at least, 512 where two share an SM (to 4 bits: 7168 x 4096 is 20 % faster on 2 than on 5, of which the device holds 56
+    // clusters; 14336 x 1024 33 % on 2; 23552 x 1024 40 % on 1 than on 3, of 93).  With few block-rows of a long x several clusters
+    // of 4 CTAs of 16 warps, so that more SMs fetch, if that are half as many CTAs again (the sums of a block-row then meet in
+    // global memory, 1.5 us: dense 1024 x 28672 to 8 bits, 31 MB, 21.0 us on 32 CTAs of 8 warps, 12.0 on 128 of 16; at n = 8192
+    // clusters of 8 are 8 to 16 % faster, at 14336 8 to 22 % slower).
+    auto resident = [&](int k, bool per_sm) {
+        const int most = kq_max_clusters<BITS, LIST, 8>(k, per_sm ? kAlone : kSmem, per_sm, sms, dev);
+        return (k & (k - 1)) == 0 ? R < most : 25 * R <= 24 * most;
+    };
+    int one = 1, two = 1, T = 1;         // CTAs per block-row with one and with two CTAs per SM
+    for (int k = 2; k <= kKqMaxCluster; ++k) {
+        if (n >= 128 * k && resident(k, true)) one = k;
+        if (k > 2 && n >= 512 * k && resident(k, false)) two = k;
+    }
+    int S = one == 1 || (one == 2 && two >= 5) ? two : one;
+    const bool alone = S > 1 && R <= kq_max_clusters<BITS, LIST, 8>(S, kAlone, true, sms, dev);
+    bool wide = S == 1 && R <= sms;
+    if (alone && n >= 1024 * S) wide = R <= kq_max_clusters<BITS, LIST, 16>(S, kSmem16, true, sms, dev);
+    if (alone && n >= 12288) {
+        int t = kq_max_clusters<BITS, LIST, 16>(4, kSmem16, true, sms, dev) / R;
+        t = t < n / 1792 ? t : n / 1792;
+        t = t < kKqMaxSplit ? t : kKqMaxSplit;
+        if (8 * t >= 3 * S && t > 1) {
+            S = 4;
+            T = t;
+            wide = true;
         }
     }
     cudaLaunchConfig_t cfg = {};
