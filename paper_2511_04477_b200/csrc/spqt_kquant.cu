@@ -243,6 +243,31 @@ __device__ __forceinline__ void kq_multiply(float (*acc)[4], unsigned st, int la
     for (int i = 0; i < kGroups; ++i) {
         unsigned c[4], d[4], a[4];
         ldsm_x4_trans(addr + 32u * i, c);
+        if (BITS == 5) {
+            // The plane's words of block i, then i + 4: entries 2t and 2t + 1 (+ 8) the halves of a word, read once for both rows of
+            // the lane and rotated so that row 2g's bit lies above its nibble, at bit 4 or 8, and row 2g + 1's one place higher.
+            // The odd bytes go one place up as well, and their sums count twice (kq_unit).  28672 x 8192 dense 64.4 -> 55.9 us, at
+            // 50 % 36.6 -> 33.1 (bound by the integer pipe; a rotation and four shared loads for each row before).
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                unsigned u[4];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const unsigned e = st + (unsigned)((2 * t4 + 8 * h) * REC + 128 + 4 * i + 16 * j);
+                    const unsigned w0 = lds_u32(e), w1 = lds_u32(e + REC);
+                    u[2 * h] = kq_rotate(__byte_perm(w0, w1, 0x5410), 2 * g, 4 + 4 * j);
+                    u[2 * h + 1] = kq_rotate(__byte_perm(w0, w1, 0x7632), 2 * g, 4 + 4 * j);
+                }
+#pragma unroll
+                for (int o = 0; o < 2; ++o) {
+                    const unsigned nibble = 0x000f000fu << (4 * j + o), bit = 0x00100010u << (4 * j + o);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) a[q] = ((o ? c[q] >> 7 : c[q]) & nibble) | (u[q] & bit);
+                    product(i + 4 * j, o, a);
+                }
+            }
+            continue;
+        }
 #pragma unroll
         for (int q = 0; q < 4; ++q) d[q] = __byte_perm(c[q], 0u, 0x4341);   // the odd bytes
 #pragma unroll
@@ -269,14 +294,6 @@ __device__ __forceinline__ void kq_multiply(float (*acc)[4], unsigned st, int la
                         hl[q] = v & 0x00300030u;
                         hh[q] = v & 0x03000300u;
                     }
-                    if (BITS == 5) {
-                        // bit row of the blocks' words of entries 2t and 2t + 1 (+ 8): the halves of one word
-                        const unsigned e = st + (unsigned)((2 * t4 + 8 * (q >> 1)) * REC + 128 + 4 * i);
-                        const unsigned sel = (q & 1) ? 0x7632u : 0x5410u;
-                        const unsigned u0 = __byte_perm(lds_u32(e), lds_u32(e + REC), sel), u4 = __byte_perm(lds_u32(e + 16u), lds_u32(e + REC + 16u), sel);
-                        hl[q] = kq_rotate(u0, 2 * g + o, 4) & 0x00100010u;
-                        hh[q] = kq_rotate(u4, 2 * g + o, 8) & 0x01000100u;
-                    }
                 }
 #pragma unroll
                 for (int q = 0; q < 4; ++q) a[q] = (s[q] & 0x000f000fu) | hl[q];
@@ -288,9 +305,10 @@ __device__ __forceinline__ void kq_multiply(float (*acc)[4], unsigned st, int la
         }
     }
 }
-__host__ __device__ constexpr float kq_unit(int bits, int blk)
+// (o: of the row's place, see kq_multiply)
+__host__ __device__ constexpr float kq_unit(int bits, int blk, int o)
 {
-    return bits == 8 ? 1.0f : bits == 2 ? (blk < 2 ? 1.0f : blk < 4 ? 0.25f : blk < 6 ? 0.0625f : 0.015625f) : (blk < 4 ? 1.0f : 0.0625f);
+    return bits == 8 ? 1.0f : bits == 2 ? (blk < 2 ? 1.0f : blk < 4 ? 0.25f : blk < 6 ? 0.0625f : 0.015625f) : (blk < 4 ? 1.0f : 0.0625f) * (bits == 5 && o ? 0.5f : 1.0f);
 }
 
 // idx == nullptr: the dense product (the list is 0, 1, .., n-1 and count is n).
@@ -436,9 +454,11 @@ kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* __restr
         ldsm_x4_trans(b_base, bb);
 #pragma unroll
         for (int j = 0; j < 4; ++j) zl[j] += zn[j];
-        const bool over = prepare(stage0 + rn, xv[1]);
+        bool over = false;
+        if (BITS != 5) over = prepare(stage0 + rn, xv[1]);
         __syncwarp();                    // (B is in registers: its place is free)
         kq_multiply<BITS>(acc, stage0 + rc, lane, bb);
+        if (BITS == 5) over = prepare(stage0 + rn, xv[1]);   // (later: its results would not fit the registers beside the product)
         if (__any_sync(0xffffffffu, over)) rescale();
         leave();
         if (regain != 1.0f) {
@@ -461,7 +481,7 @@ kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* __restr
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int o = i & 1, half = i >> 1;
-                su.red[warp][32 * blk + 16 * half + 2 * g + o] = (acc[2 * blk + o][2 * half] + acc[2 * blk + o][2 * half + 1]) * (unit * kq_unit(BITS, blk));   // hi + lo
+                su.red[warp][32 * blk + 16 * half + 2 * g + o] = (acc[2 * blk + o][2 * half] + acc[2 * blk + o][2 * half + 1]) * (unit * kq_unit(BITS, blk, o));   // hi + lo
             }
         }
 #pragma unroll
