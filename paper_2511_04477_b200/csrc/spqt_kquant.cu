@@ -592,24 +592,25 @@ static spqt_status kq_launch_mode(const void* records, int R, int n, const void*
     }
     const int sms = sm_count();
     if (sms <= 0) return SPQT_ERR_CUDA;
-    // CTAs per block-row: the rule of the one-level format's kernel (launch_gemv: the same structure), with 128 columns to a CTA
-    // at least, 512 where two share an SM (to 4 bits: 7168 x 4096 is 20 % faster on 2 than on 5, of which the device holds 56
-    // clusters; 14336 x 1024 33 % on 2; 23552 x 1024 40 % on 1 than on 3, of 93).  With few block-rows of a long x several clusters
-    // of 4 CTAs of 16 warps, so that more SMs fetch, if that are half as many CTAs again (the sums of a block-row then meet in
-    // global memory, 1.5 us: dense 1024 x 28672 to 8 bits, 31 MB, 21.0 us on 32 CTAs of 8 warps, 12.0 on 128 of 16; at n = 8192
-    // clusters of 8 are 8 to 16 % faster, at 14336 8 to 22 % slower).
+    // CTAs per block-row: the largest cluster of which all are resident at once with one CTA per SM, or, if twice as many fit with
+    // two CTAs per SM, that one (to 4 bits at n = 8192: 9216 rows 7 instead of 3 10 % faster, 11264 rows 6 instead of 2 13 %); a
+    // CTA has 128 columns at least, 512 where two share an SM.  "Resident" leaves places for four more CTAs: the previous
+    // launch's leave SM by SM (7168 x 4096 on 5, of which the device holds just 56 clusters, 27 % slower than on 2; 23552 x
+    // 1024 on 3, of 93, 40 % slower than on 1).  One CTA has 16 warps if it has an SM to itself, from n = 2048 on (25600 x 1024 8 %
+    // faster with 8).  With few block-rows of a long x several clusters of 4 CTAs of 16 warps, so that more SMs fetch, if that are
+    // half as many CTAs again (the sums of a block-row then meet in global memory, 1.5 us: dense 1024 x 28672 to 8 bits, 31 MB,
+    // 21.0 us on 32 CTAs of 8 warps, 12.0 on 128 of 16; at n = 8192 clusters of 8 are 8 to 16 % faster, at 14336 8 to 22 % slower).
     auto resident = [&](int k, bool per_sm) {
-        const int most = kq_max_clusters<BITS, LIST, 8>(k, per_sm ? kAlone : kSmem, per_sm, sms, dev);
-        return (k & (k - 1)) == 0 ? R < most : 25 * R <= 24 * most;
+        return k * (kq_max_clusters<BITS, LIST, 8>(k, per_sm ? kAlone : kSmem, per_sm, sms, dev) - R) >= 4;
     };
     int one = 1, two = 1, T = 1;         // CTAs per block-row with one and with two CTAs per SM
     for (int k = 2; k <= kKqMaxCluster; ++k) {
         if (n >= 128 * k && resident(k, true)) one = k;
         if (k > 2 && n >= 512 * k && resident(k, false)) two = k;
     }
-    int S = one == 1 || (one == 2 && two >= 5) ? two : one;
+    int S = two >= 2 * one ? two : one;
     const bool alone = S > 1 && R <= kq_max_clusters<BITS, LIST, 8>(S, kAlone, true, sms, dev);
-    bool wide = S == 1 && R <= sms;
+    bool wide = S == 1 && R <= sms && n >= 2048;
     if (alone && n >= 1024 * S) wide = R <= kq_max_clusters<BITS, LIST, 16>(S, kSmem16, true, sms, dev);
     if (alone && n >= 12288) {
         int t = kq_max_clusters<BITS, LIST, 16>(4, kSmem16, true, sms, dev) / R;
