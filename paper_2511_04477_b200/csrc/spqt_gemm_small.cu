@@ -402,21 +402,6 @@ inline size_t small_workspace_bytes(const Format& f)
     return need < 65536 ? 65536 : need;
 }
 
-// CTAs per block-row.  All of them should be resident at once (two per SM): a second wave costs more than the idle slots
-// of a first one (28672 x 4096, 4 rows: 17.4 us on 224 CTAs, 23.6 on 448).  From R = 100 up the split that this leaves,
-// two, puts two half block-rows on the busiest SMs where one whole block-row runs as fast and needs no exchange
-// (14336 x 4096, 8 rows dense: 12.3 against 14.4 us).  Below, as many as fit: 4096 x 14336, 8 rows dense 33.9 / 20.1 /
-// 16.0 / 13.4 us on 1 / 2 / 4 / 8; 8192 x 28672, 4 rows dense 51.6 / 28.6 / 26.9 us on 1 / 2 / 4; but never less than
-// one chunk per warp.
-static int small_split(const Format& f, int sms)
-{
-    int S = f.R >= 100 ? 1 : (kSmallCtasPerSm * sms) / f.R;
-    const int most = (f.n + 255) / 256;
-    if (S > most) S = most;
-    if (S > kSmallMaxSplit) S = kSmallMaxSplit;
-    return S < 1 ? 1 : S;
-}
-
 // The records of the dense product when it cannot read X with 16-byte copies: REC values per column.
 template <int REC>
 __global__ void __launch_bounds__(256) gather_rows_kernel(const unsigned short* __restrict__ X, int ldx, int batch, int n, unsigned short* __restrict__ gathered)
@@ -453,6 +438,31 @@ static spqt_status launch_gather_rows(const __half* X, int ldx, int batch, int n
     return (err == cudaSuccess && cudaGetLastError() == cudaSuccess) ? SPQT_OK : SPQT_ERR_CUDA;
 }
 
+// How many clusters of k CTAs the device holds at once, two CTAs per SM (asked once per kernel, cluster size and device).
+template <int G, int BITS, int ROWS, bool DIRECT>
+static int small_max_clusters(int k, int smem, int sms, int dev)
+{
+    static int known[64][kSmallMaxSplit + 1] = {};
+    int& at_once = known[dev][k];
+    if (at_once == 0) {
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = k;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(k, kSmallCtasPerSm * sms);
+        cfg.blockDim = dim3(kSmallThreads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int can = 0;
+        if (cudaOccupancyMaxActiveClusters(&can, gemm_small_kernel<G, BITS, ROWS, DIRECT>, &cfg) != cudaSuccess) (void)cudaGetLastError();
+        at_once = can > 0 ? can : 1;
+    }
+    return at_once;
+}
+
 template <int G, int BITS, int ROWS, bool DIRECT>
 static spqt_status launch_small(const Format& f, SmallArgs a, cudaStream_t s)
 {
@@ -467,7 +477,19 @@ static spqt_status launch_small(const Format& f, SmallArgs a, cudaStream_t s)
     }
     const int sms = sm_count();
     if (sms <= 0) return SPQT_ERR_CUDA;
-    const int S = small_split(f, sms);
+    // CTAs per block-row.  All of them should be resident at once, two per SM: a second wave costs more than the idle slots of a
+    // first one (28672 x 4096, 4 rows: 17.4 us on 224 CTAs, 23.6 on 448).  So the largest number of which the device holds R
+    // clusters and one more: clusters of 5 to 8 leave SMs over (4608 x 8192, 8 rows, on 8, of which 33 fit, 26 % slower than on
+    // 7; 12288 x 2048 on 3, of 93, 46 % slower than on 1).  4096 x 14336, 8 rows dense 33.9 / 20.1 / 16.0 / 13.4 us on 1 / 2 /
+    // 4 / 8; 8192 x 28672, 4 rows dense 51.6 / 28.6 / 26.9 us on 1 / 2 / 4.  A CTA has one chunk per warp at least, two where
+    // there are more than 32 block-rows (6144 x 1024, 3 rows: 10 % faster on 1 than on 4).  From R = 100 up two put two half
+    // block-rows on the busiest SMs, where one whole block-row runs as fast and needs no exchange (14336 x 4096, 8 rows dense:
+    // 12.3 against 14.4 us), unless x is long (12800 x 14336, 8 rows 6 %, 64-row groups 6400 x 14336, 3 rows 16 % faster on 2).
+    int S = 1;
+    for (int k = 2; k <= kSmallMaxSplit; ++k) {
+        const int columns = f.R >= 100 ? 8192 : f.R > 32 ? 512 * k : 256 * (k - 1) + 1;
+        if (f.n >= columns && f.R < small_max_clusters<G, BITS, ROWS, DIRECT>(k, smem, sms, dev)) S = k;
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(S, f.R);
     cfg.blockDim = dim3(kSmallThreads);

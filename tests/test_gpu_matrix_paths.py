@@ -211,18 +211,38 @@ def test_two_level_products_leave_the_workspace_zero(bits, m_blocks, n):
     assert torch.equal(y, binding.spqt_kqw_sparse_gemv(p, x, idx, cnt, ws)) and torch.equal(y_dense, binding.spqt_kqw_dense_gemv(p, x, ws))
 
 
+def random_matrix(bits, group, m_blocks, n):
+    """Any bytes are a packed matrix: quick for large ones."""
+    rng = np.random.Generator(np.random.PCG64(m_blocks * group + n))
+    codes = rng.integers(0, 256, binding.spqt_packed_sizes(m_blocks * group, n, bits, group).codes_bytes, dtype=np.uint8)
+    pairs = np.stack([rng.uniform(0.001, 0.01, m_blocks * n), rng.uniform(-0.1, 0.0, m_blocks * n)], axis=1).astype(np.float16)
+    p = binding.Packed(dev(codes), dev(pairs.reshape(-1)), m_blocks * group, n, bits, group)
+    return (p, codes) + tuple(np.ascontiguousarray(pairs[:, i]).reshape(m_blocks, n) for i in (0, 1))
+
+
+@pytest.mark.parametrize("bits,group,m_blocks,n,batch", [(4, 64, 101, 8192, 3), (3, 128, 100, 8193, 8), (4, 128, 36, 4097, 5), (3, 64, 99, 1536, 4)])
+def test_small_batch_at_the_lines_between_cluster_sizes(bits, group, m_blocks, n, batch):
+    p, codes, s, z = random_matrix(bits, group, m_blocks, n)
+    X = np.stack([growing_activations(n, seed=93 + b) for b in range(batch)])
+    ws = binding.new_gemm_small_workspace(p)
+    t = inputs.threshold_for_sparsity(X[0], 0.4)
+    Y, idx, cnt = binding.spqt_sparse_gemm_small(p, dev(X), t, ws)
+    Yd = binding.spqt_dense_gemm_small(p, dev(X), ws)
+    ref_idx, ref_cnt = oracle.union_sparsify(X, t)
+    assert int(cnt.item()) == ref_cnt and np.array_equal(idx.cpu().numpy()[:ref_cnt], ref_idx)
+    Y_ref, bound = oracle.sparse_gemm_small(codes, s, z, p.m, n, X, ref_idx, bits, group)
+    for b in range(batch):
+        check_y(Y.cpu().numpy()[b], Y_ref[b], bound[b], "row %d" % b)
+        check_y(Yd.cpu().numpy()[b], *oracle.dense_gemv(codes, s, z, p.m, n, X[b], bits, group), "dense row %d" % b)
+
+
 @pytest.mark.parametrize("bits,group,m_blocks,n", [(4, 128, 92, 9505), (4, 64, 95, 20049), (3, 128, 90, 5665), (3, 64, 92, 11720), (4, 128, 301, 2048),
                                                    (3, 64, 150, 4501), (3, 128, 298, 3072)])
 def test_pieces_where_the_last_round_of_block_rows_leaves_sms_idle(bits, group, m_blocks, n):
     """Equal pieces with fewer block-rows than SMs (a block-row's sums come from up to three CTAs) and with little more than one
     or two rounds of them; each just above its line."""
-    m = m_blocks * group
-    rng = np.random.Generator(np.random.PCG64(m + n))
-    sizes = binding.spqt_packed_sizes(m, n, bits, group)
-    codes = rng.integers(0, 256, sizes.codes_bytes, dtype=np.uint8)
-    pairs = np.stack([rng.uniform(0.001, 0.01, m_blocks * n), rng.uniform(-0.1, 0.0, m_blocks * n)], axis=1).astype(np.float16)
-    p = binding.Packed(dev(codes), dev(pairs.reshape(-1)), m, n, bits, group)
-    s, z = (np.ascontiguousarray(pairs[:, i]).reshape(m_blocks, n) for i in (0, 1))
+    p, codes, s, z = random_matrix(bits, group, m_blocks, n)
+    m = p.m
     x = growing_activations(n, seed=92)
     ws = binding.new_workspace(m, n, bits, group)
     t = inputs.threshold_for_sparsity(x, 0.4)
