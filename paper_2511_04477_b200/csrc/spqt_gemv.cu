@@ -1032,10 +1032,11 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
     // (a given list counts its clusters with the size of the fused call: the same slices, the same sums)
     constexpr int kSlices = MODE == kModeList ? kModeFused : MODE;
     constexpr int kSmem = (int)sizeof(GemvSmem<G, BITS, kSlices, kCluster, 8>), kSmemPlain = (int)sizeof(GemvSmem<G, BITS, MODE, kPlain, 8>);
-    constexpr int kSmem16 = (int)sizeof(GemvSmem<G, BITS, MODE, kPlain, 16>), kSmemSlice16 = (int)sizeof(GemvSmem<G, BITS, MODE, kCluster, 16>);
+    constexpr int kWideSlice = BITS == 4 ? 16 : 8;   // warps of a slice's CTA where there are more than 8 (see wide_slices)
+    constexpr int kSmem16 = (int)sizeof(GemvSmem<G, BITS, MODE, kPlain, 16>), kSmemWideSlice = (int)sizeof(GemvSmem<G, BITS, MODE, kCluster, kWideSlice>);
     constexpr int kSmemPieces = (int)sizeof(PieceSmem<G, BITS, MODE>);
     static_assert(sizeof(GemvSmem<G, BITS, MODE, kCluster, 8>) <= kSmem && sizeof(GemvSmem<G, BITS, MODE, kSerial, 8>) <= kSmem && kSmem <= kAlone, "one size for all slices");
-    static_assert(kSmem <= 115712 && kSmemPlain <= 115712 && kSmem16 <= 232448 && kSmemSlice16 <= 232448 && kSmemPieces <= 232448, "two CTAs of 8 warps per SM, or one of 16");
+    static_assert(kSmem <= 115712 && kSmemPlain <= 115712 && kSmem16 <= 232448 && kSmemWideSlice <= 232448 && kSmemPieces <= 232448, "two CTAs of 8 warps per SM, or one of 16");
     static bool configured[64] = {};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return SPQT_ERR_CUDA;
@@ -1043,9 +1044,9 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
         if (cudaFuncSetAttribute(gemv_kernel<G, BITS, MODE, kPlain, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPlain) != cudaSuccess ||
             cudaFuncSetAttribute(gemv_kernel<G, BITS, MODE, kPlain, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem16) != cudaSuccess ||
             cudaFuncSetAttribute(gemv_kernel<G, BITS, MODE, kCluster, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAlone) != cudaSuccess ||
-            cudaFuncSetAttribute(gemv_kernel<G, BITS, MODE, kCluster, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemSlice16) != cudaSuccess ||
-            cudaFuncSetAttribute(gemv_kernel<G, BITS, MODE, kSerial, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemSlice16) != cudaSuccess ||
             cudaFuncSetAttribute(gemv_kernel<G, BITS, MODE, kSerial, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess ||
+            (kWideSlice > 8 && cudaFuncSetAttribute(gemv_kernel<G, BITS, MODE, kCluster, kWideSlice>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemWideSlice) != cudaSuccess) ||
+            (kWideSlice > 8 && cudaFuncSetAttribute(gemv_kernel<G, BITS, MODE, kSerial, kWideSlice>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemWideSlice) != cudaSuccess) ||
             cudaFuncSetAttribute(gemv_pieces_kernel<G, BITS, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPieces) != cudaSuccess)
             return SPQT_ERR_CUDA;
         configured[dev] = true;
@@ -1124,7 +1125,7 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
     const bool alone = !pieces && S > 1 && f.R <= max_clusters<G, BITS, MODE>(S, kAlone, true, sms, dev);
     // a long x: 16 warps, for the scan and for the loop (4096 x 14336 at 50 % 8.1 against 8.5 us, dense 7.7 against 8.6; 3072 x
     // 28672 11.5 against 13.0; at n = 4096 and for 3-bit codes no faster)
-    const bool wide_slices = alone && BITS == 4 && f.n >= 8192;
+    const bool wide_slices = alone && kWideSlice > 8 && f.n >= 8192;
     // whole block-rows on one CTA per SM: 16 warps (14336 x 4096 6.2 against 6.5 us, 18944 x 4096 6.4 against 7.0)
     const bool wide = !pieces && kind == kPlain && f.R <= sms;
     const bool cluster = !pieces && kind == kCluster;
@@ -1151,7 +1152,7 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
     ga.static_partition = g_static_partition;
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(pieces || wide || wide_slices ? 512 : 256);
-    cfg.dynamicSmemBytes = pieces ? kSmemPieces : wide_slices ? kSmemSlice16 : alone && cluster ? kAlone : wide ? kSmem16 : kind == kPlain ? kSmemPlain : kSmem;
+    cfg.dynamicSmemBytes = pieces ? kSmemPieces : wide_slices ? kSmemWideSlice : alone && cluster ? kAlone : wide ? kSmem16 : kind == kPlain ? kSmemPlain : kSmem;
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1166,8 +1167,8 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
     auto kernel = pieces             ? gemv_pieces_kernel<G, BITS, MODE>
                   : wide             ? gemv_kernel<G, BITS, MODE, kPlain, 16>
                   : kind == kPlain   ? gemv_kernel<G, BITS, MODE, kPlain, 8>
-                  : kind == kCluster ? (wide_slices ? gemv_kernel<G, BITS, MODE, kCluster, 16> : gemv_kernel<G, BITS, MODE, kCluster, 8>)
-                  : wide_slices      ? gemv_kernel<G, BITS, MODE, kSerial, 16>
+                  : kind == kCluster ? (wide_slices ? gemv_kernel<G, BITS, MODE, kCluster, kWideSlice> : gemv_kernel<G, BITS, MODE, kCluster, 8>)
+                  : wide_slices      ? gemv_kernel<G, BITS, MODE, kSerial, kWideSlice>
                                      : gemv_kernel<G, BITS, MODE, kSerial, 8>;
     const cudaError_t err = cudaLaunchKernelEx(&cfg, kernel, ga);
     count_launch();

@@ -1,5 +1,5 @@
 // Device-side building blocks of the kernels: PTX wrappers (cp.async, shared-memory accesses by 32-bit address,
-// thread-block-cluster primitives, mbarriers with bounded waits) and the packed-FMA dequantization arithmetic.
+// thread-block-cluster primitives, mbarriers with bounded waits, two fp32 operations per instruction).
 #pragma once
 
 namespace spqt {
@@ -111,19 +111,9 @@ __device__ __forceinline__ uint2 lds_v2(unsigned addr)
     asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr) : "memory");
     return v;
 }
-__device__ __forceinline__ unsigned long long lds_u64(unsigned addr)
-{
-    unsigned long long v;
-    asm volatile("ld.shared.u64 %0, [%1];" : "=l"(v) : "r"(addr) : "memory");
-    return v;
-}
 __device__ __forceinline__ void sts_u32(unsigned addr, unsigned v)
 {
     asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
-}
-__device__ __forceinline__ void sts_u64(unsigned addr, unsigned long long v)
-{
-    asm volatile("st.shared.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
 }
 __device__ __forceinline__ void sts_u16(unsigned addr, unsigned v)
 {
@@ -133,16 +123,6 @@ __device__ __forceinline__ void sts_v4(unsigned addr, const uint4& v)
 {
     asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
-// two packed multiplier pairs (four fp32 values) of one list entry
-__device__ __forceinline__ void lds_pairs(unsigned addr, unsigned long long& a, unsigned long long& b)
-{
-    asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "r"(addr) : "memory");
-}
-__device__ __forceinline__ void sts_pairs(unsigned addr, unsigned long long a, unsigned long long b)
-{
-    asm volatile("st.shared.v2.u64 [%0], {%1, %2};" ::"r"(addr), "l"(a), "l"(b) : "memory");
-}
-
 // ---- thread-block clusters
 __device__ __forceinline__ void cluster_arrive()
 {
@@ -188,34 +168,12 @@ __device__ __forceinline__ void ffma2(unsigned long long& d, unsigned long long 
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
 }
 
-// acc[0..3] (eight fp32 sums, two per register) += the eight codes of one 32-bit word, each
-// times a*2^-56.  Codes 0..3 are masked in place, codes 4..7 after a shift by 16, so that both
-// halves use the same two multiplier pairs m01 = a*(2^93, 2^89) and m23 = a*(2^85, 2^81).
-__device__ __forceinline__ void fma_word(unsigned long long* acc, unsigned w, unsigned long long m01,
-                                         unsigned long long m23)
-{
-    const unsigned v = w >> 16;
-    ffma2(acc[0], pack2(__uint_as_float(w & 0x0000000fu), __uint_as_float(w & 0x000000f0u)), m01);
-    ffma2(acc[1], pack2(__uint_as_float(w & 0x00000f00u), __uint_as_float(w & 0x0000f000u)), m23);
-    ffma2(acc[2], pack2(__uint_as_float(v & 0x0000000fu), __uint_as_float(v & 0x000000f0u)), m01);
-    ffma2(acc[3], pack2(__uint_as_float(v & 0x00000f00u), __uint_as_float(v & 0x0000f000u)), m23);
-}
-
 // d = a * b on both lanes
 __device__ __forceinline__ unsigned long long fmul2(unsigned long long a, unsigned long long b)
 {
     unsigned long long d;
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
-}
-
-// acc (16 fp32 sums in 8 registers) += the 16 codes of a lane's 8 bytes, each times a (scaled by
-// 2^-56), given the multiplier pairs m01 = a*(2^93, 2^89) and m23 = a*(2^85, 2^81).
-__device__ __forceinline__ void fma_block8(unsigned long long* acc, const uint2& w, unsigned long long m01,
-                                           unsigned long long m23)
-{
-    fma_word(acc + 0, w.x, m01, m23);
-    fma_word(acc + 4, w.y, m01, m23);
 }
 
 // a + b on both lanes

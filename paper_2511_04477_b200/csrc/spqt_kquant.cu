@@ -40,7 +40,8 @@ __host__ __device__ constexpr int kq_code_bytes(int bits) { return kKqG * bits /
 __host__ __device__ constexpr int kq_rec_bytes(int bits) { return kq_code_bytes(bits) + 16; }
 constexpr int kKqChunk = 16;        // list entries per chunk
 constexpr int kKqMaxCluster = 8;    // the largest portable cluster
-constexpr int kKqMaxSplit = 32;     // clusters of a block-row at most (the workspace's size)
+constexpr int kKqMaxSplit = 32;     // clusters of a block-row at most,
+constexpr int kKqMaxShared = 64;    // and of all block-rows that have more than one (the workspace's size; the device holds 33 of 4 CTAs)
 
 // ---------------------------------------------------------------- conversion
 //   per block i:      lo_i = min(min_j w_j, 0),  step_i = (max_j w_j - lo_i) / 15,  neg_i = 0 - lo_i
@@ -540,7 +541,7 @@ kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* __restr
 // ---------------------------------------------------------------- host side
 
 inline size_t kq_header_bytes(int R) { return (((size_t)R * 4 + 255) / 256) * 256; }
-inline size_t kq_workspace_bytes(int R) { return kq_header_bytes(R) + (size_t)R * kKqMaxSplit * (kKqG + 8) * sizeof(float); }
+inline size_t kq_workspace_bytes(int R) { return kq_header_bytes(R) + (size_t)kKqMaxShared * kKqG * sizeof(float); }
 
 static spqt_status kq_shape(int m, int n)
 {
@@ -616,6 +617,7 @@ static spqt_status kq_launch_mode(const void* records, int R, int n, const void*
         int t = kq_max_clusters<BITS, LIST, 16>(4, kSmem16, true, sms, dev) / R;
         t = t < n / 1792 ? t : n / 1792;
         t = t < kKqMaxSplit ? t : kKqMaxSplit;
+        t = t < kKqMaxShared / R ? t : kKqMaxShared / R;
         if (8 * t >= 3 * S && t > 1) {
             S = 4;
             T = t;
