@@ -1055,9 +1055,11 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
     if (sms <= 0) return SPQT_ERR_CUDA;
     // CTAs per block-row: the largest cluster of which all are resident at once with one CTA per SM (4096 x 4096, index
     // collection inside: 6.35 / 5.57 / 4.99 / 4.61 us on 1 / 2 / 3 / 4 CTAs per block-row; 5.2 us on 7, two per SM); where that
-    // is no cluster, or one of two and five or more fit with two CTAs per SM, the largest with two per SM (9728 x 4096 6.65 us
-    // on 1, 6.57 on 3; 6144 x 14336 10.8 on 2, 10.7 on 5); else one CTA (11776 x 4096 6.8 us, 7.4 on 2, 9.0 on 3).  A CTA has
-    // 512 columns of the matrix at least, 1024 where two share an SM (2304 x 1024 of 64-row groups, dense: 3.4 us on 4, 2.6 on 1).
+    // is no cluster, or one of two or three and twice as many, five or more, fit with two CTAs per SM, the largest with two per
+    // SM (9728 x 4096 6.65 us on 1, 6.57 on 3; 6144 x 14336 10.8 on 2, 10.7 on 5; three 5120 x 5120 with one list 19.2 on 3, 18.4
+    // on 6; but 8192 x 5120 with the list 6.3 on 4, 6.0 on 2); else one CTA (11776 x 4096 6.8 us, 7.4 on 2, 9.0 on 3).  A CTA has
+    // 512 columns of the matrix at least (5632 x 2560 with the list 4.7 us on 2, 4.0 on 5; 2304 x 1024 of 64-row groups, dense:
+    // 3.4 us on 4, 2.6 on 1), 768 in a cluster of more than five where two share an SM.
     int S = 1;
     const int tuned = g_tune_ctas > 0 ? g_tune_ctas : tuned_ctas(f, MODE);
     int P = sms < kMaxPieceCtas ? sms : kMaxPieceCtas;   // CTAs of the pieces kernel
@@ -1072,18 +1074,25 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
         }
     } else {
         // "all resident" with a margin: the previous launch's CTAs leave SM by SM, and the CTAs of a cluster need places on
-        // neighbouring SMs at the same time, in odd numbers above all (7168 x 8192 on 5, of which the device holds 56: 11.1 us
-        // against 8.3 on 4 and 8.1 on 2; 11776 x 8192 on 3, of 93: 13.0 against 10.1 on 1; 4096 x 4096 on 4, of 33: no loss)
+        // neighbouring SMs at the same time, in odd numbers above all, and the less there is to do the more (7168 x 8192 on 5, of
+        // which the device holds 56: 11.1 us against 8.3 on 4 and 8.1 on 2; 64-row groups 3328 x 8192 on 5 20 % slower than on 4,
+        // at 6656 x 8192 not; 11776 x 8192 on 3, of 93: 13.0 against 10.1 on 1; 4096 x 4096 on 4, of 33: no loss).  None where
+        // there is much to do (4608 x 28672 on 7 15.0 us, 16.0 on 6, dense 14.6 / 16.3; at n = 8192 on 7 up to 10 % slower).
         auto resident = [&](int k, bool per_sm) {
             const int most = max_clusters<G, BITS, MODE>(k, per_sm ? kAlone : kSmem, per_sm, sms, dev);
-            return (k & (k - 1)) == 0 ? f.R < most : 25 * f.R <= 24 * most;
+            const long long weights = (long long)G * f.n;   // of a block-row
+            if ((k & (k - 1)) == 0) return f.R < most;
+            if (!per_sm && weights >= 1300000) return f.R <= most;
+            return per_sm || weights >= 180000ll * k ? 25 * f.R <= 24 * most : 11 * f.R <= 10 * most;
         };
         int one = 1, two = 1;            // CTAs per block-row with one and with two CTAs per SM
         for (int k = 2; k <= kMaxSplit; ++k) {
             if (f.n >= 512 * k && resident(k, true)) one = k;
-            if (k > 2 && f.n >= 1024 * k && resident(k, false)) two = k;
+            if (k > 2 && f.n >= (k > 5 ? 768 : 512) * k && resident(k, false)) two = k;
         }
-        S = one == 1 || (one == 2 && two >= 5) ? two : one;
+        S = one == 1 || (one < 4 && two >= 5 && two >= 2 * one) ? two : one;
+        // 24-byte blocks of a list: one CTA rather than three with two per SM (4864 x 8192 at 50 % 9.3 / 10.8 us, list 8.4 / 9.9)
+        if (BITS == 3 && G == 64 && MODE != kModeDense && one == 1 && f.n >= 4096) S = 1;
         if (S < least) {
             // A whole block-row does not fit a CTA: clusters of more, smaller slices if all are resident at once (14336 x 11008
             // on 2 14.5 against 16.2 us), otherwise pieces (12288 x 14589 3-bit 19.9 against 25 us with CTAs in two waves).
@@ -1102,7 +1111,9 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
         //   dense, 3 bits   36 to 51 M: 173 x 4096 14.3 / 15.5, 256 x 4096 18.3 / 16.7, 96 x 11008 17.6 / 20.2
         //   sparse          4 bits 112 M (149 x 6144 12.3 / 12.7, 173 x 6144 13.2 / 12.8; nearer to it the list's length
         //                   decides: 173 x 8192 at 25 % 18.6 / 21.4, at 65 % 13.0 / 12.9), 3 bits 96 M, 24-byte blocks 28 M
-        //                   (173 x 4096 9.6 / 9.9) and always from n = 6144 on
+        //                   (173 x 4096 at 28 % 11.7 / 12.7, at 50 % 11.0 / 11.4) and always from n = 6144 on.  The line is that of
+        //                   the index-collecting call; a given list, cut the same way for the same sums, would have it at
+        //                   n = 6144 to 8192 (173 x 4096 at 50 % 10.0 / 8.5, 28 % 10.8 / 10.7; 173 x 8192 13.1 / 13.3, 14.8 / 17.6)
         // Above two rounds whole block-rows run one after the other on few SMs: pieces from n = 2048 on (dense, 4 bits: 320 x 4096
         // 18.4 / 22.3; 64-row groups from 4096), and from 3072 on for lists (300 x 4096 13.6 / 15.1; 64-row groups of 4 bits from
         // 6144: 300 x 4096 12.0 / 12.4, but 12.9 / 11.6 with the list given).

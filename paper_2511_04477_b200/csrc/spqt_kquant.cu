@@ -593,8 +593,9 @@ static spqt_status kq_launch_mode(const void* records, int R, int n, const void*
     }
     const int sms = sm_count();
     if (sms <= 0) return SPQT_ERR_CUDA;
-    // CTAs per block-row: the largest cluster of which all are resident at once with one CTA per SM, or, if twice as many fit with
-    // two CTAs per SM, that one (to 4 bits at n = 8192: 9216 rows 7 instead of 3 10 % faster, 11264 rows 6 instead of 2 13 %); a
+    // CTAs per block-row: the largest cluster of which all are resident at once with one CTA per SM, or, if more than twice as many
+    // fit with two CTAs per SM (or four instead of two), that one (at n = 8192 to 4 bits: 9216 rows 7 instead of 3 10 % faster,
+    // 11264 rows 6 instead of 2 13 %; to 6 bits 8192 rows dense 17.3 us on 4, 18.2 on 8); a
     // CTA has 128 columns at least, 512 where two share an SM.  "Resident" leaves places for four more CTAs: the previous
     // launch's leave SM by SM (7168 x 4096 on 5, of which the device holds just 56 clusters, 27 % slower than on 2; 23552 x
     // 1024 on 3, of 93, 40 % slower than on 1).  One CTA has 16 warps if it has an SM to itself, from n = 2048 on (25600 x 1024 8 %
@@ -609,7 +610,7 @@ static spqt_status kq_launch_mode(const void* records, int R, int n, const void*
         if (n >= 128 * k && resident(k, true)) one = k;
         if (k > 2 && n >= 512 * k && resident(k, false)) two = k;
     }
-    int S = two >= 2 * one ? two : one;
+    int S = two > 2 * one || (one < 3 && two >= 4) ? two : one;
     const bool alone = S > 1 && R <= kq_max_clusters<BITS, LIST, 8>(S, kAlone, true, sms, dev);
     bool wide = S == 1 && R <= sms && n >= 2048;
     if (alone && n >= 1024 * S) wide = R <= kq_max_clusters<BITS, LIST, 16>(S, kSmem16, true, sms, dev);
