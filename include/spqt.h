@@ -118,8 +118,9 @@ spqt_status spqt_sparsify(const void* x, int n, float t,
  *   y : fp16[m], 2-byte aligned.
  *   workspace : gemv_workspace_bytes of device memory, 16-byte aligned, zeroed
  *       ONCE by the caller before its first use; every call leaves it ready for
- *       the next.  (It holds the status word that checked mode sets; sums travel through
- *       shared memory.)  Two calls that may overlap on the GPU need two
+ *       the next.  It holds the status word that checked mode sets, and, for the shapes whose block-rows are cut into
+ *       pieces that several CTAs share, their arrival counters and partial sums, which every call leaves zero again.
+ *       (Elsewhere sums travel through shared memory.)  Two calls that may overlap on the GPU therefore need two
  *       workspaces.
  * Supported: bits 4 or 3 with group 64 or 128; n <= 65535 (column numbers travel as 16 bits).
  */
@@ -256,7 +257,9 @@ spqt_status spqt_host_step_destroy(void* step);
 
 /*
  * Tuning aid: number of CTAs the GEMV calls aim at (0 restores the built-in rule): divided by the
- * number of block-rows it gives the CTAs that share a block-row, 1 to 8.  `no_overlap` is a set of bits, 0 by
+ * number of block-rows it gives the CTAs that share a block-row, 1 to 8; a value below the number of block-rows cuts
+ * all of them, laid end to end, into equal pieces for that many CTAs (at most one per SM; at least one warp, a
+ * sixteenth of a CTA, per block-row, else whole block-rows as before).  `no_overlap` is a set of bits, 0 by
  * default: bit 0 launches the GEMV kernels strictly stream-ordered instead of letting a GEMV start
  * (and wait inside the kernel) while the previous kernel of the stream drains; bit 1 never launches
  * thread-block clusters (otherwise the 2..8 CTAs that share a block-row are one, and combine their sums
@@ -278,9 +281,16 @@ spqt_status spqt_set_tuning(int gemv_ctas, int no_overlap);
  * (a row's entries at or below the threshold in columns of the union are used with their values: the
  * block is read for the batch anyway, so this is never less accurate than thresholding row by row).
  * Every active block is fetched once for the whole batch.  The dense call is the same over all n
- * columns.  Dispatch rule: with one row use spqt_sparsify_gemv; with 2..8 rows the sparse call here
- * as long as the union keeps some sparsity (the union of B sets that are each 50 % sparse is
- * 1 - 2^-B dense), the dense call otherwise and for prompts; rows beyond 8 in further calls.
+ * columns.  Dispatch rule: with one row use spqt_sparsify_gemv; with 2..8 rows the sparse call here only where
+ * the matrix is large and the union (of B independent sets that are each 50 % sparse it is 1 - 2^-B dense) keeps
+ * enough sparsity; the dense call otherwise and for prompts; rows beyond 8 in further calls.  The union list is a
+ * launch of its own (2.5 to 4 us).  Measured, cold, list included, 4-bit codes with 128 rows per group (in brackets 3-bit
+ * with 64), 2, 4 and 8 rows alike: the sparse call is the faster one
+ *   28672 x 8192           from a union sparsity of 0.2 on (0.2)
+ *   28672 x 4096           from 0.4 on (0.4; 0.3 with 8 rows)
+ *   8192 x 28672           from 0.4 on (0.3)
+ *   14336 x 4096, 8192 x 8192   at 0.6 still 0.91 to 1.01 of the dense call's speed (from 0.5 on)
+ *   4096 x 4096, 4096 x 14336   at 0.6 0.61 to 0.94 (0.68 to 1.02)
  *   X : fp16 [batch][ldx], ldx >= n, 2-byte aligned.   Y : fp16 [batch][ldy], ldy >= m.
  *   idx : int32[n], count : int32, both on the device, written by the sparse call.
  *   workspace : spqt_gemm_small_workspace bytes, 16-byte aligned, zeroed ONCE by the caller; every call

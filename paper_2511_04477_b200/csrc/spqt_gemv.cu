@@ -29,7 +29,8 @@
 // the grid is large enough, so that one computes while the other starts or ends.  The kernel before this one (one
 // persistent CTA of 18 warps per SM, fractional block-rows, packed FMAs, partial sums as tagged words in global memory;
 // 4500 instructions of code against 1600) took 6.4 us there.  Large matrices: the code stream; 28672 x 8192 dense went
-// from 26.9 to 24.2 us, 8192 x 28672 dense from 29.2 to 22.3 us (5.6 TB/s, 0.86 of the measured copy bandwidth).
+// from 26.9 to 24.2 us, 8192 x 28672 dense from 29.0 to 25.6 us among other calls in a stream (4.9 TB/s, 0.74 of the measured
+// copy bandwidth; 22.3 us in short runs).
 #include <cstddef>
 
 #include "spqt_common.cuh"

@@ -56,7 +56,7 @@ __device__ __noinline__ void convert_column(const __half* __restrict__ col, int 
 // shared memory and leave in 16-byte pieces, neighbouring lanes to neighbouring places.
 //
 // Bound by memory: 28672 x 8192 to 4 bits, 595 MB.  With an IEEE division per weight (about 20 instructions) and one
-// column per warp or thread it took 344 us, now 128 us (4.65 TB/s); with all 128 rows of a group in one thread's
+// column per warp or thread it took 344 us, now 138 us (4.3 TB/s); with all 128 rows of a group in one thread's
 // registers (12 warps per SM) 161 us.
 template <int G, int BITS, int NC>
 __global__ void __launch_bounds__(kPackThreads, NC == 2 ? 5 : 6)
