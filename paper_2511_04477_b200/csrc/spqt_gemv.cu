@@ -1077,13 +1077,14 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
         // "all resident" with a margin: the previous launch's CTAs leave SM by SM, and the CTAs of a cluster need places on
         // neighbouring SMs at the same time, in odd numbers above all, and the less there is to do the more (7168 x 8192 on 5, of
         // which the device holds 56: 11.1 us against 8.3 on 4 and 8.1 on 2; 64-row groups 3328 x 8192 on 5 20 % slower than on 4,
-        // at 6656 x 8192 not; 11776 x 8192 on 3, of 93: 13.0 against 10.1 on 1; 4096 x 4096 on 4, of 33: no loss).  None where
-        // there is much to do (4608 x 28672 on 7 15.0 us, 16.0 on 6, dense 14.6 / 16.3; at n = 8192 on 7 up to 10 % slower).
+        // at 6656 x 8192 not; 11776 x 8192 on 3, of 93: 13.0 against 10.1 on 1; 4096 x 4096 on 4, of 33: no loss).  Less
+        // where there is much to do (4608 x 28672 on 7, of 37, 15.0 us, 16.0 on 6, dense 14.6 / 16.3; at n = 8192 on 7 up to 10 %
+        // slower; but 7168 x 14336 on 5, of 56, 16.0 us against 11.4 on 4, 11776 x 14336 on 3, of 93, 19.7 against 16.4 on 2).
         auto resident = [&](int k, bool per_sm) {
             const int most = max_clusters<G, BITS, MODE>(k, per_sm ? kAlone : kSmem, per_sm, sms, dev);
             const long long weights = (long long)G * f.n;   // of a block-row
             if ((k & (k - 1)) == 0) return f.R < most;
-            if (!per_sm && weights >= 1300000) return f.R <= most;
+            if (!per_sm && weights >= 1300000) return 50 * f.R <= 49 * most;
             return per_sm || weights >= 180000ll * k ? 25 * f.R <= 24 * most : 11 * f.R <= 10 * most;
         };
         int one = 1, two = 1;            // CTAs per block-row with one and with two CTAs per SM
@@ -1101,8 +1102,9 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
             else if (!(BITS == 3 && G == 64) && resident(least, false)) S = least;
             else pieces = true;
         }
-        // (24-byte blocks: pieces rather than clusters of no more than the least; 5120 x 20480 19.6 against 17.7 us)
-        if (BITS == 3 && G == 64 && least >= 3 && S <= least) pieces = true;
+        // (24-byte blocks: pieces rather than clusters of no more than the least, 5120 x 20480 19.6 against 17.7 us, unless
+        // these have an SM for each CTA: 2048 x 28672 on 4 13.1 against 16.4 us, list 9.7 against 11.2)
+        if (BITS == 3 && G == 64 && least >= 3 && (S < least || (S == least && !resident(least, true)))) pieces = true;
         // One CTA per block-row: in the last round of block-rows some SMs have none, or one where they could run two.  Equal
         // pieces of all block-rows pay for sharing block-rows instead (2 us): worth it where what those SMs could do meanwhile,
         // in weights, is enough.  The lines are where the two times cross, between 149 and 640 block-rows and n = 2048 and

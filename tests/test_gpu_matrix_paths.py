@@ -237,10 +237,11 @@ def test_small_batch_at_the_lines_between_cluster_sizes(bits, group, m_blocks, n
 
 
 @pytest.mark.parametrize("bits,group,m_blocks,n", [(4, 128, 92, 9505), (4, 64, 95, 20049), (3, 128, 90, 5665), (3, 64, 92, 11720), (4, 128, 301, 2048),
-                                                   (3, 64, 150, 4501), (3, 128, 298, 3072)])
+                                                   (3, 64, 150, 4501), (3, 128, 298, 3072), (3, 64, 32, 28672), (3, 64, 33, 22001), (4, 64, 36, 20485)])
 def test_pieces_where_the_last_round_of_block_rows_leaves_sms_idle(bits, group, m_blocks, n):
     """Equal pieces with fewer block-rows than SMs (a block-row's sums come from up to three CTAs) and with little more than one
-    or two rounds of them; each just above its line."""
+    or two rounds of them; each just above its line.  The last three: clusters of 24-byte blocks up to the least that a long
+    x needs, pieces one block-row further on, and an odd cluster that nearly fills the device."""
     p, codes, s, z = random_matrix(bits, group, m_blocks, n)
     m = p.m
     x = growing_activations(n, seed=92)
