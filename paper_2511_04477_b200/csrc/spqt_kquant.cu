@@ -541,7 +541,11 @@ kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* __restr
 // ---------------------------------------------------------------- host side
 
 inline size_t kq_header_bytes(int R) { return (((size_t)R * 4 + 255) / 256) * 256; }
-inline size_t kq_workspace_bytes(int R) { return kq_header_bytes(R) + (size_t)kKqMaxShared * kKqG * sizeof(float); }
+// (never more than a caller who kept the size of the earlier form, 33 KB per block-row, has)
+inline size_t kq_workspace_bytes(int R)
+{
+    return kq_header_bytes(R) + (size_t)(R == 1 ? kKqMaxSplit : kKqMaxShared) * kKqG * sizeof(float);
+}
 
 static spqt_status kq_shape(int m, int n)
 {

@@ -164,3 +164,10 @@ def test_the_native_marshalling_of_another_pytorch_is_not_loaded(L, monkeypatch)
     assert build._stale(binding.native_path(), [build.NATIVE_SOURCE, build.HEADER])
     with pytest.raises(RuntimeError, match="build it"):
         binding.native()
+
+
+@pytest.mark.parametrize("bits", [2, 4, 5, 6, 8])
+def test_a_two_level_workspace_of_the_earlier_size_is_still_enough(L, bits):
+    for block_rows in (1, 2, 3, 64, 65, 1000):
+        counters = -(-block_rows * 4 // 256) * 256
+        assert binding.spqt_kqw_packed_sizes(256 * block_rows, 64, bits)[1] <= counters + block_rows * 32 * 264 * 4

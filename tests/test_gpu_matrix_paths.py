@@ -199,7 +199,7 @@ def test_two_level_sparse_product_refuses_a_missing_list():
     assert binding.spqt_launch_count() == before
 
 
-@pytest.mark.parametrize("bits,m_blocks,n", [(8, 1, 16384), (4, 3, 16421), (2, 4, 28672)])
+@pytest.mark.parametrize("bits,m_blocks,n", [(8, 1, 16384), (4, 1, 60001), (4, 3, 16421), (2, 4, 28672)])
 def test_two_level_products_leave_the_workspace_zero(bits, m_blocks, n):
     """Several clusters of a block-row: their sums lie where a shape with more block-rows has its counters."""
     p = binding.spqt_kqw_pack(dev(inputs.weights(256 * m_blocks, n, seed=n)), bits)
