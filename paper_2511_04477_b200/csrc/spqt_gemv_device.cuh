@@ -25,6 +25,16 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar)
                  : "memory");
 }
 
+// one arrival that announces `bytes` of asynchronous stores
+__device__ __forceinline__ void mbar_expect(uint64_t* bar, unsigned bytes)
+{
+    asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n\t}" ::"r"(smem_u32(bar)), "r"(bytes)
+                 : "memory");
+}
+
+// a barrier that other CTAs of the cluster use: visible to those that wait for this CTA's next cluster arrival
+__device__ __forceinline__ void mbar_publish() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
+
 __device__ __forceinline__ unsigned long long global_ns()
 {
     unsigned long long t;
@@ -139,6 +149,12 @@ __device__ __forceinline__ unsigned cluster_map(unsigned smem_addr, unsigned ran
     unsigned r;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr), "r"(rank));
     return r;
+}
+// Two values into another CTA's shared memory, counted (8 bytes) by a barrier of that CTA: the receiver waits for the
+// data itself, the sender for nothing.
+__device__ __forceinline__ void st_async_f32x2(unsigned addr, float a, float b, unsigned bar)
+{
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(addr), "f"(a), "f"(b), "r"(bar) : "memory");
 }
 __device__ __forceinline__ void st_cluster_f32(unsigned addr, float v)
 {
