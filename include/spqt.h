@@ -119,7 +119,7 @@ spqt_status spqt_sparsify(const void* x, int n, float t,
  *   workspace : gemv_workspace_bytes of device memory, 16-byte aligned, zeroed
  *       ONCE by the caller before its first use; every call leaves it ready for
  *       the next.  It holds the status word that checked mode sets, and, for the shapes whose block-rows are cut into
- *       pieces that several CTAs share, their arrival counters and partial sums, which every call leaves zero again.
+ *       pieces that several CTAs share, the places where their sums meet, which every call leaves zero again.
  *       (Elsewhere sums travel through shared memory.)  Two calls that may overlap on the GPU therefore need two
  *       workspaces.
  * Supported: bits 4 or 3 with group 64 or 128; n <= 65535 (column numbers travel as 16 bits).
@@ -168,7 +168,7 @@ spqt_status spqt_dense_gemv(const void* codes, const void* scale_zero,
  *     that device current) and keeps it; make that first call before any stream capture begins, and
  *     from one host thread (the look-up is not guarded against two threads making it at once).
  *   - All calls on a device share the one array, which still holds the previous call's contents; the
- *     part that must start at zero (the status word and the words before it) is cleared on `stream`
+ *     part that must start at zero (the status word and the places where sums meet) is cleared on `stream`
  *     before the kernel, after every argument check has passed.  Two calls that may overlap on the GPU (different streams, no
  *     ordering) race on it: order them, or use spqt_sparse_gemv with separate workspaces.
  *   - Because the status word is cleared per call, it describes the last call only: read it with

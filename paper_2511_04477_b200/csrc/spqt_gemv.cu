@@ -132,6 +132,7 @@ struct GemvSmem {
 };
 
 constexpr int kPieceWarps = 16;
+constexpr unsigned kSlotMark = 0x53705174u;   // a slot that holds a sum (no status word of another shape's header looks like it)
 template <int G, int BITS, int MODE>
 struct PieceSmem {
     using Loop = PieceLoopSmem<G, BITS, MODE, kPieceWarps>;
@@ -141,7 +142,6 @@ struct PieceSmem {
     };
     alignas(16) unsigned char area[sizeof(Area)];
     alignas(16) unsigned short ent[MODE == kModeFused ? kMaxFusedN : 8];   // fused: the columns of the whole list
-    int last[2];                                      // whether this CTA came last to its first / last block-row
 };
 
 struct GemvArgs {
@@ -152,8 +152,8 @@ struct GemvArgs {
     unsigned magic_s;           // floor((2^32 - 1) / splits)
     unsigned warps, magic_w;    // pieces: warps of the grid, floor((2^32 - 1) / warps)
     unsigned magic_r, magic_p;  // the same of R and of the number of CTAs
-    unsigned* arrived;          // per block-row: CTAs that have left their sums (zero between calls)
-    float* partial;             // sums of the first and of the last block-row of every CTA's piece (zero between calls)
+    unsigned* status;           // the workspace's status word
+    unsigned long long* slots;  // pieces: G words between every two neighbouring CTAs (zero between calls)
     const __half* x;
     const int32_t* idx;
     const int32_t* count;
@@ -664,7 +664,7 @@ gemv_kernel(const GemvArgs a)
             return;
         }
         if (tid < G / 2) {
-            if (!mbar_wait(&sm.arrival, 0u)) atomicExch(a.arrived + a.R, 1u);   // (a wait that ran out: the status word)
+            if (!mbar_wait(&sm.arrival, 0u)) atomicExch(a.status, 1u);   // (a wait that ran out)
 #pragma unroll
             for (int q = 0; q < kMaxSplit - 1; ++q)
                 if (q < a.splits - 1) {
@@ -684,11 +684,11 @@ gemv_kernel(const GemvArgs a)
 
 // N warps, R block-rows laid end to end: warp W has [W*R/N, (W+1)*R/N), the fraction of a block-row being that fraction of
 // its list entries, in units of 8.  N >= R: a warp has part of one block-row, or the end of one and the start of the next.
-// The warps' sums meet in shared memory, added in warp order; a block-row that two or more CTAs
-// share is finished by the CTA that comes last, which adds their sums in CTA order (calls are bit-reproducible).
-// What bounds it at 28672 x 8192 and 50 % (18.3 us): 17000 cycles of loop at 7 TB/s, L2 hits among them, and 12000 cycles of
-// fixed cost: x and the masks 2000, the list 2200, the first chunks' arrival 3300, the sums and their exchange 4500.  That
-// is more than whole block-rows pay, so the host takes it only where those leave SMs idle or their list does not fit.
+// The warps' sums meet in shared memory, added in warp order; those of CTAs that share a block-row in the workspace (calls are
+// bit-reproducible).
+// What bounds it at 28672 x 8192 and 50 % (16.5 us; clock stamps): x, masks and list 2.4 us, then the code stream at 5.8 TB/s
+// until the CTAs end between 12.3 and 15.1 us (the memory does not serve all SMs alike), sums and exchange 1.4.  The exchange
+// as partial sums, a fence and a counter per block-row, and the slots fetched from a busy memory, took 3 us (17.65).
 template <int G, int BITS, int MODE>
 __global__ void __launch_bounds__(kPieceWarps * 32, 1)
 gemv_pieces_kernel(const GemvArgs a)
@@ -707,6 +707,9 @@ gemv_pieces_kernel(const GemvArgs a)
     const unsigned R = (unsigned)a.R, N = a.warps, cta = blockIdx.x;
 
     prefetch_inputs<MODE, kThreads>(a, tid);
+    // (a hint too: the slots between this CTA and the one before it, which the code stream of other calls has driven from L2; an
+    // exchange that had to fetch them from a busy memory took 1 to 2 us longer)
+    if (cta > 0u && tid < G / 16) asm volatile("prefetch.global.L2::evict_last [%0];" ::"l"(a.slots + (size_t)(cta - 1u) * G + 16 * tid));
     const typename MmaStage<G, BITS>::Lane ll(lane);
     const unsigned stage0 = smem_u32(&lp.stage[warp][0]);
     constexpr unsigned kStageBytes = (unsigned)sizeof(Stage<G, BITS, Ring>), kRing = D * kStageBytes;
@@ -838,63 +841,48 @@ gemv_pieces_kernel(const GemvArgs a)
     cp_async_wait<0>();
     __syncthreads();
 
-    // ---- block-rows that several warps share: G / 2 threads each, two rows a thread
-    const int j = tid % (G / 2), group = tid / (G / 2);
+    // ---- The warps' sums of a block-row, a thread per row of it, in warp order; then the CTAs' sums.
+    const int j = tid % G, group = tid / G, low = j % (G / 2);
     const unsigned W0 = cta * NW;
     const unsigned begin_row = magic_div(W0 * R, N, a.magic_w), end_row = magic_div((W0 + NW) * R + N - 1u, N, a.magic_w);
-    auto first_warp = [&](unsigned r) { return magic_div(r * N, R, a.magic_r); };               // of the grid's, with part of r
-    auto last_warp = [&](unsigned r) { return magic_div((r + 1u) * N + R - 1u, R, a.magic_r) - 1u; };
-    auto store_y = [&](unsigned r, float v0, float v1) {
-        a.y[(size_t)r * G + j] = __float2half_rn(v0);
-        a.y[(size_t)r * G + j + G / 2] = __float2half_rn(v1);
-    };
 #pragma unroll 1
-    for (unsigned r = begin_row + (unsigned)group; r < end_row; r += kThreads / (G / 2)) {
-        const unsigned fw = first_warp(r), lw = last_warp(r);
+    for (unsigned r = begin_row + (unsigned)group; r < end_row; r += kThreads / G) {
+        // warps fw .. lw of the grid have part of r: the first one as its last block-row, unless it begins there
+        const unsigned fw = magic_div(r * N, R, a.magic_r), lw = magic_div((r + 1u) * N + R - 1u, R, a.magic_r) - 1u;
+        const int w0 = (int)max(fw, W0) - (int)W0, w1 = (int)min(lw - W0, NW - 1u), second = fw * R < r * N ? (int)fw - (int)W0 : -1;
         float v0 = 0.0f, v1 = 0.0f, z = 0.0f;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) {
+            const int s = w == second ? 1 : 0;   // (loads without a condition, so that they go together)
+            const float2 cz = lp.red_z[s][w];
+            const float r0 = lp.red[s][w][low], r1 = lp.red[s][w][low + G / 2];
+            if (w >= w0 && w <= w1) {
+                v0 += r0 * cz.x;
+                v1 += r1 * cz.x;
+                z += cz.y;
+            }
+        }
+        v1 = (v1 - ((low & 1) ? v0 : 0.0f)) * 0.0625f;   // (see add_warps)
+        float v = (j < G / 2 ? v0 : v1) + z;
+        // CTAs c0 .. c1 share r: their sums are added along a tree over their numbers, whose node between CTAs b - 1 and b is
+        // slot b - 1 of the workspace.  Of the two that meet there the one that comes second takes the other's sum (a value and
+        // a mark in one word, exchanged: no fence, no counter, nobody waits) and goes on; the order of arrival decides who
+        // adds, not what is added.
+        const unsigned c0 = fw / NW, c1 = lw / NW;
+        bool mine = true;
 #pragma unroll 1
-        for (unsigned w = max(fw, W0); w <= min(lw, W0 + NW - 1u); ++w) {
-            const int s = w * R >= r * N ? 0 : 1;   // the first or the second block-row of warp w
-            const float2 cz = lp.red_z[s][w - W0];
-            v0 += lp.red[s][w - W0][j] * cz.x;
-            v1 += lp.red[s][w - W0][j + G / 2] * cz.x;
-            z += cz.y;
+        for (unsigned step = 1; mine && step <= c1 - c0; step *= 2) {
+            const unsigned node = ((cta - c0) / (2 * step) * 2 + 1) * step;   // first CTA of the right half, from c0
+            if (node > c1 - c0) continue;                                     // (there is none)
+            unsigned long long* const slot = a.slots + (size_t)(c0 + node - 1u) * G + j;
+            const unsigned long long other = atomicExch(slot, (unsigned long long)kSlotMark << 32 | __float_as_uint(v));
+            mine = (unsigned)(other >> 32) == kSlotMark;
+            if (mine) {
+                v += __uint_as_float((unsigned)other);
+                __stcg(slot, 0ull);
+            }
         }
-        v1 = (v1 - ((j & 1) ? v0 : 0.0f)) * 0.0625f;   // (see add_warps)
-        if (fw >= W0 && lw < W0 + NW) {
-            store_y(r, v0 + z, v1 + z);
-        } else {
-            float* const p = a.partial + (size_t)(2u * cta + (fw >= W0 ? 1u : 0u)) * G;
-            __stcg(p + j, v0 + z);
-            __stcg(p + j + G / 2, v1 + z);
-        }
-    }
-    // ---- block-rows that several CTAs share: the last one there adds the sums, and leaves zeros in the workspace
-    const unsigned edge[2] = {begin_row, end_row - 1u};
-    __threadfence();
-    __syncthreads();
-    if (tid < 2) {
-        const unsigned r = tid == 0 ? edge[0] : edge[1], c0 = first_warp(r) / NW, c1 = last_warp(r) / NW;
-        int is_last = 0;
-        if (c0 != c1 && (tid == 0 || edge[1] != edge[0])) {
-            is_last = atomicAdd(a.arrived + r, 1u) == c1 - c0 ? 1 : 0;
-            if (is_last) a.arrived[r] = 0u;
-        }
-        sm.last[tid] = is_last;
-    }
-    __syncthreads();
-    if (group < 2 && sm.last[group]) {
-        __threadfence();
-        const unsigned r = group == 0 ? edge[0] : edge[1], c0 = first_warp(r) / NW, c1 = last_warp(r) / NW;
-        float v0 = 0.0f, v1 = 0.0f;
-        for (unsigned c = c0; c <= c1; ++c) {
-            float* const p = a.partial + (size_t)(2u * c + (c == c0 ? 1u : 0u)) * G;
-            v0 += __ldcg(p + j);
-            v1 += __ldcg(p + j + G / 2);
-            __stcg(p + j, 0.0f);
-            __stcg(p + j + G / 2, 0.0f);
-        }
-        store_y(r, v0, v1);
+        if (mine) a.y[(size_t)r * G + j] = __float2half_rn(v);
     }
 }
 
@@ -1158,8 +1146,8 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
     ga.magic_w = 0xffffffffu / ga.warps;
     ga.magic_r = 0xffffffffu / (unsigned)f.R;
     ga.magic_p = 0xffffffffu / (unsigned)P;
-    ga.arrived = static_cast<unsigned*>(workspace);
-    ga.partial = reinterpret_cast<float*>(static_cast<unsigned char*>(workspace) + header_bytes(f.R));
+    ga.status = static_cast<unsigned*>(workspace) + f.R;
+    ga.slots = reinterpret_cast<unsigned long long*>(static_cast<unsigned char*>(workspace) + header_bytes(f.R));
     ga.x = static_cast<const __half*>(x);
     ga.idx = idx;
     ga.count = count;
@@ -1321,9 +1309,9 @@ spqt_status spqt_sparse_gemv_static(const void* codes, const void* scale_zero,
     st = check_gemv_args(codes, scale_zero, m, n, bits, group, x, idx, count, false, y, scratch, kStaticScratchBytes, &f);
     if (st != SPQT_OK) return st;
     if (n > kMaxListN) return SPQT_ERR_UNSUPPORTED;
-    // The scratch keeps whatever the previous call left: the status word must start at zero.
+    // The scratch keeps whatever the previous call left: the status word and the slots must start at zero.
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (cudaMemsetAsync(scratch, 0, header_bytes(f.R), s) != cudaSuccess) return SPQT_ERR_CUDA;
+    if (cudaMemsetAsync(scratch, 0, header_bytes(f.R) + slots_bytes(f.group), s) != cudaSuccess) return SPQT_ERR_CUDA;
     return sparse_checked(f, codes, scale_zero, x, idx, count, y, scratch, s);
 }
 

@@ -257,3 +257,18 @@ def test_pieces_where_the_last_round_of_block_rows_leaves_sms_idle(bits, group, 
     assert torch.equal(y, y_list) and torch.equal(y_dense, again)
     check_y(y_dense.cpu().numpy(), *oracle.dense_gemv(codes, s, z, m, n, x, bits, group), "dense")
     assert int(ws.count_nonzero()) == 0
+
+
+@pytest.mark.parametrize("word", [1, 2])
+def test_status_words_of_other_shapes_are_not_taken_for_sums(word):
+    """Shapes that share a workspace have their status words where this one has the places of its sums; the entry point on the
+    built-in scratch clears both."""
+    bits, group, m_blocks, n = 3, 64, 33, 22001   # pieces
+    p, _, _, _ = random_matrix(bits, group, m_blocks, n)
+    x = dev(growing_activations(n, seed=94))
+    idx, cnt = binding.spqt_sparsify(x, 0.5)
+    want = binding.spqt_sparse_gemv(p, x, idx, cnt, binding.new_workspace(p.m, n, bits, group))
+    ws = binding.new_workspace(p.m, n, bits, group)
+    ws.view(torch.int32)[64::7] = word
+    assert torch.equal(binding.spqt_sparse_gemv(p, x, idx, cnt, ws), want)
+    assert torch.equal(binding.spqt_sparse_gemv_static(p, x, idx, cnt, torch.empty_like(want)), want)
