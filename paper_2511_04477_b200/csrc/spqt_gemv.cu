@@ -361,12 +361,19 @@ __device__ __forceinline__ void add_warps(const Warp* warp, const float2* red_z,
 template <int NW>
 struct Scan {
     ScanSmem& sc;
+    const __half2 thr;
     int n, nv, lane, warp;
     int t[4];                                         // lane l: active entries of pieces 4l .. 4l+3
 
-    __device__ __forceinline__ Scan(unsigned char* area, int n_, int lane_, int warp_)
-        : sc(*reinterpret_cast<ScanSmem*>(area)), n(n_), nv((n_ + 255) >> 8), lane(lane_), warp(warp_)
+    __device__ __forceinline__ Scan(unsigned char* area, unsigned short thr_bits, int n_, int lane_, int warp_)
+        : sc(*reinterpret_cast<ScanSmem*>(area)), thr(__half2half2(__ushort_as_half(thr_bits))), n(n_), nv((n_ + 255) >> 8), lane(lane_), warp(warp_)
     {
+    }
+    // all ones in the halves of w whose magnitude exceeds the threshold: exact in fp16, never for a NaN
+    __device__ __forceinline__ unsigned active(unsigned w) const
+    {
+        w &= 0x7fff7fffu;
+        return __hgt2_mask(*reinterpret_cast<const __half2*>(&w), thr);
     }
     __device__ __forceinline__ int below(int li) const   // active entries before piece li
     {
@@ -375,56 +382,56 @@ struct Scan {
         for (int q = 0; q < 4; ++q) v += lane * 4 + q < li ? t[q] : 0;
         return (int)__reduce_add_sync(0xffffffffu, (unsigned)v);
     }
-    // x to shared memory, and per piece of 256 entries which ones are active and how many; returns the count
-    __device__ __forceinline__ int scan_x(const __half* x, unsigned short thr_bits)
+    // x to shared memory (entries that do not exist as not-a-number: never active), and per piece of 256 entries which ones are
+    // active and how many; returns the count.  A chain of latencies that every call pays, so x goes through registers (by way
+    // of shared memory with cp.async 0.1 us longer), the loads of a warp's first four pieces together, and nothing is done for
+    // pieces that are not there (0.08 us at n = 4096).
+    __device__ __forceinline__ int scan_x(const __half* x)
     {
         const int tid = warp * 32 + lane;
         const unsigned xs_base = smem_u32(sc.xs);
         const unsigned short* const xg = reinterpret_cast<const unsigned short*>(x);
+        const bool words = (reinterpret_cast<uintptr_t>(x) & 15) == 0;
         if (tid >= nv && tid < kMaxPieces) sc.tot[tid] = 0;
-        // a warp copies its own pieces (warp, warp + NW, ..)
-        if ((reinterpret_cast<uintptr_t>(x) & 15) == 0) {
-            for (int k = tid * 8; k < nv * 256; k += NW * 256) cp_async_16_left(xs_base + 2u * k, xg + k, n - k);
-        } else {
-            for (int k = warp * 256 + lane; k < nv * 256; k += ((k & 255) < 224) ? 32 : NW * 256 - 224)
-                sts_u16(xs_base + 2u * k, k < n ? (unsigned)__ldg(xg + k) : 0u);
-        }
-        cp_async_commit();
-        cp_async_wait<0>();
-        __syncwarp();
-        // eight entries per lane and piece, two per compare, exact in fp16; false for NaN.  Two pieces at a time.
-        const __half2 thr = __half2half2(__ushort_as_half(thr_bits));
-        auto count_piece = [&](int li, const uint4& v) {
-            const unsigned w[4] = {v.x, v.y, v.z, v.w};
-            unsigned m = 0;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const unsigned ab = w[j] & 0x7fff7fffu;
-                m |= __hgt2_mask(*reinterpret_cast<const __half2*>(&ab), thr) & (0x00020001u << (2 * j));
-            }
-            m = (m | (m >> 16)) & 0xffu;
-            const int left = n - li * 256 - lane * 8;   // entries past n do not exist
-            if (left < 8) m &= left <= 0 ? 0u : (1u << left) - 1u;
-            // how many precede this lane's: bit by bit of the counts
-            const unsigned c = (unsigned)__popc(m), lt = (1u << lane) - 1u;
-            unsigned before = 0;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) before += (unsigned)__popc(__ballot_sync(0xffffffffu, (c >> i) & 1u) & lt) << i;
-            sc.mask[li][lane] = (unsigned short)(m | (before << 8));
-            if (lane == 31) sc.tot[li] = (int)(before + c);
-        };
 #pragma unroll 1
-        for (int li = warp; li < nv; li += 2 * NW) {
-            const uint4 v0 = lds_v4(xs_base + li * 512u + lane * 16u);
-            const bool two = li + NW < nv;
-            const uint4 v1 = two ? lds_v4(xs_base + (li + NW) * 512u + lane * 16u) : v0;
-            count_piece(li, v0);
-            if (two) count_piece(li + NW, v1);
+        for (int l0 = warp; l0 < nv; l0 += 4 * NW) {
+            uint4 v[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int li = l0 + i * NW, k = li * 256 + lane * 8;
+                if (li >= nv) break;                  // (uniform, as is the next condition)
+                if (words && li * 256 + 256 <= n) {
+                    v[i] = __ldg(reinterpret_cast<const uint4*>(xg + k));
+                } else {
+                    unsigned w[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {     // (no load behind a condition: they go together)
+                        const unsigned e = __ldg(xg + min(k + 2 * j, n - 1)), o = __ldg(xg + min(k + 2 * j + 1, n - 1));
+                        w[j] = (k + 2 * j < n ? e : 0x7fffu) | (k + 2 * j + 1 < n ? o : 0x7fffu) << 16;
+                    }
+                    v[i] = make_uint4(w[0], w[1], w[2], w[3]);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int li = l0 + i * NW;
+                if (li >= nv) break;
+                sts_v4(xs_base + li * 512u + lane * 16u, v[i]);
+                unsigned m = (active(v[i].x) & 0x00020001u) | (active(v[i].y) & 0x00080004u) | (active(v[i].z) & 0x00200010u) | (active(v[i].w) & 0x00800040u);
+                m = (m | (m >> 16)) & 0xffu;
+                // how many precede this lane's: bit by bit of the counts
+                const unsigned c = (unsigned)__popc(m), lt = (1u << lane) - 1u;
+                unsigned before = 0;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) before += (unsigned)__popc(__ballot_sync(0xffffffffu, (c >> q) & 1u) & lt) << q;
+                sc.mask[li][lane] = (unsigned short)(m | (before << 8));
+                if (lane == 31) sc.tot[li] = (int)(before + c);
+            }
         }
         __syncthreads();
-        const int4 v = *reinterpret_cast<const int4*>(&sc.tot[lane * 4]);
-        t[0] = v.x; t[1] = v.y; t[2] = v.z; t[3] = v.w;
-        return (int)__reduce_add_sync(0xffffffffu, (unsigned)(v.x + v.y + v.z + v.w));
+        const int4 s = *reinterpret_cast<const int4*>(&sc.tot[lane * 4]);
+        t[0] = s.x; t[1] = s.y; t[2] = s.z; t[3] = s.w;
+        return (int)__reduce_add_sync(0xffffffffu, (unsigned)(s.x + s.y + s.z + s.w));
     }
     // the list position of column kb: the number of active entries below it (the same in all lanes)
     __device__ __forceinline__ int position(int kb) const
@@ -525,11 +532,11 @@ gemv_kernel(const GemvArgs a)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-    Scan<NW> scan(sm.area, n, lane, warp);            // (fused calls only)
+    Scan<NW> scan(sm.area, a.thr, n, lane, warp);            // (fused calls only)
     int count = n;
     if (LIST) count = __ldg(a.count);
     if (FUSED) {
-        count = scan.scan_x(a.x, a.thr);
+        count = scan.scan_x(a.x);
         if (blockIdx.x == 0 && tid == 0) *a.count_out = count;
     }
 
@@ -545,7 +552,7 @@ gemv_kernel(const GemvArgs a)
             hi = min(8 * (int)magic_div((part + 1u) * units, parts, a.magic_s), count);
         }
         if (FUSED) {
-            if (KIND == kSerial && part != first_part) scan.scan_x(a.x, a.thr);
+            if (KIND == kSerial && part != first_part) scan.scan_x(a.x);
             if (a.static_partition) {
                 // Ablation, the paper's "sparse without load balancing": a slice is a fixed range of the matrix COLUMNS,
                 // and so is every warp's part of it.
@@ -724,10 +731,10 @@ gemv_pieces_kernel(const GemvArgs a)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-    Scan<NW> scan(sm.area, n, lane, warp);            // (fused calls only)
+    Scan<NW> scan(sm.area, a.thr, n, lane, warp);            // (fused calls only)
     int count = n;
     if (LIST) count = __ldg(a.count);
-    if (FUSED) count = scan.scan_x(a.x, a.thr);
+    if (FUSED) count = scan.scan_x(a.x);
     const unsigned units = (unsigned)(count + 7) >> 3;
     int first = 8 * (int)magic_div(part0 * units, N, a.magic_w), end = 8 * (int)magic_div(part1 * units, N, a.magic_w);
     if (FUSED) {
