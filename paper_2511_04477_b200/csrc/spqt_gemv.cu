@@ -401,12 +401,12 @@ struct Scan {
                 const int li = l0 + i * NW, k = li * 256 + lane * 8;
                 if (li >= nv) break;                  // (uniform, as is the next condition)
                 if (words && li * 256 + 256 <= n) {
-                    v[i] = __ldg(reinterpret_cast<const uint4*>(xg + k));
+                    v[i] = ld_global_v4(xg + k);
                 } else {
                     unsigned w[4];
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {     // (no load behind a condition: they go together)
-                        const unsigned e = __ldg(xg + min(k + 2 * j, n - 1)), o = __ldg(xg + min(k + 2 * j + 1, n - 1));
+                        const unsigned e = ld_global_u16(xg + min(k + 2 * j, n - 1)), o = ld_global_u16(xg + min(k + 2 * j + 1, n - 1));
                         w[j] = (k + 2 * j < n ? e : 0x7fffu) | (k + 2 * j + 1 < n ? o : 0x7fffu) << 16;
                     }
                     v[i] = make_uint4(w[0], w[1], w[2], w[3]);

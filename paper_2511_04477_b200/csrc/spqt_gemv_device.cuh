@@ -96,6 +96,21 @@ __device__ __forceinline__ void cp_async_wait()
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
+// ---- loads of what an earlier kernel of the stream may have written: never moved before the wait for that kernel, as a
+// load that is declared read-only may be
+__device__ __forceinline__ uint4 ld_global_v4(const void* p)
+{
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ unsigned ld_global_u16(const void* p)
+{
+    unsigned short v;
+    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p) : "memory");
+    return v;
+}
+
 // ---- shared-memory accesses by 32-bit shared address
 __device__ __forceinline__ unsigned lds_u32(unsigned addr)
 {
