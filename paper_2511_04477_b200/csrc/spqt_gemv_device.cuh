@@ -165,11 +165,20 @@ __device__ __forceinline__ unsigned cluster_map(unsigned smem_addr, unsigned ran
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr), "r"(rank));
     return r;
 }
-// Two values into another CTA's shared memory, counted (8 bytes) by a barrier of that CTA: the receiver waits for the
-// data itself, the sender for nothing.
+// Values into another CTA's shared memory, their bytes counted by a barrier of that CTA: the receiver waits for the data itself,
+// the sender for nothing.
 __device__ __forceinline__ void st_async_f32x2(unsigned addr, float a, float b, unsigned bar)
 {
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(addr), "f"(a), "f"(b), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void st_async_f32x4(unsigned addr, const float4& v, unsigned bar)
+{
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void st_async_f32(unsigned addr, float v, unsigned bar)
+{
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(addr), "f"(v), "r"(bar) : "memory");
 }
 __device__ __forceinline__ void st_cluster_f32(unsigned addr, float v)
 {
