@@ -113,20 +113,25 @@ gemm_small_kernel(const SmallArgs a)
     const uint8_t* const xsrc = DIRECT ? a.x + 2 * ((size_t)min(lane >> 2, a.batch - 1) * a.ldx + 8 * (lane & 3)) : a.x + 2 * ROWS * lane;
     const unsigned xdst = kXOff + (DIRECT ? 16u : 2u * ROWS) * lane;
 
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-
+    const uint8_t* const row_codes = a.codes + (size_t)r * (size_t)n * B;
+    const unsigned* const row_meta = a.meta + (size_t)r * (size_t)n;
     // this warp's part [pos, end) of the CTA's slice; in units of 8 entries (DIRECT: 16-byte pieces of x)
     int pos, end;
-    {
-        const int count = (!DIRECT && a.idx) ? __ldg(a.count) : n;
+    auto take_part = [&](int count) {
         const int units = (count + 7) >> 3;
         const int lo = (int)(((long long)split * units) / S), hi = (int)(((long long)(split + 1) * units) / S);
         pos = 8 * (lo + ((hi - lo) * warp) / kSmallWarps);
         end = min(8 * (lo + ((hi - lo) * (warp + 1)) / kSmallWarps), count);
-    }
-    const uint8_t* const row_codes = a.codes + (size_t)r * (size_t)n * B;
-    const unsigned* const row_meta = a.meta + (size_t)r * (size_t)n;
+    };
+    // While the previous kernel drains (hints, see prefetch_l2): the pairs of the columns that the slice is about, and the first
+    // codes where there is no list.
+    take_part(n);
+    prefetch_l2(row_meta + pos, 4 * (size_t)max(end - pos, 0), lane, 32);
+    if (DIRECT || !a.idx) prefetch_l2(row_codes + (size_t)pos * B, (size_t)max(min(end - pos, (D - 1) * CH), 0) * B, lane, 32);
+
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (!DIRECT && a.idx) take_part(__ldg(a.count));
 
     float acc[SP][4][4];
     unsigned long long zl[ROWS / 2], scale[ROWS / 2];   // pairs of rows

@@ -111,6 +111,13 @@ __device__ __forceinline__ unsigned ld_global_u16(const void* p)
     return v;
 }
 
+// a hint: `bytes` bytes from p on towards L2, thread i of `step` taking every step-th line
+__device__ __forceinline__ void prefetch_l2(const void* p, size_t bytes, int i, int step)
+{
+    for (size_t off = (size_t)i * 128; off < bytes; off += (size_t)step * 128)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const char*>(p) + off));
+}
+
 // ---- shared-memory accesses by 32-bit shared address
 __device__ __forceinline__ unsigned lds_u32(unsigned addr)
 {

@@ -345,14 +345,21 @@ kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* __restr
     const uint8_t* const row = records + (size_t)r * (size_t)n * REC;
     const unsigned short* const xg = reinterpret_cast<const unsigned short*>(x);
 
+    // this warp's part of a list of `count` entries, in units of 8
+    int first, end;
+    auto take_part = [&](int count) {
+        const unsigned units = (unsigned)(count + 7) >> 3, parts = T * S * NW, part = ((cluster - r * T) * S + rank) * NW + (unsigned)warp;
+        first = 8 * (int)((unsigned long long)units * part / parts);
+        end = min(8 * (int)((unsigned long long)units * (part + 1u) / parts), count);
+    };
+    if (!LIST) {                         // (the first records towards L2 while the previous kernel drains: a hint, see prefetch_l2)
+        take_part(n);
+        prefetch_l2(row + (size_t)first * REC, (size_t)max(min(end - first, (D - 1) * CH), 0) * REC, lane, 32);
+    }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-    const int count = LIST ? __ldg(count_ptr) : n;
-    // this warp's part of the list, in units of 8 entries
-    const unsigned units = (unsigned)(count + 7) >> 3, parts = T * S * NW, part = ((cluster - r * T) * S + rank) * NW + (unsigned)warp;
-    const int first = 8 * (int)((unsigned long long)units * part / parts);
-    const int end = min(8 * (int)((unsigned long long)units * (part + 1u) / parts), count);
+    if (LIST) take_part(__ldg(count_ptr));
 
     constexpr int kAhead = 3;
     int coming[kAhead], ahead = first;   // list: the columns of the chunks the copies come to next
