@@ -145,6 +145,13 @@ def test_conversion_at_the_edges_of_tiles_and_alignments(bits, group, m_blocks, 
     assert np.array_equal(z.view(np.uint16).reshape(-1), ref_z.view(np.uint16).reshape(-1))
 
 
+@pytest.mark.parametrize("bits,group", FORMATS)
+@pytest.mark.parametrize("m_blocks,n,pad,shift", [(1, 1, 7, 0), (1, 8, 0, 0), (2, 31, 1, 8), (3, 33, 7, 0), (1, 64, 0, 8), (2, 65, 7, 0), (99, 997, 3, 0)])
+def test_conversion_in_tiles(bits, group, m_blocks, n, pad, shift):
+    """Rows of 16-byte pieces: ragged and odd widths, and more tiles than the persistent warps take at once."""
+    test_conversion_at_the_edges_of_tiles_and_alignments(bits, group, m_blocks, n, pad, shift)
+
+
 @pytest.mark.parametrize("bits", [2, 4, 5, 6, 8])
 @pytest.mark.parametrize("m_blocks,n,pad,shift", [(1, 1, 0, 0), (2, 64, 2, 0), (1, 66, 0, 0), (2, 130, 2, 1), (2, 129, 0, 0), (1, 31, 3, 0)])
 def test_two_level_conversion_at_the_edges_of_tiles_and_alignments(bits, m_blocks, n, pad, shift):
