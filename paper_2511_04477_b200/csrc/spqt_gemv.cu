@@ -697,9 +697,10 @@ gemv_kernel(const GemvArgs a)
 // its list entries, in units of 8.  N >= R: a warp has part of one block-row, or the end of one and the start of the next.
 // The warps' sums meet in shared memory, added in warp order; those of CTAs that share a block-row in the workspace (calls are
 // bit-reproducible).
-// What bounds it at 28672 x 8192 and 50 % (16.5 us; clock stamps): x, masks and list 2.4 us, then the code stream at 5.8 TB/s
-// until the CTAs end between 12.3 and 15.1 us (the memory does not serve all SMs alike), sums and exchange 1.4.  The exchange
-// as partial sums, a fence and a counter per block-row, and the slots fetched from a busy memory, took 3 us (17.65).
+// What bounds it at 28672 x 8192 and 50 % (15.8 us; clock stamps): x, masks and list 2.4 us, then the code stream at 5.8 TB/s
+// until the CTAs end between 11.6 and 13.9 us (the memory does not serve all SMs alike), sums and exchange 1.4.  The exchange
+// as partial sums, a fence and a counter per block-row, and the slots fetched from a busy memory, took 3 us (17.65).  Whole
+// warps instead of fractions of a block-row, with the list as words, x in them: 1 % less on average, 5 to 10 % more for 24-byte blocks.
 template <int G, int BITS, int MODE>
 __global__ void __launch_bounds__(kPieceWarps * 32, 1)
 gemv_pieces_kernel(const GemvArgs a)
@@ -1118,27 +1119,30 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
         // these have an SM for each CTA: 2048 x 28672 on 4 13.1 against 16.4 us, list 9.7 against 11.2)
         if (BITS == 3 && G == 64 && least >= 3 && (S < least || (S == least && !resident(least, true)))) pieces = true;
         // One CTA per block-row: in the last round of block-rows some SMs have none, or one where they could run two.  Equal
-        // pieces of all block-rows pay for sharing block-rows instead (2 us): worth it where what those SMs could do meanwhile,
-        // in weights, is enough.  The lines are where the two times cross, between 149 and 640 block-rows and n = 2048 and
-        // 20480 (pieces against whole, us):
-        //   dense, 4 bits   66 to 77 M: 128-row groups 150 x 4096 11.9 / 12.6, 190 x 4096 14.1 / 13.3, 96 x 14336 19.7 / 21.0;
-        //                   64-row groups 224 x 8192 15.9 / 14.4, 224 x 16384 27.7 / 29.1
-        //   dense, 3 bits   36 to 51 M: 173 x 4096 14.3 / 15.5, 256 x 4096 18.3 / 16.7, 96 x 11008 17.6 / 20.2
-        //   sparse          4 bits 112 M (149 x 6144 12.3 / 12.7, 173 x 6144 13.2 / 12.8; nearer to it the list's length
-        //                   decides: 173 x 8192 at 25 % 18.6 / 21.4, at 65 % 13.0 / 12.9), 3 bits 96 M, 24-byte blocks 28 M
-        //                   (173 x 4096 at 28 % 11.7 / 12.7, at 50 % 11.0 / 11.4) and always from n = 6144 on.  The line is that of
-        //                   the index-collecting call; a given list, cut the same way for the same sums, would have it at
-        //                   n = 6144 to 8192 (173 x 4096 at 50 % 10.0 / 8.5, 28 % 10.8 / 10.7; 173 x 8192 13.1 / 13.3, 14.8 / 17.6)
-        // Above two rounds whole block-rows run one after the other on few SMs: pieces from n = 2048 on (dense, 4 bits: 320 x 4096
-        // 18.4 / 22.3; 64-row groups from 4096), and from 3072 on for lists (300 x 4096 13.6 / 15.1; 64-row groups of 4 bits from
-        // 6144: 300 x 4096 12.0 / 12.4, but 12.9 / 11.6 with the list given).
+        // pieces of all block-rows pay for sharing block-rows instead (1 us): worth it where what those SMs could do meanwhile,
+        // in weights, is enough.  The lines are where the two times cross, between 100 and 448 block-rows and n = 2048 to 14336
+        // (pieces against whole, us; every size of the sweep in random matrices):
+        //   dense, 4 bits   38 to 50 M: 128-row groups 173 x 4096 11.7 / 13.1, 200 x 4096 12.5 / 13.2, 224 x 4096 13.6 / 13.4;
+        //                   64-row groups 200 x 8192 13.1 / 14.5, 224 x 8192 15.0 / 14.9, 256 x 14336 24.4 / 24.9
+        //   dense, 3 bits   128-row groups 32 to 40 M: 149 x 2048 7.9 / 8.3, 173 x 2048 8.6 / 8.4, 224 x 4096 14.8 / 15.1; 24-byte
+        //                   blocks 25 to 32 M: 173 x 4096 9.9 / 11.2, 200 x 4096 11.2 / 11.2
+        //   sparse, 4 bits  128-row groups 65 to 75 M: 149 x 4096 9.1 / 9.6, 173 x 4096 9.6 / 9.4, 224 x 8192 16.3 / 17.1; 64-row
+        //                   groups 50 to 65 M: 173 x 8192 12.0 / 12.1, 200 x 8192 12.8 / 12.5
+        //   sparse, 3 bits  128-row groups 50 to 65 M: 173 x 4096 10.9 / 11.2, 200 x 4096 11.8 / 11.3; 24-byte blocks 28 M (173 x
+        //                   4096 9.2 / 10.6) and always from n = 6144 on
+        // The lines are those of the index-collecting call; a given list is cut the same way for the same sums (it would have them
+        // at 10 % more or less, but 24-byte blocks at n = 6144 to 8192: 173 x 4096 8.3 / 8.1; and 64-row groups of 4 bits at less:
+        // 200 x 8192 11.2 / 11.8, 256 x 8192 13.1 / 15.3).  Above two rounds whole block-rows run one after the other on few SMs:
+        // pieces from n = 2048 on (4 bits dense 320 x 4096 17.3 / 21.0, sparse 320 x 2048 9.3 / 9.9, list 8.9 / 8.6; sparse 64-row
+        // groups of 4 bits from 4096: 320 x 4096 10.7 / 12.2, and 24-byte blocks dense: 448 x 4096 19.1 / 20.8).
         if (S == 1 && !pieces) {
             const long long idle = (long long)((sms - f.R % sms) % sms) * G * f.n;
+            const bool third = f.R > 2 * sms;
             if (MODE == kModeDense) {
-                pieces = idle >= (BITS == 4 ? 68000000ll : 42000000ll) || (BITS == 4 && f.R > 2 * sms && G * f.n >= 1 << 18);
+                pieces = idle >= (BITS == 4 ? 40000000ll : G == 128 ? 37000000ll : 30000000ll) || (third && (BITS == 4 ? G * f.n >= 1 << 17 : G == 64 && f.n >= 4096));
             } else if (f.R > sms) {
-                pieces = idle >= (BITS == 4 ? 112000000ll : G == 128 ? 96000000ll : 28000000ll) || (BITS == 3 && G == 64 && f.n >= 6144) ||
-                         (f.R > 2 * sms && f.n >= (BITS == 4 && G == 64 ? 6144 : 3072));
+                pieces = idle >= (BITS == 4 ? (G == 128 ? 70000000ll : 66000000ll) : G == 128 ? 60000000ll : 28000000ll) || (BITS == 3 && G == 64 && f.n >= 6144) ||
+                         (third && f.n >= (BITS == 4 && G == 64 ? 4096 : 2048));
             }
         }
     }
