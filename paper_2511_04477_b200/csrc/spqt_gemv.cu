@@ -1049,6 +1049,7 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
     constexpr int kWideSlice = BITS == 4 ? 16 : 8;   // warps of a slice's CTA where there are more than 8 (see wide_slices)
     constexpr int kSmem16 = (int)sizeof(GemvSmem<G, BITS, MODE, kPlain, 16>), kSmemWideSlice = (int)sizeof(GemvSmem<G, BITS, MODE, kCluster, kWideSlice>);
     constexpr int kSmemPieces = (int)sizeof(PieceSmem<G, BITS, MODE>);
+    constexpr int kDenseChunk = RowRing<G, MODE>::CH;
     static_assert(sizeof(GemvSmem<G, BITS, MODE, kCluster, 8>) <= kSmem && sizeof(GemvSmem<G, BITS, MODE, kSerial, 8>) <= kSmem && kSmem <= kAlone, "one size for all slices");
     static_assert(kSmem <= 115712 && kSmemPlain <= 115712 && kSmem16 <= 232448 && kSmemWideSlice <= 232448 && kSmemPieces <= 232448, "two CTAs of 8 warps per SM, or one of 16");
     static bool configured[64] = {};
@@ -1073,7 +1074,10 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
     // SM (9728 x 4096 6.65 us on 1, 6.57 on 3; 6144 x 14336 10.8 on 2, 10.7 on 5; three 5120 x 5120 with one list 19.2 on 3, 18.4
     // on 6; but 8192 x 5120 with the list 6.3 on 4, 6.0 on 2); else one CTA (11776 x 4096 6.8 us, 7.4 on 2, 9.0 on 3).  A CTA has
     // 512 columns of the matrix at least (5632 x 2560 with the list 4.7 us on 2, 4.0 on 5; 2304 x 1024 of 64-row groups, dense:
-    // 3.4 us on 4, 2.6 on 1), 768 in a cluster of more than five where two share an SM.
+    // 3.4 us on 4, 2.6 on 1), 768 in a cluster of more than five where two share an SM.  Without a list, whose length nobody knows
+    // here, a CTA has one chunk per warp at least (1024 x 1024 2.5 us on 2, 2.1 on 4), a block-row has no more CTAs than it takes for
+    // a warp's number of chunks (3072 x 4096 on 5 4.2, on 4 3.8), and 128-row groups go to four with two per SM where two with one
+    // fit (7168 x 4096 5.7 on 2, 5.15 on 4).
     int S = 1;
     const int tuned = g_tune_ctas > 0 ? g_tune_ctas : tuned_ctas(f, MODE);
     int P = sms < kMaxPieceCtas ? sms : kMaxPieceCtas;   // CTAs of the pieces kernel
@@ -1102,10 +1106,17 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
         };
         int one = 1, two = 1;            // CTAs per block-row with one and with two CTAs per SM
         for (int k = 2; k <= kMaxSplit; ++k) {
-            if (f.n >= 512 * k && resident(k, true)) one = k;
+            if (f.n >= (MODE == kModeDense ? 8 * kDenseChunk : 512) * k && resident(k, true)) one = k;
             if (k > 2 && f.n >= (k > 5 ? 768 : 512) * k && resident(k, false)) two = k;
         }
-        S = one == 1 || (one < 4 && two >= 5 && two >= 2 * one) ? two : one;
+        S = one == 1 || (one < 4 && two >= (MODE == kModeDense && G == 128 ? 4 : 5) && two >= 2 * one) ? two : one;
+        if (MODE == kModeDense) {
+            // no more CTAs than it takes for a warp's number of chunks
+            auto chunks = [&](int k) { const int columns = k * kDenseChunk * (kWideSlice > 8 && f.n >= 8192 && S == one ? 16 : 8); return (f.n + columns - 1) / columns; };
+            int k = 1;
+            while (chunks(k) > chunks(S)) ++k;
+            S = k;
+        }
         // 24-byte blocks of a list: one CTA rather than three with two per SM (4864 x 8192 at 50 % 9.3 / 10.8 us, list 8.4 / 9.9)
         if (BITS == 3 && G == 64 && MODE != kModeDense && one == 1 && f.n >= 4096) S = 1;
         if (S < least) {
