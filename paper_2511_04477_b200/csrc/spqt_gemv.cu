@@ -162,6 +162,7 @@ struct GemvArgs {
     int32_t* idx_out;
     int32_t* count_out;
     int static_partition;
+    int small;                  // the matrix is small beside L2
 };
 
 // floor(v / d) for any 32-bit v from the multiplier m = floor((2^32 - 1) / d): the high product is
@@ -520,15 +521,15 @@ gemv_kernel(const GemvArgs a)
     const uint8_t* const row_codes = a.codes + (size_t)r * (size_t)n * B;
     const unsigned* const row_meta = a.meta + (size_t)r * (size_t)n;
 
-    // The (scale, zero) pairs of this CTA's share of the block-row: every sector of them is needed, whichever entries are active
-    // (28672 x 8192 at 50 % 17.0 -> 16.55 us).  Without a list the first chunks of codes as well (4096 x 4096 4.13 -> 3.77 us).
+    // Hints to the weights of this warp's share of the block-row, to a few entries: the (scale, zero) pairs, of which every sector
+    // is needed, whichever entries are active (28672 x 8192 at 50 % 17.3 -> 16.8 us), and without a list the first chunks of codes
+    // (both: 4096 x 4096 4.13 -> 3.8 us).  Not for a large matrix without a list: L2 has lost many of the pairs by the time they are
+    // needed, and the codes gain nothing (8192 x 28672 25.9 against 25.5 us among other calls).
     {
         const int c0 = KIND == kCluster ? (int)((unsigned long long)n * rank / parts) : 0, c1 = KIND == kCluster ? (int)((unsigned long long)n * (rank + 1u) / parts) : n;
-        prefetch_l2(row_meta + c0, 4 * (size_t)(c1 - c0), tid, kThreads);
-        if (MODE == kModeDense) {
-            const int share = (c1 - c0 + NW - 1) / NW;   // of a warp, to a few entries
-            prefetch_l2(row_codes + (size_t)(c0 + min(share * warp, c1 - c0)) * B, (size_t)max(min(c1 - c0 - share * warp, min(share, (D - 1) * CH)), 0) * B, lane, 32);
-        }
+        const int each = (c1 - c0 + NW - 1) / NW, from = c0 + min(each * warp, c1 - c0), here = min(each, c1 - from);
+        if (MODE != kModeDense || a.small) prefetch_l2(row_meta + from, 4 * (size_t)here, lane, 32);
+        if (MODE == kModeDense && a.small) prefetch_l2(row_codes + (size_t)from * B, (size_t)min(here, (D - 1) * CH) * B, lane, 32);
     }
     // Programmatic dependent launch: this grid may have been started while the previous kernel of the stream was still
     // draining.  Nothing above touches memory another kernel writes; everything below waits for that kernel to
@@ -734,13 +735,10 @@ gemv_pieces_kernel(const GemvArgs a)
     const unsigned last_row = part1 > 0u ? row1 : row1 - 1u;
 
     {
-        // (the pairs of this CTA's piece, and without a list the first codes of this warp's: as in gemv_kernel)
-        const size_t all = (size_t)R * (size_t)n, w0 = all * (cta * NW) / N, w1 = all * (cta * NW + NW) / N;
-        prefetch_l2(a.meta + w0, 4 * (w1 - w0), tid, kThreads);
-        if (MODE == kModeDense) {
-            const size_t c0 = all * W / N, c1 = all * (W + 1u) / N;
-            prefetch_l2(a.codes + c0 * B, (c1 - c0 < (size_t)((D - 1) * CH) ? c1 - c0 : (size_t)((D - 1) * CH)) * B, lane, 32);
-        }
+        // (as in gemv_kernel; here large matrices gain from the codes too: 28672 x 8192 25.5 -> 25.3 us, 24-byte blocks 14336 x 8192 18.5 -> 18.2)
+        const size_t all = (size_t)R * (size_t)n, c0 = all * W / N, here = all * (W + 1u) / N - c0;
+        if (MODE != kModeDense || a.small) prefetch_l2(a.meta + c0, 4 * here, lane, 32);
+        if (MODE == kModeDense) prefetch_l2(a.codes + c0 * B, min(here, (size_t)((D - 1) * CH)) * B, lane, 32);
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -1191,6 +1189,7 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
     ga.idx_out = fa.idx_out;
     ga.count_out = fa.count_out;
     ga.static_partition = g_static_partition;
+    ga.small = f.blocks * (size_t)f.B <= size_t(64) << 20;
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(pieces || wide || wide_slices ? 512 : 256);
     cfg.dynamicSmemBytes = pieces ? kSmemPieces : wide_slices ? kSmemWideSlice : alone && cluster ? kAlone : wide ? kSmem16 : kind == kPlain ? kSmemPlain : kSmem;
