@@ -104,6 +104,12 @@ __device__ __forceinline__ uint4 ld_global_v4(const void* p)
     asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
     return v;
 }
+__device__ __forceinline__ unsigned ld_global_u32(const void* p)
+{
+    unsigned v;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
 __device__ __forceinline__ unsigned ld_global_u16(const void* p)
 {
     unsigned short v;
@@ -182,6 +188,10 @@ __device__ __forceinline__ void st_async_f32x4(unsigned addr, const float4& v, u
 {
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(bar)
                  : "memory");
+}
+__device__ __forceinline__ void st_async_u32(unsigned addr, unsigned v, unsigned bar)
+{
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.u32 [%0], %1, [%2];" ::"r"(addr), "r"(v), "r"(bar) : "memory");
 }
 __device__ __forceinline__ void st_async_f32(unsigned addr, float v, unsigned bar)
 {

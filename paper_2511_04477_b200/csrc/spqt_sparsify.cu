@@ -1,8 +1,7 @@
 // Sparse index collection: hidden state x and a threshold t -> the ascending
 // list of the entries with |x_k| > t and its length.  Three kernels:
-//   sparsify_cluster_kernel (one row, 6144 < n <= 65536): the compaction below spread over a thread-block
-//     cluster of 8 CTAs, warp totals exchanged through distributed shared memory (3.4 against 4.9 us at
-//     n = 14336; no gain at n = 4096, where the single CTA stays).
+//   sparsify_words_kernel (one row, n <= 65536): a lane looks after pairs of neighbouring entries; one CTA, whose warps' totals meet
+//     in shared memory, or above n = 2048 a cluster of 8 CTAs, whose warps send theirs to all of them.
 //   sparsify_kernel (one row, any n): each warp owns a contiguous segment of x, counts its active entries
 //     with __ballot_sync/__popc (the loads of eight groups of 32 entries in flight together), the 32 warp
 //     totals are scanned in shared memory, and each warp then writes its indices at its base offset.
@@ -10,6 +9,7 @@
 //     also gathers the rows' values of the listed columns.
 // The output order is ascending by construction (no atomics, no arrival order).
 #include "spqt_common.cuh"
+#include "spqt_gemv_device.cuh"
 
 namespace spqt {
 
@@ -19,6 +19,115 @@ __device__ __forceinline__ bool is_active(__half v, float t)
 {
     // exact widening; NaN compares false and is therefore never active
     return fabsf(__half2float(v)) > t;
+}
+
+constexpr int kClusterCtas = 8;
+constexpr int kClusterWarps = 8;
+
+// The totals of a cluster's warps, which every warp sends to every CTA's shared memory.  The CTA's barrier counts their bytes, so
+// that a warp waits for the data alone; cluster barriers before and after reading each other's tables took 0.7 to 0.9 us more.
+template <int WARPS>
+struct ClusterTotals {
+    int total[WARPS];
+    uint64_t arrival;
+
+    // by all threads, before the wait for the previous kernel
+    __device__ __forceinline__ void open()
+    {
+        if (threadIdx.x == 0) {
+            mbar_init(&arrival, 1);
+            mbar_expect(&arrival, WARPS * 4);
+            mbar_publish();
+        }
+        __syncwarp();
+        cluster_arrive();
+        cluster_wait();                  // every CTA of the cluster runs, and its barrier is ready
+    }
+    // by every warp `me` of the cluster: what the warps before it have, and all of them (none, if the wait ran out: the
+    // count is 0 then)
+    __device__ __forceinline__ void exchange(int me, int mine, int lane, int ctas, int& below, int& all)
+    {
+        if (lane < ctas) st_async_u32(cluster_map(smem_u32(&total[me]), (unsigned)lane), (unsigned)mine, cluster_map(smem_u32(&arrival), (unsigned)lane));
+        const bool there = mbar_wait(&arrival, 0u);
+        unsigned b = 0, a = 0;
+#pragma unroll
+        for (int w = 0; w < WARPS; w += 32) {
+            const unsigned c = there ? (unsigned)total[w + lane] : 0u;
+            a += c;
+            b += w + lane < me ? c : 0u;
+        }
+        below = (int)__reduce_add_sync(0xffffffffu, b);
+        all = (int)__reduce_add_sync(0xffffffffu, a);
+    }
+};
+
+// WORDS pairs of neighbouring entries per lane, two votes for 64 entries; every warp owns a segment of x.  One CTA of 32 warps (n <=
+// 2048), or a cluster of 8 CTAs of 8 warps (n <= 4096 * WORDS), which from there on is faster (4096 on one CTA 1.5 us, 8192 2.0).
+// `thr`: the largest fp16 value not above the threshold (negative: -1, not-a-number: infinity), so that the compare is exact in
+// fp16, and false for a NaN.  Bound by latencies: launch (0.8 us), one read of x, one exchange of totals.  n = 1024 1.8 -> 1.15 us,
+// 4096 2.3 -> 1.25, 8192 2.4 -> 1.3, 14336 2.7 -> 1.4, 28672 3.7 -> 1.5 (an entry per lane; one CTA with a scan of the totals between
+// two barriers up to 6144, then a cluster with cluster barriers before and after reading each other's totals).
+template <int WORDS, bool CLUSTER>
+__global__ void __launch_bounds__(CLUSTER ? kClusterWarps * 32 : kSparsifyThreads)
+sparsify_words_kernel(const __half* __restrict__ x, int n, unsigned short thr_bits, int32_t* __restrict__ idx, int32_t* __restrict__ count)
+{
+    __shared__ ClusterTotals<CLUSTER ? kClusterCtas * kClusterWarps : 32> totals;
+    const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);
+    unsigned rank = 0;
+    if (CLUSTER) {
+        asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+        totals.open();
+    }
+    const int me = CLUSTER ? (int)rank * kClusterWarps + warp : warp;
+    const int first = me * 64 * WORDS + 2 * lane;     // this lane's entries: first + 64*j and the next
+    const unsigned short* const xg = reinterpret_cast<const unsigned short*>(x);
+    const __half2 thr = __half2half2(__ushort_as_half(thr_bits));
+    const bool words = (reinterpret_cast<uintptr_t>(x) & 3) == 0;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    unsigned w[WORDS];
+    if (words && (me + 1) * 64 * WORDS <= n) {
+#pragma unroll
+        for (int j = 0; j < WORDS; ++j) w[j] = ld_global_u32(xg + first + 64 * j);
+    } else {
+#pragma unroll
+        for (int j = 0; j < WORDS; ++j) {   // (entries that do not exist: not-a-number, never active)
+            const int k = first + 64 * j;
+            w[j] = 0x7fff7fffu;
+            if (k - 2 * lane < n) {         // (uniform)
+                const unsigned e = ld_global_u16(xg + min(k, n - 1)), o = ld_global_u16(xg + min(k + 1, n - 1));
+                w[j] = (k < n ? e : 0x7fffu) | (k + 1 < n ? o : 0x7fffu) << 16;
+            }
+        }
+    }
+    unsigned even[WORDS], odd[WORDS];
+    int total = 0;
+#pragma unroll
+    for (int j = 0; j < WORDS; ++j) {
+        const unsigned ab = w[j] & 0x7fff7fffu, m = __hgt2_mask(*reinterpret_cast<const __half2*>(&ab), thr);
+        even[j] = __ballot_sync(0xffffffffu, (m & 1u) != 0u);
+        odd[j] = __ballot_sync(0xffffffffu, (m >> 31) != 0u);
+        total += __popc(even[j]) + __popc(odd[j]);
+    }
+    int base, all;
+    if (CLUSTER) {
+        totals.exchange(me, total, lane, kClusterCtas, base, all);
+        if (me == 0 && lane == 0) *count = all;
+    } else {
+        if (lane == 0) totals.total[warp] = total;
+        __syncthreads();
+        base = (int)__reduce_add_sync(0xffffffffu, lane < warp ? (unsigned)totals.total[lane] : 0u);
+        if (warp == 31 && lane == 0) *count = base + total;
+    }
+    const unsigned lt = (1u << lane) - 1u;
+#pragma unroll
+    for (int j = 0; j < WORDS; ++j) {
+        const unsigned e = (even[j] >> lane) & 1u, o = (odd[j] >> lane) & 1u;
+        const int at = base + __popc(even[j] & lt) + __popc(odd[j] & lt);
+        if (e != 0u) idx[at] = first + 64 * j;
+        if (o != 0u) idx[at + (int)e] = first + 64 * j + 1;
+        base += __popc(even[j]) + __popc(odd[j]);
+    }
 }
 
 __global__ void __launch_bounds__(kSparsifyThreads)
@@ -90,86 +199,12 @@ sparsify_kernel(const __half* __restrict__ x, int n, float t,
     }
 }
 
-// The same compaction spread over a thread-block cluster of 8 CTAs of 8 warps (n <= 65536): one SM's
-// instruction rate is what a single CTA spends most of its time on once n reaches several thousand.  The 64
-// warps own consecutive segments of x; every CTA leaves its warps' totals in its own shared memory, the
-// cluster synchronises, and each warp adds up the totals of the warps before it, reading the other CTAs'
-// tables through distributed shared memory.  A second cluster barrier keeps every CTA's table alive until
-// all have read it.  (Hardware barriers that every CTA reaches unconditionally: nothing to time out.)
-constexpr int kClusterCtas = 8;
-constexpr int kClusterWarps = 8;
-
-__global__ void __launch_bounds__(kClusterWarps * 32)
-sparsify_cluster_kernel(const __half* __restrict__ x, int n, float t, int32_t* __restrict__ idx, int32_t* __restrict__ count)
-{
-    __shared__ int warp_total[kClusterWarps];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned rank;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-    const int gw = (int)rank * kClusterWarps + warp;      // this warp among the cluster's 64
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    constexpr int kAll = kClusterCtas * kClusterWarps;
-    const int seg = ((n + kAll * 32 - 1) / (kAll * 32)) * 32;   // at most 1024 entries: 32 groups
-    const int begin = min(gw * seg, n), end = min(begin + seg, n);
-    const int groups = (end - begin + 31) >> 5;
-    unsigned flags = 0u;
-    int total = 0;
-    for (int g0 = 0; g0 < groups; g0 += 8) {
-        __half v[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-            if (g0 + j < groups) v[j] = x[min(begin + (g0 + j) * 32 + lane, n - 1)];   // (uniform condition)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            if (g0 + j < groups) {
-                const int k = begin + (g0 + j) * 32 + lane;
-                const bool p = (k < end) && is_active(v[j], t);
-                total += __popc(__ballot_sync(0xffffffffu, p));
-                if (p) flags |= 1u << (g0 + j);
-            }
-        }
-    }
-    if (lane == 0) warp_total[warp] = total;
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    // lane l looks up the totals of warps l and l + 32 of the cluster
-    int below = 0, all = 0;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int w = lane + 32 * h;
-        unsigned remote;
-        const unsigned local = static_cast<unsigned>(__cvta_generic_to_shared(&warp_total[w % kClusterWarps]));
-        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"((unsigned)(w / kClusterWarps)));
-        int v;
-        asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(remote) : "memory");
-        below += (w < gw) ? v : 0;
-        all += v;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        below += __shfl_xor_sync(0xffffffffu, below, o);
-        all += __shfl_xor_sync(0xffffffffu, all, o);
-    }
-    if (gw == 0 && lane == 0) *count = all;
-    int base = below;
-    for (int g = 0; g < groups; ++g) {
-        const bool p = (flags >> g) & 1u;
-        const unsigned mask = __ballot_sync(0xffffffffu, p);
-        if (p) idx[base + __popc(mask & ((1u << lane) - 1u))] = begin + g * 32 + lane;
-        base += __popc(mask);
-    }
-    // nobody leaves while another CTA may still be reading its table
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
 // "Active in at least one of `batch` rows" (n < 2^16): a thread-block cluster of 8 CTAs of 16 warps; every warp owns a
 // run of groups of 32 columns, lane l column l of each group.  Behind every index goes the record the product reads
 // instead of X: the rows' values of that column, REC of them (4 or 8; zero past the batch), so that X is gathered once
 // per call and not once per block-row.  Up to kKeepGroups groups per warp (n <= 16384) the values stay in registers
-// between the counting and the writing pass.  What bounds it is latency (launch, one round trip, two cluster
-// barriers), so the columns are spread over as many lanes as a cluster has: neighbouring lanes then write
+// between the counting and the writing pass.  What bounds it is latency (launch, one round trip, the
+// totals), so the columns are spread over as many lanes as a cluster has: neighbouring lanes then write
 // neighbouring list positions.  (8 columns per lane and scattered record stores took 5.0 us at n = 4096 and 4 rows.)
 constexpr int kRowsWarps = 16;
 constexpr int kKeepGroups = 4;
@@ -179,15 +214,16 @@ __global__ void __launch_bounds__(kRowsWarps * 32)
 sparsify_rows_kernel(const unsigned short* __restrict__ X, int ldx, int batch, int n, float t,
                      int32_t* __restrict__ idx, int32_t* __restrict__ count, unsigned short* __restrict__ gathered)
 {
-    __shared__ int warp_total[kRowsWarps];
+    __shared__ ClusterTotals<kClusterCtas * kRowsWarps> totals;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned rank, nctas;
+    unsigned rank;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(nctas));
+    constexpr int nctas = kClusterCtas;
+    totals.open();
     // |x| > t as integers: magnitude bits above those of the largest fp16 value not above t (-1 if t < 0: everything is;
     // infinity if t is NaN or +inf: nothing is), and not a NaN
     const int thr = (t != t) ? 0x7c00 : (t < 0.0f ? -1 : (int)__half_as_ushort(__float2half_rd(t)));
-    const int groups = (n + (int)nctas * kRowsWarps * 32 - 1) / ((int)nctas * kRowsWarps * 32);
+    const int groups = (n + nctas * kRowsWarps * 32 - 1) / (nctas * kRowsWarps * 32);
     const int first = ((int)rank * kRowsWarps + warp) * groups * 32 + lane;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -214,26 +250,9 @@ sparsify_rows_kernel(const unsigned short* __restrict__ X, int ldx, int batch, i
 #pragma unroll
         for (int j = 0; j < kKeepGroups; ++j) total += __popc(__ballot_sync(0xffffffffu, active(g0, j)));
     }
-    if (lane == 0) warp_total[warp] = total;
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    // lane l adds up the totals of warps l, l + 32, .. of the cluster
-    int below = 0, all = 0;
     const int me = (int)rank * kRowsWarps + warp;
-#pragma unroll 4
-    for (int w = lane; w < (int)nctas * kRowsWarps; w += 32) {
-        unsigned remote;
-        const unsigned local = static_cast<unsigned>(__cvta_generic_to_shared(&warp_total[w % kRowsWarps]));
-        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"((unsigned)(w / kRowsWarps)));
-        int c;
-        asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(c) : "r"(remote) : "memory");
-        below += (w < me) ? c : 0;
-        all += c;
-    }
-    int base = __reduce_add_sync(0xffffffffu, below);
-    all = __reduce_add_sync(0xffffffffu, all);
-    // nobody leaves while another CTA may still be reading its table: arrive now, wait at the end
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    int base, all;
+    totals.exchange(me, total, lane, nctas, base, all);
     if (me == 0 && lane == 0) *count = all;
     for (int g0 = 0; g0 < groups; g0 += kKeepGroups) {
         if (groups > kKeepGroups) load(g0);
@@ -253,7 +272,6 @@ sparsify_rows_kernel(const unsigned short* __restrict__ X, int ldx, int batch, i
             base += __popc(mask);
         }
     }
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // One launch of sparsify_rows_kernel: the columns that are active in at least one of `batch` rows (n < 2^16), and
@@ -289,27 +307,34 @@ extern "C" spqt_status spqt_sparsify(const void* x, int n, float t,
     using namespace spqt;
     if (n < 0 || !count || (n > 0 && (!x || !idx))) return SPQT_ERR_INVALID_ARG;
     if (!aligned(x, 2) || !aligned(idx, 4) || !aligned(count, 4)) return SPQT_ERR_ALIGNMENT;
-    // from a few thousand entries on, the compaction spread over a cluster of 8 CTAs (falls back to the
-    // single CTA below if the cluster cannot be launched)
-    if (n > 6144 && n <= 65536) {
+    if (n > 0 && n <= 65536) {
+        static constexpr void (*spread[10])(const __half*, int, unsigned short, int32_t*, int32_t*) = {
+            sparsify_words_kernel<1, true>, sparsify_words_kernel<2, true>, sparsify_words_kernel<3, true>, sparsify_words_kernel<4, true>,
+            sparsify_words_kernel<5, true>, sparsify_words_kernel<6, true>, sparsify_words_kernel<7, true>, sparsify_words_kernel<8, true>,
+            sparsify_words_kernel<12, true>, sparsify_words_kernel<16, true>};
+        const bool cluster = n > 2048;
+        const int words = (n + 4095) / 4096;
         cudaLaunchConfig_t cc = {};
-        cc.gridDim = dim3(kClusterCtas);
-        cc.blockDim = dim3(kClusterWarps * 32);
+        cc.gridDim = dim3(cluster ? kClusterCtas : 1);
+        cc.blockDim = dim3(cluster ? kClusterWarps * 32 : kSparsifyThreads);
         cc.stream = static_cast<cudaStream_t>(stream);
         cudaLaunchAttribute ca[2];
-        ca[0].id = cudaLaunchAttributeClusterDimension;
-        ca[0].val.clusterDim.x = kClusterCtas;
-        ca[0].val.clusterDim.y = 1;
-        ca[0].val.clusterDim.z = 1;
-        ca[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        ca[1].val.programmaticStreamSerializationAllowed = 1;
-        cc.attrs = ca;
-        cc.numAttrs = g_no_pdl ? 1 : 2;
-        if (cudaLaunchKernelEx(&cc, sparsify_cluster_kernel, static_cast<const __half*>(x), n, t, idx, count) == cudaSuccess) {
+        ca[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        ca[0].val.programmaticStreamSerializationAllowed = 1;
+        ca[1].id = cudaLaunchAttributeClusterDimension;
+        ca[1].val.clusterDim.x = kClusterCtas;
+        ca[1].val.clusterDim.y = 1;
+        ca[1].val.clusterDim.z = 1;
+        cc.attrs = g_no_pdl ? ca + 1 : ca;
+        cc.numAttrs = (g_no_pdl ? 0 : 1) + (cluster ? 1 : 0);
+        auto kernel = !cluster ? sparsify_words_kernel<1, false> : spread[words <= 8 ? words - 1 : words <= 12 ? 8 : 9];
+        const unsigned short thr = t != t ? 0x7c00 : t < 0.0f ? 0xbc00 : __half_as_ushort(__float2half_rd(t));
+        const cudaError_t err = cudaLaunchKernelEx(&cc, kernel, static_cast<const __half*>(x), n, thr, idx, count);
+        if (err == cudaSuccess || !cluster) {
             count_launch();
-            return cudaGetLastError() == cudaSuccess ? SPQT_OK : SPQT_ERR_CUDA;
+            return (err == cudaSuccess && cudaGetLastError() == cudaSuccess) ? SPQT_OK : SPQT_ERR_CUDA;
         }
-        (void)cudaGetLastError();
+        (void)cudaGetLastError();         // (the cluster cannot be launched: the single CTA below)
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(1);

@@ -279,3 +279,21 @@ def test_status_words_of_other_shapes_are_not_taken_for_sums(word):
     ws.view(torch.int32)[64::7] = word
     assert torch.equal(binding.spqt_sparse_gemv(p, x, idx, cnt, ws), want)
     assert torch.equal(binding.spqt_sparse_gemv_static(p, x, idx, cnt, torch.empty_like(want)), want)
+
+
+@pytest.mark.parametrize("n", [1, 63, 64, 65, 2047, 2048, 2049, 4096, 4097, 8192, 16385, 32768, 32769, 49152, 49153, 65535, 65536, 65537])
+def test_index_collection_at_word_and_cluster_edges(n):
+    """One CTA, a cluster with 1 to 16 words per lane, and beyond; x on an odd boundary too; entries and thresholds that are
+    extreme, infinite or no numbers."""
+    x = inputs.activations(n, seed=n)
+    rng = np.random.Generator(np.random.PCG64(n))
+    for value in (np.nan, np.inf, -np.inf, -0.0, 6e-8, 65504.0, -0.5):
+        x[rng.integers(0, n, max(1, n // 50))] = value
+    for shift in (0, 1):
+        buf = torch.full((n + shift + 8,), float("inf"), dtype=torch.float16, device="cuda")   # (active, if it were read)
+        xd = buf[shift:shift + n]
+        xd.copy_(dev(x))
+        for t in (0.5, 0.0, -0.0, -1.0, 3e-8, 0.4999, 65504.0, 1e6, float("inf"), float("nan")):
+            idx, cnt = binding.spqt_sparsify(xd, t)
+            ref_idx, ref_cnt = oracle.sparsify(x, t)
+            assert int(cnt.item()) == ref_cnt and np.array_equal(idx.cpu().numpy()[:ref_cnt], ref_idx), (shift, t)
