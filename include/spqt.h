@@ -219,8 +219,9 @@ spqt_status spqt_sparse_linear_host_async(const void* codes, const void* scale_z
 
 /*
  * A token step recorded once and replayed: the host-buffer linears of a step (each described like the
- * arguments of spqt_sparse_linear_host_async: same meaning and alignment of every field) are captured,
- * in order, into one CUDA graph -- the transfer of every x from its x_host (all of them at the head of the
+ * arguments of spqt_sparse_linear_host_async: same meaning and alignment of every field) are captured
+ * into one CUDA graph (in order where one writes a buffer that another uses; otherwise in branches that may run
+ * at the same time) -- the transfer of every x from its x_host (all of them at the head of the
  * step), per linear the launch that collects the indices and multiplies, and the way y reaches y_host -- so
  * that a step costs the host one launch call.
  *   spqt_host_step_create  : builds the graph (allocates host-side CUDA objects; not a hot-path call;

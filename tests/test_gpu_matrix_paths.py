@@ -297,3 +297,31 @@ def test_index_collection_at_word_and_cluster_edges(n):
             idx, cnt = binding.spqt_sparsify(xd, t)
             ref_idx, ref_cnt = oracle.sparsify(x, t)
             assert int(cnt.item()) == ref_cnt and np.array_equal(idx.cpu().numpy()[:ref_cnt], ref_idx), (shift, t)
+
+
+@pytest.mark.parametrize("shared", [False, True])
+def test_recorded_step_in_branches(shared):
+    """More linears than a step has branches, of all formats, one with a list of its own launch; with buffers in common the
+    linears keep their order."""
+    sizes = [(4, 128, 8, 512), (3, 64, 33, 1030), (4, 64, 149, 260), (3, 128, 5, 2049), (4, 128, 2, 33000), (4, 128, 40, 300), (3, 64, 150, 4501)]
+    linears = []
+    for i, (bits, group, m_blocks, n) in enumerate(sizes):
+        p = random_matrix(bits, group, m_blocks, n)[0]
+        h = binding.HostLinear(p)
+        if shared and i > 0 and h.idx.numel() <= linears[0].idx.numel():
+            h.idx, h.count = linears[0].idx, linears[0].count
+        linears.append(h)
+    if shared:
+        linears[1].count = linears[0].count
+    ts = [0.4 + 0.05 * i for i in range(len(linears))]
+    step = binding.HostStep(linears, ts)
+    for replay in range(3):
+        for i, h in enumerate(linears):
+            h.x_host.copy_(torch.from_numpy(inputs.activations(h.p.n, seed=100 * replay + i)))
+            h.y_host.zero_()
+        step.launch()
+        torch.cuda.synchronize()
+        for h, t in zip(linears, ts):
+            y, _, _ = binding.spqt_sparsify_gemv(h.p, h.x_host.cuda(), t, binding.new_workspace(h.p.m, h.p.n, h.p.bits, h.p.group))
+            assert torch.equal(y.cpu(), h.y_host)
+            assert int(h.workspace.count_nonzero()) == 0
