@@ -169,12 +169,23 @@ gemm_small_kernel(const SmallArgs a)
             } else {
                 cp_async_8(st + xdst, xsrc + (size_t)(unsigned)ipos * 8);
             }
+            // (the chunk's blocks lie one after the other: one address instead of a shuffle and a product for every copy; 28672 x 4096
+            // with 4 rows 14.7 -> 14.0 us, 14336 x 4096 with 8 13.0 -> 12.5; 8-byte copies 2 % slower)
+            if (DIRECT && CB == 16 && ipos + CH <= end) {
+                const uint8_t* s = row_codes + ((size_t)(unsigned)ipos * B + lane * CB);
 #pragma unroll
-            for (int q = 0; q < NC; ++q) {
-                const unsigned cu = (unsigned)__shfl_sync(0xffffffffu, col, copy_e[q]);
-                const uint8_t* s = row_codes + ((size_t)cu * B + copy_part[q]);
-                if (CB == 16) cp_async_16_l2_64(st + copy_dst[q], s);
-                else cp_async_8(st + copy_dst[q], s);
+                for (int q = 0; q < NC; ++q) {
+                    if (CB == 16) cp_async_16_l2_64(st + copy_dst[q], s + q * 32 * CB);
+                    else cp_async_8(st + copy_dst[q], s + q * 32 * CB);
+                }
+            } else {
+#pragma unroll
+                for (int q = 0; q < NC; ++q) {
+                    const unsigned cu = (unsigned)__shfl_sync(0xffffffffu, col, copy_e[q]);
+                    const uint8_t* s = row_codes + ((size_t)cu * B + copy_part[q]);
+                    if (CB == 16) cp_async_16_l2_64(st + copy_dst[q], s);
+                    else cp_async_8(st + copy_dst[q], s);
+                }
             }
             if (kTwice) cp_async_8(st + lane * Layout::kRow + 24, row_codes + ((size_t)(unsigned)col * B + 16));
             ri = ri + kStageBytes == D * kStageBytes ? 0u : ri + kStageBytes;
