@@ -469,12 +469,15 @@ static spqt_status launch_gather_rows(const __half* X, int ldx, int batch, int n
     return (err == cudaSuccess && cudaGetLastError() == cudaSuccess) ? SPQT_OK : SPQT_ERR_CUDA;
 }
 
-// How many clusters of k CTAs the device holds at once, two CTAs per SM (asked once per kernel, cluster size and device).
+constexpr int kSmallAlone = 120 * 1024;   // shared memory that keeps a second CTA off the SM
+
+// How many clusters of k CTAs the device holds at once, one or two CTAs per SM (asked once per kernel, cluster size and device).
 template <int G, int BITS, int ROWS, bool DIRECT>
-static int small_max_clusters(int k, int smem, int sms, int dev)
+static int small_max_clusters(int k, bool alone, int sms, int dev)
 {
-    static int known[64][kSmallMaxSplit + 1] = {};
-    int& at_once = known[dev][k];
+    constexpr int smem = (int)sizeof(SmallSmem<G, BITS, ROWS>);
+    static int known[64][2][kSmallMaxSplit + 1] = {};
+    int& at_once = known[dev][alone ? 1 : 0][k];
     if (at_once == 0) {
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -484,7 +487,7 @@ static int small_max_clusters(int k, int smem, int sms, int dev)
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(k, kSmallCtasPerSm * sms);
         cfg.blockDim = dim3(kSmallThreads);
-        cfg.dynamicSmemBytes = smem;
+        cfg.dynamicSmemBytes = alone ? kSmallAlone : smem;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int can = 0;
@@ -501,9 +504,10 @@ static spqt_status launch_small(const Format& f, SmallArgs a, cudaStream_t s)
     static bool configured[64] = {};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return SPQT_ERR_CUDA;
-    const int smem = (int)sizeof(SmallSmem<G, BITS, ROWS>);
+    constexpr int smem = (int)sizeof(SmallSmem<G, BITS, ROWS>);
+    static_assert(smem <= 115712, "two CTAs per SM");
     if (!configured[dev]) {
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return SPQT_ERR_CUDA;
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallAlone) != cudaSuccess) return SPQT_ERR_CUDA;
         configured[dev] = true;
     }
     const int sms = sm_count();
@@ -516,10 +520,34 @@ static spqt_status launch_small(const Format& f, SmallArgs a, cudaStream_t s)
     // there are more than 32 block-rows (6144 x 1024, 3 rows: 10 % faster on 1 than on 4).  From R = 100 up two put two half
     // block-rows on the busiest SMs, where one whole block-row runs as fast and needs no exchange (14336 x 4096, 8 rows dense:
     // 12.3 against 14.4 us), unless x is long (12800 x 14336, 8 rows 6 %, 64-row groups 6400 x 14336, 3 rows 16 % faster on 2).
+    // Without a list, where the same call may come next, odd clusters that nearly fill the device wait for one another, and the best
+    // is the least load of an SM: a block-row over k CTAs with an SM each, 1.6 times that where two share one (three with two per
+    // SM at most where two are alone: 9216 x 2048, 8 rows 7.1 us on 3, 5.3 on 2; 6912 x 8192 15.0 on 5, 12.7 on 4), and with a long x
+    // clusters of four in more than one wave rather than one or two CTAs (11776 x 8192, 8 rows 24.0 on 3, 23.3 on 1, 19.3 on 4).  Over 297
+    // sizes the choice is 2 % slower than the best cluster, the largest that fits was 7 %.
     int S = 1;
-    for (int k = 2; k <= kSmallMaxSplit; ++k) {
-        const int columns = f.R >= 100 ? 8192 : f.R > 32 ? 512 * k : 256 * (k - 1) + 1;
-        if (f.n >= columns && f.R < small_max_clusters<G, BITS, ROWS, DIRECT>(k, smem, sms, dev)) S = k;
+    if (DIRECT || !a.idx) {
+        float least = 0.0f;
+        for (int k = 1; k <= kSmallMaxSplit && (k == 1 || f.n >= 512 * k); ++k) {
+            const bool even = (k & (k - 1)) == 0;
+            const int one = k == 1 ? sms : small_max_clusters<G, BITS, ROWS, DIRECT>(k, true, sms, dev);
+            const int two = k == 1 ? 2 * sms : small_max_clusters<G, BITS, ROWS, DIRECT>(k, false, sms, dev);
+            float load = 0.0f;                // of an SM, in block-rows
+            if (even ? f.R <= one : 10 * f.R <= 9 * one) load = 1.0f / k;
+            else if (k == 2 && f.n < 8192) continue;   // (two halves on the busiest SMs: no less than a whole)
+            else if (even ? f.R <= two : 25 * f.R <= 24 * two || (k >= 6 && f.n >= 8192 && f.R < two)) load = 1.6f / k;
+            else if (k == 4 && f.n >= 8192 && 2 * f.R > sms && f.R <= sms) load = 2.0f * f.R / (4.0f * two);
+            else if (k > 1) continue;
+            if (k == 1 || load < least) {
+                least = load;
+                S = k;
+            }
+        }
+    } else {
+        for (int k = 2; k <= kSmallMaxSplit; ++k) {
+            const int columns = f.R >= 100 ? 8192 : f.R > 32 ? 512 * k : 256 * (k - 1) + 1;
+            if (f.n >= columns && f.R < small_max_clusters<G, BITS, ROWS, DIRECT>(k, false, sms, dev)) S = k;
+        }
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(S, f.R);
