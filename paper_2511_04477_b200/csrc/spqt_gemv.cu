@@ -22,15 +22,15 @@
 // codes being operands as they are.  y[j] = sum_k a_k * code_jk + sum_k x_k * zero_rk.
 //
 // What bounds it.  Small and medium matrices: the fixed cost of a launch (a 4096 x 4096 call at 50 % needs 4.5 MB, 0.7 us
-// of DRAM time, and takes 4.6 us), most of it chains of dependent instructions that every warp of every CTA goes
-// through: clock stamps put 600 cycles on fetching x, 600 on the activity masks, 500 on the list, 400 on the first
-// copies, 500 on their arrival, 600 on a first chunk, 500 on the sums.  Hence whole block-rows instead of fractions (no
+// of DRAM time, and takes 4.2 us), a chain of dependent steps.  Clock stamps from the end of the launch before: 0.6 us to
+// the end of the wait for it, 0.6 x and the masks, 0.1 the count, 0.4 the list, 0.6 to 1.1 the first copies (all of the matrix is on
+// its way then), 0.8 the loop and the sums, 0.4 the cluster's exchange.  Hence whole block-rows instead of fractions (no
 // work map), one instance of every code path, few warps with much work each rather than many, and two CTAs per SM where
-// the grid is large enough, so that one computes while the other starts or ends.  The kernel before this one (one
+// the grid is large enough, so that one computes while the other starts or ends.  The kernel before the tensor cores (one
 // persistent CTA of 18 warps per SM, fractional block-rows, packed FMAs, partial sums as tagged words in global memory;
 // 4500 instructions of code against 1600) took 6.4 us there.  Large matrices: the code stream; 28672 x 8192 dense went
-// from 26.9 to 24.2 us, 8192 x 28672 dense from 29.0 to 25.6 us among other calls in a stream (4.9 TB/s, 0.74 of the measured
-// copy bandwidth; 22.3 us in short runs).
+// from 26.9 to 21.6 us, 8192 x 28672 dense from 29.0 to 24.6 us among other calls in a stream (5.1 TB/s, 0.78 of the measured
+// copy bandwidth; 21.2 us in short runs).
 #include <cstddef>
 
 #include "spqt_common.cuh"

@@ -19,10 +19,11 @@
 //                    records are an odd number of 16-byte pieces, so that ldmatrix.trans reads them as they lie; the
 //                    eight columns of B are hi and lo of the multipliers of four blocks, a second set those of the other
 //                    four.  Sums: warps through shared memory, CTAs through the cluster's, in a fixed order.
-//                    What bounds it: the fixed cost of the call and of the list's launch before it, then latency: 12 to 16
-//                    warps per SM with 2 to 5 chunks in flight each.  28672 x 4096 to 4 bits at 50 %, list included, takes
-//                    15.9 us (19.4 with packed FMAs, partial sums in global memory and chunks dealt in turn), 8192 x 8192
-//                    to 6 bits dense 16.6 us (20.4; 55 MB), 28672 x 4096 to 2 bits dense 17.3 us (24.7).
+//                    What bounds it: the integer pipe in the loop (masks, shifts: 53 to 61 % busy over the whole call), the fixed
+//                    cost of the call and of the list's launch before it, then latency: 12 to 16 warps per SM with 2 to 5
+//                    chunks in flight each.  28672 x 4096 to 4 bits at 50 %, list included, takes 14.2 us (19.4 with packed
+//                    FMAs, partial sums in global memory and chunks dealt in turn), 8192 x 8192 to 6 bits dense 14.3 us (20.4;
+//                    55 MB), 28672 x 8192 to 4 bits dense 31.1 us.
 //                    A multiplier x*(d*sc) is rounded to fp32 and goes in as two fp16 values, off by 2^-26 of the warp's
 //                    largest at most (spqt_mma.cuh; their rounding and rescaling cost 2 to 3 %: 28672 x 8192 dense to 4 bits 34.4 -> 35.4 us).
 #include <cstddef>
@@ -653,8 +654,14 @@ static spqt_status kq_launch_mode(const void* records, int R, int n, const void*
     // faster with 8).  With few block-rows of a long x several clusters of 4 CTAs of 16 warps, so that more SMs fetch, if that are
     // half as many CTAs again (the sums of a block-row then meet in global memory, 1.5 us: dense 1024 x 28672 to 8 bits, 31 MB,
     // 21.0 us on 32 CTAs of 8 warps, 12.0 on 128 of 16; at n = 8192 clusters of 8 are 8 to 16 % faster, at 14336 8 to 22 % slower).
+    // Powers of two with an SM for each CTA fit neighbouring SMs without (18944 x 8192 to 6 bits dense 34.7 us on 3, 25.7 on 2, of
+    // which the device holds 74); with two per SM, odd numbers take 8 % unless there is much to do (13312 x 4096 dense 14.2 on 5, of 56, 10.8
+    // on 4; 13312 x 14336 to 6 bits with the list 25.4 on 5, 28.2 on 4).
     auto resident = [&](int k, bool per_sm) {
-        return k * (kq_max_clusters<BITS, LIST, 8>(k, per_sm ? kAlone : kSmem, per_sm, sms, dev) - R) >= 4;
+        const int most = kq_max_clusters<BITS, LIST, 8>(k, per_sm ? kAlone : kSmem, per_sm, sms, dev);
+        if (per_sm && (k & (k - 1)) == 0) return R <= most;
+        if (!per_sm && (k & 1) != 0 && 100 * R > 92 * most && n < (k == 3 ? 4096 : 12288)) return false;
+        return k * (most - R) >= 4;
     };
     int one = 1, two = 1, T = 1;         // CTAs per block-row with one and with two CTAs per SM
     for (int k = 2; k <= kKqMaxCluster; ++k) {
