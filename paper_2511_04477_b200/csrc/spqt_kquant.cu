@@ -655,12 +655,12 @@ static spqt_status kq_launch_mode(const void* records, int R, int n, const void*
     // half as many CTAs again (the sums of a block-row then meet in global memory, 1.5 us: dense 1024 x 28672 to 8 bits, 31 MB,
     // 21.0 us on 32 CTAs of 8 warps, 12.0 on 128 of 16; at n = 8192 clusters of 8 are 8 to 16 % faster, at 14336 8 to 22 % slower).
     // Powers of two with an SM for each CTA fit neighbouring SMs without (18944 x 8192 to 6 bits dense 34.7 us on 3, 25.7 on 2, of
-    // which the device holds 74); with two per SM, odd numbers take 8 % unless there is much to do (13312 x 4096 dense 14.2 on 5, of 56, 10.8
-    // on 4; 13312 x 14336 to 6 bits with the list 25.4 on 5, 28.2 on 4).
+    // which the device holds 74); with two per SM, five and seven take 8 %, three
+    // where there is little to do (13312 x 4096 dense 14.2 on 5, of 56, 10.8 on 4; 22528 x 2048 dense 12.0 on 3, of 93, 10.5 on 1).
     auto resident = [&](int k, bool per_sm) {
         const int most = kq_max_clusters<BITS, LIST, 8>(k, per_sm ? kAlone : kSmem, per_sm, sms, dev);
         if (per_sm && (k & (k - 1)) == 0) return R <= most;
-        if (!per_sm && (k & 1) != 0 && 100 * R > 92 * most && n < (k == 3 ? 4096 : 12288)) return false;
+        if (!per_sm && (k & 1) != 0 && 100 * R > 92 * most && (k > 3 || n < 4096)) return false;
         return k * (most - R) >= 4;
     };
     int one = 1, two = 1, T = 1;         // CTAs per block-row with one and with two CTAs per SM
