@@ -454,8 +454,8 @@ spqt_status spqt_set_debug(int on);
 /*
  * Reads the workspace's status word into *status_host (a host int) and waits for
  * the stream: 0 = every GEMV that used this workspace ran to completion;
- * 1 = a bounded wait expired inside a GEMV kernel (no present kernel has one; it would return early,
- * leaving y unspecified); 2 = checked mode found a bad index list.  The word is
+ * 1 = a bounded wait expired inside a GEMV kernel (one second, for the sums of a cluster's other CTAs; that block-row of
+ * y is then unspecified); 2 = checked mode found a bad index list.  The word is
  * sticky until the caller zeroes the workspace again.  Returns SPQT_OK for 0,
  * SPQT_ERR_TIMEOUT for 1 and SPQT_ERR_INVALID_ARG for 2 (after writing *status_host).
  */

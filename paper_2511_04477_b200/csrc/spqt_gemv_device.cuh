@@ -153,10 +153,6 @@ __device__ __forceinline__ void sts_u32(unsigned addr, unsigned v)
 {
     asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
-__device__ __forceinline__ void sts_u16(unsigned addr, unsigned v)
-{
-    asm volatile("st.shared.u16 [%0], %1;" ::"r"(addr), "h"((unsigned short)v) : "memory");
-}
 __device__ __forceinline__ void sts_v4(unsigned addr, const uint4& v)
 {
     asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
@@ -196,16 +192,6 @@ __device__ __forceinline__ void st_async_u32(unsigned addr, unsigned v, unsigned
 __device__ __forceinline__ void st_async_f32(unsigned addr, float v, unsigned bar)
 {
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(addr), "f"(v), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void st_cluster_f32(unsigned addr, float v)
-{
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
-}
-__device__ __forceinline__ float ld_cluster_f32(unsigned addr)
-{
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
-    return v;
 }
 
 // Two fp32 lanes in one 64-bit register, the operand form of the packed FMA.
