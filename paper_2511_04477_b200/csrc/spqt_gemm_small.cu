@@ -403,7 +403,7 @@ gemm_small_kernel(const SmallArgs a)
             st_async_f32x4(cluster_map(dst, (unsigned)owner), v, cluster_map(smem_u32(&sm.arrival), (unsigned)owner));
             return;
         }
-        const float start = mbar_wait(&sm.arrival, 0u) ? 0.0f : __int_as_float(0x7fffffff);   // (a wait that ran out: not-a-number)
+        const float start = mbar_wait_cluster(&sm.arrival, 0u) ? 0.0f : __int_as_float(0x7fffffff);   // (a wait that ran out: not-a-number)
         float4 sum = make_float4(start, start, start, start);
 #pragma unroll
         for (int q = 0; q < kSmallMaxSplit; ++q) {

@@ -688,7 +688,7 @@ gemv_kernel(const GemvArgs a)
             return;
         }
         if (tid < G / 2) {
-            if (!mbar_wait(&sm.arrival, 0u)) atomicExch(a.status, 1u);   // (a wait that ran out)
+            if (!mbar_wait_cluster(&sm.arrival, 0u)) atomicExch(a.status, 1u);   // (a wait that ran out)
 #pragma unroll
             for (int q = 0; q < kMaxSplit - 1; ++q)
                 if (q < a.splits - 1) {

@@ -11,7 +11,7 @@ __device__ __forceinline__ unsigned smem_u32(const void* p)
     return static_cast<unsigned>(__cvta_generic_to_shared(p));
 }
 
-// ---- mbarriers (the row-wise kernel's ring)
+// ---- mbarriers (the row-wise kernel's ring; what the CTAs of a cluster send one another)
 constexpr unsigned long long kWaitNs = 1000000000ull;  // bound on every wait: one second of wall time
 
 __device__ __forceinline__ void mbar_init(uint64_t* bar, unsigned count)
@@ -44,26 +44,41 @@ __device__ __forceinline__ unsigned long long global_ns()
 
 // Bounded wait for the phase with the given parity; false when the bound
 // (wall time, so that a logic error can never hold the GPU) expires.  One try_wait
-// blocks for up to about 4 us on this GPU (with or without the time hint).
+// blocks for up to about 4 us on this GPU (with or without the time hint).  CLUSTER: what the barrier announces comes from other
+// CTAs of the cluster, and the acquire has to reach as far (left out, its scope is the CTA).
 constexpr unsigned kSuspendNs = 100000u;  // the time hint of one try_wait
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity)
+template <bool CLUSTER>
+__device__ __forceinline__ bool mbar_wait_scope(uint64_t* bar, unsigned parity)
 {
     const unsigned addr = smem_u32(bar);
     unsigned long long t0 = 0;
     for (unsigned it = 0;; ++it) {
         unsigned done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done)
-            : "r"(addr), "r"(parity), "r"(kSuspendNs)
-            : "memory");
+        if (CLUSTER)
+            asm volatile(
+                "{\n\t.reg .pred p;\n\t"
+                "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
+                "selp.u32 %0, 1, 0, p;\n\t}"
+                : "=r"(done)
+                : "r"(addr), "r"(parity), "r"(kSuspendNs)
+                : "memory");
+        else
+            asm volatile(
+                "{\n\t.reg .pred p;\n\t"
+                "mbarrier.try_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2, %3;\n\t"
+                "selp.u32 %0, 1, 0, p;\n\t}"
+                : "=r"(done)
+                : "r"(addr), "r"(parity), "r"(kSuspendNs)
+                : "memory");
         if (done) return true;
         if (it == 0) t0 = global_ns();
         else if (global_ns() - t0 > kWaitNs) return false;
     }
 }
+// for arrivals of this CTA's threads
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity) { return mbar_wait_scope<false>(bar, parity); }
+// for asynchronous stores of other CTAs of the cluster
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, unsigned parity) { return mbar_wait_scope<true>(bar, parity); }
 
 // ---- asynchronous copies
 __device__ __forceinline__ void cp_async_16(unsigned smem_dst, const void* gmem_src)

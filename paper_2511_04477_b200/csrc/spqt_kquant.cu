@@ -555,7 +555,7 @@ kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* __restr
             return;
         }
         if (tid < kKqG) {
-            if (!mbar_wait(&sm.arrival, 0u)) total = __int_as_float(0x7fffffff);   // (a wait that ran out: not-a-number)
+            if (!mbar_wait_cluster(&sm.arrival, 0u)) total = __int_as_float(0x7fffffff);   // (a wait that ran out: not-a-number)
 #pragma unroll
             for (unsigned q = 0; q < kKqMaxCluster - 1; ++q)
                 if (q < S - 1u) total += sm.xred[q][tid];

@@ -48,7 +48,7 @@ struct ClusterTotals {
     __device__ __forceinline__ void exchange(int me, int mine, int lane, int ctas, int& below, int& all)
     {
         if (lane < ctas) st_async_u32(cluster_map(smem_u32(&total[me]), (unsigned)lane), (unsigned)mine, cluster_map(smem_u32(&arrival), (unsigned)lane));
-        const bool there = mbar_wait(&arrival, 0u);
+        const bool there = mbar_wait_cluster(&arrival, 0u);
         unsigned b = 0, a = 0;
 #pragma unroll
         for (int w = 0; w < WARPS; w += 32) {
