@@ -3,6 +3,7 @@
 #include <atomic>
 
 #include "spqt_common.cuh"
+#include "spqt_gemv_device.cuh"
 
 namespace spqt {
 
@@ -38,8 +39,8 @@ __global__ void __launch_bounds__(256) fetch_x_kernel(FetchList fl)
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const unsigned short* __restrict__ src = fl.src[blockIdx.x];
-    unsigned short* __restrict__ dst = fl.dst[blockIdx.x];
+    const unsigned short* const src = fl.src[blockIdx.x];
+    unsigned short* const dst = fl.dst[blockIdx.x];
     const int n = fl.n[blockIdx.x];
     const int tid = threadIdx.x;
     if (((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) == 0) {
@@ -51,7 +52,7 @@ __global__ void __launch_bounds__(256) fetch_x_kernel(FetchList fl)
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const int i = i0 + j * 256 + tid;
-                if (i < nv) v[j] = s4[i];
+                v[j] = ld_global_v4(s4 + min(i, nv - 1));   // (no load behind a condition: they go together)
             }
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
@@ -59,9 +60,9 @@ __global__ void __launch_bounds__(256) fetch_x_kernel(FetchList fl)
                 if (i < nv) d4[i] = v[j];
             }
         }
-        for (int i = (nv << 3) + tid; i < n; i += 256) dst[i] = src[i];
+        for (int i = (nv << 3) + tid; i < n; i += 256) dst[i] = (unsigned short)ld_global_u16(src + i);
     } else {
-        for (int i = tid; i < n; i += 256) dst[i] = src[i];
+        for (int i = tid; i < n; i += 256) dst[i] = (unsigned short)ld_global_u16(src + i);
     }
 }
 

@@ -131,7 +131,7 @@ gemm_small_kernel(const SmallArgs a)
 
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (!DIRECT && a.idx) take_part(__ldg(a.count));
+    if (!DIRECT && a.idx) take_part((int)ld_global_u32(a.count));
 
     float acc[SP][4][4];
     unsigned long long zl[ROWS / 2], scale[ROWS / 2];   // pairs of rows
@@ -152,7 +152,7 @@ gemm_small_kernel(const SmallArgs a)
     int ipos = pos;               // where the copies stand; the arithmetic is D - 1 chunks behind
     auto column_at = [&](int p) -> int {
         const int e = min(p + lane, end - 1);
-        return (!DIRECT && a.idx) ? __ldg(a.idx + e) : e;
+        return (!DIRECT && a.idx) ? (int)ld_global_u32(a.idx + e) : e;
     };
 #pragma unroll
     for (int d = 0; d < kAhead; ++d) coming[d] = pos < end ? column_at(pos + d * CH) : 0;
@@ -435,7 +435,7 @@ inline size_t small_workspace_bytes(const Format& f)
 
 // The records of the dense product when it cannot read X with 16-byte copies: REC values per column.
 template <int REC>
-__global__ void __launch_bounds__(256) gather_rows_kernel(const unsigned short* __restrict__ X, int ldx, int batch, int n, unsigned short* __restrict__ gathered)
+__global__ void __launch_bounds__(256) gather_rows_kernel(const unsigned short* X, int ldx, int batch, int n, unsigned short* gathered)
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -444,8 +444,8 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const unsigned short* 
     unsigned rec[REC / 2];
 #pragma unroll
     for (int b = 0; b < REC; b += 2) {
-        const unsigned lo = b < batch ? __ldg(X + (size_t)b * ldx + k) : 0u;
-        const unsigned hi = b + 1 < batch ? __ldg(X + (size_t)(b + 1) * ldx + k) : 0u;
+        const unsigned lo = b < batch ? ld_global_u16(X + (size_t)b * ldx + k) : 0u;
+        const unsigned hi = b + 1 < batch ? ld_global_u16(X + (size_t)(b + 1) * ldx + k) : 0u;
         rec[b / 2] = lo | (hi << 16);
     }
     if (REC == 8) *reinterpret_cast<uint4*>(gathered + (size_t)k * 8) = make_uint4(rec[0], rec[1], rec[REC / 2 - 2], rec[REC / 2 - 1]);

@@ -551,7 +551,7 @@ gemv_kernel(const GemvArgs a)
 
     Scan<NW> scan(sm.area, a.thr, n, lane, warp);            // (fused calls only)
     int count = n;
-    if (LIST) count = __ldg(a.count);
+    if (LIST) count = (int)ld_global_u32(a.count);
     if (FUSED) {
         count = scan.scan_x(a.x);
         if (blockIdx.x == 0 && tid == 0) *a.count_out = count;
@@ -598,7 +598,7 @@ gemv_kernel(const GemvArgs a)
         int coming[kAhead][EPL], ahead = first;
         auto fetch_ahead = [&](int d) {
 #pragma unroll
-            for (int q = 0; q < EPL; ++q) coming[d][q] = __ldg(a.idx + min(ahead + 32 * q + lane, end - 1));
+            for (int q = 0; q < EPL; ++q) coming[d][q] = (int)ld_global_u32(a.idx + min(ahead + 32 * q + lane, end - 1));
             ahead = ahead + CH >= end ? first : ahead + CH;
         };
         if (LIST && first < end) {
@@ -621,7 +621,7 @@ gemv_kernel(const GemvArgs a)
                 for (int q = 0; q < EPL; ++q) {       // (past the end: the last entry again, with x = 0)
                     const int e = ipos + 32 * q + lane;
                     col[q] = LIST ? (unsigned)coming[0][q] : FUSED ? lds_u16(ent_base + 4u * (unsigned)(min(e, end - 1) - lo)) : (unsigned)min(e, end - 1);
-                    if (!FUSED) xv[D - 1][q] = e < end ? (unsigned)__ldg(xg + col[q]) : 0u;
+                    if (!FUSED) xv[D - 1][q] = ld_global_u16_if(e < end, xg + col[q]);
                 }
                 copy_chunk<G, BITS, Ring>(stage0 + ri, row_codes, row_meta, col, lane, MODE == kModeDense && ipos + CH <= end);
                 ri = ri + kStageBytes == kRing ? 0u : ri + kStageBytes;
@@ -757,7 +757,7 @@ gemv_pieces_kernel(const GemvArgs a)
 
     Scan<NW> scan(sm.area, a.thr, n, lane, warp);            // (fused calls only)
     int count = n;
-    if (LIST) count = __ldg(a.count);
+    if (LIST) count = (int)ld_global_u32(a.count);
     if (FUSED) count = scan.scan_x(a.x);
     const unsigned units = (unsigned)(count + 7) >> 3;
     int first = 8 * (int)magic_div(part0 * units, N, a.magic_w), end = 8 * (int)magic_div(part1 * units, N, a.magic_w);
@@ -801,7 +801,7 @@ gemv_pieces_kernel(const GemvArgs a)
     auto fetch_ahead = [&](int d) {
         if (ahead.pos < ahead.hi) {
 #pragma unroll
-            for (int q = 0; q < EPL; ++q) coming[d][q] = __ldg(a.idx + min(ahead.pos + 32 * q + lane, ahead.hi - 1));
+            for (int q = 0; q < EPL; ++q) coming[d][q] = (int)ld_global_u32(a.idx + min(ahead.pos + 32 * q + lane, ahead.hi - 1));
         }
         advance(ahead);
     };
@@ -822,7 +822,7 @@ gemv_pieces_kernel(const GemvArgs a)
             for (int q = 0; q < EPL; ++q) {           // (past the end: the last entry again, with x = 0)
                 const int e = at.pos + 32 * q + lane, in = min(e, at.hi - 1);
                 col[q] = LIST ? (unsigned)coming[0][q] : FUSED ? lds_u16(ent_base + 2u * (unsigned)in) : (unsigned)in;
-                xv[D - 1][q] = e < at.hi ? (unsigned)__ldg(xg + col[q]) : 0u;
+                xv[D - 1][q] = ld_global_u16_if(e < at.hi, xg + col[q]);
             }
             copy_chunk<G, BITS, Ring>(stage0 + ri, row_codes, row_meta, col, lane, false);
             ri = ri + kStageBytes == kRing ? 0u : ri + kStageBytes;

@@ -317,8 +317,8 @@ __host__ __device__ constexpr float kq_unit(int bits, int blk, int o)
 // idx == nullptr: the dense product (the list is 0, 1, .., n-1 and count is n).
 template <int BITS, bool LIST, int NW>
 __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1)
-kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* __restrict__ x, const int32_t* __restrict__ idx,
-               const int32_t* __restrict__ count_ptr, __half* __restrict__ y, int splits, int clusters, unsigned* arrived, float* partial)
+kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* x, const int32_t* idx,
+               const int32_t* count_ptr, __half* y, int splits, int clusters, unsigned* arrived, float* partial)
 {
     constexpr int REC = kq_rec_bytes(BITS), NCB = kq_code_bytes(BITS), PPR = REC / 16, CH = kKqChunk, D = kq_depth(BITS);
     constexpr int kPieces = CH * PPR, NC = (kPieces + 31) / 32;
@@ -360,12 +360,12 @@ kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* __restr
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-    if (LIST) take_part(__ldg(count_ptr));
+    if (LIST) take_part((int)ld_global_u32(count_ptr));
 
     constexpr int kAhead = 2;            // (a third costs registers: 28672 x 4096 to 4 bits 13.2 against 12.8 us, to 8 bits 16.8 against 16.3)
     int coming[kAhead], ahead = first;   // list: the columns of the chunks the copies come to next
     auto fetch_ahead = [&](int d) {
-        coming[d] = __ldg(idx + min(ahead + e, end - 1));
+        coming[d] = (int)ld_global_u32(idx + min(ahead + e, end - 1));
         ahead = ahead + CH >= end ? first : ahead + CH;
     };
     if (LIST && first < end) {
@@ -383,7 +383,7 @@ kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* __restr
         xv[D - 1] = 0u;
         if (ipos < end) {                // (past the end: the last entry again, with x = 0)
             const unsigned col = LIST ? (unsigned)coming[0] : (unsigned)min(ipos + e, end - 1);
-            if (ipos + e < end) xv[D - 1] = (unsigned)__ldg(xg + col);
+            xv[D - 1] = ld_global_u16_if(ipos + e < end, xg + col);
             // (the chunk's records lie one after the other: one address instead of a shuffle and a product for every copy; 28672 x 8192
             // to 6 bits 50.0 -> 44.4 us, 5 bits 53.0 -> 51.0; to 4 bits 2 % slower)
             if (!LIST && BITS >= 5 && ipos + CH <= end) {

@@ -135,7 +135,7 @@ __device__ __forceinline__ float reduce_rows(const float* v, int lane, int* row)
 template <int G, int ROWS>
 __global__ void __launch_bounds__(kRwThreads, 1)
 rowwise_gemv_kernel(const uint8_t* __restrict__ codes, const unsigned* __restrict__ meta, int m, int n,
-                    const __half* __restrict__ x, __half* __restrict__ y, int Wc, int Rg, int sparse, float thr)
+                    const __half* x, __half* y, int Wc, int Rg, int sparse, float thr)
 {
     using Smem = RwSmem<G, ROWS>;
     constexpr int B = G / 2, NG = Smem::NG, D = kRwDepth;
@@ -194,9 +194,7 @@ rowwise_gemv_kernel(const uint8_t* __restrict__ codes, const unsigned* __restric
     {
         unsigned short xl[16], xh[16];
         if (live && (reinterpret_cast<uintptr_t>(x) & 15) == 0) {
-            const uint4* pl = reinterpret_cast<const uint4*>(x + c_lo);
-            const uint4* ph = reinterpret_cast<const uint4*>(x + c_lo + G / 2);
-            const uint4 v[4] = {__ldg(pl), __ldg(pl + 1), __ldg(ph), __ldg(ph + 1)};
+            const uint4 v[4] = {ld_global_v4(x + c_lo), ld_global_v4(x + c_lo + 8), ld_global_v4(x + c_lo + G / 2), ld_global_v4(x + c_lo + G / 2 + 8)};
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const unsigned wl[4] = {v[h].x, v[h].y, v[h].z, v[h].w};
@@ -213,8 +211,8 @@ rowwise_gemv_kernel(const uint8_t* __restrict__ codes, const unsigned* __restric
             const unsigned short* xb = reinterpret_cast<const unsigned short*>(x);
 #pragma unroll
             for (int t = 0; t < 16; ++t) {
-                xl[t] = live ? __ldg(xb + c_lo + t) : (unsigned short)0;
-                xh[t] = live ? __ldg(xb + c_lo + t + G / 2) : (unsigned short)0;
+                xl[t] = live ? (unsigned short)ld_global_u16(xb + c_lo + t) : (unsigned short)0;
+                xh[t] = live ? (unsigned short)ld_global_u16(xb + c_lo + t + G / 2) : (unsigned short)0;
             }
         }
 #pragma unroll

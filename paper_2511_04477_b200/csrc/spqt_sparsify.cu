@@ -69,7 +69,7 @@ struct ClusterTotals {
 // two barriers up to 6144, then a cluster with cluster barriers before and after reading each other's totals).
 template <int WORDS, bool CLUSTER>
 __global__ void __launch_bounds__(CLUSTER ? kClusterWarps * 32 : kSparsifyThreads)
-sparsify_words_kernel(const __half* __restrict__ x, int n, unsigned short thr_bits, int32_t* __restrict__ idx, int32_t* __restrict__ count)
+sparsify_words_kernel(const __half* x, int n, unsigned short thr_bits, int32_t* idx, int32_t* count)
 {
     __shared__ ClusterTotals<CLUSTER ? kClusterCtas * kClusterWarps : 32> totals;
     const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);
@@ -131,8 +131,7 @@ sparsify_words_kernel(const __half* __restrict__ x, int n, unsigned short thr_bi
 }
 
 __global__ void __launch_bounds__(kSparsifyThreads)
-sparsify_kernel(const __half* __restrict__ x, int n, float t,
-                int32_t* __restrict__ idx, int32_t* __restrict__ count)
+sparsify_kernel(const __half* x, int n, float t, int32_t* idx, int32_t* count)
 {
     __shared__ int warp_total[32];
     __shared__ int warp_base[32];
@@ -156,7 +155,7 @@ sparsify_kernel(const __half* __restrict__ x, int n, float t,
         __half v[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j)
-            if (g0 + j < groups) v[j] = x[min(begin + (g0 + j) * 32 + lane, n - 1)];   // (uniform condition)
+            if (g0 + j < groups) v[j] = __ushort_as_half((unsigned short)ld_global_u16(x + min(begin + (g0 + j) * 32 + lane, n - 1)));   // (uniform condition)
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             if (g0 + j < groups) {
@@ -192,7 +191,7 @@ sparsify_kernel(const __half* __restrict__ x, int n, float t,
     }
     for (int k0 = begin; k0 < end; k0 += 32) {
         const int k = k0 + lane;
-        const bool p = (k < end) && is_active(x[k], t);
+        const bool p = k < end && is_active(__ushort_as_half((unsigned short)ld_global_u16(x + k)), t);
         const unsigned mask = __ballot_sync(0xffffffffu, p);
         if (p) idx[base + __popc(mask & ((1u << lane) - 1u))] = k;
         base += __popc(mask);
@@ -211,8 +210,7 @@ constexpr int kKeepGroups = 4;
 
 template <int REC>
 __global__ void __launch_bounds__(kRowsWarps * 32)
-sparsify_rows_kernel(const unsigned short* __restrict__ X, int ldx, int batch, int n, float t,
-                     int32_t* __restrict__ idx, int32_t* __restrict__ count, unsigned short* __restrict__ gathered)
+sparsify_rows_kernel(const unsigned short* X, int ldx, int batch, int n, float t, int32_t* idx, int32_t* count, unsigned short* gathered)
 {
     __shared__ ClusterTotals<kClusterCtas * kRowsWarps> totals;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -234,7 +232,7 @@ sparsify_rows_kernel(const unsigned short* __restrict__ X, int ldx, int batch, i
         for (int j = 0; j < kKeepGroups; ++j) {
             const int k = min(first + (g0 + j) * 32, n - 1);
 #pragma unroll
-            for (int b = 0; b < REC; ++b) v[j][b] = (g0 + j < groups && b < batch) ? __ldg(X + (size_t)b * ldx + k) : (unsigned short)0;
+            for (int b = 0; b < REC; ++b) v[j][b] = (g0 + j < groups && b < batch) ? (unsigned short)ld_global_u16(X + (size_t)b * ldx + k) : (unsigned short)0;
         }
     };
     auto active = [&](int g0, int j) -> bool {

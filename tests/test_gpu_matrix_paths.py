@@ -325,3 +325,49 @@ def test_recorded_step_in_branches(shared):
             y, _, _ = binding.spqt_sparsify_gemv(h.p, h.x_host.cuda(), t, binding.new_workspace(h.p.m, h.p.n, h.p.bits, h.p.group))
             assert torch.equal(y.cpu(), h.y_host)
             assert int(h.workspace.count_nonzero()) == 0
+
+
+def test_calls_behind_one_another_see_what_the_previous_one_wrote():
+    """Every call starts while the previous one of the stream drains: a list, its length and x that the previous call has just
+    written, other ones each time, give what the same calls give one at a time."""
+    m = n = 2048
+    W = inputs.weights(m, n, seed=5, std=n ** -0.5)   # (y is about as large as x)
+    p, pr, pk = pack_on_gpu(W, 4, 128), binding.spqt_rowwise_pack(dev(W), 4, 128), binding.spqt_kqw_pack(dev(W), 6)
+    ws, wk, wsm = binding.new_workspace(m, n), binding.new_kq_workspace(pk), binding.new_gemm_small_workspace(p)
+    idx, cnt = torch.empty(n, dtype=torch.int32, device="cuda"), torch.empty(1, dtype=torch.int32, device="cuda")
+    Y = torch.empty((5, 2, m), dtype=torch.float16, device="cuda")
+    starts = dev(np.stack([inputs.activations(n, seed=80 + i) for i in range(12)]))
+
+    def chain(wait):
+        """Products whose x is the y of the call before; lists that are collected over and over into the same places."""
+        outs = []
+
+        def call(f, *a, **k):
+            r = f(*a, **k)
+            if wait:
+                torch.cuda.synchronize()
+            return r
+
+        for i, x in enumerate(starts):
+            t = 0.1 + 0.05 * (i % 5)
+            call(binding.spqt_sparsify, x, t, idx, cnt)
+            a = call(binding.spqt_sparse_gemv, p, x, idx, cnt, ws)
+            call(binding.spqt_sparsify, a, 2 * t, idx, cnt)
+            b = call(binding.spqt_kqw_sparse_gemv, pk, a, idx, cnt, wk)
+            c = call(binding.spqt_dense_gemv, p, b, ws)
+            d = call(binding.spqt_kqw_dense_gemv, pk, c, wk)
+            e = call(binding.spqt_rowwise_dense_gemv, pr, d)
+            f = call(binding.spqt_sparsify_gemv, p, e, t, ws, idx=idx, count=cnt)[0]
+            Z = Y[i % 5]
+            call(binding.spqt_dense_gemv, p, f, ws, y=Z[0])
+            call(binding.spqt_dense_gemv, p, a, ws, y=Z[1])
+            g = call(binding.spqt_sparse_gemm_small, p, Z, t, wsm, idx=idx, count=cnt)[0]
+            h = call(binding.spqt_dense_gemm_small, p, g, wsm)
+            outs += [a, b, c, d, e, f, g, h]
+        torch.cuda.synchronize()
+        return outs
+
+    want = chain(True)
+    assert all(bool(v.isfinite().all()) and float(v.float().std()) > 1e-2 for v in want)
+    for got in (chain(False), chain(False)):
+        assert all(torch.equal(a, b) for a, b in zip(want, got))

@@ -26,3 +26,20 @@ def test_waits_for_stores_of_other_ctas_acquire_at_cluster_scope():
     helpers = open(os.path.join(ROOT, "paper_2511_04477_b200", "csrc", "spqt_gemv_device.cuh")).read()
     forms = re.findall(r"mbarrier\.try_wait\.[a-z0-9_.:]*", helpers)
     assert sorted(forms) == ["mbarrier.try_wait.parity.acquire.%s.shared::cta.b64" % s for s in ("cluster", "cta")]
+
+
+def test_what_the_previous_kernel_may_write_is_not_read_as_read_only():
+    """A kernel that starts while the previous one of its stream drains reads x, lists and their lengths behind
+    griddepcontrol.wait.  A load that is declared read-only may be moved in front of it: these kernels have none but of weights."""
+    waiting = [p for p in SOURCES if "griddepcontrol.wait" in code(p)]
+    assert len(waiting) >= 6
+    for path in waiting:
+        text = code(path)
+        assert "__ldg(" not in text, path
+        kernels = re.split(r"__global__", text)[1:]
+        for kernel in kernels:
+            if "griddepcontrol.wait" not in kernel:
+                continue
+            read_only = re.findall(r"\bconst\s+\w+\s*\*\s*(?:const\s+)?__restrict__\s+(\w+)", kernel[:kernel.rindex("griddepcontrol.wait")])
+            read_only += re.findall(r"\bconst\s+[\w\s]+\*\s*(?:const\s+)?__restrict__\s+(\w+)", kernel.split("static", 1)[0])
+            assert set(read_only) <= {"codes", "meta", "records"}, (path, read_only)
