@@ -118,7 +118,7 @@ spqt_status spqt_sparsify(const void* x, int n, float t,
  *   y : fp16[m], 2-byte aligned.
  *   workspace : gemv_workspace_bytes of device memory, 16-byte aligned, zeroed
  *       ONCE by the caller before its first use; every call leaves it ready for
- *       the next.  It holds the status word that checked mode sets, and, for the shapes whose block-rows are cut into
+ *       the next.  It holds the status word (see spqt_workspace_status), the same one for every shape, and, for the shapes whose block-rows are cut into
  *       pieces that several CTAs share, the places where their sums meet, which every call leaves zero again.
  *       (Elsewhere sums travel through shared memory.)  Two calls that may overlap on the GPU therefore need two
  *       workspaces.
@@ -455,8 +455,8 @@ spqt_status spqt_set_debug(int on);
  * Reads the workspace's status word into *status_host (a host int) and waits for
  * the stream: 0 = every GEMV that used this workspace ran to completion;
  * 1 = a bounded wait expired inside a GEMV kernel (one second, for the sums of a cluster's other CTAs; that block-row of
- * y is then unspecified); 2 = checked mode found a bad index list.  The word is
- * sticky until the caller zeroes the workspace again.  Returns SPQT_OK for 0,
+ * y is then unspecified); 2 = checked mode found a bad index list.  The word is one for the calls of
+ * all shapes, and sticky until the caller zeroes the workspace again.  Returns SPQT_OK for 0,
  * SPQT_ERR_TIMEOUT for 1 and SPQT_ERR_INVALID_ARG for 2 (after writing *status_host).
  */
 spqt_status spqt_workspace_status(const void* workspace, int m, int group, int* status_host, void* stream);

@@ -33,19 +33,21 @@ inline spqt_status make_format(int m, int n, int bits, int group, Format* f)
 
 inline bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 
-// Workspace layout: [R] int32 words that are not used, one int32 status word, padded to 256 B; then the slots in which CTAs
-// that share a block-row leave their sums, 8 bytes for each of its rows between every two neighbouring CTAs.  All zero between
-// calls, so that calls of different shapes may use one workspace.  (The size is that of the first form, which had counters in
-// the words and at least one fp32 value per output row and block-row behind them.)
+// Workspace layout, the same for every shape, so that calls of different shapes may use one workspace: the status word, the last
+// one of the first 256 bytes (the others are not used); then the slots in which CTAs that share a block-row leave their sums, 8
+// bytes for each of its rows between every two neighbouring CTAs, zero between calls.  (The size is that of the first form, which
+// had counters for the block-rows and at least one fp32 value per output row and block-row behind them.)
 constexpr int kMaxPieceCtas = 160;
-inline size_t header_bytes(int R) { return (((size_t)(R + 1) * 4 + 255) / 256) * 256; }
-inline size_t slots_bytes(int group) { return (size_t)kMaxPieceCtas * (size_t)group * sizeof(unsigned long long); }
+constexpr size_t kSlotsOffset = 256, kStatusOffset = kSlotsOffset - sizeof(int);
 
 inline size_t workspace_bytes(const Format& f)
 {
-    const size_t rows = ((size_t)f.m + (size_t)f.R) * sizeof(float), slots = slots_bytes(f.group);
-    return header_bytes(f.R) + (rows > slots ? rows : slots);
+    const size_t header = (((size_t)(f.R + 1) * 4 + 255) / 256) * 256;   // (not less than kSlotsOffset)
+    const size_t rows = ((size_t)f.m + (size_t)f.R) * sizeof(float), slots = (size_t)kMaxPieceCtas * (size_t)f.group * sizeof(unsigned long long);
+    return header + (rows > slots ? rows : slots);
 }
+
+inline void* status_word(void* workspace) { return static_cast<unsigned char*>(workspace) + kStatusOffset; }
 
 extern int g_no_pdl;          // 1 = launch strictly stream-ordered (spqt_set_tuning)
 int sm_count();               // SMs of the current device (cached per device); <= 0 on error

@@ -132,7 +132,7 @@ struct GemvSmem {
 };
 
 constexpr int kPieceWarps = 16;
-constexpr unsigned kSlotMark = 0x53705174u;   // a slot that holds a sum (no status word of another shape's header looks like it)
+constexpr unsigned kSlotMark = 0x53705174u;   // a slot that holds a sum
 template <int G, int BITS, int MODE>
 struct PieceSmem {
     using Loop = PieceLoopSmem<G, BITS, MODE, kPieceWarps>;
@@ -1193,8 +1193,8 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
     ga.magic_w = 0xffffffffu / ga.warps;
     ga.magic_r = 0xffffffffu / (unsigned)f.R;
     ga.magic_p = 0xffffffffu / (unsigned)P;
-    ga.status = static_cast<unsigned*>(workspace) + f.R;
-    ga.slots = reinterpret_cast<unsigned long long*>(static_cast<unsigned char*>(workspace) + header_bytes(f.R));
+    ga.status = static_cast<unsigned*>(status_word(workspace));
+    ga.slots = reinterpret_cast<unsigned long long*>(static_cast<unsigned char*>(workspace) + kSlotsOffset);
     ga.x = static_cast<const __half*>(x);
     ga.idx = idx;
     ga.count = count;
@@ -1264,7 +1264,7 @@ static spqt_status sparse_checked(const Format& f, const void* codes, const void
 {
     if (f.n > kMaxListN) return SPQT_ERR_UNSUPPORTED;
     if (g_debug) {
-        spqt_status st = debug_check(idx, count, f.n, static_cast<int*>(workspace) + f.R, s, &count);
+        spqt_status st = debug_check(idx, count, f.n, static_cast<int*>(status_word(workspace)), s, &count);
         if (st != SPQT_OK) return st;
     }
     return gemv_dispatch<kModeList>(f, codes, meta, x, idx, count, y, workspace, s, FusedArgs{0.0f, nullptr, nullptr});
@@ -1359,7 +1359,7 @@ spqt_status spqt_sparse_gemv_static(const void* codes, const void* scale_zero,
     if (n > kMaxListN) return SPQT_ERR_UNSUPPORTED;
     // The scratch keeps whatever the previous call left: the status word and the slots must start at zero.
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (cudaMemsetAsync(scratch, 0, header_bytes(f.R) + slots_bytes(f.group), s) != cudaSuccess) return SPQT_ERR_CUDA;
+    if (cudaMemsetAsync(scratch, 0, kSlotsOffset + (size_t)kMaxPieceCtas * f.group * sizeof(unsigned long long), s) != cudaSuccess) return SPQT_ERR_CUDA;
     return sparse_checked(f, codes, scale_zero, x, idx, count, y, scratch, s);
 }
 
@@ -1376,7 +1376,7 @@ spqt_status spqt_static_status(int m, int group, int* status_host, void* stream)
     if (!status_host || m <= 0 || (group != 64 && group != 128) || m % group) return SPQT_ERR_INVALID_ARG;
     void* const scratch = static_scratch_address();
     if (scratch == nullptr) return SPQT_ERR_CUDA;
-    return read_status_word(static_cast<const int*>(scratch) + m / group, status_host, static_cast<cudaStream_t>(stream));
+    return read_status_word(static_cast<const int*>(spqt::status_word(scratch)), status_host, static_cast<cudaStream_t>(stream));
 }
 
 spqt_status spqt_autotune(const void* codes, const void* scale_zero, int m, int n, int bits, int group,
@@ -1457,7 +1457,8 @@ spqt_status spqt_set_tuning(int gemv_ctas, int reserved)
 spqt_status spqt_workspace_status(const void* workspace, int m, int group, int* status_host, void* stream)
 {
     if (!workspace || !status_host || m <= 0 || (group != 64 && group != 128) || m % group) return SPQT_ERR_INVALID_ARG;
-    return read_status_word(static_cast<const int*>(workspace) + m / group, status_host, static_cast<cudaStream_t>(stream));
+    const void* const word = static_cast<const unsigned char*>(workspace) + spqt::kStatusOffset;
+    return read_status_word(static_cast<const int*>(word), status_host, static_cast<cudaStream_t>(stream));
 }
 
 }  // extern "C"

@@ -268,8 +268,7 @@ def test_pieces_where_the_last_round_of_block_rows_leaves_sms_idle(bits, group, 
 
 @pytest.mark.parametrize("word", [1, 2])
 def test_status_words_of_other_shapes_are_not_taken_for_sums(word):
-    """Shapes that share a workspace have their status words where this one has the places of its sums; the entry point on the
-    built-in scratch clears both."""
+    """A word that is no sum, where CTAs' sums meet, does not get into y; nor does what the built-in scratch still holds."""
     bits, group, m_blocks, n = 3, 64, 33, 22001   # pieces
     p, _, _, _ = random_matrix(bits, group, m_blocks, n)
     x = dev(growing_activations(n, seed=94))
@@ -279,6 +278,26 @@ def test_status_words_of_other_shapes_are_not_taken_for_sums(word):
     ws.view(torch.int32)[64::7] = word
     assert torch.equal(binding.spqt_sparse_gemv(p, x, idx, cnt, ws), want)
     assert torch.equal(binding.spqt_sparse_gemv_static(p, x, idx, cnt, torch.empty_like(want)), want)
+
+
+def test_status_word_survives_calls_of_other_shapes():
+    """One workspace for a shape with more block-rows, whose list checked mode refuses, and one with fewer that CTAs share in pieces:
+    the status stays until the workspace is zeroed, and the sums have other places."""
+    bits, group = 3, 64
+    many, few = random_matrix(bits, group, 150, 512)[0], random_matrix(bits, group, 33, 22001)[0]
+    ws = torch.zeros(max(w.numel() for w in (binding.new_workspace(p.m, p.n, bits, group) for p in (many, few))), dtype=torch.uint8, device="cuda")
+    x = dev(growing_activations(few.n, seed=95))
+    idx, cnt = binding.spqt_sparsify(x, 0.5)
+    want = binding.spqt_sparse_gemv(few, x, idx, cnt, ws)
+    assert int(ws.count_nonzero()) == 0
+    binding.spqt_set_debug(True)
+    try:
+        binding.spqt_sparse_gemv(many, x[:512].clone(), torch.full((512,), 3, dtype=torch.int32, device="cuda"), torch.full((1,), 2, dtype=torch.int32, device="cuda"), ws)
+    finally:
+        binding.spqt_set_debug(False)
+    for _ in range(2):
+        assert binding.spqt_workspace_status(ws, many.m, group) == 2 and binding.spqt_workspace_status(ws, few.m, group) == 2
+        assert torch.equal(binding.spqt_sparse_gemv(few, x, idx, cnt, ws), want)
 
 
 @pytest.mark.parametrize("n", [1, 63, 64, 65, 2047, 2048, 2049, 4096, 4097, 8192, 16385, 32768, 32769, 49152, 49153, 65535, 65536, 65537])
