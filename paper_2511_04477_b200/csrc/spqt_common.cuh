@@ -39,11 +39,12 @@ inline bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_
 // had counters for the block-rows and at least one fp32 value per output row and block-row behind them.)
 constexpr int kMaxPieceCtas = 160;
 constexpr size_t kSlotsOffset = 256, kStatusOffset = kSlotsOffset - sizeof(int);
+inline size_t slots_bytes(int group) { return (size_t)kMaxPieceCtas * (size_t)group * sizeof(unsigned long long); }
 
 inline size_t workspace_bytes(const Format& f)
 {
     const size_t header = (((size_t)(f.R + 1) * 4 + 255) / 256) * 256;   // (not less than kSlotsOffset)
-    const size_t rows = ((size_t)f.m + (size_t)f.R) * sizeof(float), slots = (size_t)kMaxPieceCtas * (size_t)f.group * sizeof(unsigned long long);
+    const size_t rows = ((size_t)f.m + (size_t)f.R) * sizeof(float), slots = slots_bytes(f.group);
     return header + (rows > slots ? rows : slots);
 }
 
