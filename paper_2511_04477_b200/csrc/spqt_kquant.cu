@@ -220,9 +220,12 @@ struct KqSmem {
         unsigned char sums[sizeof(Sums)];
     };
     alignas(16) unsigned char area[sizeof(Area)];
-    alignas(16) uint64_t arrival;                      // first CTA of a cluster: the arrival of the other CTAs' sums
-    alignas(16) float xred[kKqMaxCluster - 1][kKqG];   // and the sums (in a smaller cluster the memory may end before the last ones)
+    alignas(16) uint64_t arrival;                      // first CTA of a cluster: the arrival of the other CTAs' sums, which lie behind
 };
+
+// with the sums of the k - 1 other CTAs of a cluster
+template <int BITS, int NW>
+constexpr int kq_smem_bytes(int k) { return (int)sizeof(KqSmem<BITS, NW>) + (k - 1) * kKqG * (int)sizeof(float); }
 
 // The rotation that brings bit `from` of both halves to bit `to`.
 __device__ __forceinline__ unsigned kq_rotate(unsigned v, int from, int to) { return __funnelshift_r(v, v, from - to); }
@@ -325,6 +328,7 @@ kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* x, cons
     using Smem = KqSmem<BITS, NW>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem& sm = *reinterpret_cast<Smem*>(smem_raw);
+    float* const xred = reinterpret_cast<float*>(smem_raw + sizeof(Smem));   // [S - 1][kKqG]
     typename Smem::Loop& lp = *reinterpret_cast<typename Smem::Loop*>(sm.area);
     typename Smem::Sums& su = *reinterpret_cast<typename Smem::Sums*>(sm.area);
     const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
@@ -333,7 +337,7 @@ kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* x, cons
     if (S > 1) {
         if (tid == 0) {
             mbar_init(&sm.arrival, 1);
-            mbar_expect(&sm.arrival, (S - 1u) * (unsigned)sizeof(sm.xred[0]));
+            mbar_expect(&sm.arrival, (S - 1u) * kKqG * (unsigned)sizeof(float));
             mbar_publish();
         }
         __syncwarp();
@@ -551,14 +555,14 @@ kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* x, cons
         // gemv_kernel; 8192 x 8192 to 6 bits dense 17.1 -> 16.5 us)
         cluster_wait();                  // (every CTA of the cluster runs)
         if (rank != 0) {
-            if (tid < kKqG) st_async_f32(cluster_map(smem_u32(&sm.xred[rank - 1][tid]), 0u), total, cluster_map(smem_u32(&sm.arrival), 0u));
+            if (tid < kKqG) st_async_f32(cluster_map(smem_u32(xred + (rank - 1u) * kKqG + tid), 0u), total, cluster_map(smem_u32(&sm.arrival), 0u));
             return;
         }
         if (tid < kKqG) {
             if (!mbar_wait_cluster(&sm.arrival, 0u)) total = __int_as_float(0x7fffffff);   // (a wait that ran out: not-a-number)
 #pragma unroll
             for (unsigned q = 0; q < kKqMaxCluster - 1; ++q)
-                if (q < S - 1u) total += sm.xred[q][tid];
+                if (q < S - 1u) total += xred[q * kKqG + tid];
         }
     }
     if (T > 1) {
@@ -631,9 +635,10 @@ static spqt_status kq_launch_mode(const void* records, int R, int n, const void*
 {
     constexpr int kAlone = 120 * 1024;   // shared memory that keeps a second CTA of 8 warps off the SM
     // (8-bit codes: two CTAs per SM have memory for the sums of a cluster of seven)
-    constexpr int kMostTwo = sizeof(KqSmem<BITS, 8>) <= 115712 ? kKqMaxCluster : kKqMaxCluster - 1;
-    constexpr int kSmem = (int)(sizeof(KqSmem<BITS, 8>) - (kKqMaxCluster - kMostTwo) * sizeof(KqSmem<BITS, 8>::xred[0])), kSmem16 = (int)sizeof(KqSmem<BITS, 16>);
+    constexpr int kMostTwo = kq_smem_bytes<BITS, 8>(kKqMaxCluster) <= 115712 ? kKqMaxCluster : kKqMaxCluster - 1;
+    constexpr int kSmem = kq_smem_bytes<BITS, 8>(kMostTwo), kSmem16 = kq_smem_bytes<BITS, 16>(kKqMaxCluster);
     static_assert(kSmem <= 115712 && kSmem16 <= 232448, "two CTAs of 8 warps per SM, or one of 16");
+    static_assert(kq_smem_bytes<BITS, 8>(kKqMaxCluster) <= kAlone, "any cluster with an SM for each CTA");
     static bool configured[64] = {};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return SPQT_ERR_CUDA;

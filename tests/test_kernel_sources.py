@@ -43,3 +43,12 @@ def test_what_the_previous_kernel_may_write_is_not_read_as_read_only():
             read_only = re.findall(r"\bconst\s+\w+\s*\*\s*(?:const\s+)?__restrict__\s+(\w+)", kernel[:kernel.rindex("griddepcontrol.wait")])
             read_only += re.findall(r"\bconst\s+[\w\s]+\*\s*(?:const\s+)?__restrict__\s+(\w+)", kernel.split("static", 1)[0])
             assert set(read_only) <= {"codes", "meta", "records"}, (path, read_only)
+
+
+def test_no_launch_has_less_shared_memory_than_the_kernel_may_assume():
+    """A kernel that sees its shared memory as one object may have any part of it read early, behind a condition or not: what a
+    launch can do without lies behind the object."""
+    sizes = [(p, m) for p in SOURCES for m in re.findall(r"sizeof\(\w*Smem<[^()]*>\)[^;]*;", code(p))]
+    assert len(sizes) >= 8
+    for path, text in sizes:
+        assert not re.search(r"sizeof\(\w*Smem<[^()]*>\)\s*-", text), (path, text)
