@@ -101,7 +101,9 @@ spqt_status spqt_unpack(const void* codes, int m, int n, int bits, int group,
  * idx[0:*count] = every k with |x_k| > t, in ascending order; *count = how many.
  * The comparison is strict and exact (fp16 widened); NaN entries are never
  * active.  idx must hold n entries.  x: fp16[n], 2-byte aligned.  idx, count:
- * int32, 4-byte aligned.  n == 0 is allowed and writes *count = 0.
+ * int32, 4-byte aligned.  n == 0 is allowed and writes *count = 0.  (*count = -1: the totals that the
+ * kernel's CTAs send one another did not arrive within its bounded waits, seconds; idx is then not to
+ * be used, and the products give not-a-number for it.  Not seen so far.)
  */
 spqt_status spqt_sparsify(const void* x, int n, float t,
                           int32_t* idx, int32_t* count, void* stream);
@@ -454,8 +456,9 @@ spqt_status spqt_set_debug(int on);
 /*
  * Reads the workspace's status word into *status_host (a host int) and waits for
  * the stream: 0 = every GEMV that used this workspace ran to completion;
- * 1 = a bounded wait expired inside a GEMV kernel (one second, for the sums of a cluster's other CTAs; that block-row of
- * y is then unspecified); 2 = checked mode found a bad index list.  The word is one for the calls of
+ * 1 = a bounded wait expired inside a GEMV kernel (seconds, for the sums of a cluster's other CTAs; that block-row of
+ * y is then not-a-number), or the list had a negative length (all of y is not-a-number); the two-level and small-batch
+ * products say the same by not-a-number alone; 2 = checked mode found a bad index list.  The word is one for the calls of
  * all shapes, and sticky until the caller zeroes the workspace again.  Returns SPQT_OK for 0,
  * SPQT_ERR_TIMEOUT for 1 and SPQT_ERR_INVALID_ARG for 2 (after writing *status_host).
  */

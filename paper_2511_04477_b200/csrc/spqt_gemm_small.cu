@@ -131,7 +131,12 @@ gemm_small_kernel(const SmallArgs a)
 
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (!DIRECT && a.idx) take_part((int)ld_global_u32(a.count));
+    bool lost = false;                   // (a list without a length, see kListLost)
+    if (!DIRECT && a.idx) {
+        const int count = (int)ld_global_u32(a.count);
+        lost = count < 0;
+        take_part(max(count, 0));
+    }
 
     float acc[SP][4][4];
     unsigned long long zl[ROWS / 2], scale[ROWS / 2];   // pairs of rows
@@ -379,7 +384,10 @@ gemm_small_kernel(const SmallArgs a)
     // the cluster before and after reading each other's shared memory took 0.5 to 0.9 us longer: 4096 x 14336, 8 rows dense 13.1
     // against 12.1 us, 1024 x 4096, 4 rows dense 3.8 against 3.3).
     if (S > 1) cluster_wait();           // (every CTA of the cluster runs)
-    if (tid >= groups) return;
+    if (tid >= groups) {
+        if (S > 1) cluster_sent();
+        return;
+    }
     const int b = tid / (G / 4), j = tid % (G / 4) * 4;
     float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     float z = 0.0f;
@@ -401,9 +409,10 @@ gemm_small_kernel(const SmallArgs a)
         if (owner != split) {
             const unsigned dst = smem_u32(&sm.others[split * stride + tid - groups * owner / S]);
             st_async_f32x4(cluster_map(dst, (unsigned)owner), v, cluster_map(smem_u32(&sm.arrival), (unsigned)owner));
-            return;
         }
-        const float start = mbar_wait_cluster(&sm.arrival, 0u) ? 0.0f : __int_as_float(0x7fffffff);   // (a wait that ran out: not-a-number)
+        cluster_sent();
+        if (owner != split) return;
+        const float start = mbar_wait_cluster(&sm.arrival, 0u) ? 0.0f : __int_as_float(0x7fffffff);
         float4 sum = make_float4(start, start, start, start);
 #pragma unroll
         for (int q = 0; q < kSmallMaxSplit; ++q) {
@@ -418,10 +427,10 @@ gemm_small_kernel(const SmallArgs a)
         v = sum;
     }
     __half* const y = a.Y + (size_t)b * a.ldy + (size_t)r * G + j;
-    y[0] = __float2half_rn(v.x);
-    y[1] = __float2half_rn(v.y);
-    y[2] = __float2half_rn(v.z);
-    y[3] = __float2half_rn(v.w);
+    y[0] = __float2half_rn(not_a_number_if(lost, v.x));
+    y[1] = __float2half_rn(not_a_number_if(lost, v.y));
+    y[2] = __float2half_rn(not_a_number_if(lost, v.z));
+    y[3] = __float2half_rn(not_a_number_if(lost, v.w));
 }
 
 // Workspace: one word per block-row (zero, kept for callers that look at it), then the gathered x: 16 bytes per list

@@ -552,6 +552,11 @@ gemv_kernel(const GemvArgs a)
     Scan<NW> scan(sm.area, a.thr, n, lane, warp);            // (fused calls only)
     int count = n;
     if (LIST) count = (int)ld_global_u32(a.count);
+    const bool lost = LIST && count < 0;
+    if (lost) {
+        count = 0;
+        if (blockIdx.x == 0 && tid == 0) atomicExch(a.status, 1u);
+    }
     if (FUSED) {
         count = scan.scan_x(a.x);
         if (blockIdx.x == 0 && tid == 0) *a.count_out = count;
@@ -683,12 +688,14 @@ gemv_kernel(const GemvArgs a)
         // senders wait for their stores and everybody for everybody, took 1.2 to 1.3 us from the warps' sums to y, this 0.4 to
         // 0.5 (1024 x 4096 at 50 % 4.1 -> 3.6 us, 4096 x 4096 4.8 -> 4.4, with the list 4.0 -> 3.6).
         cluster_wait();                  // (every CTA of the cluster runs)
-        if (rank != 0) {
-            if (tid < G / 2) st_async_f32x2(cluster_map(smem_u32(&sm.xred[rank - 1][tid]), 0u), total[0], total[1], cluster_map(smem_u32(&sm.arrival), 0u));
-            return;
-        }
+        if (rank != 0 && tid < G / 2) st_async_f32x2(cluster_map(smem_u32(&sm.xred[rank - 1][tid]), 0u), total[0], total[1], cluster_map(smem_u32(&sm.arrival), 0u));
+        cluster_sent();
+        if (rank != 0) return;
         if (tid < G / 2) {
-            if (!mbar_wait_cluster(&sm.arrival, 0u)) atomicExch(a.status, 1u);   // (a wait that ran out)
+            if (!mbar_wait_cluster(&sm.arrival, 0u)) {
+                atomicExch(a.status, 1u);
+                total[0] = total[1] = __int_as_float(0x7fffffff);
+            }
 #pragma unroll
             for (int q = 0; q < kMaxSplit - 1; ++q)
                 if (q < a.splits - 1) {
@@ -699,8 +706,8 @@ gemv_kernel(const GemvArgs a)
         }
     }
     if (tid < G / 2) {
-        a.y[(size_t)r * G + tid] = __float2half_rn(total[0]);
-        a.y[(size_t)r * G + tid + G / 2] = __float2half_rn(total[1]);
+        a.y[(size_t)r * G + tid] = __float2half_rn(not_a_number_if(lost, total[0]));
+        a.y[(size_t)r * G + tid + G / 2] = __float2half_rn(not_a_number_if(lost, total[1]));
     }
 }
 
@@ -758,6 +765,11 @@ gemv_pieces_kernel(const GemvArgs a)
     Scan<NW> scan(sm.area, a.thr, n, lane, warp);            // (fused calls only)
     int count = n;
     if (LIST) count = (int)ld_global_u32(a.count);
+    const bool lost = LIST && count < 0;
+    if (lost) {
+        count = 0;
+        if (blockIdx.x == 0 && tid == 0) atomicExch(a.status, 1u);
+    }
     if (FUSED) count = scan.scan_x(a.x);
     const unsigned units = (unsigned)(count + 7) >> 3;
     int first = 8 * (int)magic_div(part0 * units, N, a.magic_w), end = 8 * (int)magic_div(part1 * units, N, a.magic_w);
@@ -913,7 +925,7 @@ gemv_pieces_kernel(const GemvArgs a)
                 __stcg(slot, 0ull);
             }
         }
-        if (mine) a.y[(size_t)r * G + j] = __float2half_rn(v);
+        if (mine) a.y[(size_t)r * G + j] = __float2half_rn(not_a_number_if(lost, v));
     }
 }
 

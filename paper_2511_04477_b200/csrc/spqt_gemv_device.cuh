@@ -77,8 +77,16 @@ __device__ __forceinline__ bool mbar_wait_scope(uint64_t* bar, unsigned parity)
 }
 // for arrivals of this CTA's threads
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity) { return mbar_wait_scope<false>(bar, parity); }
-// for asynchronous stores of other CTAs of the cluster
-__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, unsigned parity) { return mbar_wait_scope<true>(bar, parity); }
+// For asynchronous stores of other CTAs of the cluster, by threads that have called cluster_sent() as every thread of the cluster
+// does.  If they have not come within the bound, a CTA that left now would leave stores on their way to memory that has ended:
+// the hardware's barrier tells when all CTAs have sent theirs (no later than the kernel could end in any case: none of them waits
+// for another one before that), and then they have a second bound to arrive.  False: stores are lost.
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, unsigned parity)
+{
+    if (mbar_wait_scope<true>(bar, parity)) return true;
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    return mbar_wait_scope<true>(bar, parity);
+}
 
 // ---- asynchronous copies
 __device__ __forceinline__ void cp_async_16(unsigned smem_dst, const void* gmem_src)
@@ -191,6 +199,12 @@ __device__ __forceinline__ void cluster_wait()
 {
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// By every thread of the cluster, once, between the stores that it sends to other CTAs, if any, and its wait for theirs, if any (see
+// mbar_wait_cluster; nobody waits here).
+__device__ __forceinline__ void cluster_sent()
+{
+    asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
+}
 // address of the same shared-memory location in the CTA of the given rank
 __device__ __forceinline__ unsigned cluster_map(unsigned smem_addr, unsigned rank)
 {
@@ -217,6 +231,12 @@ __device__ __forceinline__ void st_async_f32(unsigned addr, float v, unsigned ba
 {
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(addr), "f"(v), "r"(bar) : "memory");
 }
+
+// The length that the index collection gives a list whose places it could not find (totals of its warps were lost, see
+// mbar_wait_cluster; the warps concerned write no entry).  The products take a negative length for an empty list and give
+// not-a-number.
+constexpr int kListLost = -1;
+__device__ __forceinline__ float not_a_number_if(bool lost, float v) { return lost ? __int_as_float(0x7fffffff) : v; }
 
 // Two fp32 lanes in one 64-bit register, the operand form of the packed FMA.
 __device__ __forceinline__ unsigned long long pack2(float lo, float hi)

@@ -364,7 +364,12 @@ kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* x, cons
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-    if (LIST) take_part((int)ld_global_u32(count_ptr));
+    bool lost = false;                   // (a list without a length, see kListLost)
+    if (LIST) {
+        const int count = (int)ld_global_u32(count_ptr);
+        lost = count < 0;
+        take_part(max(count, 0));
+    }
 
     constexpr int kAhead = 2;            // (a third costs registers: 28672 x 4096 to 4 bits 13.2 against 12.8 us, to 8 bits 16.8 against 16.3)
     int coming[kAhead], ahead = first;   // list: the columns of the chunks the copies come to next
@@ -554,12 +559,11 @@ kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* x, cons
         // the other CTAs send their sums to the first one's shared memory, which counts the bytes and adds them in CTA order (see
         // gemv_kernel; 8192 x 8192 to 6 bits dense 17.1 -> 16.5 us)
         cluster_wait();                  // (every CTA of the cluster runs)
-        if (rank != 0) {
-            if (tid < kKqG) st_async_f32(cluster_map(smem_u32(xred + (rank - 1u) * kKqG + tid), 0u), total, cluster_map(smem_u32(&sm.arrival), 0u));
-            return;
-        }
+        if (rank != 0 && tid < kKqG) st_async_f32(cluster_map(smem_u32(xred + (rank - 1u) * kKqG + tid), 0u), total, cluster_map(smem_u32(&sm.arrival), 0u));
+        cluster_sent();
+        if (rank != 0) return;
         if (tid < kKqG) {
-            if (!mbar_wait_cluster(&sm.arrival, 0u)) total = __int_as_float(0x7fffffff);   // (a wait that ran out: not-a-number)
+            if (!mbar_wait_cluster(&sm.arrival, 0u)) total = __int_as_float(0x7fffffff);
 #pragma unroll
             for (unsigned q = 0; q < kKqMaxCluster - 1; ++q)
                 if (q < S - 1u) total += xred[q * kKqG + tid];
@@ -585,7 +589,7 @@ kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* x, cons
             for (unsigned t = 0; t < T; ++t) __stcg(row_sums + t * kKqG + tid, 0.0f);   // (a loop of its own: the loads go together)
         }
     }
-    if (tid < kKqG) y[(size_t)r * kKqG + tid] = __float2half_rn(total);
+    if (tid < kKqG) y[(size_t)r * kKqG + tid] = __float2half_rn(not_a_number_if(lost, total));
 }
 
 // ---------------------------------------------------------------- host side

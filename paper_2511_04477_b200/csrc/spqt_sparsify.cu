@@ -43,21 +43,22 @@ struct ClusterTotals {
         cluster_arrive();
         cluster_wait();                  // every CTA of the cluster runs, and its barrier is ready
     }
-    // by every warp `me` of the cluster: what the warps before it have, and all of them (none, if the wait ran out: the
-    // count is 0 then)
-    __device__ __forceinline__ void exchange(int me, int mine, int lane, int ctas, int& below, int& all)
+    // by every warp `me` of the cluster: what the warps before it have, and all of them; false if that is lost
+    __device__ __forceinline__ bool exchange(int me, int mine, int lane, int ctas, int& below, int& all)
     {
         if (lane < ctas) st_async_u32(cluster_map(smem_u32(&total[me]), (unsigned)lane), (unsigned)mine, cluster_map(smem_u32(&arrival), (unsigned)lane));
-        const bool there = mbar_wait_cluster(&arrival, 0u);
+        cluster_sent();
+        const bool there = __all_sync(0xffffffffu, mbar_wait_cluster(&arrival, 0u));
         unsigned b = 0, a = 0;
 #pragma unroll
         for (int w = 0; w < WARPS; w += 32) {
-            const unsigned c = there ? (unsigned)total[w + lane] : 0u;
+            const unsigned c = (unsigned)total[w + lane];
             a += c;
             b += w + lane < me ? c : 0u;
         }
         below = (int)__reduce_add_sync(0xffffffffu, b);
         all = (int)__reduce_add_sync(0xffffffffu, a);
+        return there;
     }
 };
 
@@ -111,8 +112,9 @@ sparsify_words_kernel(const __half* x, int n, unsigned short thr_bits, int32_t* 
     }
     int base, all;
     if (CLUSTER) {
-        totals.exchange(me, total, lane, kClusterCtas, base, all);
-        if (me == 0 && lane == 0) *count = all;
+        const bool there = totals.exchange(me, total, lane, kClusterCtas, base, all);
+        if ((me == 0 || !there) && lane == 0) *count = there ? all : kListLost;
+        if (!there) return;
     } else {
         if (lane == 0) totals.total[warp] = total;
         __syncthreads();
@@ -250,8 +252,9 @@ sparsify_rows_kernel(const unsigned short* X, int ldx, int batch, int n, float t
     }
     const int me = (int)rank * kRowsWarps + warp;
     int base, all;
-    totals.exchange(me, total, lane, nctas, base, all);
-    if (me == 0 && lane == 0) *count = all;
+    const bool there = totals.exchange(me, total, lane, nctas, base, all);
+    if ((me == 0 || !there) && lane == 0) *count = there ? all : kListLost;
+    if (!there) return;
     for (int g0 = 0; g0 < groups; g0 += kKeepGroups) {
         if (groups > kKeepGroups) load(g0);
 #pragma unroll

@@ -300,6 +300,24 @@ def test_status_word_survives_calls_of_other_shapes():
         assert torch.equal(binding.spqt_sparse_gemv(few, x, idx, cnt, ws), want)
 
 
+@pytest.mark.parametrize("length", [-1, -9, -2 ** 31])
+def test_list_without_a_length_gives_not_a_number(length):
+    """What the index collection leaves if it finds no places: block-rows in clusters, whole, in pieces, and of the two-level format
+    in one cluster and in several; the next call is as if nothing had been."""
+    cnt = torch.full((1,), length, dtype=torch.int32, device="cuda")
+    for bits, group, m_blocks, n in [(4, 128, 8, 4096), (4, 64, 300, 512), (3, 64, 33, 22001)]:
+        p = random_matrix(bits, group, m_blocks, n)[0]
+        ws, x, idx = binding.new_workspace(p.m, n, bits, group), dev(inputs.activations(n, seed=96)), torch.zeros(n, dtype=torch.int32, device="cuda")
+        assert bool(binding.spqt_sparse_gemv(p, x, idx, cnt, ws).isnan().all())
+        assert binding.spqt_workspace_status(ws, p.m, group) == 1
+        assert bool((binding.spqt_sparse_gemv(p, x, idx, cnt * 0, ws) == 0).all())
+    for bits, m_blocks, n in [(4, 8, 512), (8, 4, 28672), (5, 300, 64)]:
+        p = binding.spqt_kqw_pack(dev(inputs.weights(256 * m_blocks, n, seed=6)), bits)
+        ws, x, idx = binding.new_kq_workspace(p), dev(inputs.activations(n, seed=97)), torch.zeros(n, dtype=torch.int32, device="cuda")
+        assert bool(binding.spqt_kqw_sparse_gemv(p, x, idx, cnt, ws).isnan().all()) and int(ws.count_nonzero()) == 0
+        assert bool((binding.spqt_kqw_sparse_gemv(p, x, idx, cnt * 0, ws) == 0).all())
+
+
 @pytest.mark.parametrize("n", [1, 63, 64, 65, 2047, 2048, 2049, 4096, 4097, 8192, 16385, 32768, 32769, 49152, 49153, 65535, 65536, 65537])
 def test_index_collection_at_word_and_cluster_edges(n):
     """One CTA, a cluster with 1 to 16 words per lane, and beyond; x on an odd boundary too; entries and thresholds that are

@@ -52,3 +52,32 @@ def test_no_launch_has_less_shared_memory_than_the_kernel_may_assume():
     assert len(sizes) >= 8
     for path, text in sizes:
         assert not re.search(r"sizeof\(\w*Smem<[^()]*>\)\s*-", text), (path, text)
+
+
+def test_a_cta_whose_bounded_wait_ran_out_stays_until_the_others_have_sent():
+    """Every thread says that it has sent before any waits, a late wait is for that first and then for the data, and nobody
+    takes an answer for granted."""
+    helpers = code(os.path.join(ROOT, "paper_2511_04477_b200", "csrc", "spqt_gemv_device.cuh"))
+    body = helpers[helpers.index("bool mbar_wait_cluster("):]
+    body = body[:body.index("\n}")]
+    assert re.search(r"mbar_wait_scope<true>.*barrier\.cluster\.wait.*mbar_wait_scope<true>", body, flags=re.S)
+    for path in SOURCES:
+        text = code(path)
+        if not path.endswith(".cu") or "st_async_" not in text:
+            continue
+        for wait in re.finditer(r"mbar_wait_cluster\(", text):
+            before = text[:wait.start()]
+            assert before.rindex("cluster_sent();") > before.rindex("st_async_"), path
+            assert re.search(r"[!=,(]\s*$", before), (path, "an answer that nobody looks at")
+
+
+def test_a_list_without_a_length_is_no_list():
+    """The index collection leaves no length where totals were lost, and the products that take a list look for that."""
+    csrc = os.path.join(ROOT, "paper_2511_04477_b200", "csrc")
+    collect = code(os.path.join(csrc, "spqt_sparsify.cu"))
+    assert len(re.findall(r"there \? all : kListLost", collect)) == collect.count("totals.exchange(") == len(re.findall(r"if \(!there\) return;", collect))
+    for name in ("spqt_gemv.cu", "spqt_kquant.cu", "spqt_gemm_small.cu"):
+        text = code(os.path.join(csrc, name))
+        reads = len(re.findall(r"ld_global_u32\((?:a\.count|count_ptr)\)", text))
+        assert reads >= 1 and len(re.findall(r"lost = (?:LIST && )?count < 0;", text)) == reads, name
+        assert "not_a_number_if(lost" in text, name
