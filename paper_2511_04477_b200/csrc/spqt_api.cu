@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(256) fetch_x_kernel(FetchList fl)
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const int i = i0 + j * 256 + tid;
-                v[j] = ld_global_v4(s4 + min(i, nv - 1));   // (no load behind a condition: they go together)
+                v[j] = ld_global_v4_if(i < nv, s4 + i);   // (not one more than needed: the bus is what takes the time)
             }
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
@@ -60,9 +60,17 @@ __global__ void __launch_bounds__(256) fetch_x_kernel(FetchList fl)
                 if (i < nv) d4[i] = v[j];
             }
         }
-        for (int i = (nv << 3) + tid; i < n; i += 256) dst[i] = (unsigned short)ld_global_u16(src + i);
+        const int i = (nv << 3) + tid;
+        if (i < n) dst[i] = (unsigned short)ld_global_u16(src + i);
     } else {
-        for (int i = tid; i < n; i += 256) dst[i] = (unsigned short)ld_global_u16(src + i);
+        for (int i0 = 0; i0 < n; i0 += 256 * 8) {
+            unsigned v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[j] = ld_global_u16_if(i0 + j * 256 + tid < n, src + i0 + j * 256 + tid);
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (i0 + j * 256 + tid < n) dst[i0 + j * 256 + tid] = (unsigned short)v[j];
+        }
     }
 }
 

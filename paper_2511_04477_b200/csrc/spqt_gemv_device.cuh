@@ -128,6 +128,13 @@ __device__ __forceinline__ uint4 ld_global_v4(const void* p)
     asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
     return v;
 }
+__device__ __forceinline__ uint4 ld_global_v4_if(bool on, const void* p)   // (or zeros; see ld_global_u16_if)
+{
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %5, 0;\n\t@p ld.global.v4.u32 {%0, %1, %2, %3}, [%4];\n\t}"
+                 : "+r"(v.x), "+r"(v.y), "+r"(v.z), "+r"(v.w) : "l"(p), "r"((unsigned)on) : "memory");
+    return v;
+}
 __device__ __forceinline__ unsigned ld_global_u32(const void* p)
 {
     unsigned v;
