@@ -131,10 +131,10 @@ gemm_small_kernel(const SmallArgs a)
 
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    bool lost = false;                   // (a list without a length, see kListLost)
+    float nothing = 0.0f;                // what the sums of x*zero begin with: not-a-number for a list without a length (see kListLost)
     if (!DIRECT && a.idx) {
         const int count = (int)ld_global_u32(a.count);
-        lost = count < 0;
+        nothing = not_a_number_if(count < 0, 0.0f);
         take_part(max(count, 0));
     }
 
@@ -146,7 +146,7 @@ gemm_small_kernel(const SmallArgs a)
         for (int i = 0; i < 16; ++i) acc[s][i >> 2][i & 3] = 0.0f;
 #pragma unroll
     for (int b = 0; b < ROWS / 2; ++b) {
-        zl[b] = 0ull;
+        zl[b] = pack2(nothing, nothing);
         scale[b] = pack2(kMmaNoScale, kMmaNoScale);
     }
 
@@ -427,10 +427,10 @@ gemm_small_kernel(const SmallArgs a)
         v = sum;
     }
     __half* const y = a.Y + (size_t)b * a.ldy + (size_t)r * G + j;
-    y[0] = __float2half_rn(not_a_number_if(lost, v.x));
-    y[1] = __float2half_rn(not_a_number_if(lost, v.y));
-    y[2] = __float2half_rn(not_a_number_if(lost, v.z));
-    y[3] = __float2half_rn(not_a_number_if(lost, v.w));
+    y[0] = __float2half_rn(v.x);
+    y[1] = __float2half_rn(v.y);
+    y[2] = __float2half_rn(v.z);
+    y[3] = __float2half_rn(v.w);
 }
 
 // Workspace: one word per block-row (zero, kept for callers that look at it), then the gathered x: 16 bytes per list

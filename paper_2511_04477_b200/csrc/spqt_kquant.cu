@@ -364,10 +364,10 @@ kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* x, cons
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-    bool lost = false;                   // (a list without a length, see kListLost)
+    float nothing = 0.0f;                // what the sums of x*(dmin*m) begin with: not-a-number for a list without a length (see kListLost)
     if (LIST) {
         const int count = (int)ld_global_u32(count_ptr);
-        lost = count < 0;
+        nothing = not_a_number_if(count < 0, 0.0f);
         take_part(max(count, 0));
     }
 
@@ -428,7 +428,7 @@ kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* x, cons
 #pragma unroll
     for (int i = 0; i < 64; ++i) acc[i >> 2][i & 3] = 0.0f;
     float scale = kMmaNoScale, regain = 1.0f;
-    unsigned long long zl[2] = {0ull, 0ull}, zn[2] = {0ull, 0ull}, am[2], pm[2];   // pairs of blocks
+    unsigned long long zl[2] = {pack2(nothing, nothing), pack2(nothing, nothing)}, zn[2] = {0ull, 0ull}, am[2], pm[2];   // pairs of blocks
     auto prepare = [&](unsigned st, unsigned xb) -> bool {
         const uint4 f = lds_v4(st + (unsigned)(e * REC + NCB));
         const unsigned sc = lane < 16 ? f.x : __funnelshift_r(f.x, f.y, 24), mn = lane < 16 ? __funnelshift_r(f.y, f.z, 16) : f.z >> 8;
@@ -589,7 +589,7 @@ kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* x, cons
             for (unsigned t = 0; t < T; ++t) __stcg(row_sums + t * kKqG + tid, 0.0f);   // (a loop of its own: the loads go together)
         }
     }
-    if (tid < kKqG) y[(size_t)r * kKqG + tid] = __float2half_rn(not_a_number_if(lost, total));
+    if (tid < kKqG) y[(size_t)r * kKqG + tid] = __float2half_rn(total);
 }
 
 // ---------------------------------------------------------------- host side
