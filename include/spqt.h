@@ -222,14 +222,19 @@ spqt_status spqt_sparse_linear_host_async(const void* codes, const void* scale_z
 /*
  * A token step recorded once and replayed: the host-buffer linears of a step (each described like the
  * arguments of spqt_sparse_linear_host_async: same meaning and alignment of every field) are captured
- * into one CUDA graph (in order where one writes a buffer that another uses; otherwise in branches that may run
- * at the same time) -- the transfer of every x from its x_host (all of them at the head of the
+ * into one CUDA graph (in branches that may run at the same time, or in the order given, see below) -- the transfer of every x from its x_host (all of them at the head of the
  * step), per linear the launch that collects the indices and multiplies, and the way y reaches y_host -- so
  * that a step costs the host one launch call.
  *   spqt_host_step_create  : builds the graph (allocates host-side CUDA objects; not a hot-path call;
  *                            nothing runs on the device).  The pointers, shapes and thresholds are fixed
  *                            from here on; the CONTENTS of the x_host buffers are read at every launch.
- *                            The linears must not share staging buffers or workspaces; x_host and y_host
+ *                            Linears that are to run at the same time have staging buffers, workspaces
+ *                            and y_host of their own.  If any two overlap in y_host, y_dev, idx_dev, count_dev
+ *                            or workspace (or one's y_host, y_dev, .. in what another reads), by the addresses
+ *                            given here, all linears of the step run one after the other in the order given.
+ *                            That does not hold for x: every x_dev is filled from its x_host at the head of the
+ *                            step, so linears must not share an x_dev, and no x_host sees a y_host of the
+ *                            same step.  x_host and y_host
  *                            must be pinned memory (a copy from pageable memory cannot be recorded:
  *                            SPQT_ERR_CUDA).  Returns a handle
  *                            in *step; SPQT_ERR_CUDA if the capture fails, the failing linear's status if

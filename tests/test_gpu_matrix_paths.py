@@ -338,8 +338,8 @@ def test_index_collection_at_word_and_cluster_edges(n):
 
 @pytest.mark.parametrize("shared", [False, True])
 def test_recorded_step_in_branches(shared):
-    """More linears than a step has branches, of all formats, one with a list of its own launch; with buffers in common the
-    linears keep their order."""
+    """More linears than a step has branches, of all formats, one with a list of its own launch; also where linears write their
+    lists to the same place."""
     sizes = [(4, 128, 8, 512), (3, 64, 33, 1030), (4, 64, 149, 260), (3, 128, 5, 2049), (4, 128, 2, 33000), (4, 128, 40, 300), (3, 64, 150, 4501)]
     linears = []
     for i, (bits, group, m_blocks, n) in enumerate(sizes):
@@ -408,3 +408,31 @@ def test_calls_behind_one_another_see_what_the_previous_one_wrote():
     assert all(bool(v.isfinite().all()) and float(v.float().std()) > 1e-2 for v in want)
     for got in (chain(False), chain(False)):
         assert all(torch.equal(a, b) for a, b in zip(want, got))
+
+
+@pytest.mark.parametrize("shared", ["idx", "count", "workspace", "y_host"])
+def test_recorded_step_keeps_the_order_of_linears_with_a_buffer_in_common(shared):
+    """Linear 5, whose predecessors in a branch of its own would be quick, has a buffer in common with linear 4, which a large one
+    would hold up: what the buffer holds in the end, and what the linears read from it meanwhile, is as in the order given."""
+    sizes = [(4, 128, 400, 8192)] + 3 * [(4, 128, 2, 256)] + 2 * [(3, 64, 33, 33001)] + [(4, 64, 3, 300)]
+    linears = [binding.HostLinear(random_matrix(*size)[0]) for size in sizes]
+    setattr(linears[5], shared, getattr(linears[4], shared))
+    ts = [0.6] * 4 + [1.5, 0.3, 0.6]
+    xs = [inputs.activations(h.p.n, seed=110 + i) for i, h in enumerate(linears)]
+    for h, x in zip(linears, xs):
+        h.x_host.copy_(torch.from_numpy(x))
+    step = binding.HostStep(linears, ts)
+    for _ in range(5):
+        for h in linears:
+            h.y_host.zero_()
+        step.launch()
+        torch.cuda.synchronize()
+        for i, (h, x, t) in enumerate(zip(linears, xs, ts)):
+            y, idx, cnt = binding.spqt_sparsify_gemv(h.p, dev(x), t, binding.new_workspace(h.p.m, h.p.n, h.p.bits, h.p.group))
+            if i != 4 or shared != "y_host":
+                assert torch.equal(y.cpu(), h.y_host), i
+            if i != 4 or shared != "count":
+                assert int(h.count) == int(cnt), i
+            if i != 4 or shared != "idx":
+                assert torch.equal(h.idx[:int(cnt)], idx[:int(cnt)]), i
+            assert int(h.workspace.count_nonzero()) == 0
