@@ -534,7 +534,13 @@ static spqt_status launch_small(const Format& f, SmallArgs a, cudaStream_t s)
     // SM at most where two are alone: 9216 x 2048, 8 rows 7.1 us on 3, 5.3 on 2; 6912 x 8192 15.0 on 5, 12.7 on 4), and with a long x
     // clusters of four in more than one wave rather than one or two CTAs (11776 x 8192, 8 rows 24.0 on 3, 23.3 on 1, 19.3 on 4).  Over 297
     // sizes the choice is 2 % slower than the best cluster, the largest that fits was 7 %.
+    // Nothing keeps the CTAs of a cluster that were counted with an SM each from sharing some: a launch that lets a second CTA onto its
+    // SMs starts earlier, which gains more as long as the device spreads the clusters.  It does not where they fill its parts: four
+    // from a fourth cluster in one of eight parts on, six from a second one in all of them (2048 x 8192, 8 rows on 16 clusters of
+    // 6: 8.4 us, 6.9 with all shared memory; 3328 x 3072, 4 rows on 26 of 4: 4.2 / 3.9; but 1920 x 4096, 4 rows on 15 of 8: 3.4 / 3.75,
+    // 2816 x 4096 on 22 of 5 4.2 / 4.3, 5120 x 2048 on 40 of 3 3.7 / 4.0, 9216 x 2048, 8 rows on 72 of 2 5.2 / 5.4).
     int S = 1;
+    bool alone = false;
     if (DIRECT || !a.idx) {
         float least = 0.0f;
         for (int k = 1; k <= kSmallMaxSplit && (k == 1 || f.n >= 512 * k); ++k) {
@@ -542,7 +548,8 @@ static spqt_status launch_small(const Format& f, SmallArgs a, cudaStream_t s)
             const int one = k == 1 ? sms : small_max_clusters<G, BITS, ROWS, DIRECT>(k, true, sms, dev);
             const int two = k == 1 ? 2 * sms : small_max_clusters<G, BITS, ROWS, DIRECT>(k, false, sms, dev);
             float load = 0.0f;                // of an SM, in block-rows
-            if (even ? f.R <= one : 10 * f.R <= 9 * one) load = 1.0f / k;
+            const bool apart = even ? f.R <= one : 10 * f.R <= 9 * one;
+            if (apart) load = 1.0f / k;
             else if (k == 2 && f.n < 8192) continue;   // (two halves on the busiest SMs: no less than a whole)
             else if (even ? f.R <= two : 25 * f.R <= 24 * two || (k >= 6 && f.n >= 8192 && f.R < two)) load = 1.6f / k;
             else if (k == 4 && f.n >= 8192 && 2 * f.R > sms && f.R <= sms) load = 2.0f * f.R / (4.0f * two);
@@ -550,6 +557,7 @@ static spqt_status launch_small(const Format& f, SmallArgs a, cudaStream_t s)
             if (k == 1 || load < least) {
                 least = load;
                 S = k;
+                alone = apart && ((k == 4 && 4 * f.R > 3 * one) || (k == 6 && 11 * f.R >= 8 * one));
             }
         }
     } else {
@@ -561,7 +569,7 @@ static spqt_status launch_small(const Format& f, SmallArgs a, cudaStream_t s)
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(S, f.R);
     cfg.blockDim = dim3(kSmallThreads);
-    cfg.dynamicSmemBytes = smem;
+    cfg.dynamicSmemBytes = alone ? kSmallAlone : smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;

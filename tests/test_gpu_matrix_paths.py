@@ -43,6 +43,11 @@ def test_small_batch_at_chunk_part_and_split_edges(bits, group, m_blocks, n, bat
         check_y(Ys.cpu().numpy()[b], Ys_ref[b], bound[b], "row %d" % b)
 
 
+@pytest.mark.parametrize("bits,group,m_blocks,n,batch", [(4, 128, 16, 3072, 8), (3, 64, 19, 3080, 3), (4, 64, 25, 2055, 6), (3, 128, 33, 2048, 2)])
+def test_small_batch_in_clusters_with_an_sm_for_each_cta(bits, group, m_blocks, n, batch):
+    test_small_batch_at_chunk_part_and_split_edges(bits, group, m_blocks, n, batch)
+
+
 def share_not_nearest(y, exact):
     """Share of the outputs that are not the fp16 nearest to the exact value.  A value lands on the other side of a rounding
     boundary with a probability of its error before the rounding over the spacing of fp16: the mean error in those units."""
