@@ -174,13 +174,13 @@ __device__ __forceinline__ unsigned magic_div(unsigned v, unsigned d, unsigned m
 }
 
 // Hints only (no data is consumed before the wait for the previous kernel, and a prefetched line is as coherent as any other in
-// L2), given while that kernel drains and the memory has little to do.  x, and a given list: a few CTAs do it for all.
-template <int MODE, int THREADS>
+// L2), given while that kernel drains and the memory has little to do.  x: a few CTAs do it for all.  (Not a given list: how much
+// of it there is to read is known only behind the wait.)
+template <int THREADS>
 __device__ __forceinline__ void prefetch_inputs(const GemvArgs& a, int tid)
 {
     if ((blockIdx.x & 15) != 0) return;
     prefetch_l2(a.x, 2 * (size_t)a.n, tid, THREADS);
-    if (MODE == kModeList) prefetch_l2(a.idx, 4 * (size_t)a.n, tid, THREADS);
 }
 
 // ---------------------------------------------------------------- copies
@@ -523,7 +523,7 @@ gemv_kernel(const GemvArgs a)
     // the slices of the list this CTA works on: first_part .. last_part - 1 of `parts`
     const unsigned parts = (unsigned)a.splits, first_part = rank, last_part = KIND == kCluster ? rank + 1u : parts;
 
-    prefetch_inputs<MODE, kThreads>(a, tid);
+    prefetch_inputs<kThreads>(a, tid);
     // constants of the loop that need no data
     const typename MmaStage<G, BITS>::Lane ll(lane);
     const unsigned stage0 = smem_u32(&lp.stage[warp][0]);
@@ -738,7 +738,7 @@ gemv_pieces_kernel(const GemvArgs a)
     const int n = a.n;
     const unsigned R = (unsigned)a.R, N = a.warps, cta = blockIdx.x;
 
-    prefetch_inputs<MODE, kThreads>(a, tid);
+    prefetch_inputs<kThreads>(a, tid);
     // (a hint too: the slots between this CTA and the one before it, which the code stream of other calls has driven from L2; an
     // exchange that had to fetch them from a busy memory took 1 to 2 us longer)
     if (cta > 0u && tid < G / 16) asm volatile("prefetch.global.L2::evict_last [%0];" ::"l"(a.slots + (size_t)(cta - 1u) * G + 16 * tid));

@@ -80,3 +80,10 @@ def test_a_list_without_a_length_is_no_list():
         text = code(os.path.join(csrc, name))
         reads = len(re.findall(r"ld_global_u32\((?:a\.count|count_ptr)\)", text))
         assert reads >= 1 and len(re.findall(r"lost = LIST && count < 0;|not_a_number_if\(count < 0, ", text)) == reads, name
+
+
+def test_hints_stay_within_buffers_whose_size_is_known():
+    """A given list has as many entries as its length says, which is read behind the wait; hints are given before it."""
+    for path in SOURCES:
+        for what in re.findall(r"\bprefetch_l2\(([^,]*),", code(path)):
+            assert "idx" not in what, (path, what)
