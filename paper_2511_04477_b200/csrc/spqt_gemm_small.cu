@@ -179,10 +179,7 @@ gemm_small_kernel(const SmallArgs a)
             if (DIRECT && CB == 16 && ipos + CH <= end) {
                 const uint8_t* s = row_codes + ((size_t)(unsigned)ipos * B + lane * CB);
 #pragma unroll
-                for (int q = 0; q < NC; ++q) {
-                    if (CB == 16) cp_async_16_l2_64(st + copy_dst[q], s + q * 32 * CB);
-                    else cp_async_8(st + copy_dst[q], s + q * 32 * CB);
-                }
+                for (int q = 0; q < NC; ++q) cp_async_16_l2_64(st + copy_dst[q], s + q * 32 * CB);
             } else {
 #pragma unroll
                 for (int q = 0; q < NC; ++q) {

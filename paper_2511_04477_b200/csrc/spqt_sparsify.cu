@@ -2,7 +2,7 @@
 // list of the entries with |x_k| > t and its length.  Three kernels:
 //   sparsify_words_kernel (one row, n <= 65536): a lane looks after pairs of neighbouring entries; one CTA, whose warps' totals meet
 //     in shared memory, or above n = 2048 a cluster of 8 CTAs, whose warps send theirs to all of them.
-//   sparsify_kernel (one row, any n): each warp owns a contiguous segment of x, counts its active entries
+//   sparsify_kernel (one row, n above 65536, or where no cluster can be launched): each warp owns a contiguous segment of x, counts its active entries
 //     with __ballot_sync/__popc (the loads of eight groups of 32 entries in flight together), the 32 warp
 //     totals are scanned in shared memory, and each warp then writes its indices at its base offset.
 //   sparsify_rows_kernel (the small batch, n < 2^16: "active in at least one of B rows"): a cluster of 8 CTAs, which
@@ -147,11 +147,8 @@ sparsify_kernel(const __half* x, int n, float t, int32_t* idx, int32_t* count)
     const int begin = min(warp * seg, n), end = min(begin + seg, n);
 
     // Eight groups of 32 entries at a time: their loads are issued together (addresses clamped into x instead
-    // of guarded, so that nothing makes one load wait for another), then one ballot per group.  Up to 64
-    // groups per warp (n <= 65536) the lane's activity bits stay in a register for the writing phase.
+    // of guarded, so that nothing makes one load wait for another), then one ballot per group.
     const int groups = (end - begin + 31) >> 5;
-    const bool in_regs = groups <= 64;
-    unsigned long long flags = 0ull;
     int total = 0;
     for (int g0 = 0; g0 < groups; g0 += 8) {
         __half v[8];
@@ -164,7 +161,6 @@ sparsify_kernel(const __half* x, int n, float t, int32_t* idx, int32_t* count)
                 const int k = begin + (g0 + j) * 32 + lane;
                 const bool p = (k < end) && is_active(v[j], t);
                 total += __popc(__ballot_sync(0xffffffffu, p));
-                if (p) flags |= 1ull << ((g0 + j) & 63);
             }
         }
     }
@@ -182,15 +178,6 @@ sparsify_kernel(const __half* x, int n, float t, int32_t* idx, int32_t* count)
     }
     __syncthreads();
     int base = warp_base[warp];
-    if (in_regs) {
-        for (int g = 0; g < groups; ++g) {
-            const bool p = (flags >> g) & 1ull;
-            const unsigned mask = __ballot_sync(0xffffffffu, p);
-            if (p) idx[base + __popc(mask & ((1u << lane) - 1u))] = begin + g * 32 + lane;
-            base += __popc(mask);
-        }
-        return;
-    }
     for (int k0 = begin; k0 < end; k0 += 32) {
         const int k = k0 + lane;
         const bool p = k < end && is_active(__ushort_as_half((unsigned short)ld_global_u16(x + k)), t);
