@@ -381,10 +381,7 @@ gemm_small_kernel(const SmallArgs a)
     // the cluster before and after reading each other's shared memory took 0.5 to 0.9 us longer: 4096 x 14336, 8 rows dense 13.1
     // against 12.1 us, 1024 x 4096, 4 rows dense 3.8 against 3.3).
     if (S > 1) cluster_wait();           // (every CTA of the cluster runs)
-    if (tid >= groups) {
-        if (S > 1) cluster_sent();
-        return;
-    }
+    if (tid >= groups) return;
     const int b = tid / (G / 4), j = tid % (G / 4) * 4;
     float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     float z = 0.0f;
@@ -406,9 +403,8 @@ gemm_small_kernel(const SmallArgs a)
         if (owner != split) {
             const unsigned dst = smem_u32(&sm.others[split * stride + tid - groups * owner / S]);
             st_async_f32x4(cluster_map(dst, (unsigned)owner), v, cluster_map(smem_u32(&sm.arrival), (unsigned)owner));
+            return;
         }
-        cluster_sent();
-        if (owner != split) return;
         const float start = mbar_wait_cluster(&sm.arrival, 0u) ? 0.0f : __int_as_float(0x7fffffff);
         float4 sum = make_float4(start, start, start, start);
 #pragma unroll

@@ -688,9 +688,10 @@ gemv_kernel(const GemvArgs a)
         // senders wait for their stores and everybody for everybody, took 1.2 to 1.3 us from the warps' sums to y, this 0.4 to
         // 0.5 (1024 x 4096 at 50 % 4.1 -> 3.6 us, 4096 x 4096 4.8 -> 4.4, with the list 4.0 -> 3.6).
         cluster_wait();                  // (every CTA of the cluster runs)
-        if (rank != 0 && tid < G / 2) st_async_f32x2(cluster_map(smem_u32(&sm.xred[rank - 1][tid]), 0u), total[0], total[1], cluster_map(smem_u32(&sm.arrival), 0u));
-        cluster_sent();
-        if (rank != 0) return;
+        if (rank != 0) {
+            if (tid < G / 2) st_async_f32x2(cluster_map(smem_u32(&sm.xred[rank - 1][tid]), 0u), total[0], total[1], cluster_map(smem_u32(&sm.arrival), 0u));
+            return;
+        }
         if (tid < G / 2) {
             if (!mbar_wait_cluster(&sm.arrival, 0u)) {
                 atomicExch(a.status, 1u);

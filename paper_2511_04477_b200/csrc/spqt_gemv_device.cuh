@@ -42,50 +42,72 @@ __device__ __forceinline__ unsigned long long global_ns()
     return t;
 }
 
-// Bounded wait for the phase with the given parity; false when the bound
-// (wall time, so that a logic error can never hold the GPU) expires.  One try_wait
-// blocks for up to about 4 us on this GPU (with or without the time hint).  CLUSTER: what the barrier announces comes from other
-// CTAs of the cluster, and the acquire has to reach as far (left out, its scope is the CTA).
-constexpr unsigned kSuspendNs = 100000u;  // the time hint of one try_wait
+// One attempt to see the phase with the given parity, which blocks for up to about 4 us on this GPU (with or without the time hint).
+// CLUSTER: what the barrier announces comes from other CTAs of the cluster, and the acquire has to reach as far (left out, its
+// scope is the CTA).
+constexpr unsigned kSuspendNs = 100000u;  // the time hint
 template <bool CLUSTER>
-__device__ __forceinline__ bool mbar_wait_scope(uint64_t* bar, unsigned parity)
+__device__ __forceinline__ bool mbar_try(unsigned addr, unsigned parity)
+{
+    unsigned done;
+    if (CLUSTER)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done)
+            : "r"(addr), "r"(parity), "r"(kSuspendNs)
+            : "memory");
+    else
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2, %3;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done)
+            : "r"(addr), "r"(parity), "r"(kSuspendNs)
+            : "memory");
+    return done != 0u;
+}
+
+// Bounded wait for the arrivals of this CTA's threads; false when the bound (wall time, so that a logic error can never hold the
+// GPU) expires.
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity)
 {
     const unsigned addr = smem_u32(bar);
     unsigned long long t0 = 0;
     for (unsigned it = 0;; ++it) {
-        unsigned done;
-        if (CLUSTER)
-            asm volatile(
-                "{\n\t.reg .pred p;\n\t"
-                "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
-                "selp.u32 %0, 1, 0, p;\n\t}"
-                : "=r"(done)
-                : "r"(addr), "r"(parity), "r"(kSuspendNs)
-                : "memory");
-        else
-            asm volatile(
-                "{\n\t.reg .pred p;\n\t"
-                "mbarrier.try_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2, %3;\n\t"
-                "selp.u32 %0, 1, 0, p;\n\t}"
-                : "=r"(done)
-                : "r"(addr), "r"(parity), "r"(kSuspendNs)
-                : "memory");
-        if (done) return true;
+        if (mbar_try<false>(addr, parity)) return true;
         if (it == 0) t0 = global_ns();
         else if (global_ns() - t0 > kWaitNs) return false;
     }
 }
-// for arrivals of this CTA's threads
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity) { return mbar_wait_scope<false>(bar, parity); }
-// For asynchronous stores of other CTAs of the cluster, by threads that have called cluster_sent() as every thread of the cluster
-// does.  If they have not come within the bound, a CTA that left now would leave stores on their way to memory that has ended:
-// the hardware's barrier tells when all CTAs have sent theirs (no later than the kernel could end in any case: none of them waits
-// for another one before that), and then they have a second bound to arrive.  False: stores are lost.
+
+// By a thread of a cluster that sends nothing more to other CTAs and does not end at once: see mbar_wait_cluster.  Nobody waits here.
+__device__ __forceinline__ void cluster_sent() { asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory"); }
+
+// Bounded wait for the asynchronous stores of other CTAs of the cluster, once, after this thread's own.  If they have not come within
+// the bound, a CTA that left now would leave stores on their way to memory that has ended.  So the thread waits for the hardware's
+// barrier of the cluster first, which threads that have ended do not hold up; every other one has said cluster_sent() before it
+// waits for anything (here: it is the first thing done).  All stores have been sent then, and have a second bound to arrive.  False:
+// they are lost.  (Arrivals of the threads that end after sending as well: 1 to 2 % of a small call, 1024 x 4096 3.66 -> 3.71 us.)
 __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, unsigned parity)
 {
-    if (mbar_wait_scope<true>(bar, parity)) return true;
-    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-    return mbar_wait_scope<true>(bar, parity);
+    cluster_sent();
+    const unsigned addr = smem_u32(bar);
+    unsigned long long t0 = 0;
+    bool late = false;
+#pragma unroll 1
+    while (!mbar_try<true>(addr, parity)) {
+        if (t0 == 0) {
+            t0 = global_ns();
+        } else if (global_ns() - t0 > kWaitNs) {
+            if (late) return false;
+            asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+            late = true;
+            t0 = 0;
+        }
+    }
+    return true;
 }
 
 // ---- asynchronous copies
@@ -206,12 +228,6 @@ __device__ __forceinline__ void cluster_wait()
 {
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// By every thread of the cluster, once, between the stores that it sends to other CTAs, if any, and its wait for theirs, if any (see
-// mbar_wait_cluster; nobody waits here).
-__device__ __forceinline__ void cluster_sent()
-{
-    asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
-}
 // address of the same shared-memory location in the CTA of the given rank
 __device__ __forceinline__ unsigned cluster_map(unsigned smem_addr, unsigned rank)
 {
@@ -240,7 +256,7 @@ __device__ __forceinline__ void st_async_f32(unsigned addr, float v, unsigned ba
 }
 
 // The length that the index collection gives a list whose places it could not find (totals of its warps were lost, see
-// mbar_wait_cluster; the warps concerned write no entry).  The products take a negative length for an empty list and give
+// mbar_wait_cluster).  The products take a negative length for an empty list and give
 // not-a-number.
 constexpr int kListLost = -1;
 __device__ __forceinline__ float not_a_number_if(bool lost, float v) { return lost ? __int_as_float(0x7fffffff) : v; }

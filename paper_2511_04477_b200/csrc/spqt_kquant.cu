@@ -559,10 +559,13 @@ kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* x, cons
         // the other CTAs send their sums to the first one's shared memory, which counts the bytes and adds them in CTA order (see
         // gemv_kernel; 8192 x 8192 to 6 bits dense 17.1 -> 16.5 us)
         cluster_wait();                  // (every CTA of the cluster runs)
-        if (rank != 0 && tid < kKqG) st_async_f32(cluster_map(smem_u32(xred + (rank - 1u) * kKqG + tid), 0u), total, cluster_map(smem_u32(&sm.arrival), 0u));
-        cluster_sent();
-        if (rank != 0) return;
-        if (tid < kKqG) {
+        if (rank != 0) {
+            if (tid < kKqG) st_async_f32(cluster_map(smem_u32(xred + (rank - 1u) * kKqG + tid), 0u), total, cluster_map(smem_u32(&sm.arrival), 0u));
+            return;
+        }
+        if (tid >= kKqG) {
+            cluster_sent();              // (there are barriers of the CTA to come)
+        } else {
             if (!mbar_wait_cluster(&sm.arrival, 0u)) total = __int_as_float(0x7fffffff);
 #pragma unroll
             for (unsigned q = 0; q < kKqMaxCluster - 1; ++q)

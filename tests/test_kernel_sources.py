@@ -55,27 +55,33 @@ def test_no_launch_has_less_shared_memory_than_the_kernel_may_assume():
 
 
 def test_a_cta_whose_bounded_wait_ran_out_stays_until_the_others_have_sent():
-    """Every thread says that it has sent before any waits, a late wait is for that first and then for the data, and nobody
-    takes an answer for granted."""
+    """The wait arrives at the cluster's barrier first, a late one is for that barrier and then for the data; a thread that sends
+    waits afterwards or ends; and nobody takes an answer for granted."""
     helpers = code(os.path.join(ROOT, "paper_2511_04477_b200", "csrc", "spqt_gemv_device.cuh"))
     body = helpers[helpers.index("bool mbar_wait_cluster("):]
     body = body[:body.index("\n}")]
-    assert re.search(r"mbar_wait_scope<true>.*barrier\.cluster\.wait.*mbar_wait_scope<true>", body, flags=re.S)
+    assert re.search(r"cluster_sent\(\);.*while \(!mbar_try<true>.*> kWaitNs.*if \(late\) return false;.*barrier\.cluster\.wait.*late = true;", body, flags=re.S)
     for path in SOURCES:
         text = code(path)
         if not path.endswith(".cu") or "st_async_" not in text:
             continue
-        for wait in re.finditer(r"mbar_wait_cluster\(", text):
-            before = text[:wait.start()]
-            assert before.rindex("cluster_sent();") > before.rindex("st_async_"), path
-            assert re.search(r"[!=,(]\s*$", before), (path, "an answer that nobody looks at")
+        sends = [m.start() for m in re.finditer(r"\bst_async_\w+\(", text)]
+        waits = [m.start() for m in re.finditer(r"\bmbar_wait_cluster\(", text)]
+        assert len(sends) == len(waits) == 1 and sends[0] < waits[0], path
+        between = text[sends[0]:waits[0]]
+        assert not re.search(r"__sync|cluster_wait\(", between), (path, "a wait for something else in between")
+        assert re.search(r"[!=,(]\s*$", text[:waits[0]]), (path, "an answer that nobody looks at")
+        behind = text[waits[0]:text.index("__global__", waits[0])] if "__global__" in text[waits[0]:] else text[waits[0]:]
+        if "__syncthreads" in behind:    # those that do not wait for stores but go on
+            assert re.search(r"if \(tid >= \w+\) \{\s*cluster_sent\(\);\s*\} else \{", between), path
 
 
 def test_a_list_without_a_length_is_no_list():
     """The index collection leaves no length where totals were lost, and the products that take a list look for that."""
     csrc = os.path.join(ROOT, "paper_2511_04477_b200", "csrc")
     collect = code(os.path.join(csrc, "spqt_sparsify.cu"))
-    assert len(re.findall(r"there \? all : kListLost", collect)) == collect.count("totals.exchange(") == len(re.findall(r"if \(!there\) return;", collect))
+    assert re.search(r"if \(!there\) \*count = kListLost;.*\*count = all < kNone \? \(int\)all : kListLost;", collect, flags=re.S)
+    assert collect.count("totals.exchange(") == len(re.findall(r"totals\.exchange\([^;]*, count\);", collect)) == 2
     for name in ("spqt_gemv.cu", "spqt_kquant.cu", "spqt_gemm_small.cu"):
         text = code(os.path.join(csrc, name))
         reads = len(re.findall(r"ld_global_u32\((?:a\.count|count_ptr)\)", text))
