@@ -149,6 +149,7 @@ struct GemvArgs {
     const unsigned* meta;       // (scale, zero) pairs
     int n, R;
     int splits;                 // slices of the list
+    int together;               // whether a cluster's CTAs leave together (see cluster_leave_together)
     unsigned magic_s;           // floor((2^32 - 1) / splits)
     unsigned warps, magic_w;    // pieces: warps of the grid, floor((2^32 - 1) / warps)
     unsigned magic_r, magic_p;  // the same of R and of the number of CTAs
@@ -694,6 +695,7 @@ gemv_kernel(const GemvArgs a)
         cluster_wait();                  // (every CTA of the cluster runs)
         if (rank != 0) {
             if (tid < G / 2) st_async_f32x2(cluster_map(smem_u32(&sm.xred[rank - 1][tid]), 0u), total[0], total[1], cluster_map(smem_u32(&sm.arrival), 0u));
+            if (a.together) cluster_leave_together();
             return;
         }
         if (tid < G / 2) {
@@ -1123,11 +1125,14 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
         // which the device holds 56: 11.1 us against 8.3 on 4 and 8.1 on 2; 64-row groups 3328 x 8192 on 5 20 % slower than on 4,
         // at 6656 x 8192 not; 11776 x 8192 on 3, of 93: 13.0 against 10.1 on 1; 4096 x 4096 on 4, of 33: no loss).  Less
         // where there is much to do (4608 x 28672 on 7, of 37, 15.0 us, 16.0 on 6, dense 14.6 / 16.3; at n = 8192 on 7 up to 10 %
-        // slower; but 7168 x 14336 on 5, of 56, 16.0 us against 11.4 on 4, 11776 x 14336 on 3, of 93, 19.7 against 16.4 on 2).
+        // slower; but 7168 x 14336 on 5, of 56, 16.0 us against 11.4 on 4).  Three with two per SM go to 95 %, lists of a long x to 97 (of
+        // 93, dense n = 8192 on 88 / 90 / 92 10.0 / 11.6 / 14.4 us where one CTA or pieces take 11.6; n = 14336 16.3 / 16.9 / 21.6, pieces 16.6
+        // to 17.2; with the list 10.9 / 12.0 / 15.4, 13.3 on 1).
         auto resident = [&](int k, bool per_sm) {
             const int most = max_clusters<G, BITS, MODE>(k, per_sm ? kAlone : kSmem, per_sm, sms, dev);
             const long long weights = (long long)G * f.n;   // of a block-row
             if ((k & (k - 1)) == 0) return f.R < most;
+            if (!per_sm && k == 3 && 100 * f.R > (weights >= 1300000 && MODE != kModeDense ? 97 : 95) * most) return false;
             if (!per_sm && weights >= 1300000) return 50 * f.R <= 49 * most;
             return per_sm || weights >= 180000ll * k ? 25 * f.R <= 24 * most : 11 * f.R <= 10 * most;
         };
@@ -1205,6 +1210,7 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
     ga.n = f.n;
     ga.R = f.R;
     ga.splits = S;
+    ga.together = cluster && 100 * f.R > 91 * max_clusters<G, BITS, MODE>(S, alone ? kAlone : kSmem, alone, sms, dev);
     ga.magic_s = 0xffffffffu / (unsigned)S;
     ga.warps = (unsigned)warps;
     ga.magic_w = 0xffffffffu / ga.warps;

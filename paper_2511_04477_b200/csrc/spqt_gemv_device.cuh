@@ -110,6 +110,14 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, unsigned parity
     return true;
 }
 
+// By every thread of a CTA that has sent and is done: it leaves when the CTA that waits for the stores is about to, not before (its
+// wait arrives at the same barrier).  A cluster whose CTAs leave one by one leaves places that the next launch's clusters do not fit.
+__device__ __forceinline__ void cluster_leave_together()
+{
+    cluster_sent();
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+
 // ---- asynchronous copies
 __device__ __forceinline__ void cp_async_16(unsigned smem_dst, const void* gmem_src)
 {

@@ -321,7 +321,7 @@ __host__ __device__ constexpr float kq_unit(int bits, int blk, int o)
 template <int BITS, bool LIST, int NW>
 __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1)
 kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* x, const int32_t* idx,
-               const int32_t* count_ptr, __half* y, int splits, int clusters, unsigned* arrived, float* partial)
+               const int32_t* count_ptr, __half* y, int splits, int clusters, int together, unsigned* arrived, float* partial)
 {
     constexpr int REC = kq_rec_bytes(BITS), NCB = kq_code_bytes(BITS), PPR = REC / 16, CH = kKqChunk, D = kq_depth(BITS);
     constexpr int kPieces = CH * PPR, NC = (kPieces + 31) / 32;
@@ -561,6 +561,7 @@ kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* x, cons
         cluster_wait();                  // (every CTA of the cluster runs)
         if (rank != 0) {
             if (tid < kKqG) st_async_f32(cluster_map(smem_u32(xred + (rank - 1u) * kKqG + tid), 0u), total, cluster_map(smem_u32(&sm.arrival), 0u));
+            if (together) cluster_leave_together();
             return;
         }
         if (tid >= kKqG) {
@@ -667,12 +668,15 @@ static spqt_status kq_launch_mode(const void* records, int R, int n, const void*
     // half as many CTAs again (the sums of a block-row then meet in global memory, 1.5 us: dense 1024 x 28672 to 8 bits, 31 MB,
     // 21.0 us on 32 CTAs of 8 warps, 12.0 on 128 of 16; at n = 8192 clusters of 8 are 8 to 16 % faster, at 14336 8 to 22 % slower).
     // Powers of two with an SM for each CTA fit neighbouring SMs without (18944 x 8192 to 6 bits dense 34.7 us on 3, 25.7 on 2, of
-    // which the device holds 74); with two per SM, five and seven take 8 %, three
-    // where there is little to do (13312 x 4096 dense 14.2 on 5, of 56, 10.8 on 4; 22528 x 2048 dense 12.0 on 3, of 93, 10.5 on 1).
+    // which the device holds 74); with two per SM, and the CTAs of a cluster leaving together, odd ones take most of what the device holds
+    // (of 56 clusters of five, 6 bits dense n = 2560 on 52 / 53 / 54 9.4 / 9.8 / 10.4 us, 10.5 on 4; 4 bits 7.3 / 8.3 / 9.4, 7.7 on 4; n = 14336
+    // 6 bits 35.8 / 36.0 / 37.2, 42.5 on 4; 36 of 37 of seven n = 8192 12.3, 13.1 on 6; of 93 of three n = 2048 dense on 88 / 90 9.0 / 9.9, 10.3
+    // on 1, with the list 7.65 / 8.75, 8.3 on 1; n = 8192 dense on 90 25.2, 31.5 on 1).
     auto resident = [&](int k, bool per_sm) {
         const int most = kq_max_clusters<BITS, LIST, 8>(k, per_sm ? kAlone : kSmem, per_sm, sms, dev);
         if (per_sm && (k & (k - 1)) == 0) return R <= most;
-        if (!per_sm && (k & 1) != 0 && 100 * R > 92 * most && (k > 3 || n < 4096)) return false;
+        const int percent = k == 7 ? 98 : k == 5 ? (n < 8192 ? 93 : 95) : (n < 4096 ? 95 : 97);
+        if (!per_sm && (k & 1) != 0 && 100 * R > percent * most) return false;
         return k * (most - R) >= 4;
     };
     int one = 1, two = 1, T = 1;         // CTAs per block-row with one and with two CTAs per SM
@@ -695,6 +699,8 @@ static spqt_status kq_launch_mode(const void* records, int R, int n, const void*
             wide = true;
         }
     }
+    // (see cluster_leave_together)
+    const int together = !wide && S > 1 && 100 * R > 91 * kq_max_clusters<BITS, LIST, 8>(S, alone ? kAlone : kSmem, alone, sms, dev);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)S * (unsigned)T * (unsigned)R);
     cfg.blockDim = dim3(wide ? 512 : 256);
@@ -711,7 +717,7 @@ static spqt_status kq_launch_mode(const void* records, int R, int n, const void*
     cfg.numAttrs = (g_no_pdl ? 0 : 1) + (S > 1 ? 1 : 0);
     auto kernel = wide ? kq_gemv_kernel<BITS, LIST, 16> : kq_gemv_kernel<BITS, LIST, 8>;
     const cudaError_t err = cudaLaunchKernelEx(&cfg, kernel, static_cast<const uint8_t*>(records), n, static_cast<const __half*>(x), idx, count,
-                                               static_cast<__half*>(y), S, T, static_cast<unsigned*>(workspace),
+                                               static_cast<__half*>(y), S, T, together, static_cast<unsigned*>(workspace),
                                                reinterpret_cast<float*>(static_cast<char*>(workspace) + kq_header_bytes(R)));
     count_launch();
     return (err == cudaSuccess && cudaGetLastError() == cudaSuccess) ? SPQT_OK : SPQT_ERR_CUDA;

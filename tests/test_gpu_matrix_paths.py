@@ -441,3 +441,37 @@ def test_recorded_step_keeps_the_order_of_linears_with_a_buffer_in_common(shared
             if i != 4 or shared != "idx":
                 assert torch.equal(h.idx[:int(cnt)], idx[:int(cnt)]), i
             assert int(h.workspace.count_nonzero()) == 0
+
+
+@pytest.mark.parametrize("bits,group,m_blocks,n", [(4, 128, 88, 8200), (3, 128, 53, 14337), (4, 64, 36, 14336), (3, 64, 25, 4099), (4, 128, 24, 4096)])
+def test_clusters_that_leave_together(bits, group, m_blocks, n):
+    """Clusters that nearly fill the device, calls behind one another."""
+    p, codes, s, z = random_matrix(bits, group, m_blocks, n)
+    m, ws = p.m, binding.new_workspace(p.m, n, bits, group)
+    x = growing_activations(n, seed=98)
+    t = inputs.threshold_for_sparsity(x, 0.5)
+    y, idx, cnt = binding.spqt_sparsify_gemv(p, dev(x), t, ws)
+    ref_idx, ref_cnt = oracle.sparsify(x, t)
+    assert int(cnt.item()) == ref_cnt and np.array_equal(idx.cpu().numpy()[:ref_cnt], ref_idx)
+    y_dense = binding.spqt_dense_gemv(p, dev(x), ws)
+    check_y(y.cpu().numpy(), *oracle.sparse_gemv(codes, s, z, m, n, x, ref_idx, bits, group), "list collected")
+    check_y(y_dense.cpu().numpy(), *oracle.dense_gemv(codes, s, z, m, n, x, bits, group), "dense")
+    for _ in range(20):
+        assert torch.equal(binding.spqt_sparse_gemv(p, dev(x), idx, cnt, ws), y) and torch.equal(binding.spqt_dense_gemv(p, dev(x), ws), y_dense)
+    assert binding.spqt_workspace_status(ws, m, group) == 0 and int(ws.count_nonzero()) == 0
+
+
+@pytest.mark.parametrize("bits,m_blocks,n", [(4, 53, 8192), (8, 36, 4100), (6, 90, 4097), (2, 88, 1537), (5, 52, 2560)])
+def test_two_level_clusters_that_leave_together(bits, m_blocks, n):
+    m = 256 * m_blocks
+    W = inputs.weights(m, n, seed=m + n)
+    p, parts = binding.spqt_kqw_pack(dev(W), bits), oracle.kq_quantize(W, bits=bits)
+    x, ws = growing_activations(n, seed=99), binding.new_kq_workspace(p)
+    idx, cnt = binding.spqt_sparsify(dev(x), 0.5)
+    ref_idx, _ = oracle.sparsify(x, 0.5)
+    rows = np.unique(np.concatenate([np.arange(0, m, 97), np.arange(256), np.arange(m - 256, m)]))
+    y, y_dense = binding.spqt_kqw_sparse_gemv(p, dev(x), idx, cnt, ws), binding.spqt_kqw_dense_gemv(p, dev(x), ws)
+    check_y(y.cpu().numpy()[rows], *oracle.kq_gemv(*parts, x, ref_idx, rows=rows), "list")
+    check_y(y_dense.cpu().numpy()[rows], *oracle.kq_gemv(*parts, x, rows=rows), "dense")
+    for _ in range(20):
+        assert torch.equal(binding.spqt_kqw_sparse_gemv(p, dev(x), idx, cnt, ws), y) and torch.equal(binding.spqt_kqw_dense_gemv(p, dev(x), ws), y_dense)
