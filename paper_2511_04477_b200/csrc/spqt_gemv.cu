@@ -149,7 +149,6 @@ struct GemvArgs {
     const unsigned* meta;       // (scale, zero) pairs
     int n, R;
     int splits;                 // slices of the list
-    int together;               // whether a cluster's CTAs leave together (see cluster_leave_together)
     unsigned magic_s;           // floor((2^32 - 1) / splits)
     unsigned warps, magic_w;    // pieces: warps of the grid, floor((2^32 - 1) / warps)
     unsigned magic_r, magic_p;  // the same of R and of the number of CTAs
@@ -164,6 +163,8 @@ struct GemvArgs {
     int32_t* count_out;
     int static_partition;
     int small;                  // the matrix is small beside L2
+    int together;               // whether a cluster's CTAs leave together (see cluster_leave_together; the last member: before the
+                                // others it moved some that every call needs to another line, 0.05 us a call)
 };
 
 // floor(v / d) for any 32-bit v from the multiplier m = floor((2^32 - 1) / d): the high product is
@@ -1121,7 +1122,8 @@ static spqt_status launch_gemv(const Format& f, const void* codes, const void* m
         }
     } else {
         // "all resident" with a margin: the previous launch's CTAs leave SM by SM, and the CTAs of a cluster need places on
-        // neighbouring SMs at the same time, in odd numbers above all, and the less there is to do the more (7168 x 8192 on 5, of
+        // neighbouring SMs at the same time, in odd numbers above all, and the less there is to do the more (figures up to the last two
+        // lines from before clusters that nearly fill the device left together, which the lines still hold for; 7168 x 8192 on 5, of
         // which the device holds 56: 11.1 us against 8.3 on 4 and 8.1 on 2; 64-row groups 3328 x 8192 on 5 20 % slower than on 4,
         // at 6656 x 8192 not; 11776 x 8192 on 3, of 93: 13.0 against 10.1 on 1; 4096 x 4096 on 4, of 33: no loss).  Less
         // where there is much to do (4608 x 28672 on 7, of 37, 15.0 us, 16.0 on 6, dense 14.6 / 16.3; at n = 8192 on 7 up to 10 %

@@ -21,7 +21,7 @@
 //                    four.  Sums: warps through shared memory, CTAs through the cluster's, in a fixed order.
 //                    What bounds it: the integer pipe in the loop (masks, shifts: 53 to 61 % busy over the whole call), the fixed
 //                    cost of the call and of the list's launch before it, then latency: 12 to 16 warps per SM with 2 to 5
-//                    chunks in flight each.  28672 x 4096 to 4 bits at 50 %, list included, takes 14.2 us (19.4 with packed
+//                    chunks in flight each.  28672 x 4096 to 4 bits at 50 %, list included, takes 13.8 us (19.4 with packed
 //                    FMAs, partial sums in global memory and chunks dealt in turn), 8192 x 8192 to 6 bits dense 14.3 us (20.4;
 //                    55 MB), 28672 x 8192 to 4 bits dense 31.1 us.
 //                    A multiplier x*(d*sc) is rounded to fp32 and goes in as two fp16 values, off by 2^-26 of the warp's
@@ -321,7 +321,7 @@ __host__ __device__ constexpr float kq_unit(int bits, int blk, int o)
 template <int BITS, bool LIST, int NW>
 __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1)
 kq_gemv_kernel(const uint8_t* __restrict__ records, int n, const __half* x, const int32_t* idx,
-               const int32_t* count_ptr, __half* y, int splits, int clusters, int together, unsigned* arrived, float* partial)
+               const int32_t* count_ptr, __half* y, int splits, int clusters, unsigned* arrived, float* partial, int together)
 {
     constexpr int REC = kq_rec_bytes(BITS), NCB = kq_code_bytes(BITS), PPR = REC / 16, CH = kKqChunk, D = kq_depth(BITS);
     constexpr int kPieces = CH * PPR, NC = (kPieces + 31) / 32;
@@ -717,8 +717,8 @@ static spqt_status kq_launch_mode(const void* records, int R, int n, const void*
     cfg.numAttrs = (g_no_pdl ? 0 : 1) + (S > 1 ? 1 : 0);
     auto kernel = wide ? kq_gemv_kernel<BITS, LIST, 16> : kq_gemv_kernel<BITS, LIST, 8>;
     const cudaError_t err = cudaLaunchKernelEx(&cfg, kernel, static_cast<const uint8_t*>(records), n, static_cast<const __half*>(x), idx, count,
-                                               static_cast<__half*>(y), S, T, together, static_cast<unsigned*>(workspace),
-                                               reinterpret_cast<float*>(static_cast<char*>(workspace) + kq_header_bytes(R)));
+                                               static_cast<__half*>(y), S, T, static_cast<unsigned*>(workspace),
+                                               reinterpret_cast<float*>(static_cast<char*>(workspace) + kq_header_bytes(R)), together);
     count_launch();
     return (err == cudaSuccess && cudaGetLastError() == cudaSuccess) ? SPQT_OK : SPQT_ERR_CUDA;
 }
