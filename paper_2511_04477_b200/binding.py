@@ -511,8 +511,8 @@ def _status_word(rc: int, out: ctypes.c_int, where: str) -> int:
 
 
 def spqt_workspace_status(workspace: torch.Tensor, m: int, group: int = 128, stream=None) -> int:
-    """The workspace's status word: 0, 1 (a bounded on-chip wait expired in a GEMV that used this workspace)
-    or 2 (checked mode refused an index list).  Synchronises."""
+    """The workspace's status word: 0, 1 (a bounded on-chip wait expired in a GEMV that used this workspace, or its
+    list had a negative length) or 2 (checked mode refused an index list).  Synchronises."""
     out = ctypes.c_int(-1)
     rc = lib().spqt_workspace_status(_dev(workspace, torch.uint8, "workspace"), m, group,
                                      ctypes.byref(out), _stream(stream))

@@ -10,7 +10,7 @@
 //                           (spqt_mma.cuh), which take the codes as they are.  At the end the warps' sums meet in
 //                           shared memory and are sent to the CTA that finishes them, which adds them in a fixed order.
 //
-// What bounds it: instruction issue around the code stream (270 warp instructions per chunk), then the fixed cost of a
+// What bounds it: instruction issue around the code stream (240 to 280 warp instructions per chunk, 400 with five to eight rows), then the fixed cost of a
 // launch.  The batch is the N = 8 side of the matrix instructions, so the instruction count hardly grows with the
 // rows (the packed-FMA form before it paid 64 FMAs per chunk and row and two passes from five rows up).
 #include <cstddef>

@@ -176,9 +176,9 @@ struct PackTile {
 // W with rows of 16-byte pieces (W on a 16-byte boundary, ldw a multiple of 8).  A persistent warp takes tiles of 64 rows per
 // lane: 128 rows x 32 columns, or 64 x 64, 8 KB.  While a tile is converted, from registers, the next one comes by cp.async
 // into the shared memory that it left: 160 KB in flight per SM, and half the instructions of loads by the lane, whose addresses
-// take more than the loads (22 instructions for two weights, now 19).  Bound by memory: 28672 x 8192 to 4 bits, 595 MB, in
-// 105 us = 5.7 TB/s, where loads by the lane, in phases with the rest, took 125 us (and 345 us with an IEEE division per weight);
-// from 8 M weights on 5 to 20 % faster, below that the same.
+// take more than the loads (22 instructions for two weights, now 19).  Bound by memory: 28672 x 8192 to 4 bits, 595 MB, alone in
+// 105 us = 5.7 TB/s, where loads by the lane, in phases with the rest, took 125 us (and 345 us with an IEEE division per weight); one
+// call after the other for longer, under the power limit, 121 and 132 us; from 8 M weights on 5 to 20 % faster, below that the same.
 constexpr int kTileCtas = 5;             // per SM
 template <int G, int BITS>
 __global__ void __launch_bounds__(kPackThreads, kTileCtas)
