@@ -155,7 +155,7 @@ sparsify_kernel(const __half* x, int n, float t, int32_t* idx, int32_t* count)
         auto load = [&](int k) { return __ushort_as_half((unsigned short)ld_global_u16(x + min(k + lane, n - 1))); };
         auto vote = [&](int k, __half v) { each(k, __ballot_sync(0xffffffffu, k + lane < end && is_active(v, t))); };
         int k = begin;
-        for (; k + 256 <= end; k += 256) {
+        for (; end - k >= 256; k += 256) {
             __half v[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) v[j] = load(k + 32 * j);
